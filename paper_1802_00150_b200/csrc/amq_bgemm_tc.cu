@@ -222,6 +222,17 @@ __device__ __forceinline__ void mma_i8_stage(uint32_t d_tmem, uint32_t a_lo, uin
         :: "r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(acc_first) : "memory");
 }
 
+// true in one lane of the (converged) warp.  The issuing warp runs its loop as a whole and only the tensor-core instructions are
+// under this predicate: their operands then stay in uniform registers.  With the loop inside `if (lane == 0)` the compiler moved
+// every operand of every MMA into them one by one, and a pipeline step of four MMAs cost the issuing thread 676 clocks whatever
+// its N; this way it costs 230-300 (N <= 128: below the pace of the tensor pipe from N = 128 up).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t one;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(one));
+    return one != 0;
+}
+
 __device__ __forceinline__ void mma_commit(uint32_t bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(bar) : "memory");
@@ -796,8 +807,10 @@ bgemm_tc_kernel(TcParams p)
             *coef_dst = coef_val;
             if (has_corr) sBcorr[(r_all - MT * TILE_M) / KA] = -(float)p.pad * corr_sum;
         }
-    } else if (lane == 0) {
-        // ---- MMA issuer ----
+    } else {
+        // ---- MMA issuer (whole warp; one elected lane issues) ----
+        const bool issues = elect_one();
+        const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
         // instruction descriptor: int8 (s32 accumulators, signed 8-bit operands), or block-scaled E2M1 (operand format 1,
         // scale format E8M0); N >> 3 at bit 17, M >> 4 at bit 24, both operands K-major
         const uint32_t idesc = fp4 ? ((1u << 7) | (1u << 10) | ((uint32_t)(n_mma >> 3) << 17) | (1u << 23) | ((uint32_t)(TILE_M >> 4) << 24))
@@ -813,6 +826,7 @@ bgemm_tc_kernel(TcParams p)
             const uint64_t adesc0 = desc_base + (uint64_t)((buf * stage_bytes) >> 4);
             const uint64_t bdesc0 = adesc0 + (uint64_t)(a_stage_bytes >> 4);
             const int word0 = c * step_words;
+            if (issues) {
             if (fp4 || word0 >= split_word || word0 + step_words <= split_word) {
                 // the whole stage lies in one column segment (always in the 4-bit form; else unless a GRU's input width is
                 // not a multiple of 128)
@@ -845,9 +859,11 @@ bgemm_tc_kernel(TcParams p)
                 }
             }
             mma_commit(smem_u32(&empty_bar[buf]));
+            }
+            __syncwarp();
             if (++buf == S) { buf = 0; full_parity ^= 1u; }
         }
-        if (!*failed) mma_commit(smem_u32(done_bar));               // covers every MMA issued above
+        if (issues && !*failed) mma_commit(smem_u32(done_bar));               // covers every MMA issued above
     }
     __syncwarp();
 
@@ -1041,8 +1057,10 @@ bgemm_tc_persistent_kernel(TcParams p)
             if (buf >= S) { buf -= S; empty_parity ^= 1u; }
         }
     } else if (warp == mma_warp) {
-        if (lane == 0) {
-            // ---- MMA issuer ----
+        {
+            // ---- MMA issuer (whole warp; one elected lane issues) ----
+            const bool issues = elect_one();
+            const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
             const uint32_t idesc = fp4 ? ((1u << 7) | (1u << 10) | ((uint32_t)(n_mma >> 3) << 17) | (1u << 23) | ((uint32_t)(TILE_M >> 4) << 24))
                                        : ((2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n_mma >> 3) << 17) | ((uint32_t)(TILE_M >> 4) << 24));
             const uint64_t desc_base = smem_desc(smem_u32(stage_base));
@@ -1064,6 +1082,7 @@ bgemm_tc_persistent_kernel(TcParams p)
                     const uint64_t adesc0 = desc_base + (uint64_t)((buf * stage_bytes) >> 4);
                     const uint64_t bdesc0 = adesc0 + (uint64_t)(a_stage_bytes >> 4);
                     const int word0 = c * step_words;
+                    if (issues) {
                     if (fp4 || word0 >= split_word || word0 + step_words <= split_word) {
                         const int seg = word0 >= split_word ? 1 : 0;
                         const uint32_t acc_first = (word0 != 0 && word0 != split_word) ? 1u : 0u;
@@ -1094,9 +1113,11 @@ bgemm_tc_persistent_kernel(TcParams p)
                         }
                     }
                     mma_commit(smem_u32(&empty_bar[buf]));
+                    }
+                    __syncwarp();
                     if (++buf == S) { buf = 0; full_parity ^= 1u; }
                 }
-                if (ok) mma_commit(smem_u32(&tfull_bar[ab]));       // covers every MMA of the tile
+                if (ok && issues) mma_commit(smem_u32(&tfull_bar[ab]));       // covers every MMA of the tile
             }
             if (!ok) *failed = 1;
         }
