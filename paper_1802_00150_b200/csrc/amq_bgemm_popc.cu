@@ -204,6 +204,7 @@ bgemm_popc_kernel(PopcParams p)
 amq_status launch_binary_gemm(const GemmArgs& a, cudaStream_t st)
 {
     if (gemv_supported(a)) return launch_binary_gemv(a, st);
+    if (gemm_resident_supported(a)) return launch_binary_gemm_resident(a, st);
     if (gemm_tc_supported(a)) return launch_binary_gemm_tc(a, st);
     PopcParams p;
     p.a = a;

@@ -1,0 +1,283 @@
+// Batched binary product (Sec. 4, Fig. 3 right; y = sum_i sum_j alpha_i beta_j D_ij + bias) with a resident activation operand
+// (amq_resident.cuh).  One CTA per SM; the work is the list of (block of vectors, tile of 128 weight rows) pairs, dealt out in
+// equal contiguous shares, so that a CTA expands the activation operand once or twice and streams weight tiles past it.
+//
+// What bounds it: the pace of the pipeline steps (240-265 clocks per 256 bit positions of 128 plane-rows) times the number of
+// blocks the batch is cut into; outputs leave as 128-byte stores of consecutive rows from registers.
+#include "amq_resident.cuh"
+
+namespace amq {
+
+namespace {
+
+struct ResGemmParams {
+    ResProblem p;
+    const uint32_t* xcodes; const float* xbeta; const float* bias;
+    float* y; int ldy;
+    int mtiles, blocks;         // tiles of 128 rows, blocks of TB vectors
+    int b_bytes;                // expanded activation operand
+    int vec_out;                // rows of y start on 16 bytes
+    uint32_t* status;           // set when a bounded wait ran out
+};
+
+// Row stride of the results staged for the stores: 8 mod 32 words for two vectors (conflict-free in the m16n8 layout), 16-byte rows.
+constexpr int Y_LD = 132;
+// groups of eight vectors per epilogue thread: TB <= 64, or 32 (registers)
+__host__ __device__ constexpr int res_ng(int k_a) { return k_a <= 2 ? 2 : 1; }
+
+template <int KA>
+__global__ void __launch_bounds__(RES_THREADS, 1)
+bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
+{
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    const ResProblem& p = a.p;
+    constexpr int NG = res_ng(KA);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    float* sBeta = reinterpret_cast<float*>(smem_raw + a.b_bytes);                  // [256] per operand row
+    float* sRow = sBeta + 256;                                                      // [3][256]
+    int* sSum = reinterpret_cast<int*>(sRow + 3 * 256);                             // [2][256]
+    float* sAlpha = reinterpret_cast<float*>(sSum + 2 * 256);                       // [2][k_w][128]
+    uint32_t* table = reinterpret_cast<uint32_t*>(sAlpha + 2 * AMQ_MAX_K * 128);
+    float* sY = reinterpret_cast<float*>(table + RES_TABLE);                        // [TB][Y_LD] results of a tile
+    ResSync& sy = *reinterpret_cast<ResSync*>(sY + p.TB * Y_LD);
+    const uint32_t sB = smem_u32(smem_raw);
+
+    // this CTA's share of the (block, tile) list; a pass is the part of it that lies in one block of vectors
+    const long long total = (long long)a.blocks * a.mtiles;
+    long long w = total * blockIdx.x / gridDim.x;
+    const long long w_end = total * (blockIdx.x + 1) / gridDim.x;
+    auto pass_tiles = [&](long long at) {
+        const int tile0 = (int)(at % a.mtiles);
+        return (int)(w_end - at < a.mtiles - tile0 ? w_end - at : a.mtiles - tile0);
+    };
+
+    if (tid == 0) res_sync_init(sy);
+    if (warp == RES_MMA_WARP) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     :: "r"(smem_u32(&sy.tmem_slot)), "r"((uint32_t)RES_TMEM_COLS) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = __shfl_sync(0xffffffffu, sy.tmem_slot, 0);
+    if (warp < 4) res_write_scales(p, tmem, warp);
+
+    for (int q = tid; q < 512; q += RES_THREADS) sSum[q] = 0;
+    res_fill_table(p, table);
+    __syncthreads();
+
+    // expand the activations of block bb; all threads, ends with a CTA barrier
+    auto load_block = [&](int bb) {
+        const int b0 = bb * p.TB;
+        for (int q = tid; q < p.N; q += RES_THREADS) {
+            const int b = b0 + res_row_vector<KA>(q), j = res_row_plane<KA>(q);
+            sBeta[q] = q < p.TB * KA && b < p.batch ? __ldcg(a.xbeta + (size_t)b * KA + j) : 0.0f;
+        }
+        res_expand_activations<KA>(p, a.xcodes, b0, sB, sSum);
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    };
+    // Every role runs its own loop over the passes (the registers of one role are then not held through another's code); a pass
+    // ends with a barrier, after which every MMA that read the operand has completed (the epilogue has waited for all
+    // accumulators), so the operand may be overwritten.
+    bool ok = true;
+    if (warp < RES_EXP_WARPS) {
+        const int r = (warp & 3) * 32 + lane, steps_per_tile = p.k_w * ((p.NS + 1) >> 1);
+        int first_step = 0;                         // pipeline steps so far, mod the number of groups
+        ResFeedState fs{warp >> 2, 1u};
+        ResFeeder<RES_PLAIN> feed;
+        auto start = [&](long long at) {
+            feed.start(p, table, (int)(at % a.mtiles), 1, pass_tiles(at), r, ((warp >> 2) - first_step + RES_GROUPS) % RES_GROUPS);
+        };
+        if (w < w_end) start(w);                    // (weights: no kernel of a chain writes them)
+        grid_dependency_wait();                     // the planes and coefficients may come from the preceding kernel
+        while (w < w_end) {
+            load_block((int)(w / a.mtiles));
+            ok = res_feed(p, sy, table, feed, tmem, fs);
+            const int tiles = pass_tiles(w);
+            w += tiles;
+            first_step = (int)((first_step + (long long)tiles * steps_per_tile) % RES_GROUPS);
+            if (w < w_end) start(w);
+            if (__syncthreads_or(!ok)) { ok = false; break; }
+        }
+    } else if (warp == RES_MMA_WARP) {
+        ResIssueState issue{0, 0, 0, 1};
+        grid_dependency_wait();
+        while (w < w_end) {
+            load_block((int)(w / a.mtiles));
+            const int tiles = pass_tiles(w);
+            ok = res_issue(p, sy, tiles, tmem, sB, issue);
+            w += tiles;
+            if (__syncthreads_or(!ok)) { ok = false; break; }
+        }
+    } else if (warp < RES_MMA_WARP) {
+        const int te = tid - 32 * RES_EXP_WARPS, quarter = warp & 3, sub = (warp - RES_EXP_WARPS) >> 2, rl = quarter * 32 + (lane >> 2);
+        ResDrainState drain{0, 0};
+        ResColumns<KA, NG> col;
+        uint32_t y_parity = 1;
+        // coefficients of a tile's rows: thread te takes one of the 128 k_w, a tile ahead
+        auto alpha_of = [&](int tile) {
+            const int row = tile * 128 + (te & 127), plane = te >> 7;
+            return plane < p.k_w && row < p.units ? __ldg(p.Walpha + (size_t)row * p.k_w + plane) : 0.0f;
+        };
+        grid_dependency_wait();
+        while (w < w_end) {
+            const int bb = (int)(w / a.mtiles), tile0 = (int)(w % a.mtiles), tiles = pass_tiles(w);
+            float next_alpha = alpha_of(tile0);
+            load_block(bb);
+            res_row_constants(p, sSum, sRow);
+            for (int t = 0; t < tiles; ++t) {
+                float* sa = sAlpha + (t & 1) * AMQ_MAX_K * 128;
+                sa[te] = next_alpha;
+                if (res_epi_bar(!ok)) { ok = false; break; }        // (also: everybody is past the tile before last, whose buffer this is)
+                if (t == 0) { col.load(p, sBeta, sub, col.beta); col.load(p, sRow, sub, col.row); }
+                if (t + 1 < tiles) next_alpha = alpha_of(tile0 + t + 1);
+                f32x2 y[NG][4];
+                ok = res_drain_tile<KA, NG>(p, sy, sa, quarter, sub, tmem, col, drain, y);
+                // Results leave through shared memory and three warps of their own: in this layout a store from the registers is four
+                // 32-byte pieces, and stores from the epilogue warps held them up for longer than a tile's MMAs take.
+                ok = ok && res_group_wait(sy, smem_u32(&sy.yempty), y_parity, warp == RES_EXP_WARPS, 1, 32 * RES_EPI_WARPS);
+                y_parity ^= 1u;
+#pragma unroll
+                for (int g = 0; g < NG; ++g) {
+                    const int e = (RES_EPI_SPLIT * g + sub) * 8 + 2 * (lane & 3);
+                    if (e >= p.TB) break;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        float y0, y1;
+                        unpack2(y[g][i], y0, y1);
+                        sY[e * Y_LD + rl + 8 * i] = y0;
+                        sY[(e + 1) * Y_LD + rl + 8 * i] = y1;
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(&sy.yfull)) : "memory");
+            }
+            w += tiles;
+            if (__syncthreads_or(!ok)) { ok = false; break; }
+        }
+    } else {
+        uint32_t y_parity = 0;
+        while (w < w_end) {
+            const int bb = (int)(w / a.mtiles), tile0 = (int)(w % a.mtiles), b0 = bb * p.TB, tiles = pass_tiles(w);
+            grid_dependency_wait();
+            load_block(bb);
+            const int last = p.batch - b0 < p.TB ? p.batch - b0 : p.TB;
+            for (int t = 0; t < tiles && ok; ++t) {
+                const int row = (tile0 + t) * 128 + 4 * lane;
+                float4 bias = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                if (a.bias) {
+                    if (row < p.units) bias.x = __ldg(a.bias + row);
+                    if (row + 1 < p.units) bias.y = __ldg(a.bias + row + 1);
+                    if (row + 2 < p.units) bias.z = __ldg(a.bias + row + 2);
+                    if (row + 3 < p.units) bias.w = __ldg(a.bias + row + 3);
+                }
+                ok = __all_sync(0xffffffffu, mbar_wait_relaxed(smem_u32(&sy.yfull), y_parity, &sy.failed));
+                y_parity ^= 1u;
+                if (!ok) { *(volatile int*)&sy.failed = 1; break; }
+                const bool vec = a.vec_out && row + 3 < p.units;
+#pragma unroll 4
+                for (int e = warp - RES_MMA_WARP - 1; e < last; e += RES_OUT_WARPS) {
+                    float4 v = *reinterpret_cast<const float4*>(sY + e * Y_LD + 4 * lane);
+                    v.x += bias.x; v.y += bias.y; v.z += bias.z; v.w += bias.w;
+                    float* out = a.y + (size_t)(b0 + e) * a.ldy + row;
+                    if (vec) {
+                        *reinterpret_cast<float4*>(out) = v;
+                    } else {
+                        if (row < p.units) out[0] = v.x;
+                        if (row + 1 < p.units) out[1] = v.y;
+                        if (row + 2 < p.units) out[2] = v.z;
+                        if (row + 3 < p.units) out[3] = v.w;
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(&sy.yempty)) : "memory");
+            }
+            w += tiles;
+            if (__syncthreads_or(!ok)) { ok = false; break; }
+        }
+    }
+    __syncwarp();
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (!ok) {      // (uniform) give the tensor core time to drain before tensor memory is released
+        if (tid == 0) atomicExch(a.status, 1u);
+        __nanosleep(1000000);
+        __syncthreads();
+    }
+    if (warp == RES_MMA_WARP)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"((uint32_t)RES_TMEM_COLS) : "memory");
+}
+
+struct ResGemmPlan { ResGemmParams a; int grid; size_t smem; };
+
+bool plan(const GemmArgs& g, ResGemmPlan* out)
+{
+    if (g.epilogue != EPI_Y) return false;
+    const int sms = res_sm_count();
+    ResGemmParams a{};
+    ResProblem& p = a.p;
+    p.W = g.Wcodes; p.Walpha = g.Walpha; p.k_w = g.k_w; p.wpr = words_per_row(g.n);
+    p.vec32 = p.wpr % 8 == 0 && (reinterpret_cast<uintptr_t>(g.Wcodes) & 31) == 0;
+    p.cell = RES_PLAIN; p.units = g.m; p.ut = 128; p.tpu = 1;
+    p.n = g.n; p.NS = (g.n + 255) / 256; p.batch = g.batch;
+    a.mtiles = (g.m + 127) / 128;
+    // block of vectors: the size with the least estimated time (shares of tiles x steps, plus the expansion of the operand,
+    // which a share pays at least once); sizes whose operand does not fit shared memory are out (n > 28000 or so: none fits)
+    double best = 0.0;
+    for (int TB = 8; TB <= 8 * res_ng(g.k_a) * RES_EPI_SPLIT; TB += 8) {
+        ResProblem q = p;
+        if (!res_set_block(q, TB, g.k_a, (size_t)TB * Y_LD * 4)) break;
+        const long long blocks = (g.batch + TB - 1) / TB, per_cta = (blocks * a.mtiles + sms - 1) / sms;
+        const double expand = (double)q.N * q.NS * 128 / 80.0 + 1500.0;
+        const double t = (double)per_cta * q.k_w * q.NS * res_slot_clocks(q) + expand * (1.0 + (double)per_cta / a.mtiles);
+        if (best == 0.0 || t < best) { best = t; a.p = q; a.blocks = (int)blocks; }
+        if (TB >= g.batch) break;
+    }
+    if (best == 0.0) return false;
+    a.b_bytes = a.p.NS * a.p.N * 128;
+    a.xcodes = g.xcodes; a.xbeta = g.xbeta; a.bias = g.bias; a.y = g.y; a.ldy = g.ldy;
+    const long long total = (long long)a.blocks * a.mtiles;
+    out->grid = (int)(total < sms ? total : sms);
+    out->smem = res_smem_bytes(a.p, g.k_a) + (size_t)a.p.TB * Y_LD * 4;
+    a.vec_out = (reinterpret_cast<uintptr_t>(g.y) & 15) == 0 && g.ldy % 4 == 0;
+    out->a = a;
+    return true;
+}
+
+template <int KA>
+amq_status launch(const ResGemmPlan& pl, bool overlap, cudaStream_t st)
+{
+    auto kernel = bgemm_resident_kernel<KA>;
+    AMQ_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem));
+    AMQ_CUDA_TRY(launch_kernel(kernel, dim3((unsigned)pl.grid), dim3(RES_THREADS), pl.smem, st, overlap, pl.a));
+    AMQ_LAUNCH_CHECK();
+    return AMQ_OK;
+}
+
+}  // namespace
+
+bool gemm_resident_supported(const GemmArgs& g)
+{
+    ResGemmPlan pl;
+    return g.batch >= 2 && plan(g, &pl);
+}
+
+amq_status launch_binary_gemm_resident(const GemmArgs& g, cudaStream_t st)
+{
+    ResGemmPlan pl;
+    if (!plan(g, &pl)) return AMQ_ERR_UNSUPPORTED;
+    amq_status s = tc_status_word(&pl.a.status);
+    if (s != AMQ_OK) return s;
+    switch (g.k_a) {
+        case 1: return launch<1>(pl, g.overlap_with_previous, st);
+        case 2: return launch<2>(pl, g.overlap_with_previous, st);
+        case 3: return launch<3>(pl, g.overlap_with_previous, st);
+        case 4: return launch<4>(pl, g.overlap_with_previous, st);
+    }
+    return AMQ_ERR_UNSUPPORTED;
+}
+
+}  // namespace amq

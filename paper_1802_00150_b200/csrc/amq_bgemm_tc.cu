@@ -43,6 +43,7 @@
 // loop of the next).  Both may be launched as programmatic dependents of the kernel that produces the
 // activation planes: they set themselves up and fetch weight rows, then wait for it.
 #include "amq_common.cuh"
+#include "amq_tcgen05.cuh"
 
 namespace amq {
 
@@ -52,7 +53,6 @@ constexpr int MAX_THREADS = 1024;           // expander threads (one or two per 
 constexpr int TILE_M = 128;                 // stacked weight plane-rows per M tile (= TMEM lanes)
 constexpr int STAGE_WORDS = 4;              // packed words of K per pipeline stage (128 bit positions)
 constexpr int MAX_STAGES = 4;
-constexpr unsigned WAIT_LIMIT = 1u << 20;   // attempts on an mbarrier before giving up
 
 __device__ uint32_t g_tc_status;            // nonzero after a bounded wait ran out (sticky until read)
 __device__ uint32_t g_tc_status_taken;      // what the last read found
@@ -101,55 +101,6 @@ struct TcParams {
 // read it entry by entry with unit-strided rows and keep the odd stride.
 __host__ __device__ __forceinline__ int staging_stride(int TB, int epilogue) { return epilogue == EPI_Y ? TB + 4 : TB + 1; }
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(bar), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
-{
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.b32 %0, 1, 0, p;\n\t}"
-        : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-    return done != 0;
-}
-
-// bounded wait of the single MMA-issuing thread; false when it ran out
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
-{
-    for (unsigned i = 0; i < WAIT_LIMIT; ++i)
-        if (mbar_try_wait(bar, parity)) return true;
-    return false;
-}
-
-// the same for the many expander threads: between attempts the thread sleeps, so that waiters do not take
-// issue slots from the warps that have work
-__device__ __forceinline__ bool mbar_wait_relaxed(uint32_t bar, uint32_t parity)
-{
-    if (mbar_try_wait(bar, parity)) return true;
-    for (unsigned i = 0; i < WAIT_LIMIT; ++i) {
-        __nanosleep(40);
-        if (mbar_try_wait(bar, parity)) return true;
-    }
-    return false;
-}
-
-// the same, giving up early once another role of the CTA has recorded a failure
-__device__ __forceinline__ bool mbar_wait_relaxed(uint32_t bar, uint32_t parity, volatile int* failed)
-{
-    if (mbar_try_wait(bar, parity)) return true;
-    for (unsigned i = 0; i < WAIT_LIMIT && !*failed; ++i) {
-        __nanosleep(40);
-        if (mbar_try_wait(bar, parity)) return true;
-    }
-    return false;
-}
-
 // barrier 1 joins the epilogue warps only (barrier 0 is the CTA-wide one)
 __device__ __forceinline__ void epi_bar(int nthreads)
 {
@@ -167,13 +118,6 @@ __device__ __forceinline__ bool epi_bar_or(int nthreads, bool flag)
         "selp.b32 %0, 1, 0, q;\n\t}"
         : "=r"(out) : "r"((uint32_t)flag), "r"(nthreads) : "memory");
     return out != 0;
-}
-
-// K-major, 128-byte swizzle: start address (the tile base is 1024-byte aligned), leading byte offset unused (1),
-// stride byte offset = 1024 bytes between groups of 8 rows, descriptor version 1, layout type 2
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr)
-{
-    return (uint64_t)((addr >> 4) & 0x3fffu) | (1ull << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
 }
 
 __device__ __forceinline__ void mma_i8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
@@ -220,35 +164,6 @@ __device__ __forceinline__ void mma_i8_stage(uint32_t d_tmem, uint32_t a_lo, uin
         "tcgen05.mma.cta_group::1.kind::i8 [%0], da, db, %4, q;\n\t"
         "}"
         :: "r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(acc_first) : "memory");
-}
-
-// true in one lane of the (converged) warp.  The issuing warp runs its loop as a whole and only the tensor-core instructions are
-// under this predicate: their operands then stay in uniform registers.  With the loop inside `if (lane == 0)` the compiler moved
-// every operand of every MMA into them one by one, and a pipeline step of four MMAs cost the issuing thread 676 clocks whatever
-// its N; this way it costs 230-300 (N <= 128: below the pace of the tensor pipe from N = 128 up).
-__device__ __forceinline__ bool elect_one()
-{
-    uint32_t one;
-    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(one));
-    return one != 0;
-}
-
-__device__ __forceinline__ void mma_commit(uint32_t bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(bar) : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, int (&v)[8])
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-        : "r"(taddr) : "memory");
-}
-
-__device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t x, uint32_t y, uint32_t z, uint32_t w)
-{
-    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" :: "r"(addr), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
 }
 
 // (x & a) ^ b in one three-input logic instruction
@@ -354,35 +269,6 @@ __device__ __forceinline__ void mma_mxf4_stage(uint32_t d_tmem, uint32_t a_lo, u
         :: "r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(acc_first), "r"(sf_tmem) : "memory");
 }
 
-// The same with the weight operand in tensor memory (lanes 0..127, 8 columns = 64 nibbles per MMA).
-__device__ __forceinline__ void mma_mxf4_stage_ta(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc,
-                                                  uint32_t acc_first, uint32_t sf_tmem)
-{
-    asm volatile(
-        "{\n\t"
-        ".reg .pred p, q;\n\t"
-        ".reg .b64 db;\n\t"
-        ".reg .b32 al, bl;\n\t"
-        "setp.ne.b32 p, %5, 0;\n\t"
-        "setp.eq.b32 q, %5, %5;\n\t"
-        "mov.b64 db, {%2, %3};\n\t"
-        "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.block32 [%0], [%1], db, %4, [%6], [%6], p;\n\t"
-        "add.u32 al, %1, 8;\n\t"
-        "add.u32 bl, %2, 2;\n\t"
-        "mov.b64 db, {bl, %3};\n\t"
-        "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.block32 [%0], [al], db, %4, [%6], [%6], q;\n\t"
-        "add.u32 al, %1, 16;\n\t"
-        "add.u32 bl, %2, 4;\n\t"
-        "mov.b64 db, {bl, %3};\n\t"
-        "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.block32 [%0], [al], db, %4, [%6], [%6], q;\n\t"
-        "add.u32 al, %1, 24;\n\t"
-        "add.u32 bl, %2, 6;\n\t"
-        "mov.b64 db, {bl, %3};\n\t"
-        "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.block32 [%0], [al], db, %4, [%6], [%6], q;\n\t"
-        "}"
-        :: "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(acc_first), "r"(sf_tmem) : "memory");
-}
-
 // 4-bit form, weight operand in tensor memory: one 128-bit chunk of a packed row -> 16 columns of the thread's lane, in
 // the word order of the shared-memory row (word 4 q + s keeps bits s, s + 4, .. of packed word q).  Warp-collective.
 __device__ __forceinline__ void expand_chunk_fp4_tmem(uint32_t taddr, const uint4& v)
@@ -402,26 +288,11 @@ __device__ __forceinline__ void expand_chunk_fp4_tmem(uint32_t taddr, const uint
            "r"(y[8]), "r"(y[9]), "r"(y[10]), "r"(y[11]), "r"(y[12]), "r"(y[13]), "r"(y[14]), "r"(y[15]) : "memory");
 }
 
-// Scale factors of the 4-bit form: 16 tensor-memory columns, every byte 0x7F (2^0 in E8M0), written by four warps (one per
-// lane quarter); both operands' scale addresses point at this region, whose every byte is the same.
-__device__ __forceinline__ void write_unit_scales(uint32_t tmem_base, int sf_col, int warp)
-{
-    const uint32_t t = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)sf_col;
-    const uint32_t one = 0x7F7F7F7Fu;
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1};"
-        :: "r"(t), "r"(one) : "memory");
-    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-
 // an accumulator as the epilogue reads it from tensor memory -> the exact integer dot product (pad positions included)
 __device__ __forceinline__ float acc_to_float(int acc, bool fp4)
 {
     return fp4 ? __int_as_float(acc) : small_int_to_float(acc >> 12);
 }
-
-__device__ __forceinline__ float logistic(float v) { return 1.0f / (1.0f + __expf(-v)); }
 
 // x / d for x >= 0 and the small divisors that occur in the row bookkeeping (bits per weight 1..4; gates 1, 3, 4): inside the
 // switch the divisor is a constant, so each case is a shift or one multiplication instead of the generic division sequence
@@ -1414,6 +1285,14 @@ amq_status launch_binary_gemm_tc(const GemmArgs& a, cudaStream_t st)
 __global__ void take_tc_status_kernel()
 {
     g_tc_status_taken = atomicExch(&g_tc_status, 0u);
+}
+
+amq_status tc_status_word(uint32_t** word)
+{
+    void* p = nullptr;
+    AMQ_CUDA_TRY(cudaGetSymbolAddress(&p, g_tc_status));
+    *word = static_cast<uint32_t*>(p);
+    return AMQ_OK;
 }
 
 amq_status read_tc_status(cudaStream_t st, uint32_t* out)

@@ -153,6 +153,11 @@ amq_status launch_quantized_gemv(const uint32_t* Wcodes, const float* Walpha, in
 bool gemm_tc_supported(const GemmArgs& a);
 amq_status launch_binary_gemm_tc(const GemmArgs& a, cudaStream_t st);
 amq_status read_tc_status(cudaStream_t st, uint32_t* out);
+amq_status tc_status_word(uint32_t** word);       // device address of the status word, for kernels of other files
+
+// Tensor-core product with a resident activation operand (EPI_Y): whether it covers a problem, and its launch.
+bool gemm_resident_supported(const GemmArgs& a);
+amq_status launch_binary_gemm_resident(const GemmArgs& a, cudaStream_t st);
 
 // Persistent batch-1 recurrent kernel: whether it covers a problem (sizes, shared memory), and its launch.
 bool persistent_supported(int I, int H, int batch, int k_w, int k_a, bool gru, int* grid_out, int* upc_out,

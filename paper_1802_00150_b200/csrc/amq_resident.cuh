@@ -1,0 +1,541 @@
+// Tensor-core product with a RESIDENT activation operand: the pieces shared by the batched product (amq_bgemm_resident.cu) and
+// the batched sequence kernel (amq_rnn_batched.cu).
+//
+// A CTA owns a block of TB activation vectors.  Their k_a planes are expanded ONCE, over the whole length of the vectors, into
+// E2M1 nibbles in shared memory (N rows of n / 2 bytes, row (g, j, e) = plane j of vector 8 g + e; positions past the end of a
+// vector hold zero nibbles, which add nothing to a dot product), and stay there while packed weight rows stream past: expander warps turn 512 bit positions of
+// 128 plane-rows per pipeline step into tensor memory, one warp issues the MMAs (kind::mxf4, unit block scales, M = 128), and
+// epilogue warps fold finished accumulators.  Against expanding both operands stage by stage this takes the activation
+// operand's shared-memory stores (40-60 % of a stage's, repeated for every weight tile) out of the main loop.
+//
+// The k_w planes of a tile of 128 weight rows are k_w accumulators one after the other in a ring, not neighbouring lanes of one
+// accumulator: a lane of tensor memory IS a weight row, so an epilogue thread adds up the planes of its row in registers
+// and lanes store consecutive rows.  (The former layout, k_w plane-rows side by side, needed a pass through shared memory per
+// tile that took longer than the tile's MMAs.)
+//
+// Nibbles.  Output word s of a packed word keeps its bits s, s + 4, .., s + 28.  With bit 1 = -1 on both operands (a dot
+// product of +-1 vectors does not see the common sign), a weight bit needs no shift at all: nibble 0x1, 0x2 or 0x4 for s = 0, 1,
+// 2 is {0, 0.5}, {0, 1} or {0, 2}, which the block scales 4, 2, 1 (32 elements of one s) make {0, 2}; for s = 3 the bit is the
+// sign of 1.0.  The activation operand is b = +-1 for s = 3 and -b for s < 3, so the accumulator is the +-1 dot product minus
+// sum_{s < 3} b, a constant of the operand row that the epilogue adds back before anything is rounded.  Four logic
+// operations per packed word instead of seven: the expanders share the issue slots with the epilogue.
+//
+// Along K the vector is cut into slots of 256 positions (128 bytes of every expanded row, 128-byte swizzle: eight rows per 1024
+// bytes).  For the GRU, whose candidate keeps the columns [0, I) and [I, n) apart, the slot that holds column I exists twice,
+// once with only the x columns and once with only the h columns, so any I works and the x part is slots [0, nx), the h part
+// [nx, NS); a full product runs over all of them.
+//
+// Pace, measured in isolation (one CTA per SM): 240 clocks per slot at N <= 96, 265 at N = 128 (256 is the tensor pipe's own
+// time), bound by the issue and synchronisation of the steps below N = 96 (an MMA takes 46 clocks however small N is).
+#pragma once
+
+#include "amq_common.cuh"
+#include "amq_tcgen05.cuh"
+
+namespace amq {
+
+constexpr int RES_GROUPS = 3;                       // groups of four expander warps, which take the slots in turn
+constexpr int RES_EXP_WARPS = 4 * RES_GROUPS;       // warps 0 .. 11
+constexpr int RES_EPI_WARPS = 16;                   // warps 12 .. 27: lane quarter = warp mod 4, four warps per quarter
+constexpr int RES_EPI_SPLIT = RES_EPI_WARPS / 4;    // warps that share a quarter: groups of eight vectors in turn
+constexpr int RES_MMA_WARP = RES_EXP_WARPS + RES_EPI_WARPS;        // warp 28
+constexpr int RES_OUT_WARPS = 3;                    // warps 29 .. 31: a plain product's stores
+constexpr int RES_THREADS = 1024;
+constexpr int RES_STAGE_COLS = 64;                  // tensor-memory columns of a stage: two slots of the weight operand
+constexpr int RES_MAX_STAGES = 4;
+constexpr int RES_MAX_RING = 2;                     // accumulator buffers
+constexpr int RES_TMEM_COLS = 512;
+constexpr int RES_ROW_BYTES = (256 + 3 * 256 + 2 * 256) * 4;    // per operand row: coefficient, constants as fp32, as they are summed up
+constexpr int RES_ALPHA_BYTES = 2 * AMQ_MAX_K * 128 * 4;         // weight coefficients of a tile, double-buffered
+constexpr int RES_SMEM_LIMIT = 225 * 1024;
+
+enum ResCell { RES_PLAIN = 0, RES_LSTM = 1, RES_GRU = 2 };
+
+struct ResProblem {
+    const uint32_t* W; const float* Walpha; int k_w, wpr;
+    int vec32;          // every plane-row is whole 32-byte pieces (256-bit loads)
+    int cell;           // ResCell
+    int units;          // rows of a plain product, hidden units of a cell
+    int ut;             // units per block: 128 (lane = unit; a cell's gates are four tiles one after the other), or 32 (a
+                        // cell only: lane quarter = gate)
+    int tpu;            // tiles per block of units: 1, or 4
+    int n, I;           // vector length; first column of the h part (GRU)
+    int NS, nx, xw;     // slots; slots of the x part (0: no split); whole x slots before the doubled one
+    int TB, N, ring;    // activation vectors per CTA, operand rows (TB * k_a rounded up to 16), accumulator buffers
+    int stages;         // weight-operand stages in tensor memory
+    int batch;
+};
+
+// gate order of the four tiles of a 128-unit block, chosen so that an epilogue thread keeps one value per (unit, vector) alive:
+// LSTM i, g, f, o; GRU r, nh, nx, z
+__device__ __forceinline__ int res_gate_of_tile(int cell, int tt)
+{
+    return cell == RES_LSTM ? (tt == 0 ? 0 : tt == 1 ? 3 : tt == 2 ? 1 : 2) : (tt == 0 ? 0 : tt == 3 ? 1 : 2);
+}
+
+__device__ __forceinline__ void res_tile_slots(const ResProblem& p, int tt, int& s0, int& s1)
+{
+    s0 = 0; s1 = p.NS;
+    if (p.cell == RES_GRU && p.tpu == 4) {
+        if (tt == 1) s0 = p.nx;
+        if (tt == 2) s1 = p.nx;
+    }
+}
+
+__device__ __forceinline__ int res_slot_word(const ResProblem& p, int s) { return 8 * (s < p.nx ? s : p.xw + s - p.nx); }
+
+// weight row of lane r of tile tt of unit block ub; -1: none
+__device__ __forceinline__ int res_row(const ResProblem& p, int ub, int tt, int r)
+{
+    if (p.ut == 32) {
+        const int u = ub * 32 + (r & 31), q = r >> 5;
+        return u < p.units ? ((p.cell == RES_GRU && q == 3) ? 2 : q) * p.units + u : -1;
+    }
+    const int u = ub * 128 + r;
+    if (u >= p.units) return -1;
+    return p.cell == RES_PLAIN ? u : res_gate_of_tile(p.cell, tt) * p.units + u;
+}
+
+// Synchronisation block in shared memory.
+struct ResSync {
+    uint64_t full[RES_MAX_STAGES], empty[RES_MAX_STAGES];           // stage filled / read by the MMAs
+    uint64_t tfull[RES_MAX_RING], tempty[RES_MAX_RING];     // accumulator complete / read out
+    uint64_t yfull, yempty;                                 // results of a tile staged / stored (plain product)
+    uint32_t tmem_slot;
+    int failed;                                             // a bounded wait ran out
+};
+
+__device__ __forceinline__ void res_sync_init(ResSync& sy)
+{
+    for (int g = 0; g < RES_MAX_STAGES; ++g) { mbar_init(smem_u32(&sy.full[g]), 4); mbar_init(smem_u32(&sy.empty[g]), 1); }
+    for (int q = 0; q < RES_MAX_RING; ++q) { mbar_init(smem_u32(&sy.tfull[q]), 1); mbar_init(smem_u32(&sy.tempty[q]), RES_EPI_WARPS); }
+    mbar_init(smem_u32(&sy.yfull), RES_EPI_WARPS); mbar_init(smem_u32(&sy.yempty), RES_OUT_WARPS);
+    sy.failed = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+
+// barrier of `threads` threads; true when `bad` is true in any of them
+__device__ __forceinline__ bool res_bar(int id, int threads, bool bad)
+{
+    uint32_t out;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\tbar.red.or.pred q, %2, %3, p;\n\tselp.b32 %0, 1, 0, q;\n\t}"
+        : "=r"(out) : "r"((uint32_t)bad), "r"(id), "r"(threads) : "memory");
+    return out != 0;
+}
+__device__ __forceinline__ bool res_epi_bar(bool bad) { return res_bar(1, 32 * RES_EPI_WARPS, bad); }
+
+// Wait of a whole group of warps on one mbarrier: one warp polls, the others wait at a hardware barrier.  (With every warp polling,
+// the polls alone took half of the SM's issue slots and the synchronisation of a slot, without any work in it, 370 clocks.)
+__device__ __forceinline__ bool res_group_wait(ResSync& sy, uint32_t bar, uint32_t parity, bool polls, int id, int threads)
+{
+    bool ok = true;
+    if (polls) {
+        ok = mbar_wait(bar, parity);
+        if (!ok) *(volatile int*)&sy.failed = 1;
+    }
+    return !res_bar(id, threads, !ok);
+}
+
+// ---- activation operand ---------------------------------------------------------------------------------------------------
+
+// 256 bit positions of one packed row -> the 128 nibble bytes of operand row `row` in one slot.  `lo`, `hi`: valid element range.
+// Returns sum of b over the valid positions with s < 3 (bit 1 = -1).
+__device__ __forceinline__ int res_expand_row(uint32_t slot_addr, int row, const uint32_t (&w)[8], int first, int lo, int hi)
+{
+    const uint32_t base = slot_addr + (uint32_t)row * 128u;
+    int sum = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        uint32_t vm[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int e = first + 32 * (4 * h + q);
+            vm[q] = 0xffffffffu;
+            if (lo > e) vm[q] = lo - e >= 32 ? 0u : vm[q] << (lo - e);
+            if (hi < e + 32) vm[q] = hi <= e ? 0u : vm[q] & (0xffffffffu >> (e + 32 - hi));
+            const uint32_t m3 = vm[q] & 0x77777777u;
+            sum += __popc(m3) - 2 * __popc(w[4 * h + q] & m3);
+        }
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            uint32_t y[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t sign = (w[4 * h + q] << (3 - s)) & 0x88888888u;                          // nibble i: bit 4 i + s
+                y[q] = (s < 3 ? sign ^ 0xAAAAAAAAu : sign | 0x22222222u) & (((vm[q] >> s) & 0x11111111u) * 15u);
+            }
+            st_shared_v4(base + (uint32_t)(((4 * h + s) ^ (row & 7)) << 4), y[0], y[1], y[2], y[3]);
+        }
+    }
+    return sum;
+}
+
+// operand row -> (vector of the block, plane): rows of a group of eight vectors are plane-major
+template <int KA> __device__ __forceinline__ int res_row_vector(int row) { return row / (8 * KA) * 8 + (row & 7); }
+template <int KA> __device__ __forceinline__ int res_row_plane(int row) { return row / 8 % KA; }
+
+// Expand the planes of vectors b0 .. b0 + TB - 1 (all threads of the CTA; rows past the batch are zero nibbles), add up the
+// constants of the rows (sSum[part][row], zeroed by the caller; part 1: the h part of a GRU's split).  The caller makes the stores
+// visible to the MMAs: every thread executes the proxy fence at the end, then a CTA barrier.
+template <int KA>
+__device__ __forceinline__ void res_expand_activations(const ResProblem& p, const uint32_t* xcodes, int b0, uint32_t sB, int* sSum)
+{
+    const int N = p.N;
+    int row = (int)threadIdx.x % N, slot = (int)threadIdx.x / N;
+    const int drow = (int)blockDim.x % N, dslot = (int)blockDim.x / N;
+    while (slot < p.NS) {
+        const int b = b0 + res_row_vector<KA>(row), j = res_row_plane<KA>(row);
+        const int w0 = res_slot_word(p, slot);
+        const bool in_x = slot < p.nx;
+        uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        const bool live = row < p.TB * KA && b < p.batch;
+        if (live) {
+            const uint4* src = reinterpret_cast<const uint4*>(xcodes + ((size_t)b * KA + j) * p.wpr + w0);
+            const uint4 v0 = __ldcg(src);               // (other SMs wrote the planes: not through the read-only path)
+            w[0] = v0.x; w[1] = v0.y; w[2] = v0.z; w[3] = v0.w;
+            if (w0 + 4 < p.wpr) { const uint4 v1 = __ldcg(src + 1); w[4] = v1.x; w[5] = v1.y; w[6] = v1.z; w[7] = v1.w; }
+        }
+        const int lo = (p.nx > 0 && !in_x) ? p.I : 0, hi = !live ? 0 : (in_x ? p.I : p.n);
+        const int sum = res_expand_row(sB + (uint32_t)(slot * N * 128), row, w, w0 * 32, live ? lo : 0, hi);
+        if (live) atomicAdd(&sSum[(p.nx > 0 && !in_x ? 256 : 0) + row], sum);
+        row += drow; slot += dslot;
+        if (row >= N) { row -= N; ++slot; }
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+
+// Epilogue warps, after the barrier that completes sSum: the constants as fp32, sRow[0] of the whole vector, and of the x and the h
+// part, sRow[1], sRow[2], where the columns are split; clears sSum for the next block.
+__device__ __forceinline__ void res_row_constants(const ResProblem& p, int* sSum, float* sRow)
+{
+    for (int i = (int)threadIdx.x - 32 * RES_EXP_WARPS; i < p.N; i += 32 * RES_EPI_WARPS) {
+        const int x = sSum[i], h = p.nx > 0 ? sSum[256 + i] : 0;
+        sSum[i] = 0; sSum[256 + i] = 0;
+        sRow[i] = (float)(x + h);
+        if (p.nx > 0) { sRow[256 + i] = (float)x; sRow[512 + i] = (float)h; }
+    }
+}
+
+// ---- weight operand -------------------------------------------------------------------------------------------------------
+
+// The steps of a tile (two consecutive slots of one plane each) as a table in shared memory, two words per step: word offset in
+// the row's planes, bit 29: no such slot, bit 30: the slot has only 16 bytes of the row, bit 31: it belongs to the h part of a split.
+constexpr int RES_KIND = AMQ_MAX_K * 34;            // entries of one kind of tile: AMQ_MAX_N / 256 + 1 slots, in pairs
+constexpr int RES_TABLE = 4 * RES_KIND;             // up to four kinds (a GRU block of 128 units)
+constexpr uint32_t RES_STEP_NONE = 1u << 29, RES_STEP_HALF = 1u << 30, RES_STEP_H = 1u << 31;
+
+__device__ __forceinline__ int res_tile_steps(const ResProblem& p, int tt)
+{
+    int s0, s1;
+    res_tile_slots(p, tt, s0, s1);
+    return p.k_w * ((s1 - s0 + 1) >> 1);
+}
+
+// One group's share of the CTA's steps: the steps of all tiles in order are dealt to the groups in turn.  Thread = plane-row.  The
+// packed words of a step are fetched one of the group's steps ahead.  (Every instruction counts here: the expander warps
+// issue about one in ten clocks beside the other roles, and a group has three steps' time, some 1500 clocks, per step.)
+template <int CELL>
+struct ResFeeder {
+    const uint32_t* row;            // plane 0 of this thread's row in the cursor's tile (a lane without a weight row takes the last one:
+                                    // its accumulators are read by nobody)
+    int i, n;                       // the cursor's step in its tile, steps of the tile
+    int it, nitems;                 // tile counter of the CTA
+    int base;                       // the tile kind's part of the table
+    int ub0, ub_step;
+    uint4 v[2][2];                  // the next step's packed words, and its table entries
+    uint2 e;
+    bool live;                      // there is a next step
+
+    __device__ __forceinline__ void tile(const ResProblem& p, int r)
+    {
+        const int ub = ub0 + (CELL != RES_PLAIN && p.tpu == 4 ? it >> 2 : it) * ub_step, tt = CELL != RES_PLAIN && p.tpu == 4 ? it & 3 : 0;
+        const int wr = CELL == RES_PLAIN ? ub * 128 + r : res_row(p, ub, tt, r);
+        row = p.W + (size_t)(wr < 0 || (CELL == RES_PLAIN && wr >= p.units) ? p.units - 1 : wr) * (p.k_w * p.wpr);
+        if (CELL == RES_GRU && p.tpu == 4) { n = res_tile_steps(p, tt); base = tt * RES_KIND; }
+    }
+    // position on the first own step of a pass over tiles ub0, ub0 + ub_step, ..; `skip` steps of other groups come first
+    __device__ __forceinline__ void start(const ResProblem& p, const uint32_t* table, int first_block, int block_step, int tiles, int r, int skip)
+    {
+        it = 0; nitems = tiles; ub0 = first_block; ub_step = block_step; base = 0;
+        n = p.k_w * ((p.NS + 1) >> 1); i = skip;
+        if (nitems > 0) tile(p, r);
+        next_tile(p, r);
+        fetch(p, table, r);
+    }
+    __device__ __forceinline__ void next_tile(const ResProblem& p, int r)
+    {
+        while (i >= n && it < nitems) {
+            i -= n;
+            if (++it < nitems) tile(p, r);
+        }
+    }
+    // whether this lane's row is zero in the slot of table entry `entry` (candidate rows of a 32-unit GRU block)
+    __device__ __forceinline__ static bool zero_row(const ResProblem& p, uint32_t entry, int r)
+    {
+        return CELL == RES_GRU && p.ut == 32 && (r >> 5) == ((entry & RES_STEP_H) ? 2 : 3);
+    }
+    // packed words of the cursor's step, and on to the group's next step
+    __device__ __forceinline__ void fetch(const ResProblem& p, const uint32_t* table, int r)
+    {
+        live = it < nitems;
+        if (!live) return;
+        e = *reinterpret_cast<const uint2*>(table + base + 2 * i);
+        const uint4* src0 = reinterpret_cast<const uint4*>(row + (e.x & (RES_STEP_NONE - 1)));
+        const uint4* src1 = reinterpret_cast<const uint4*>(row + (e.y & (RES_STEP_NONE - 1)));
+        if (p.vec32) {
+            asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                         : "=r"(v[0][0].x), "=r"(v[0][0].y), "=r"(v[0][0].z), "=r"(v[0][0].w),
+                           "=r"(v[0][1].x), "=r"(v[0][1].y), "=r"(v[0][1].z), "=r"(v[0][1].w) : "l"(src0));
+            asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                         : "=r"(v[1][0].x), "=r"(v[1][0].y), "=r"(v[1][0].z), "=r"(v[1][0].w),
+                           "=r"(v[1][1].x), "=r"(v[1][1].y), "=r"(v[1][1].z), "=r"(v[1][1].w) : "l"(src1));
+        } else {        // (a missing half keeps whatever was there: it meets zeros of the activation operand)
+            v[0][0] = __ldg(src0);
+            if (!(e.x & RES_STEP_HALF)) v[0][1] = __ldg(src0 + 1);
+            v[1][0] = __ldg(src1);
+            if (!(e.y & RES_STEP_HALF)) v[1][1] = __ldg(src1 + 1);
+        }
+        i += RES_GROUPS;
+        if (i >= n) next_tile(p, r);
+    }
+};
+
+// fill the table (all threads; a CTA barrier follows)
+__device__ __forceinline__ void res_fill_table(const ResProblem& p, uint32_t* table)
+{
+    const int kinds = p.cell == RES_GRU && p.tpu == 4 ? 4 : 1;
+    for (int tt = 0; tt < kinds; ++tt) {
+        int s0, s1;
+        res_tile_slots(p, tt, s0, s1);
+        const int per_plane = (s1 - s0 + 1) & ~1;
+        for (int q = threadIdx.x; q < p.k_w * per_plane; q += blockDim.x) {
+            const int plane = q / per_plane, s = s0 + q - plane * per_plane, w0 = res_slot_word(p, s);
+            table[tt * RES_KIND + q] = s >= s1 ? RES_STEP_NONE | RES_STEP_HALF          // (offset 0: loads what is there, used by nobody)
+                : (uint32_t)(plane * p.wpr + w0) | (w0 + 8 > p.wpr ? RES_STEP_HALF : 0u) | (p.nx > 0 && s >= p.nx ? RES_STEP_H : 0u);
+        }
+    }
+}
+
+// 256 bit positions of this lane's row -> 32 tensor-memory columns (the same order inside a slot as the activation rows)
+__device__ __forceinline__ void res_store_slot(uint32_t taddr, const uint4& a, const uint4& b, bool zero)
+{
+    const uint32_t one = zero ? 0u : 0x22222222u, keep = zero ? 0u : 0xffffffffu;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        uint32_t w[4] = {h ? b.x : a.x, h ? b.y : a.y, h ? b.z : a.z, h ? b.w : a.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) w[q] &= keep;                   // (all ones where no row can be zero: nothing is executed)
+        uint32_t y[16];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            y[q] = w[q] & 0x11111111u;
+            y[4 + q] = w[q] & 0x22222222u;
+            y[8 + q] = w[q] & 0x44444444u;
+            y[12 + q] = (w[q] & 0x88888888u) | one;
+        }
+        asm volatile(
+            "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+            :: "r"(taddr + 16 * h), "r"(y[0]), "r"(y[1]), "r"(y[2]), "r"(y[3]), "r"(y[4]), "r"(y[5]), "r"(y[6]), "r"(y[7]),
+               "r"(y[8]), "r"(y[9]), "r"(y[10]), "r"(y[11]), "r"(y[12]), "r"(y[13]), "r"(y[14]), "r"(y[15]) : "memory");
+    }
+}
+
+struct ResFeedState { int stage; uint32_t parity; };       // the group's next stage and the parity of its "empty" barrier: start {group, 1}
+
+// The expander warps' part of one pass (f has been started).  False when a wait ran out.
+template <int CELL>
+__device__ __forceinline__ bool res_feed(const ResProblem& p, ResSync& sy, const uint32_t* table, ResFeeder<CELL>& f, uint32_t tmem, ResFeedState& st)
+{
+    const int grp = (int)threadIdx.x >> 7, r = (int)threadIdx.x & 127;
+    const uint32_t taddr = tmem + ((uint32_t)(r & 96) << 16) + (uint32_t)(p.ring * p.N + 16);
+    while (f.live) {
+        if (!res_group_wait(sy, smem_u32(&sy.empty[st.stage]), st.parity, r < 32, 2 + grp, 128)) return false;
+        const uint32_t t = taddr + (uint32_t)(st.stage * RES_STAGE_COLS);
+        res_store_slot(t, f.v[0][0], f.v[0][1], f.zero_row(p, f.e.x, r));
+        if (!(f.e.y & RES_STEP_NONE)) res_store_slot(t + 32, f.v[1][0], f.v[1][1], f.zero_row(p, f.e.y, r));
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(&sy.full[st.stage])) : "memory");
+        f.fetch(p, table, r);                       // (into the registers just expanded)
+        st.stage += RES_GROUPS;
+        if (st.stage >= p.stages) { st.stage -= p.stages; st.parity ^= 1u; }
+    }
+    return true;
+}
+
+// ---- MMA issue ------------------------------------------------------------------------------------------------------------
+
+struct ResIssueState { int stage; uint32_t full_parity; int ring; uint32_t ring_parity; };      // start: {0, 0, 0, 1}
+
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
+{
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.b32 %0, 1, 0, p;\n\t}"
+        : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    return done != 0;
+}
+
+// Scale factors: eight columns of ones (both operands), eight of the pair (4, 2) for weight blocks s = 0, 1; every lane and word
+// alike.  Four warps, one per lane quarter.
+__device__ __forceinline__ void res_write_scales(const ResProblem& p, uint32_t tmem, int warp)
+{
+    const uint32_t t = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(p.ring * p.N);
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1, %2, %2, %2, %2, %2, %2, %2, %2};"
+        :: "r"(t), "r"(0x7F7F7F7Fu), "r"(0x80818081u) : "memory");
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+}
+
+// The issuing warp's part of one pass over `nitems` tiles (whole warp, one elected lane issues).
+__device__ __forceinline__ bool res_issue(const ResProblem& p, ResSync& sy, int nitems, uint32_t tmem, uint32_t sB, ResIssueState& st)
+{
+    const bool issues = elect_one();
+    const uint32_t idesc = (1u << 7) | (1u << 10) | ((uint32_t)(p.N >> 3) << 17) | (1u << 23) | (8u << 24);     // E2M1, E8M0, M 128
+    const uint64_t desc = smem_desc(sB);
+    const uint32_t lo = (uint32_t)desc, hi = (uint32_t)(desc >> 32), slot_units = (uint32_t)(p.N * 8);      // N * 128 bytes / 16
+    const uint32_t sf = tmem + (uint32_t)(p.ring * p.N), sfa = sf + 8, a0 = sf + 16;
+    const uint32_t full0 = smem_u32(&sy.full[0]), empty0 = smem_u32(&sy.empty[0]);
+    // The next step's barrier is looked at between the two halves of a step, while the MMAs of the first half are in the queue: with the
+    // look after the last MMA the tensor pipe ran dry for 250-400 clocks between steps.
+    bool ready = false;
+    for (int it = 0; it < nitems; ++it) {
+        int s0, s1;
+        res_tile_slots(p, p.tpu == 4 ? it & 3 : 0, s0, s1);
+        for (int plane = 0; plane < p.k_w; ++plane) {
+            if (!mbar_wait(smem_u32(&sy.tempty[st.ring]), st.ring_parity)) { *(volatile int*)&sy.failed = 1; return false; }
+            const uint32_t acc = tmem + (uint32_t)(st.ring * p.N);
+            uint32_t b = lo + (uint32_t)s0 * slot_units;
+            for (int s = s0; s < s1; s += 2) {
+                if (!ready && !mbar_wait(full0 + 8 * st.stage, st.full_parity)) { *(volatile int*)&sy.failed = 1; return false; }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint32_t a = a0 + (uint32_t)(st.stage * RES_STAGE_COLS), empty = empty0 + 8 * st.stage;
+                if (issues) mma_mxf4_slot(acc, a, b, hi, idesc, s != s0 ? 1u : 0u, sfa, sf);
+                if (++st.stage == p.stages) { st.stage = 0; st.full_parity ^= 1u; }
+                ready = mbar_test(full0 + 8 * st.stage, st.full_parity);
+                if (issues) {
+                    if (s + 1 < s1) mma_mxf4_slot(acc, a + 32, b + slot_units, hi, idesc, 1u, sfa, sf);
+                    mma_commit(empty);
+                }
+                b += 2 * slot_units;
+            }
+            if (issues) mma_commit(smem_u32(&sy.tfull[st.ring]));
+            __syncwarp();
+            if (++st.ring == p.ring) { st.ring = 0; st.ring_parity ^= 1u; }
+        }
+    }
+    return true;
+}
+
+// ---- accumulators ---------------------------------------------------------------------------------------------------------
+//
+// An epilogue warp reads its 32 rows in the m16n8 layout: a thread then holds, of every group of eight vectors, the two vectors
+// 2 (lane mod 4) + {0, 1} for the four rows lane / 4 + 8 i.  Its activation coefficients and row constants depend on the vectors only
+// and stay in registers for the whole pass, and two vectors share every instruction.
+
+template <int KA, int NG>
+struct ResColumns {
+    f32x2 beta[NG][KA], row[NG][KA];        // of this thread's two vectors in the groups sub, sub + 4, ..
+
+    __device__ __forceinline__ static void load(const ResProblem& p, const float* src, int sub, f32x2 (&dst)[NG][KA])
+    {
+#pragma unroll
+        for (int g = 0; g < NG; ++g)
+#pragma unroll
+            for (int j = 0; j < KA; ++j) {
+                const int gg = RES_EPI_SPLIT * g + sub;
+                dst[g][j] = gg * 8 < p.TB ? *reinterpret_cast<const f32x2*>(src + (gg * KA + j) * 8 + 2 * (threadIdx.x & 3)) : 0ull;
+            }
+    }
+};
+
+struct ResDrainState { int ring; uint32_t parity; };        // start: {0, 0}
+
+// One tile: the k_w accumulators of this warp's 32 rows, y[g][i] = sum over planes of alpha * sum_j beta_j D_j for row lane / 4 + 8 i
+// and the two vectors, D_j = accumulator + row constant (exact integers).  `sAlpha`: coefficients [plane][128] of the tile.
+template <int KA, int NG>
+__device__ __forceinline__ bool res_drain_tile(const ResProblem& p, ResSync& sy, const float* sAlpha, int quarter, int sub, uint32_t tmem,
+                                               const ResColumns<KA, NG>& col, ResDrainState& st, f32x2 (&y)[NG][4])
+{
+    const int lane = (int)threadIdx.x & 31;
+#pragma unroll
+    for (int g = 0; g < NG; ++g)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) y[g][i] = 0ull;
+#pragma unroll 1
+    for (int plane = 0; plane < p.k_w; ++plane) {
+        f32x2 al[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float v = sAlpha[plane * 128 + quarter * 32 + (lane >> 2) + 8 * i];
+            al[i] = pack2(v, v);
+        }
+        if (!res_group_wait(sy, smem_u32(&sy.tfull[st.ring]), st.parity, threadIdx.x >> 5 == RES_EXP_WARPS, 1, 32 * RES_EPI_WARPS)) return false;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(st.ring * p.N);
+#pragma unroll
+        for (int g = 0; g < NG; ++g) {
+            const int gg = RES_EPI_SPLIT * g + sub;
+            if (gg * 8 >= p.TB) break;
+            f32x2 v[4][KA];
+            tmem_ld_pairs<KA>(acc + (uint32_t)(gg * 8 * KA), v);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                f32x2 s = mul2(col.beta[g][0], add2(v[i][0], col.row[g][0]));
+#pragma unroll
+                for (int j = 1; j < KA; ++j) s = fma2(col.beta[g][j], add2(v[i][j], col.row[g][j]), s);
+                y[g][i] = fma2(al[i], s, y[g][i]);
+            }
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0)
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(&sy.tempty[st.ring])) : "memory");
+        if (++st.ring == p.ring) { st.ring = 0; st.parity ^= 1u; }
+    }
+    return true;
+}
+
+// ---- host -----------------------------------------------------------------------------------------------------------------
+
+inline int res_sm_count()
+{
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0) return v;
+    return 1;
+}
+
+// shared memory: operand, coefficients, synchronisation block, and what the caller adds behind them
+inline size_t res_smem_bytes(const ResProblem& p, int k_a)
+{
+    (void)k_a;
+    return (size_t)p.NS * p.N * 128 + RES_ROW_BYTES + RES_ALPHA_BYTES + RES_TABLE * 4 + sizeof(ResSync);
+}
+
+// block of TB vectors: operand rows and accumulator buffers; false when they fit neither tensor nor shared memory
+inline bool res_set_block(ResProblem& p, int TB, int k_a, size_t more_smem = 0)
+{
+    p.TB = TB;
+    p.N = (TB * k_a + 15) / 16 * 16;
+    if (p.N > 256 || p.NS > 33) return false;
+    // two accumulator buffers where that leaves a stage per group
+    p.ring = (RES_TMEM_COLS - 16 - 2 * p.N) / RES_STAGE_COLS >= RES_GROUPS ? 2 : 1;
+    const int stages = (RES_TMEM_COLS - 16 - p.ring * p.N) / RES_STAGE_COLS;
+    p.stages = stages < RES_MAX_STAGES ? stages : RES_MAX_STAGES;
+    return res_smem_bytes(p, k_a) + more_smem <= (size_t)RES_SMEM_LIMIT;
+}
+
+// estimated clocks per slot of 128 plane-rows (measured: 240 up to N = 96, 265 at N = 128, then the tensor pipe's own pace); with
+// one accumulator buffer the MMAs of the next plane wait while the epilogue reads the last one out
+inline double res_slot_clocks(const ResProblem& p)
+{
+    const double t = 2.0 * p.N + 10.0 > 240.0 ? 2.0 * p.N + 10.0 : 240.0;
+    return p.ring > 1 ? t : t + 600.0 / p.NS;
+}
+
+}  // namespace amq
