@@ -261,8 +261,11 @@ amq_status launch(const ResGemmPlan& pl, bool overlap, cudaStream_t st)
 
 bool gemm_resident_supported(const GemmArgs& g)
 {
+    // from 16 vectors on always; for 2..15 vectors when the weight matrix is large enough that the CUDA-core kernel's tile loop
+    // costs more than this kernel's set-up
     ResGemmPlan pl;
-    return g.batch >= 2 && plan(g, &pl);
+    const bool big = (long long)g.m * g.k_w * words_per_row(g.n) >= (1ll << 17);
+    return (g.batch >= 16 || (g.batch >= 2 && big)) && plan(g, &pl);
 }
 
 amq_status launch_binary_gemm_resident(const GemmArgs& g, cudaStream_t st)

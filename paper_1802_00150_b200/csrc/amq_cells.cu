@@ -55,6 +55,13 @@ __global__ void lstm_gates_kernel(const float* pre, const float* addend, const f
     h_out[u] = og * tanhf(c);
 }
 
+BatchedSequence batched_call(const CellCall& c, const CellWorkspace& ws, const float* x_seq, int steps, const float* h0, const float* c0,
+                             float* h_seq, float* h_last, float* c_last)
+{
+    return BatchedSequence{c.Wcodes, c.Walpha, c.bias, c.I, c.H, c.I + c.H, c.k_w, c.k_a, c.T, c.batch, steps, c.gru, x_seq, h0, c0,
+                           h_seq, h_last, c_last, {ws.h[0], ws.h[1]}, ws.c, nullptr, ws.zcodes, ws.zbeta, ws.counters, ws.status};
+}
+
 // quantize z = [x ; h_in] into the workspace, then product + gates
 amq_status enqueue_step(const CellCall& c, const CellWorkspace& ws, const float* x, const float* h_in,
                         const float* c_in, float* h_out, float* c_out, cudaStream_t st)
@@ -76,23 +83,45 @@ amq_status enqueue_step(const CellCall& c, const CellWorkspace& ws, const float*
     return launch_binary_gemm(a, st);
 }
 
-// `chunk_ready` (may be NULL): events after which the inputs of steps [q * steps_per_chunk, (q + 1) * steps_per_chunk) are
-// in place; the stream waits for event q before the first kernel of that chunk (batched chains only).
+// Inputs that arrive in chunks of timesteps: chunk q holds the steps begin[q] .. begin[q + 1] - 1, complete after ready[q].
+constexpr int MAX_CHUNKS = 8;
+struct Chunks {
+    int count;
+    int begin[MAX_CHUNKS + 1];
+    cudaEvent_t ready[MAX_CHUNKS + 1];      // (one more, for the start of the copy stream)
+};
+
+// `chunks` (may be NULL): the stream waits for a chunk's event before the first kernel that reads it (batched calls only).
 amq_status enqueue_sequence(const CellCall& c, const CellWorkspace& ws, const float* x_seq, int steps,
                             const float* h0, const float* c0, float* h_seq, float* h_last, float* c_last,
-                            cudaStream_t st, const cudaEvent_t* chunk_ready = nullptr, int steps_per_chunk = 0)
+                            cudaStream_t st, const Chunks* chunks = nullptr)
 {
-    const size_t state_bytes = (size_t)c.batch * c.H * sizeof(float);
+    const size_t state = (size_t)c.batch * c.H, state_bytes = state * sizeof(float);
     const bool persistent = steps > 0 && use_persistent(c);
-    AMQ_CUDA_TRY(cudaMemsetAsync(ws.status, 0, 256 + ((persistent && steps > 1) ? ws.hx_bytes : 0), st));
+    // (the exchange words or the counters lie directly behind the status words: one clear)
+    AMQ_CUDA_TRY(cudaMemsetAsync(ws.status, 0, 256 + ((persistent && steps > 1) ? ws.hx_bytes : 0) + ws.counter_bytes, st));
     if (persistent)
         return enqueue_persistent(c, ws, x_seq, steps, h0, c0, h_seq, h_last, c_last, st);
+    if (steps > 0 && batched_sequence_supported(batched_call(c, ws, x_seq, steps, h0, c0, h_seq, h_last, c_last))) {
+        // one launch for all steps, or one per chunk, the state handed on in the caller's h_last / c_last
+        for (int q = 0; q < (chunks ? chunks->count : 1); ++q) {
+            const int s0 = chunks ? chunks->begin[q] : 0, s1 = chunks ? chunks->begin[q + 1] : steps;
+            if (chunks) AMQ_CUDA_TRY(cudaStreamWaitEvent(st, chunks->ready[q], 0));
+            if (q > 0) AMQ_CUDA_TRY(cudaMemsetAsync(ws.counters, 0, ws.counter_bytes, st));
+            const amq_status r = launch_batched_sequence(
+                batched_call(c, ws, x_seq + (size_t)s0 * c.batch * c.I, s1 - s0, q ? h_last : h0, q ? c_last : c0,
+                             h_seq ? h_seq + (size_t)s0 * state : nullptr, h_last, c_last), st);
+            if (r != AMQ_OK) return r;
+        }
+        return AMQ_OK;
+    }
     if (!c.gru) AMQ_CUDA_TRY(cudaMemcpyAsync(ws.c, c0, state_bytes, cudaMemcpyDeviceToDevice, st));
     const float* h_prev = h0;
     for (int s = 0; s < steps; ++s) {
         float* h_next = h_seq ? h_seq + (size_t)s * c.batch * c.H : ws.h[s & 1];
         const float* x = x_seq + (size_t)s * c.batch * c.I;
-        if (chunk_ready && s % steps_per_chunk == 0) AMQ_CUDA_TRY(cudaStreamWaitEvent(st, chunk_ready[s / steps_per_chunk], 0));
+        for (int q = 0; chunks && q < chunks->count; ++q)
+            if (s == chunks->begin[q]) AMQ_CUDA_TRY(cudaStreamWaitEvent(st, chunks->ready[q], 0));
         amq_status r = enqueue_step(c, ws, x, h_prev, ws.c, h_next, ws.c, st);
         if (r != AMQ_OK) return r;
         h_prev = h_next;
@@ -100,6 +129,15 @@ amq_status enqueue_sequence(const CellCall& c, const CellWorkspace& ws, const fl
     AMQ_CUDA_TRY(cudaMemcpyAsync(h_last, h_prev, state_bytes, cudaMemcpyDeviceToDevice, st));
     if (!c.gru) AMQ_CUDA_TRY(cudaMemcpyAsync(c_last, ws.c, state_bytes, cudaMemcpyDeviceToDevice, st));
     return AMQ_OK;
+}
+
+amq_status step_entry(const CellCall& c, const CellWorkspace& ws, const float* x, const float* h_in, const float* c_in, float* h_out,
+                      float* c_out, cudaStream_t st)
+{
+    AMQ_CUDA_TRY(cudaMemsetAsync(ws.status, 0, 256 + ws.counter_bytes, st));
+    const BatchedSequence b = batched_call(c, ws, x, 1, h_in, c_in, nullptr, h_out, c_out);
+    if (batched_sequence_supported(b)) return launch_batched_sequence(b, st);
+    return enqueue_step(c, ws, x, h_in, c_in, h_out, c_out, st);
 }
 
 amq_status sequence_entry(const CellCall& c, const float* x_seq, int steps, const float* h0, const float* c0,
@@ -154,16 +192,15 @@ amq_status sequence_host_entry(const CellCall& c, const float* x_seq_host, int s
     HostStaging hs = carve_staging(staging, c.I, c.H, c.batch, steps);
     const size_t state_bytes = (size_t)c.batch * c.H * sizeof(float);
     const size_t x_bytes = (size_t)steps * c.batch * c.I * sizeof(float);
-    // Large inputs of a batched chain travel in chunks of timesteps on a stream of their own, so that the copy of the later
-    // timesteps runs beside the kernels of the earlier ones (C4: 73 MB of inputs against 1.7 ms of kernels); the chain waits
-    // for a chunk's event before its first step.  The copy stream and the events live for the duration of the call.
-    constexpr int MAX_CHUNKS = 8;
+    // Large inputs of a batched call travel in chunks of timesteps on a stream of their own, so that the copy of the later
+    // timesteps runs beside the kernels of the earlier ones (C4: 73 MB of inputs); the kernels wait for a chunk's event before
+    // its first step.  The copy stream and the events live for the duration of the call.  Chunks grow from a twelfth of the
+    // sequence by 1.6 to a quarter: nothing runs during the first copy, and every chunk is a launch.
     const bool chunked = x_bytes >= ((size_t)4 << 20) && steps >= 2 && !(steps > 0 && use_persistent(c));
     cudaStream_t copy_stream = nullptr;
-    cudaEvent_t ready[MAX_CHUNKS + 1] = {};
-    int nchunks = 0, steps_per_chunk = 0;
+    Chunks chunks{};
     auto release = [&]() {
-        for (int q = 0; q <= MAX_CHUNKS; ++q) if (ready[q]) cudaEventDestroy(ready[q]);
+        for (cudaEvent_t e : chunks.ready) if (e) cudaEventDestroy(e);
         if (copy_stream) cudaStreamDestroy(copy_stream);
     };
     // the small copies of the initial state go first: host-to-device copies are served in the order they were submitted,
@@ -172,27 +209,32 @@ amq_status sequence_host_entry(const CellCall& c, const float* x_seq_host, int s
     if (e == cudaSuccess && !c.gru) e = cudaMemcpyAsync(hs.c0, c0_host, state_bytes, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return AMQ_ERR_CUDA;
     if (chunked) {
-        steps_per_chunk = (steps + MAX_CHUNKS - 1) / MAX_CHUNKS;
-        nchunks = (steps + steps_per_chunk - 1) / steps_per_chunk;
+        for (int done = 0, size = (steps + 11) / 12; done < steps; ++chunks.count) {
+            chunks.begin[chunks.count] = done;
+            done = chunks.count == MAX_CHUNKS - 1 || done + size > steps ? steps : done + size;
+            chunks.begin[chunks.count + 1] = done;
+            size = (size * 8 + 4) / 5;
+            if (size > (steps + 3) / 4) size = (steps + 3) / 4;
+        }
         e = cudaStreamCreateWithFlags(&copy_stream, cudaStreamNonBlocking);
-        for (int q = 0; q <= nchunks && e == cudaSuccess; ++q) e = cudaEventCreateWithFlags(&ready[q], cudaEventDisableTiming);
+        for (int q = 0; q <= chunks.count && e == cudaSuccess; ++q) e = cudaEventCreateWithFlags(&chunks.ready[q], cudaEventDisableTiming);
         // the copy stream starts after what the caller's stream holds so far (the staging buffer may still be in use there)
-        if (e == cudaSuccess) e = cudaEventRecord(ready[nchunks], st);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(copy_stream, ready[nchunks], 0);
+        if (e == cudaSuccess) e = cudaEventRecord(chunks.ready[chunks.count], st);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(copy_stream, chunks.ready[chunks.count], 0);
         const size_t step_bytes = (size_t)c.batch * c.I * sizeof(float);
-        for (int q = 0; q < nchunks && e == cudaSuccess; ++q) {
-            const int s0 = q * steps_per_chunk, s1 = (s0 + steps_per_chunk < steps) ? s0 + steps_per_chunk : steps;
+        for (int q = 0; q < chunks.count && e == cudaSuccess; ++q) {
+            const int s0 = chunks.begin[q], s1 = chunks.begin[q + 1];
             e = cudaMemcpyAsync(reinterpret_cast<char*>(hs.x_seq) + s0 * step_bytes,
                                 reinterpret_cast<const char*>(x_seq_host) + s0 * step_bytes, (size_t)(s1 - s0) * step_bytes,
                                 cudaMemcpyHostToDevice, copy_stream);
-            if (e == cudaSuccess) e = cudaEventRecord(ready[q], copy_stream);
+            if (e == cudaSuccess) e = cudaEventRecord(chunks.ready[q], copy_stream);
         }
         if (e != cudaSuccess) { cudaStreamSynchronize(copy_stream); release(); return AMQ_ERR_CUDA; }
     } else if (x_bytes) {
         AMQ_CUDA_TRY(cudaMemcpyAsync(hs.x_seq, x_seq_host, x_bytes, cudaMemcpyHostToDevice, st));
     }
     s = enqueue_sequence(c, ws, hs.x_seq, steps, hs.h0, hs.c0, h_seq_host ? hs.h_seq : nullptr, hs.h_last, hs.c_last, st,
-                         chunked ? ready : nullptr, steps_per_chunk);
+                         chunked ? &chunks : nullptr);
     if (chunked) {
         // the events and the stream may go once both streams have drained
         cudaStreamSynchronize(copy_stream);
@@ -245,8 +287,7 @@ amq_status amq_lstm_step(const uint32_t* Wcodes, const float* Walpha, const floa
     if (!h_in || !c_in || !h_out || !c_out || (I > 0 && !x) || h_out == h_in) return AMQ_ERR_INVALID_ARG;
     if (batch == 0) return AMQ_OK;
     amq::CellWorkspace ws = amq::carve_cell_workspace(workspace, I, H, batch, k_a);
-    AMQ_CUDA_TRY(cudaMemsetAsync(ws.status, 0, 256, (cudaStream_t)stream));
-    return amq::enqueue_step(c, ws, x, h_in, c_in, h_out, c_out, (cudaStream_t)stream);
+    return amq::step_entry(c, ws, x, h_in, c_in, h_out, c_out, (cudaStream_t)stream);
 }
 
 amq_status amq_gru_step(const uint32_t* Wcodes, const float* Walpha, const float* bias, int I, int H, int k_w,
@@ -259,8 +300,7 @@ amq_status amq_gru_step(const uint32_t* Wcodes, const float* Walpha, const float
     if (!h_in || !h_out || (I > 0 && !x) || h_out == h_in) return AMQ_ERR_INVALID_ARG;
     if (batch == 0) return AMQ_OK;
     amq::CellWorkspace ws = amq::carve_cell_workspace(workspace, I, H, batch, k_a);
-    AMQ_CUDA_TRY(cudaMemsetAsync(ws.status, 0, 256, (cudaStream_t)stream));
-    return amq::enqueue_step(c, ws, x, h_in, nullptr, h_out, nullptr, (cudaStream_t)stream);
+    return amq::step_entry(c, ws, x, h_in, nullptr, h_out, nullptr, (cudaStream_t)stream);
 }
 
 amq_status amq_lstm_sequence(const uint32_t* Wcodes, const float* Walpha, const float* bias, int I, int H, int k_w,

@@ -52,8 +52,13 @@ struct CellWorkspace {
     float* c;           // [batch][H]
     unsigned long long* hx;   // [2][copies][H] exchange words {fp32 bits, step tag} of the persistent kernel
     size_t hx_bytes;
+    uint32_t* counters;       // progress counters of the batched sequence kernel, 64 words per block of vectors (batch > 1)
+    size_t counter_bytes;
     size_t bytes;
 };
+
+// progress counters of the batched sequence kernel: blocks have at least eight vectors
+inline size_t batched_counter_bytes(int batch) { return batch > 1 ? (size_t)((batch + 7) / 8) * 256 : 0; }
 
 inline CellWorkspace carve_cell_workspace(void* base, int I, int H, int batch, int k_a)
 {
@@ -65,6 +70,9 @@ inline CellWorkspace carve_cell_workspace(void* base, int I, int H, int batch, i
     w.hx = reinterpret_cast<unsigned long long*>(p + off);
     w.hx_bytes = batch == 1 ? round_up((size_t)2 * PERSISTENT_EXCHANGE_COPIES * persistent_exchange_stride(H) * 8, 256) : 0;   // batch 1 only
     off += w.hx_bytes;
+    w.counters = reinterpret_cast<uint32_t*>(p + off);
+    w.counter_bytes = batched_counter_bytes(batch);
+    off += w.counter_bytes;
     w.zcodes = reinterpret_cast<uint32_t*>(p + off);            off += round_up((size_t)batch * k_a * words_per_row(I + H) * 4, 256);
     w.zbeta = reinterpret_cast<float*>(p + off);                off += round_up((size_t)batch * k_a * 4, 256);
     w.h[0] = reinterpret_cast<float*>(p + off);                 off += round_up((size_t)batch * H * 4, 256);
@@ -158,6 +166,21 @@ amq_status tc_status_word(uint32_t** word);       // device address of the statu
 // Tensor-core product with a resident activation operand (EPI_Y): whether it covers a problem, and its launch.
 bool gemm_resident_supported(const GemmArgs& a);
 amq_status launch_binary_gemm_resident(const GemmArgs& a, cudaStream_t st);
+
+// Batched recurrent kernel: all timesteps of a batch of sequences in one cooperative launch.  z = [x ; h] (LSTM, GRU) or h alone with
+// the input projections as `addend` (paper form: I = 0, n = H).  `counters` cleared by the caller.
+struct BatchedSequence {
+    const uint32_t* Wcodes; const float* Walpha; const float* bias;
+    int I, H, n, k_w, k_a, T, batch, steps;
+    bool gru;
+    const float* x_seq; const float* h0; const float* c0;
+    float* h_seq; float* h_last; float* c_last;
+    float* h[2]; float* c;
+    const float* addend;
+    uint32_t* zcodes; float* zbeta; uint32_t* counters; uint32_t* status;
+};
+bool batched_sequence_supported(const BatchedSequence& s);
+amq_status launch_batched_sequence(const BatchedSequence& s, cudaStream_t st);
 
 // Persistent batch-1 recurrent kernel: whether it covers a problem (sizes, shared memory), and its launch.
 bool persistent_supported(int I, int H, int batch, int k_w, int k_a, bool gru, int* grid_out, int* upc_out,

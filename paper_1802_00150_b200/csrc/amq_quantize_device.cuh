@@ -49,24 +49,38 @@ struct __align__(16) QuantScratch {
     int code[NW][1 << K];
 };
 
-// To be called once by every thread of a CTA-wide group before its first quantize_group (no barrier needed
+// The threads of a group of several warps: the whole CTA, or some consecutive warps of it with a hardware barrier of their own.
+struct QuantTeam {
+    int warp, bar, threads;         // this warp's number in the team, barrier, threads of the team
+    __device__ __forceinline__ static QuantTeam cta() { return QuantTeam{(int)(threadIdx.x >> 5), 0, (int)blockDim.x}; }
+    __device__ __forceinline__ void sync() const { asm volatile("bar.sync %0, %1;" :: "r"(bar), "r"(threads) : "memory"); }
+    __device__ __forceinline__ int sync_or(int flag) const
+    {
+        int out;
+        asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\tbar.red.or.pred q, %2, %3, p;\n\tselp.b32 %0, 1, 0, q;\n\t}"
+                     : "=r"(out) : "r"(flag), "r"(bar), "r"(threads) : "memory");
+        return out;
+    }
+};
+
+// To be called once by every thread of a team before its first quantize_group (no barrier needed
 // afterwards): partial-sum slots of warps that do not exist are read as zeros by every reduction.
 template <int K, int NW>
-__device__ __forceinline__ void quant_scratch_init(QuantScratch<K, NW>& sc)
+__device__ __forceinline__ void quant_scratch_init(QuantScratch<K, NW>& sc, const QuantTeam& team = QuantTeam::cta())
 {
     constexpr int V = QuantScratch<K, NW>::V, SLOTS = QuantScratch<K, NW>::SLOTS;
-    const int warps = blockDim.x >> 5;
+    const int warps = team.threads >> 5;
     float* flat = &sc.red[0][0][0];
-    for (int idx = threadIdx.x; idx < 2 * V * SLOTS; idx += blockDim.x)
+    for (int idx = team.warp * 32 + (threadIdx.x & 31); idx < 2 * V * SLOTS; idx += team.threads)
         if ((idx % SLOTS) >= warps) flat[idx] = 0.0f;
 }
 
 // Totals over the group of VF floats and VI ints (ints are carried exactly); every thread of the group holds
-// them afterwards.  NW > 1: the group is the CTA and the call contains exactly one CTA barrier; when `flag`
-// is given, that barrier also ORs *flag over the CTA (every thread gets the result).
+// them afterwards.  NW > 1: the group is a team and the call contains exactly one barrier of it; when `flag`
+// is given, that barrier also ORs *flag over the team (every thread gets the result).
 template <int VF, int VI, int K, int NW>
 __device__ __forceinline__ void group_totals(float (&f)[VF], int (&iv)[VI > 0 ? VI : 1], QuantScratch<K, NW>& sc,
-                                             int parity, int* flag = nullptr)
+                                             int parity, int* flag, const QuantTeam& team)
 {
 #pragma unroll
     for (int i = 0; i < VF; ++i) {
@@ -77,15 +91,15 @@ __device__ __forceinline__ void group_totals(float (&f)[VF], int (&iv)[VI > 0 ? 
     for (int i = 0; i < VI; ++i) iv[i] = __reduce_add_sync(0xffffffffu, iv[i]);
     if (NW == 1) return;
     constexpr int SLOTS = QuantScratch<K, NW>::SLOTS;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = team.warp, lane = threadIdx.x & 31;
     if (lane == 0) {
 #pragma unroll
         for (int i = 0; i < VF; ++i) sc.red[parity][i][warp] = f[i];
 #pragma unroll
         for (int i = 0; i < VI; ++i) sc.red[parity][VF + i][warp] = __int_as_float(iv[i]);
     }
-    if (flag) *flag = __syncthreads_or(*flag);
-    else __syncthreads();
+    if (flag) *flag = team.sync_or(*flag);
+    else team.sync();
     // every thread: the partials of all warps, added in a fixed tree (slots of absent warps hold zeros)
 #pragma unroll
     for (int i = 0; i < VF; ++i) {
@@ -338,13 +352,14 @@ __host__ __device__ inline int quant_padding_strided32(int n, int ept) { return 
 template <int K, int EPT, int NW>
 __device__ __forceinline__ void quantize_group(const float (&w_in)[EPT], uint32_t valid, int n, int pad_elems, int T,
                                                float (&alpha)[K], uint32_t (&bits)[K], QuantScratch<K, NW>& sc,
-                                               int* flag = nullptr, int* parity_io = nullptr)
+                                               int* flag = nullptr, int* parity_io = nullptr,
+                                               const QuantTeam& team = QuantTeam::cta())
 {
     constexpr int M = 1 << K;
     constexpr int NG = K * (K - 1) / 2;
     constexpr uint32_t SIGN = 0x80000000u;
     const int lane = threadIdx.x & 31;
-    const int slot = NW > 1 ? (int)(threadIdx.x >> 5) : 0;
+    const int slot = NW > 1 ? team.warp : 0;
     const int nvalid = __popc(valid);
     const float inv_n = 1.0f / (float)n;
     const float padding = (float)pad_elems;                      // zero elements past the end that are summed along
@@ -379,7 +394,7 @@ __device__ __forceinline__ void quantize_group(const float (&w_in)[EPT], uint32_
             if (i == K - 1 && T > 0) { last_abs = part; alpha[i] = 0.0f; break; }
             float tot[1] = {part};
             int none[1] = {0};
-            group_totals<1, 0, K, NW>(tot, none, sc, parity, flag);
+            group_totals<1, 0, K, NW>(tot, none, sc, parity, flag, team);
             flag = nullptr;
             parity ^= 1;
             const float a = (tot[0] - padding * fabsf(rho)) * inv_n;
@@ -409,7 +424,7 @@ __device__ __forceinline__ void quantize_group(const float (&w_in)[EPT], uint32_
                     gram[q++] = nvalid - 2 * __popc((bits[i] ^ bits[j]) & valid);
             if (NG == 0) gram[0] = 0;
         }
-        group_totals<1 + K, NG, K, NW>(fsum, gram, sc, parity, flag);
+        group_totals<1 + K, NG, K, NW>(fsum, gram, sc, parity, flag, team);
         flag = nullptr;
         parity ^= 1;
         float thr[M - 1];

@@ -252,7 +252,7 @@ struct ResFeeder {
         const int ub = ub0 + (CELL != RES_PLAIN && p.tpu == 4 ? it >> 2 : it) * ub_step, tt = CELL != RES_PLAIN && p.tpu == 4 ? it & 3 : 0;
         const int wr = CELL == RES_PLAIN ? ub * 128 + r : res_row(p, ub, tt, r);
         row = p.W + (size_t)(wr < 0 || (CELL == RES_PLAIN && wr >= p.units) ? p.units - 1 : wr) * (p.k_w * p.wpr);
-        if (CELL == RES_GRU && p.tpu == 4) { n = res_tile_steps(p, tt); base = tt * RES_KIND; }
+        if (CELL != RES_PLAIN && p.tpu == 4) { n = res_tile_steps(p, tt); base = tt * RES_KIND; }
     }
     // position on the first own step of a pass over tiles ub0, ub0 + ub_step, ..; `skip` steps of other groups come first
     __device__ __forceinline__ void start(const ResProblem& p, const uint32_t* table, int first_block, int block_step, int tiles, int r, int skip)
@@ -273,7 +273,7 @@ struct ResFeeder {
     // whether this lane's row is zero in the slot of table entry `entry` (candidate rows of a 32-unit GRU block)
     __device__ __forceinline__ static bool zero_row(const ResProblem& p, uint32_t entry, int r)
     {
-        return CELL == RES_GRU && p.ut == 32 && (r >> 5) == ((entry & RES_STEP_H) ? 2 : 3);
+        return CELL != RES_PLAIN && p.cell == RES_GRU && p.ut == 32 && (r >> 5) == ((entry & RES_STEP_H) ? 2 : 3);
     }
     // packed words of the cursor's step, and on to the group's next step
     __device__ __forceinline__ void fetch(const ResProblem& p, const uint32_t* table, int r)
