@@ -25,8 +25,10 @@ constexpr int Y_LD = 132;
 // groups of eight vectors per epilogue thread: TB <= 64, or 32 (registers)
 __host__ __device__ constexpr int res_ng(int k_a) { return k_a <= 2 ? 2 : 1; }
 
+using R = ResRoles<3, 16, 3>;
+
 template <int KA>
-__global__ void __launch_bounds__(RES_THREADS, 1)
+__global__ void __launch_bounds__(R::THREADS, 1)
 bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -51,8 +53,8 @@ bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
         return (int)(w_end - at < a.mtiles - tile0 ? w_end - at : a.mtiles - tile0);
     };
 
-    if (tid == 0) res_sync_init(sy);
-    if (warp == RES_MMA_WARP) {
+    if (tid == 0) res_sync_init<R>(sy);
+    if (warp == R::MMA_WARP) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      :: "r"(smem_u32(&sy.tmem_slot)), "r"((uint32_t)RES_TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -63,14 +65,14 @@ bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
     const uint32_t tmem = __shfl_sync(0xffffffffu, sy.tmem_slot, 0);
     if (warp < 4) res_write_scales(p, tmem, warp);
 
-    for (int q = tid; q < 512; q += RES_THREADS) sSum[q] = 0;
+    for (int q = tid; q < 512; q += R::THREADS) sSum[q] = 0;
     res_fill_table(p, table);
     __syncthreads();
 
     // expand the activations of block bb; all threads, ends with a CTA barrier
     auto load_block = [&](int bb) {
         const int b0 = bb * p.TB;
-        for (int q = tid; q < p.N; q += RES_THREADS) {
+        for (int q = tid; q < p.N; q += R::THREADS) {
             const int b = b0 + res_row_vector<KA>(q), j = res_row_plane<KA>(q);
             sBeta[q] = q < p.TB * KA && b < p.batch ? __ldcg(a.xbeta + (size_t)b * KA + j) : 0.0f;
         }
@@ -83,13 +85,13 @@ bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
     // ends with a barrier, after which every MMA that read the operand has completed (the epilogue has waited for all
     // accumulators), so the operand may be overwritten.
     bool ok = true;
-    if (warp < RES_EXP_WARPS) {
+    if (warp < R::EXP_WARPS) {
         const int r = (warp & 3) * 32 + lane, steps_per_tile = p.k_w * ((p.NS + 1) >> 1);
         int first_step = 0;                         // pipeline steps so far, mod the number of groups
         ResFeedState fs{warp >> 2, 1u};
-        ResFeeder<RES_PLAIN> feed;
+        ResFeeder<R, RES_PLAIN> feed;
         auto start = [&](long long at) {
-            feed.start(p, table, (int)(at % a.mtiles), 1, pass_tiles(at), r, ((warp >> 2) - first_step + RES_GROUPS) % RES_GROUPS);
+            feed.start(p, table, (int)(at % a.mtiles), 1, pass_tiles(at), r, ((warp >> 2) - first_step + R::GROUPS) % R::GROUPS);
         };
         if (w < w_end) start(w);                    // (weights: no kernel of a chain writes them)
         grid_dependency_wait();                     // the planes and coefficients may come from the preceding kernel
@@ -98,11 +100,11 @@ bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
             ok = res_feed(p, sy, table, feed, tmem, fs);
             const int tiles = pass_tiles(w);
             w += tiles;
-            first_step = (int)((first_step + (long long)tiles * steps_per_tile) % RES_GROUPS);
+            first_step = (int)((first_step + (long long)tiles * steps_per_tile) % R::GROUPS);
             if (w < w_end) start(w);
             if (__syncthreads_or(!ok)) { ok = false; break; }
         }
-    } else if (warp == RES_MMA_WARP) {
+    } else if (warp == R::MMA_WARP) {
         ResIssueState issue{0, 0, 0, 1};
         grid_dependency_wait();
         while (w < w_end) {
@@ -112,10 +114,9 @@ bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
             w += tiles;
             if (__syncthreads_or(!ok)) { ok = false; break; }
         }
-    } else if (warp < RES_MMA_WARP) {
-        const int te = tid - 32 * RES_EXP_WARPS, quarter = warp & 3, sub = (warp - RES_EXP_WARPS) >> 2, rl = quarter * 32 + (lane >> 2);
+    } else if (warp < R::MMA_WARP) {
+        const int te = tid - 32 * R::EXP_WARPS, quarter = warp & 3, sub = (warp - R::EXP_WARPS) >> 2, rl = quarter * 32 + (lane >> 2);
         ResDrainState drain{0, 0};
-        ResColumns<KA, NG> col;
         uint32_t y_parity = 1;
         // coefficients of a tile's rows: thread te takes one of the 128 k_w, a tile ahead
         auto alpha_of = [&](int tile) {
@@ -127,22 +128,21 @@ bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
             const int bb = (int)(w / a.mtiles), tile0 = (int)(w % a.mtiles), tiles = pass_tiles(w);
             float next_alpha = alpha_of(tile0);
             load_block(bb);
-            res_row_constants(p, sSum, sRow);
+            res_row_constants<R>(p, sSum, sRow);
             for (int t = 0; t < tiles; ++t) {
                 float* sa = sAlpha + (t & 1) * AMQ_MAX_K * 128;
                 sa[te] = next_alpha;
-                if (res_epi_bar(!ok)) { ok = false; break; }        // (also: everybody is past the tile before last, whose buffer this is)
-                if (t == 0) { col.load(p, sBeta, sub, col.beta); col.load(p, sRow, sub, col.row); }
+                if (res_epi_bar<R>(!ok)) { ok = false; break; }        // (also: everybody is past the tile before last, whose buffer this is)
                 if (t + 1 < tiles) next_alpha = alpha_of(tile0 + t + 1);
                 f32x2 y[NG][4];
-                ok = res_drain_tile<KA, NG>(p, sy, sa, quarter, sub, tmem, col, drain, y);
+                ok = res_drain_tile<R, KA, NG>(p, sy, sa, quarter, sub, tmem, sBeta, sRow, drain, y);
                 // Results leave through shared memory and three warps of their own: in this layout a store from the registers is four
                 // 32-byte pieces, and stores from the epilogue warps held them up for longer than a tile's MMAs take.
-                ok = ok && res_group_wait(sy, smem_u32(&sy.yempty), y_parity, warp == RES_EXP_WARPS, 1, 32 * RES_EPI_WARPS);
+                ok = ok && res_group_wait(sy, smem_u32(&sy.yempty), y_parity, warp == R::EXP_WARPS, 1, 32 * R::EPI_WARPS);
                 y_parity ^= 1u;
 #pragma unroll
                 for (int g = 0; g < NG; ++g) {
-                    const int e = (RES_EPI_SPLIT * g + sub) * 8 + 2 * (lane & 3);
+                    const int e = (R::SPLIT * g + sub) * 8 + 2 * (lane & 3);
                     if (e >= p.TB) break;
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
@@ -179,7 +179,7 @@ bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
                 if (!ok) { *(volatile int*)&sy.failed = 1; break; }
                 const bool vec = a.vec_out && row + 3 < p.units;
 #pragma unroll 4
-                for (int e = warp - RES_MMA_WARP - 1; e < last; e += RES_OUT_WARPS) {
+                for (int e = warp - R::MMA_WARP - 1; e < last; e += R::OUT_WARPS) {
                     float4 v = *reinterpret_cast<const float4*>(sY + e * Y_LD + 4 * lane);
                     v.x += bias.x; v.y += bias.y; v.z += bias.z; v.w += bias.w;
                     float* out = a.y + (size_t)(b0 + e) * a.ldy + row;
@@ -207,7 +207,7 @@ bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
         __nanosleep(1000000);
         __syncthreads();
     }
-    if (warp == RES_MMA_WARP)
+    if (warp == R::MMA_WARP)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"((uint32_t)RES_TMEM_COLS) : "memory");
 }
 
@@ -227,9 +227,9 @@ bool plan(const GemmArgs& g, ResGemmPlan* out)
     // block of vectors: the size with the least estimated time (shares of tiles x steps, plus the expansion of the operand,
     // which a share pays at least once); sizes whose operand does not fit shared memory are out (n > 28000 or so: none fits)
     double best = 0.0;
-    for (int TB = 8; TB <= 8 * res_ng(g.k_a) * RES_EPI_SPLIT; TB += 8) {
+    for (int TB = 8; TB <= 8 * res_ng(g.k_a) * R::SPLIT; TB += 8) {
         ResProblem q = p;
-        if (!res_set_block(q, TB, g.k_a, (size_t)TB * Y_LD * 4)) break;
+        if (!res_set_block<R>(q, TB, g.k_a, (size_t)TB * Y_LD * 4)) break;
         const long long blocks = (g.batch + TB - 1) / TB, per_cta = (blocks * a.mtiles + sms - 1) / sms;
         const double expand = (double)q.N * q.NS * 128 / 80.0 + 1500.0;
         const double t = (double)per_cta * q.k_w * q.NS * res_slot_clocks(q) + expand * (1.0 + (double)per_cta / a.mtiles);
@@ -252,7 +252,7 @@ amq_status launch(const ResGemmPlan& pl, bool overlap, cudaStream_t st)
 {
     auto kernel = bgemm_resident_kernel<KA>;
     AMQ_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem));
-    AMQ_CUDA_TRY(launch_kernel(kernel, dim3((unsigned)pl.grid), dim3(RES_THREADS), pl.smem, st, overlap, pl.a));
+    AMQ_CUDA_TRY(launch_kernel(kernel, dim3((unsigned)pl.grid), dim3(R::THREADS), pl.smem, st, overlap, pl.a));
     AMQ_LAUNCH_CHECK();
     return AMQ_OK;
 }

@@ -106,6 +106,7 @@ __device__ __forceinline__ void group_totals(float (&f)[VF], int (&iv)[VI > 0 ? 
         float tot = 0.0f;
 #pragma unroll
         for (int q = 0; q < SLOTS / 4; ++q) {
+            if (q > 0 && 4 * q >= team.threads >> 5) break;         // (slots of warps that a smaller team does not have)
             const float4 v = *reinterpret_cast<const float4*>(&sc.red[parity][i][4 * q]);
             const float s = (v.x + v.y) + (v.z + v.w);
             tot = (q == 0) ? s : tot + s;
@@ -117,6 +118,7 @@ __device__ __forceinline__ void group_totals(float (&f)[VF], int (&iv)[VI > 0 ? 
         int tot = 0;
 #pragma unroll
         for (int q = 0; q < SLOTS / 4; ++q) {
+            if (q > 0 && 4 * q >= team.threads >> 5) break;
             const int4 v = *reinterpret_cast<const int4*>(&sc.red[parity][VF + i][4 * q]);
             tot += (v.x + v.y) + (v.z + v.w);
         }

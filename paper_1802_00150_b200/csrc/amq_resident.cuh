@@ -27,6 +27,10 @@
 //
 // Pace, measured in isolation (one CTA per SM): 240 clocks per slot at N <= 96, 265 at N = 128 (256 is the tensor pipe's own
 // time), bound by the issue and synchronisation of the steps below N = 96 (an MMA takes 46 clocks however small N is).
+//
+// Code size matters as much as anything above: with the operand's expansion inlined into every role and its loops unrolled the kernels
+// were 95 and 210 KB of instructions, and every role waited for instruction fetches (some ten clocks per instruction).  Bodies that
+// run once per pass appear once and are not unrolled.
 #pragma once
 
 #include "amq_common.cuh"
@@ -34,13 +38,13 @@
 
 namespace amq {
 
-constexpr int RES_GROUPS = 3;                       // groups of four expander warps, which take the slots in turn
-constexpr int RES_EXP_WARPS = 4 * RES_GROUPS;       // warps 0 .. 11
-constexpr int RES_EPI_WARPS = 16;                   // warps 12 .. 27: lane quarter = warp mod 4, four warps per quarter
-constexpr int RES_EPI_SPLIT = RES_EPI_WARPS / 4;    // warps that share a quarter: groups of eight vectors in turn
-constexpr int RES_MMA_WARP = RES_EXP_WARPS + RES_EPI_WARPS;        // warp 28
-constexpr int RES_OUT_WARPS = 3;                    // warps 29 .. 31: a plain product's stores
-constexpr int RES_THREADS = 1024;
+// Roles of a CTA: groups of four expander warps (which take the pipeline steps in turn), epilogue warps (lane quarter = warp mod 4,
+// SPLIT warps per quarter, groups of eight vectors in turn), one warp that issues the MMAs, others.
+template <int GROUPS_, int EPI_WARPS_, int OUT_WARPS_>
+struct ResRoles {
+    static constexpr int GROUPS = GROUPS_, EXP_WARPS = 4 * GROUPS_, EPI_WARPS = EPI_WARPS_, SPLIT = EPI_WARPS_ / 4,
+                         MMA_WARP = EXP_WARPS + EPI_WARPS, OUT_WARPS = OUT_WARPS_, THREADS = 32 * (MMA_WARP + 1 + OUT_WARPS_);
+};
 constexpr int RES_STAGE_COLS = 64;                  // tensor-memory columns of a stage: two slots of the weight operand
 constexpr int RES_MAX_STAGES = 4;
 constexpr int RES_MAX_RING = 2;                     // accumulator buffers
@@ -105,11 +109,14 @@ struct ResSync {
     int failed;                                             // a bounded wait ran out
 };
 
+template <typename R>
 __device__ __forceinline__ void res_sync_init(ResSync& sy)
 {
+#pragma unroll 1
     for (int g = 0; g < RES_MAX_STAGES; ++g) { mbar_init(smem_u32(&sy.full[g]), 4); mbar_init(smem_u32(&sy.empty[g]), 1); }
-    for (int q = 0; q < RES_MAX_RING; ++q) { mbar_init(smem_u32(&sy.tfull[q]), 1); mbar_init(smem_u32(&sy.tempty[q]), RES_EPI_WARPS); }
-    mbar_init(smem_u32(&sy.yfull), RES_EPI_WARPS); mbar_init(smem_u32(&sy.yempty), RES_OUT_WARPS);
+#pragma unroll 1
+    for (int q = 0; q < RES_MAX_RING; ++q) { mbar_init(smem_u32(&sy.tfull[q]), 1); mbar_init(smem_u32(&sy.tempty[q]), R::EPI_WARPS); }
+    mbar_init(smem_u32(&sy.yfull), R::EPI_WARPS); mbar_init(smem_u32(&sy.yempty), R::OUT_WARPS);
     sy.failed = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
@@ -123,7 +130,7 @@ __device__ __forceinline__ bool res_bar(int id, int threads, bool bad)
         : "=r"(out) : "r"((uint32_t)bad), "r"(id), "r"(threads) : "memory");
     return out != 0;
 }
-__device__ __forceinline__ bool res_epi_bar(bool bad) { return res_bar(1, 32 * RES_EPI_WARPS, bad); }
+template <typename R> __device__ __forceinline__ bool res_epi_bar(bool bad) { return res_bar(1, 32 * R::EPI_WARPS, bad); }
 
 // Wait of a whole group of warps on one mbarrier: one warp polls, the others wait at a hardware barrier.  (With every warp polling,
 // the polls alone took half of the SM's issue slots and the synchronisation of a slot, without any work in it, 370 clocks.)
@@ -139,6 +146,9 @@ __device__ __forceinline__ bool res_group_wait(ResSync& sy, uint32_t bar, uint32
 
 // ---- activation operand ---------------------------------------------------------------------------------------------------
 
+// bits n .. 31 (all of them for n <= 0, none for n >= 32)
+__device__ __forceinline__ uint32_t upper_bits(int n) { return n >= 32 ? 0u : 0xffffffffu << (n < 0 ? 0 : n); }
+
 // 256 bit positions of one packed row -> the 128 nibble bytes of operand row `row` in one slot.  `lo`, `hi`: valid element range.
 // Returns sum of b over the valid positions with s < 3 (bit 1 = -1).
 __device__ __forceinline__ int res_expand_row(uint32_t slot_addr, int row, const uint32_t (&w)[8], int first, int lo, int hi)
@@ -151,20 +161,18 @@ __device__ __forceinline__ int res_expand_row(uint32_t slot_addr, int row, const
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int e = first + 32 * (4 * h + q);
-            vm[q] = 0xffffffffu;
-            if (lo > e) vm[q] = lo - e >= 32 ? 0u : vm[q] << (lo - e);
-            if (hi < e + 32) vm[q] = hi <= e ? 0u : vm[q] & (0xffffffffu >> (e + 32 - hi));
+            // bits of the word inside [lo, hi): everything from lo - e up, less everything from hi - e up
+            vm[q] = upper_bits(lo - e) & ~upper_bits(hi - e);
             const uint32_t m3 = vm[q] & 0x77777777u;
             sum += __popc(m3) - 2 * __popc(w[4 * h + q] & m3);
         }
-#pragma unroll
+#pragma unroll 1
         for (int s = 0; s < 4; ++s) {
+            const uint32_t flip = s < 3 ? 0xAAAAAAAAu : 0x22222222u;        // s < 3: -b (bit 1 -> +1); s = 3: b
             uint32_t y[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const uint32_t sign = (w[4 * h + q] << (3 - s)) & 0x88888888u;                          // nibble i: bit 4 i + s
-                y[q] = (s < 3 ? sign ^ 0xAAAAAAAAu : sign | 0x22222222u) & (((vm[q] >> s) & 0x11111111u) * 15u);
-            }
+            for (int q = 0; q < 4; ++q)
+                y[q] = (((w[4 * h + q] << (3 - s)) & 0x88888888u) ^ flip) & (((vm[q] >> s) & 0x11111111u) * 15u);      // nibble i: bit 4 i + s
             st_shared_v4(base + (uint32_t)(((4 * h + s) ^ (row & 7)) << 4), y[0], y[1], y[2], y[3]);
         }
     }
@@ -184,6 +192,7 @@ __device__ __forceinline__ void res_expand_activations(const ResProblem& p, cons
     const int N = p.N;
     int row = (int)threadIdx.x % N, slot = (int)threadIdx.x / N;
     const int drow = (int)blockDim.x % N, dslot = (int)blockDim.x / N;
+#pragma unroll 1
     while (slot < p.NS) {
         const int b = b0 + res_row_vector<KA>(row), j = res_row_plane<KA>(row);
         const int w0 = res_slot_word(p, slot);
@@ -207,9 +216,11 @@ __device__ __forceinline__ void res_expand_activations(const ResProblem& p, cons
 
 // Epilogue warps, after the barrier that completes sSum: the constants as fp32, sRow[0] of the whole vector, and of the x and the h
 // part, sRow[1], sRow[2], where the columns are split; clears sSum for the next block.
+template <typename R>
 __device__ __forceinline__ void res_row_constants(const ResProblem& p, int* sSum, float* sRow)
 {
-    for (int i = (int)threadIdx.x - 32 * RES_EXP_WARPS; i < p.N; i += 32 * RES_EPI_WARPS) {
+#pragma unroll 1
+    for (int i = (int)threadIdx.x - 32 * R::EXP_WARPS; i < p.N; i += 32 * R::EPI_WARPS) {
         const int x = sSum[i], h = p.nx > 0 ? sSum[256 + i] : 0;
         sSum[i] = 0; sSum[256 + i] = 0;
         sRow[i] = (float)(x + h);
@@ -235,7 +246,7 @@ __device__ __forceinline__ int res_tile_steps(const ResProblem& p, int tt)
 // One group's share of the CTA's steps: the steps of all tiles in order are dealt to the groups in turn.  Thread = plane-row.  The
 // packed words of a step are fetched one of the group's steps ahead.  (Every instruction counts here: the expander warps
 // issue about one in ten clocks beside the other roles, and a group has three steps' time, some 1500 clocks, per step.)
-template <int CELL>
+template <typename R, int CELL>
 struct ResFeeder {
     const uint32_t* row;            // plane 0 of this thread's row in the cursor's tile (a lane without a weight row takes the last one:
                                     // its accumulators are read by nobody)
@@ -265,6 +276,7 @@ struct ResFeeder {
     }
     __device__ __forceinline__ void next_tile(const ResProblem& p, int r)
     {
+#pragma unroll 1
         while (i >= n && it < nitems) {
             i -= n;
             if (++it < nitems) tile(p, r);
@@ -296,7 +308,7 @@ struct ResFeeder {
             v[1][0] = __ldg(src1);
             if (!(e.y & RES_STEP_HALF)) v[1][1] = __ldg(src1 + 1);
         }
-        i += RES_GROUPS;
+        i += R::GROUPS;
         if (i >= n) next_tile(p, r);
     }
 };
@@ -305,10 +317,12 @@ struct ResFeeder {
 __device__ __forceinline__ void res_fill_table(const ResProblem& p, uint32_t* table)
 {
     const int kinds = p.cell == RES_GRU && p.tpu == 4 ? 4 : 1;
+#pragma unroll 1
     for (int tt = 0; tt < kinds; ++tt) {
         int s0, s1;
         res_tile_slots(p, tt, s0, s1);
         const int per_plane = (s1 - s0 + 1) & ~1;
+#pragma unroll 1
         for (int q = threadIdx.x; q < p.k_w * per_plane; q += blockDim.x) {
             const int plane = q / per_plane, s = s0 + q - plane * per_plane, w0 = res_slot_word(p, s);
             table[tt * RES_KIND + q] = s >= s1 ? RES_STEP_NONE | RES_STEP_HALF          // (offset 0: loads what is there, used by nobody)
@@ -344,13 +358,14 @@ __device__ __forceinline__ void res_store_slot(uint32_t taddr, const uint4& a, c
 struct ResFeedState { int stage; uint32_t parity; };       // the group's next stage and the parity of its "empty" barrier: start {group, 1}
 
 // The expander warps' part of one pass (f has been started).  False when a wait ran out.
-template <int CELL>
-__device__ __forceinline__ bool res_feed(const ResProblem& p, ResSync& sy, const uint32_t* table, ResFeeder<CELL>& f, uint32_t tmem, ResFeedState& st)
+template <typename R, int CELL>
+__device__ __forceinline__ bool res_feed(const ResProblem& p, ResSync& sy, const uint32_t* table, ResFeeder<R, CELL>& f, uint32_t tmem, ResFeedState& st)
 {
-    const int grp = (int)threadIdx.x >> 7, r = (int)threadIdx.x & 127;
+    const int r = (int)threadIdx.x & 127;
     const uint32_t taddr = tmem + ((uint32_t)(r & 96) << 16) + (uint32_t)(p.ring * p.N + 16);
+#pragma unroll 1
     while (f.live) {
-        if (!res_group_wait(sy, smem_u32(&sy.empty[st.stage]), st.parity, r < 32, 2 + grp, 128)) return false;
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&sy.empty[st.stage]), st.parity))) { *(volatile int*)&sy.failed = 1; return false; }
         const uint32_t t = taddr + (uint32_t)(st.stage * RES_STAGE_COLS);
         res_store_slot(t, f.v[0][0], f.v[0][1], f.zero_row(p, f.e.x, r));
         if (!(f.e.y & RES_STEP_NONE)) res_store_slot(t + 32, f.v[1][0], f.v[1][1], f.zero_row(p, f.e.y, r));
@@ -359,7 +374,7 @@ __device__ __forceinline__ bool res_feed(const ResProblem& p, ResSync& sy, const
         __syncwarp();
         if ((threadIdx.x & 31) == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(&sy.full[st.stage])) : "memory");
         f.fetch(p, table, r);                       // (into the registers just expanded)
-        st.stage += RES_GROUPS;
+        st.stage += R::GROUPS;
         if (st.stage >= p.stages) { st.stage -= p.stages; st.parity ^= 1u; }
     }
     return true;
@@ -404,13 +419,16 @@ __device__ __forceinline__ bool res_issue(const ResProblem& p, ResSync& sy, int 
     // The next step's barrier is looked at between the two halves of a step, while the MMAs of the first half are in the queue: with the
     // look after the last MMA the tensor pipe ran dry for 250-400 clocks between steps.
     bool ready = false;
+#pragma unroll 1
     for (int it = 0; it < nitems; ++it) {
         int s0, s1;
         res_tile_slots(p, p.tpu == 4 ? it & 3 : 0, s0, s1);
+#pragma unroll 1
         for (int plane = 0; plane < p.k_w; ++plane) {
             if (!mbar_wait(smem_u32(&sy.tempty[st.ring]), st.ring_parity)) { *(volatile int*)&sy.failed = 1; return false; }
             const uint32_t acc = tmem + (uint32_t)(st.ring * p.N);
             uint32_t b = lo + (uint32_t)s0 * slot_units;
+#pragma unroll 1
             for (int s = s0; s < s1; s += 2) {
                 if (!ready && !mbar_wait(full0 + 8 * st.stage, st.full_parity)) { *(volatile int*)&sy.failed = 1; return false; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -435,32 +453,17 @@ __device__ __forceinline__ bool res_issue(const ResProblem& p, ResSync& sy, int 
 // ---- accumulators ---------------------------------------------------------------------------------------------------------
 //
 // An epilogue warp reads its 32 rows in the m16n8 layout: a thread then holds, of every group of eight vectors, the two vectors
-// 2 (lane mod 4) + {0, 1} for the four rows lane / 4 + 8 i.  Its activation coefficients and row constants depend on the vectors only
-// and stay in registers for the whole pass, and two vectors share every instruction.
-
-template <int KA, int NG>
-struct ResColumns {
-    f32x2 beta[NG][KA], row[NG][KA];        // of this thread's two vectors in the groups sub, sub + 4, ..
-
-    __device__ __forceinline__ static void load(const ResProblem& p, const float* src, int sub, f32x2 (&dst)[NG][KA])
-    {
-#pragma unroll
-        for (int g = 0; g < NG; ++g)
-#pragma unroll
-            for (int j = 0; j < KA; ++j) {
-                const int gg = RES_EPI_SPLIT * g + sub;
-                dst[g][j] = gg * 8 < p.TB ? *reinterpret_cast<const f32x2*>(src + (gg * KA + j) * 8 + 2 * (threadIdx.x & 3)) : 0ull;
-            }
-    }
-};
+// 2 (lane mod 4) + {0, 1} for the four rows lane / 4 + 8 i.  A pair of vectors shares every instruction, and four rows every load
+// of the activation coefficients and row constants.
 
 struct ResDrainState { int ring; uint32_t parity; };        // start: {0, 0}
 
 // One tile: the k_w accumulators of this warp's 32 rows, y[g][i] = sum over planes of alpha * sum_j beta_j D_j for row lane / 4 + 8 i
-// and the two vectors, D_j = accumulator + row constant (exact integers).  `sAlpha`: coefficients [plane][128] of the tile.
-template <int KA, int NG>
+// and the two vectors, D_j = accumulator + row constant (exact integers).  `sAlpha`: coefficients [plane][128] of the tile; `sRow`: the
+// row constants that go with the lane's slots.
+template <typename R, int KA, int NG>
 __device__ __forceinline__ bool res_drain_tile(const ResProblem& p, ResSync& sy, const float* sAlpha, int quarter, int sub, uint32_t tmem,
-                                               const ResColumns<KA, NG>& col, ResDrainState& st, f32x2 (&y)[NG][4])
+                                               const float* sBeta, const float* sRow, ResDrainState& st, f32x2 (&y)[NG][4])
 {
     const int lane = (int)threadIdx.x & 31;
 #pragma unroll
@@ -475,20 +478,26 @@ __device__ __forceinline__ bool res_drain_tile(const ResProblem& p, ResSync& sy,
             const float v = sAlpha[plane * 128 + quarter * 32 + (lane >> 2) + 8 * i];
             al[i] = pack2(v, v);
         }
-        if (!res_group_wait(sy, smem_u32(&sy.tfull[st.ring]), st.parity, threadIdx.x >> 5 == RES_EXP_WARPS, 1, 32 * RES_EPI_WARPS)) return false;
+        if (!res_group_wait(sy, smem_u32(&sy.tfull[st.ring]), st.parity, threadIdx.x >> 5 == R::EXP_WARPS, 1, 32 * R::EPI_WARPS)) return false;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(st.ring * p.N);
 #pragma unroll
         for (int g = 0; g < NG; ++g) {
-            const int gg = RES_EPI_SPLIT * g + sub;
+            const int gg = R::SPLIT * g + sub;
             if (gg * 8 >= p.TB) break;
-            f32x2 v[4][KA];
+            f32x2 v[4][KA], beta[KA], row[KA];
+            const int c0 = gg * 8 * KA + 2 * (lane & 3);
+#pragma unroll
+            for (int j = 0; j < KA; ++j) {
+                beta[j] = *reinterpret_cast<const f32x2*>(sBeta + c0 + 8 * j);
+                row[j] = *reinterpret_cast<const f32x2*>(sRow + c0 + 8 * j);
+            }
             tmem_ld_pairs<KA>(acc + (uint32_t)(gg * 8 * KA), v);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                f32x2 s = mul2(col.beta[g][0], add2(v[i][0], col.row[g][0]));
+                f32x2 s = mul2(beta[0], add2(v[i][0], row[0]));
 #pragma unroll
-                for (int j = 1; j < KA; ++j) s = fma2(col.beta[g][j], add2(v[i][j], col.row[g][j]), s);
+                for (int j = 1; j < KA; ++j) s = fma2(beta[j], add2(v[i][j], row[j]), s);
                 y[g][i] = fma2(al[i], s, y[g][i]);
             }
         }
@@ -518,13 +527,14 @@ inline size_t res_smem_bytes(const ResProblem& p, int k_a)
 }
 
 // block of TB vectors: operand rows and accumulator buffers; false when they fit neither tensor nor shared memory
+template <typename R>
 inline bool res_set_block(ResProblem& p, int TB, int k_a, size_t more_smem = 0)
 {
     p.TB = TB;
     p.N = (TB * k_a + 15) / 16 * 16;
     if (p.N > 256 || p.NS > 33) return false;
     // two accumulator buffers where that leaves a stage per group
-    p.ring = (RES_TMEM_COLS - 16 - 2 * p.N) / RES_STAGE_COLS >= RES_GROUPS ? 2 : 1;
+    p.ring = (RES_TMEM_COLS - 16 - 2 * p.N) / RES_STAGE_COLS >= R::GROUPS ? 2 : 1;
     const int stages = (RES_TMEM_COLS - 16 - p.ring * p.N) / RES_STAGE_COLS;
     p.stages = stages < RES_MAX_STAGES ? stages : RES_MAX_STAGES;
     return res_smem_bytes(p, k_a) + more_smem <= (size_t)RES_SMEM_LIMIT;

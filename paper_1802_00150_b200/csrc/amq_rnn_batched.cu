@@ -1,7 +1,7 @@
 // Batched quantized LSTM / GRU sequences (Eq. 6; stacked form of Fig. 3, right): ONE cooperative launch for all timesteps.
 //
 // The batch is cut into blocks of TB vectors; P CTAs (one per SM) share a block, each with its own blocks of hidden units.  A
-// timestep is, in every CTA: quantize this CTA's share of the block's vectors z = [x_t ; h_{t-1}] (Algorithm 2, teams of 8 to 32
+// timestep is, in every CTA: quantize this CTA's share of the block's vectors z = [x_t ; h_{t-1}] (Algorithm 2, teams of 8 or 16
 // warps), wait for the other P - 1 CTAs' shares, expand the planes of the whole block into shared memory, run the product of the own
 // gate rows (amq_resident.cuh) with the gates in the epilogue, wait for the other CTAs' h.  The two waits are counters in the
 // workspace, one pair per block of vectors: blocks never wait for one another.
@@ -19,7 +19,9 @@ namespace {
 
 constexpr int SEQ_Y_LD = 132;                   // row stride of the staged pre-activations
 constexpr unsigned SEQ_POLL_LIMIT = 1u << 21;   // looks at a counter before giving up (a second or so)
-constexpr int SEQ_EPT = 8;                      // elements per thread of a quantizer team
+using R = ResRoles<2, 8, 3>;                     // (640 threads: 96 registers each; the quantizer and the epilogue spill with 64)
+constexpr int SEQ_QUANT_WARPS = 16;             // warps that quantize: two teams of 8, or one of 16
+constexpr int SEQ_NG = 2;                       // groups of eight vectors per epilogue thread: blocks of up to 32 vectors
 
 struct SeqParams {
     ResProblem p;               // units = H
@@ -35,10 +37,8 @@ struct SeqParams {
     uint32_t* status;
     int P, unit_blocks, b_bytes;
     int team_warps;             // warps per quantized vector
+    int unit_steps;             // pipeline steps of a block of units
 };
-
-// groups of eight vectors per epilogue thread (registers)
-__host__ __device__ constexpr int seq_ng(int k_a) { return k_a <= 2 ? 2 : 1; }
 
 __device__ __forceinline__ void seq_publish(uint32_t* counter)
 {
@@ -66,18 +66,18 @@ struct __align__(16) SeqShared {
     ResSync sync;
 };
 
-// Quantize one vector with a team of NW warps, thread g of the team owning the elements 8 g .. 8 g + 7.
-template <int KA, int NW>
-__device__ __forceinline__ void seq_quantize(const SeqParams& a, const float* x, const float* h, int vector, QuantScratch<KA, NW>& sc,
-                                             const QuantTeam& team, int& parity)
+// Quantize one vector with a team of warps, thread g of the team owning the elements EPT g .. EPT g + EPT - 1.
+template <int KA, int EPT>
+__device__ __forceinline__ void seq_quantize(const SeqParams& a, const float* x, const float* h, int vector,
+                                             QuantScratch<KA, SEQ_QUANT_WARPS>& sc, const QuantTeam& team, int& parity)
 {
-    const int n = a.p.n, g = team.warp * 32 + ((int)threadIdx.x & 31), t0 = g * SEQ_EPT;
-    float w[SEQ_EPT];
+    const int n = a.p.n, g = team.warp * 32 + ((int)threadIdx.x & 31), t0 = g * EPT;
+    float w[EPT];
     uint32_t valid = 0;
     const float* xr = x + (size_t)vector * a.xn;
     const float* hr = h + (size_t)vector * a.H - a.xn;
 #pragma unroll
-    for (int q = 0; q < SEQ_EPT / 4; ++q) {
+    for (int q = 0; q < EPT / 4; ++q) {
         const int t = t0 + 4 * q;
         const float* p = (t < a.xn ? xr : hr) + t;
         const bool one_piece = t + 3 < n && (t + 3 < a.xn || t >= a.xn) && (reinterpret_cast<uintptr_t>(p) & 15u) == 0;
@@ -96,12 +96,13 @@ __device__ __forceinline__ void seq_quantize(const SeqParams& a, const float* x,
     }
     float beta[KA];
     uint32_t bits[KA];
-    quantize_group<KA, SEQ_EPT, NW>(w, valid, n, quant_padding_consecutive(n, SEQ_EPT), a.T, beta, bits, sc, nullptr, &parity, team);
+    quantize_group<KA, EPT, SEQ_QUANT_WARPS>(w, valid, n, quant_padding_consecutive(n, EPT), a.T, beta, bits, sc, nullptr, &parity, team);
     const int wpr = a.p.wpr;
     if (t0 < wpr * 32) {
 #pragma unroll
         for (int i = 0; i < KA; ++i)
-            reinterpret_cast<uint8_t*>(a.zcodes + ((size_t)vector * KA + i) * wpr)[g] = (uint8_t)bits[i];
+            if (EPT == 8) reinterpret_cast<uint8_t*>(a.zcodes + ((size_t)vector * KA + i) * wpr)[g] = (uint8_t)bits[i];
+            else reinterpret_cast<uint16_t*>(a.zcodes + ((size_t)vector * KA + i) * wpr)[g] = (uint16_t)bits[i];
     }
     if (g < KA) {
         float b = beta[0];
@@ -113,149 +114,51 @@ __device__ __forceinline__ void seq_quantize(const SeqParams& a, const float* x,
 
 __device__ __forceinline__ float seq_logistic(float v) { return 1.0f / (1.0f + __expf(-v)); }
 
-// Epilogue over 32-unit blocks (lane quarter = gate): pre-activations meet in shared memory, then lane = unit, one vector per warp.
-template <int KA, int NG, typename AlphaOf>
-__device__ __forceinline__ bool seq_tiles32(const SeqParams& a, SeqShared& sh, float* sY, uint32_t tmem, int te, int tiles, int part, int b0,
-                                            int in_block, int t, int quarter, int sub, int rl, float next_alpha, const AlphaOf& alpha_of,
-                                            ResColumns<KA, NG>& col, ResDrainState& drain, const float* h_prev, const float* c_prev,
-                                            float* h_next, float* h_also, float* c_next)
+// The state update of one (unit, vector) from its staged pre-activations `yv` (gate g at yv[32 g]) and biases.
+__device__ __forceinline__ void seq_cell(const SeqParams& a, const float* yv, const float (&bias)[4], const float* addend, size_t o,
+                                         const float* h_prev, const float* c_prev, float* h_next, float* h_also, float* c_next)
 {
-    const ResProblem& p = a.p;
-    const int lane = te & 31, H = a.H;
-    for (int it = 0; it < tiles; ++it) {
-        float* sa = sh.alpha[it & 1];
-        sa[te] = next_alpha;
-        res_epi_bar(false);                         // (also: the constants; everybody is past the tile before last, whose buffer this is)
-        if (it == 0) {
-            col.load(p, sh.beta, sub, col.beta);
-            col.load(p, sh.row[p.cell == RES_GRU && quarter >= 2 ? quarter - 1 : 0], sub, col.row);
+    float g4[4], h;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) g4[g] = yv[32 * g] + bias[g];
+    if (a.p.cell == RES_LSTM) {
+        if (addend) {
+#pragma unroll
+            for (int g = 0; g < 4; ++g) g4[g] += __ldcg(addend + (size_t)g * a.H);
         }
-        if (it + 1 < tiles) next_alpha = alpha_of(it + 1);
-        const int u = (part + it * a.P) * 32 + lane;
-        float bias[4];
-#pragma unroll
-        for (int g = 0; g < 4; ++g) bias[g] = (a.bias && u < H) ? __ldg(a.bias + g * H + u) : 0.0f;
-        {
-            f32x2 y[NG][4];
-            if (!res_drain_tile<KA, NG>(p, sh.sync, sa, quarter, sub, tmem, col, drain, y)) return false;
-#pragma unroll
-            for (int g = 0; g < NG; ++g) {
-                const int e = (RES_EPI_SPLIT * g + sub) * 8 + 2 * (lane & 3);
-                if (e >= p.TB) break;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    float y0, y1;
-                    unpack2(y[g][i], y0, y1);
-                    sY[e * SEQ_Y_LD + rl + 8 * i] = y0;
-                    sY[(e + 1) * SEQ_Y_LD + rl + 8 * i] = y1;
-                }
-            }
-        }
-        res_epi_bar(false);
-        for (int e = te >> 5; e < in_block; e += RES_EPI_WARPS) {
-            if (u >= H) break;
-            const float* yv = sY + e * SEQ_Y_LD + lane;
-            const size_t o = (size_t)(b0 + e) * H + u;
-            float h;
-            if (p.cell == RES_LSTM) {
-                float g4[4];
-#pragma unroll
-                for (int g = 0; g < 4; ++g) g4[g] = yv[32 * g] + bias[g];
-                if (a.addend) {
-                    const float* ad = a.addend + ((size_t)t * p.batch + b0 + e) * 4 * H + u;
-#pragma unroll
-                    for (int g = 0; g < 4; ++g) g4[g] += __ldcg(ad + (size_t)g * H);
-                }
-                const float ig = seq_logistic(g4[0]), fg = seq_logistic(g4[1]), og = seq_logistic(g4[2]), gg = tanhf(g4[3]);
-                const float c = fg * __ldcg(c_prev + o) + ig * gg;
-                c_next[o] = c;
-                h = og * tanhf(c);
-            } else {
-                const float rg = seq_logistic(yv[0] + bias[0]), zg = seq_logistic(yv[32] + bias[1]);
-                const float cand = tanhf(yv[64] + bias[2] + rg * (yv[96] + bias[3]));
-                h = (1.0f - zg) * cand + zg * __ldcg(h_prev + o);
-            }
-            h_next[o] = h;
-            if (h_also) h_also[o] = h;
-        }
-        // (the next tile's values are staged behind the barrier inside its drain)
+        const float ig = seq_logistic(g4[0]), fg = seq_logistic(g4[1]), og = seq_logistic(g4[2]), gg = tanhf(g4[3]);
+        const float c = fg * __ldcg(c_prev + o) + ig * gg;
+        c_next[o] = c;
+        h = og * tanhf(c);
+    } else {
+        const float rg = seq_logistic(g4[0]), zg = seq_logistic(g4[1]), cand = tanhf(g4[2] + rg * g4[3]);
+        h = (1.0f - zg) * cand + zg * __ldcg(h_prev + o);
     }
-    return true;
+    h_next[o] = h;
+    if (h_also) h_also[o] = h;
 }
 
-// Epilogue over 128-unit blocks of a GRU: the gates r, n (h part), n (x part), z of a unit come to the same thread one after the other,
-// with one value per unit and vector kept between them.
-template <int KA, int NG, typename AlphaOf>
-__device__ __forceinline__ bool seq_tiles128(const SeqParams& a, SeqShared& sh, uint32_t tmem, int te, int tiles, int part, int b0, int t,
-                                             int quarter, int sub, int rl, float next_alpha, const AlphaOf& alpha_of,
-                                             ResColumns<KA, NG>& col, ResDrainState& drain, const float* h_prev, float* h_next, float* h_also)
-{
-    const ResProblem& p = a.p;
-    const int lane = te & 31, H = a.H;
-    (void)t;
-    float keep[NG][4][2];
-    for (int it = 0; it < tiles; ++it) {
-        const int tt = it & 3, unit0 = (part + (it >> 2) * a.P) * 128 + rl;
-        float* sa = sh.alpha[it & 1];
-        sa[te] = next_alpha;
-        res_epi_bar(false);
-        if (it == 0) col.load(p, sh.beta, sub, col.beta);
-        col.load(p, sh.row[tt == 1 ? 2 : tt == 2 ? 1 : 0], sub, col.row);
-        if (it + 1 < tiles) next_alpha = alpha_of(it + 1);
-        const int bias_row = (tt == 0 ? 0 : tt == 1 ? 3 : tt == 2 ? 2 : 1) * H;
-        float bias[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) bias[i] = (a.bias && unit0 + 8 * i < H) ? __ldg(a.bias + bias_row + unit0 + 8 * i) : 0.0f;
-        f32x2 y[NG][4];
-        if (!res_drain_tile<KA, NG>(p, sh.sync, sa, quarter, sub, tmem, col, drain, y)) return false;
-#pragma unroll
-        for (int g = 0; g < NG; ++g) {
-            const int b = b0 + (RES_EPI_SPLIT * g + sub) * 8 + 2 * (lane & 3);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                float v[2];
-                unpack2(y[g][i], v[0], v[1]);
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const float s = v[q] + bias[i];
-                    if (tt == 0) keep[g][i][q] = seq_logistic(s);
-                    else if (tt == 1) keep[g][i][q] *= s;
-                    else if (tt == 2) keep[g][i][q] = tanhf(s + keep[g][i][q]);
-                    else if (b + q < p.batch && (b + q - b0) < p.TB && unit0 + 8 * i < H) {
-                        const size_t o = (size_t)(b + q) * H + unit0 + 8 * i;
-                        const float zg = seq_logistic(s), h = (1.0f - zg) * keep[g][i][q] + zg * __ldcg(h_prev + o);
-                        h_next[o] = h;
-                        if (h_also) h_also[o] = h;
-                    }
-                }
-            }
-        }
-        __syncwarp();
-    }
-    return true;
-}
-
-template <int KA>
-__global__ void __launch_bounds__(RES_THREADS, 1)
+template <int KA, int EPT>
+__global__ void __launch_bounds__(R::THREADS, 1)
 rnn_batched_kernel(const __grid_constant__ SeqParams a)
 {
-    constexpr int NG = seq_ng(KA);
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     const ResProblem& p = a.p;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, H = a.H;
     const int bb = (int)blockIdx.x / a.P, part = (int)blockIdx.x - bb * a.P, b0 = bb * p.TB;
     const int in_block = p.batch - b0 < p.TB ? p.batch - b0 : p.TB;         // vectors of this block
     const int my_blocks = (a.unit_blocks - part + a.P - 1) / a.P, tiles = my_blocks * p.tpu;
     SeqShared& sh = *reinterpret_cast<SeqShared*>(smem_raw + a.b_bytes);
-    float* sY = reinterpret_cast<float*>(&sh + 1);                          // [TB][SEQ_Y_LD] (32-unit blocks)
-    unsigned char* quant_raw = reinterpret_cast<unsigned char*>(&sh + 1);   // the quantizer's scratch (the staged values are dead then)
+    float* sY = reinterpret_cast<float*>(&sh + 1);                          // [TB][SEQ_Y_LD] pre-activations of a tile
+    QuantScratch<KA, SEQ_QUANT_WARPS>* scratch = reinterpret_cast<QuantScratch<KA, SEQ_QUANT_WARPS>*>(&sh + 1);    // (they are dead then)
     const uint32_t sB = smem_u32(smem_raw);
     uint32_t* counter = a.counters + (size_t)bb * 64;
 
-    for (int q = tid; q < 512; q += RES_THREADS) sh.sum[0][q] = 0;
+#pragma unroll 1
+    for (int q = tid; q < 512; q += R::THREADS) sh.sum[0][q] = 0;
     res_fill_table(p, sh.table);
-    if (tid == 0) res_sync_init(sh.sync);
-    if (warp == RES_MMA_WARP) {
+    if (tid == 0) res_sync_init<R>(sh.sync);
+    if (warp == R::MMA_WARP) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      :: "r"(smem_u32(&sh.sync.tmem_slot)), "r"((uint32_t)RES_TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -266,87 +169,128 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
     const uint32_t tmem = __shfl_sync(0xffffffffu, sh.sync.tmem_slot, 0);
     if (warp < 4) res_write_scales(p, tmem, warp);
 
-    int steps_per_pass = 0;
-    for (int tt = 0; tt < p.tpu; ++tt) steps_per_pass += my_blocks * res_tile_steps(p, tt);
     int first_step = 0;                             // pipeline steps so far, mod the number of groups
     ResFeedState feed_state{warp >> 2, 1u};
     ResIssueState issue{0, 0, 0, 1};
     ResDrainState drain{0, 0};
-    const int teams = 32 / a.team_warps, team = warp / a.team_warps;
+    const int team = warp / a.team_warps, teams = SEQ_QUANT_WARPS / a.team_warps;
     const QuantTeam quant{warp - team * a.team_warps, 8 + team, a.team_warps * 32};
     int quant_parity = 0;
     bool ok = true;
 
+#pragma unroll 1
     for (int t = 0; t < a.steps; ++t) {
         const bool last = t + 1 == a.steps;
-        const float* h_prev = t == 0 ? a.h0 : (a.h_seq ? a.h_seq + (size_t)(t - 1) * p.batch * a.H : a.h[(t - 1) & 1]);
+        const float* h_prev = t == 0 ? a.h0 : (a.h_seq ? a.h_seq + (size_t)(t - 1) * p.batch * H : a.h[(t - 1) & 1]);
 
         // ---- 1. this CTA's share of the block's vectors ----
         if (t > 0) {
             if (tid == 0) ok = seq_wait(counter + 32, (uint32_t)(t * a.P));
             if (__syncthreads_or(!ok)) { ok = false; break; }
         }
-        {
+        if (warp < SEQ_QUANT_WARPS) {
             const float* x = a.x_seq + (size_t)t * p.batch * a.xn;
-            for (int v = part + team * a.P; v < in_block; v += teams * a.P) {
-                if (a.team_warps == 8)
-                    seq_quantize<KA, 8>(a, x, h_prev, b0 + v, reinterpret_cast<QuantScratch<KA, 8>*>(quant_raw)[team], quant, quant_parity);
-                else if (a.team_warps == 16)
-                    seq_quantize<KA, 16>(a, x, h_prev, b0 + v, reinterpret_cast<QuantScratch<KA, 16>*>(quant_raw)[team], quant, quant_parity);
-                else
-                    seq_quantize<KA, 32>(a, x, h_prev, b0 + v, *reinterpret_cast<QuantScratch<KA, 32>*>(quant_raw), quant, quant_parity);
-            }
+#pragma unroll 1
+            for (int v = part + team * a.P; v < in_block; v += teams * a.P)
+                seq_quantize<KA, EPT>(a, x, h_prev, b0 + v, scratch[team], quant, quant_parity);
         }
         __syncthreads();
-        if (tid == 0) seq_publish(counter);
+        if (tid == 0) {
+            seq_publish(counter);
+            ok = seq_wait(counter, (uint32_t)((t + 1) * a.P));
+        }
+        if (__syncthreads_or(!ok)) { ok = false; break; }
 
-        // the block's planes, once every share is there; ends with a CTA barrier.  False when a wait ran out.
-        auto load_block = [&]() {
-            bool there = true;
-            if (tid == 32 * RES_MMA_WARP) there = seq_wait(counter, (uint32_t)((t + 1) * a.P));
-            if (__syncthreads_or(!there)) return false;
-            for (int q = tid; q < p.N; q += RES_THREADS) {
-                const int b = b0 + res_row_vector<KA>(q), j = res_row_plane<KA>(q);
-                sh.beta[q] = q < p.TB * KA && b < p.batch ? __ldcg(a.zbeta + (size_t)b * KA + j) : 0.0f;
-            }
-            res_expand_activations<KA>(p, a.zcodes, b0, sB, sh.sum[0]);
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncthreads();
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            return true;
-        };
+        // ---- 2. the planes of the whole block as the activation operand ----
+        if (tid < p.N) {
+            const int b = b0 + res_row_vector<KA>(tid), j = res_row_plane<KA>(tid);
+            sh.beta[tid] = tid < p.TB * KA && b < p.batch ? __ldcg(a.zbeta + (size_t)b * KA + j) : 0.0f;
+        }
+        res_expand_activations<KA>(p, a.zcodes, b0, sB, sh.sum[0]);
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
-        // ---- 2. product, gates ----
-        if (warp < RES_EXP_WARPS) {
-            ResFeeder<RES_GRU> feed;
-            feed.start(p, sh.table, part, a.P, tiles, tid & 127, ((warp >> 2) - first_step + RES_GROUPS) % RES_GROUPS);
-            ok = load_block() && res_feed(p, sh.sync, sh.table, feed, tmem, feed_state);
-        } else if (warp == RES_MMA_WARP) {
-            ok = load_block() && res_issue(p, sh.sync, tiles, tmem, sB, issue);
-        } else if (warp > RES_MMA_WARP) {
-            ok = load_block();
-        } else {
-            const int te = tid - 32 * RES_EXP_WARPS, quarter = warp & 3, sub = (warp - RES_EXP_WARPS) >> 2, rl = quarter * 32 + (lane >> 2);
-            float* h_next = last ? a.h_last : (a.h_seq ? a.h_seq + (size_t)t * p.batch * a.H : a.h[t & 1]);
-            float* h_also = last && a.h_seq ? a.h_seq + (size_t)t * p.batch * a.H : nullptr;
+        // ---- 3. product, gates ----
+        if (warp < R::EXP_WARPS) {
+            ResFeeder<R, RES_GRU> feed;
+            feed.start(p, sh.table, part, a.P, tiles, tid & 127, ((warp >> 2) - first_step) & (R::GROUPS - 1));
+            ok = res_feed(p, sh.sync, sh.table, feed, tmem, feed_state);
+        } else if (warp == R::MMA_WARP) {
+            ok = res_issue(p, sh.sync, tiles, tmem, sB, issue);
+        } else if (warp < R::MMA_WARP) {
+            const int te = tid - 32 * R::EXP_WARPS, quarter = warp & 3, sub = (warp - R::EXP_WARPS) >> 2, rl = quarter * 32 + (lane >> 2);
+            float* h_next = last ? a.h_last : (a.h_seq ? a.h_seq + (size_t)t * p.batch * H : a.h[t & 1]);
+            float* h_also = last && a.h_seq ? a.h_seq + (size_t)t * p.batch * H : nullptr;
             const float* c_prev = t == 0 ? a.c0 : a.c;
             float* c_next = last ? a.c_last : a.c;
-            ResColumns<KA, NG> col;
-            auto alpha_of = [&](int it) {           // coefficient of plane te / 128, row te mod 128 of tile `it` of this CTA
-                const int row = res_row(p, part + (p.tpu == 4 ? it >> 2 : it) * a.P, p.tpu == 4 ? it & 3 : 0, te & 127), plane = te >> 7;
-                return plane < p.k_w && row >= 0 ? __ldg(p.Walpha + (size_t)row * p.k_w + plane) : 0.0f;
-            };
-            float next_alpha = alpha_of(0);
-            ok = load_block();
-            if (ok) res_row_constants(p, sh.sum[0], sh.row[0]);
-            if (p.tpu == 1)
-                ok = ok && seq_tiles32<KA, NG>(a, sh, sY, tmem, te, tiles, part, b0, in_block, t, quarter, sub, rl, next_alpha, alpha_of, col, drain,
-                                               h_prev, c_prev, h_next, h_also, c_next);
-            else
-                ok = ok && seq_tiles128<KA, NG>(a, sh, tmem, te, tiles, part, b0, t, quarter, sub, rl, next_alpha, alpha_of, col, drain,
-                                                h_prev, h_next, h_also);
+            res_row_constants<R>(p, sh.sum[0], sh.row[0]);
+            float keep[16];                         // 128-unit blocks: one value per (unit, vector) of this thread, from gate to gate
+#pragma unroll 1
+            for (int it = 0; it < tiles && ok; ++it) {
+                const int tt = p.tpu == 4 ? it & 3 : 0, ub = part + (p.tpu == 4 ? it >> 2 : it) * a.P;
+                float* sa = sh.alpha[it & 1];
+                {
+                    const int wr = res_row(p, ub, tt, te & 127);
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        const int plane = (te >> 7) + 2 * q;
+                        sa[plane * 128 + (te & 127)] = plane < p.k_w && wr >= 0 ? __ldg(p.Walpha + (size_t)wr * p.k_w + plane) : 0.0f;
+                    }
+                }
+                res_epi_bar<R>(false);              // (also: everybody is past the tile before last, whose buffer this is)
+                const int kind = p.cell != RES_GRU ? 0 : p.tpu == 4 ? (tt == 1 ? 2 : tt == 2 ? 1 : 0) : quarter >= 2 ? quarter - 1 : 0;
+                f32x2 y[SEQ_NG][4];
+                ok = res_drain_tile<R, KA, SEQ_NG>(p, sh.sync, sa, quarter, sub, tmem, sh.beta, sh.row[kind], drain, y);
+#pragma unroll
+                for (int g = 0; g < SEQ_NG; ++g) {
+                    const int e = (R::SPLIT * g + sub) * 8 + 2 * (lane & 3);
+                    if (e >= p.TB) break;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        float y0, y1;
+                        unpack2(y[g][i], y0, y1);
+                        sY[e * SEQ_Y_LD + rl + 8 * i] = y0;
+                        sY[(e + 1) * SEQ_Y_LD + rl + 8 * i] = y1;
+                    }
+                }
+                if (p.tpu == 1) {                   // lane quarter = gate: lane = unit, one vector per warp
+                    const int u = ub * 32 + lane;
+                    float bias[4];
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) bias[g] = (a.bias && u < H) ? __ldg(a.bias + g * H + u) : 0.0f;
+                    res_epi_bar<R>(false);
+                    const float* addend = a.addend ? a.addend + ((size_t)t * p.batch + b0) * 4 * H + u : nullptr;
+                    if (u < H) {
+#pragma unroll 1
+                        for (int e = te >> 5; e < in_block; e += R::EPI_WARPS)
+                            seq_cell(a, sY + e * SEQ_Y_LD + lane, bias, addend ? addend + (size_t)e * 4 * H : nullptr, (size_t)(b0 + e) * H + u,
+                                     h_prev, c_prev, h_next, h_also, c_next);
+                    }
+                } else {                            // the gates r, n (h part), n (x part), z of 128 units one after the other
+                    const int u = ub * 128 + (te & 127), bias_row = (tt == 0 ? 0 : tt == 1 ? 3 : tt == 2 ? 2 : 1) * H;
+                    const float bias = (a.bias && u < H) ? __ldg(a.bias + bias_row + u) : 0.0f;
+                    res_epi_bar<R>(false);
+#pragma unroll 1
+                    for (int e = te >> 7; e < in_block; e += 2) {
+                        const float s = sY[e * SEQ_Y_LD + (te & 127)] + bias;
+                        float k = keep[e >> 1];
+                        if (tt == 0) k = seq_logistic(s);
+                        else if (tt == 1) k *= s;
+                        else if (tt == 2) k = tanhf(s + k);
+                        else if (u < H) {
+                            const size_t o = (size_t)(b0 + e) * H + u;
+                            const float zg = seq_logistic(s), h = (1.0f - zg) * k + zg * __ldcg(h_prev + o);
+                            h_next[o] = h;
+                            if (h_also) h_also[o] = h;
+                        }
+                        keep[e >> 1] = k;
+                    }
+                }
+                __syncwarp();                       // (the next tile's values are staged behind the barrier inside its drain)
+            }
         }
-        first_step = (first_step + steps_per_pass) % RES_GROUPS;
+        first_step = (first_step + my_blocks * a.unit_steps) & (R::GROUPS - 1);
         if (__syncthreads_or(!ok)) { ok = false; break; }
         if (tid == 0 && !last) seq_publish(counter + 32);
     }
@@ -359,19 +303,17 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
         __nanosleep(1000000);
         __syncthreads();
     }
-    if (warp == RES_MMA_WARP)
+    if (warp == R::MMA_WARP)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"((uint32_t)RES_TMEM_COLS) : "memory");
 }
 
 struct SeqPlan { SeqParams a; int grid; size_t smem; };
 
-size_t seq_more_smem(const ResProblem& p, int k_a)
+size_t seq_more_smem(const ResProblem& p)
 {
-    // the staged pre-activations of a 32-unit block; the quantizer's scratch uses the same bytes
-    const size_t scratch = k_a == 4 ? 8192 : 6144;
-    static_assert(4 * sizeof(QuantScratch<4, 8>) <= 8192 && 2 * sizeof(QuantScratch<4, 16>) <= 8192 && sizeof(QuantScratch<4, 32>) <= 8192, "");
-    static_assert(4 * sizeof(QuantScratch<3, 8>) <= 6144 && 2 * sizeof(QuantScratch<3, 16>) <= 6144 && sizeof(QuantScratch<3, 32>) <= 6144, "");
-    const size_t y = p.tpu == 1 ? (size_t)p.TB * SEQ_Y_LD * 4 : 0;
+    // the staged pre-activations; the quantizer's scratch uses the same bytes
+    constexpr size_t scratch = 2 * sizeof(QuantScratch<4, SEQ_QUANT_WARPS>);
+    const size_t y = (size_t)p.TB * SEQ_Y_LD * 4;
     return sizeof(SeqShared) + (y > scratch ? y : scratch);
 }
 
@@ -380,7 +322,7 @@ bool plan(const BatchedSequence& s, SeqPlan* out)
     if (s.batch < 2 || s.H < 1 || s.n > AMQ_MAX_N || (s.gru && s.I < 1)) return false;
     const int sms = res_sm_count();
     SeqParams a{};
-    a.team_warps = s.n <= 2048 ? 8 : s.n <= 4096 ? 16 : 32;
+    a.team_warps = s.n <= 2048 ? 8 : 16;
     ResProblem p{};
     p.W = s.Wcodes; p.Walpha = s.Walpha; p.k_w = s.k_w; p.wpr = words_per_row(s.n);
     p.vec32 = p.wpr % 8 == 0 && (reinterpret_cast<uintptr_t>(s.Wcodes) & 31) == 0;
@@ -395,18 +337,18 @@ bool plan(const BatchedSequence& s, SeqPlan* out)
     // the weight steps that 32-unit blocks spend on the zero halves of the candidate rows, 32-unit blocks divide more finely.
     double best = 0.0;
     for (int wide = 0; wide <= (s.gru ? 1 : 0); ++wide)
-        for (int TB = 8; TB <= 8 * seq_ng(s.k_a) * RES_EPI_SPLIT; TB += 8) {
+        for (int TB = 8; TB <= 8 * SEQ_NG * R::SPLIT; TB += 8) {
             ResProblem q = p;
             q.ut = wide ? 128 : 32; q.tpu = wide ? 4 : 1; q.TB = TB;
-            if (!res_set_block(q, TB, s.k_a, seq_more_smem(q, s.k_a))) break;
+            if (!res_set_block<R>(q, TB, s.k_a, seq_more_smem(q))) break;
             const int blocks = (s.batch + TB - 1) / TB, ub = (s.H + q.ut - 1) / q.ut;
             if (blocks > sms) continue;
             const int P = ub < sms / blocks ? ub : sms / blocks, per_cta = (ub + P - 1) / P;
-            const double steps = wide ? 2.0 * ((q.NS + 1) / 2) + (q.nx + 1) / 2 + (q.NS - q.nx + 1) / 2 : (q.NS + 1) / 2;
-            const int vectors = (TB + P - 1) / P, teams = 32 / a.team_warps;
-            const double t = per_cta * (steps * 2 * q.k_w * res_slot_clocks(q) + 1500.0 * q.tpu) + (double)q.N * q.NS * 128 / 60.0 +
+            const int steps = q.k_w * (wide ? 2 * ((q.NS + 1) / 2) + (q.nx + 1) / 2 + (q.NS - q.nx + 1) / 2 : (q.NS + 1) / 2);
+            const int vectors = (TB + P - 1) / P, teams = SEQ_QUANT_WARPS / a.team_warps;
+            const double t = per_cta * (steps * 2 * res_slot_clocks(q) + 1500.0 * q.tpu) + (double)q.N * q.NS * 128 / 60.0 +
                              (vectors + teams - 1) / teams * (s.k_a >= 3 ? 4500.0 : 3500.0);
-            if (best == 0.0 || t < best) { best = t; a.p = q; a.P = P; a.unit_blocks = ub; }
+            if (best == 0.0 || t < best) { best = t; a.p = q; a.P = P; a.unit_blocks = ub; a.unit_steps = steps; }
             if (TB >= s.batch) break;
         }
     if (best == 0.0) return false;
@@ -417,7 +359,7 @@ bool plan(const BatchedSequence& s, SeqPlan* out)
     a.h[0] = s.h[0]; a.h[1] = s.h[1]; a.c = s.c; a.addend = s.addend;
     a.zcodes = s.zcodes; a.zbeta = s.zbeta; a.counters = s.counters; a.status = s.status;
     out->grid = blocks * a.P;
-    out->smem = (size_t)a.b_bytes + seq_more_smem(a.p, s.k_a);
+    out->smem = (size_t)a.b_bytes + seq_more_smem(a.p);
     out->a = a;
     return true;
 }
@@ -425,11 +367,11 @@ bool plan(const BatchedSequence& s, SeqPlan* out)
 template <int KA>
 amq_status launch(const SeqPlan& pl, cudaStream_t st)
 {
-    auto kernel = rnn_batched_kernel<KA>;
+    auto kernel = pl.a.p.n <= 4096 ? rnn_batched_kernel<KA, 8> : rnn_batched_kernel<KA, 16>;
     AMQ_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem));
     SeqParams args = pl.a;
     void* params[] = {&args};
-    AMQ_CUDA_TRY(cudaLaunchCooperativeKernel((void*)kernel, dim3((unsigned)pl.grid), dim3(RES_THREADS), params, pl.smem, st));
+    AMQ_CUDA_TRY(cudaLaunchCooperativeKernel((void*)kernel, dim3((unsigned)pl.grid), dim3(R::THREADS), params, pl.smem, st));
     __atomic_fetch_add(&g_kernel_launches, 1ull, __ATOMIC_RELAXED);
     return AMQ_OK;
 }

@@ -30,6 +30,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
 // bounded wait of the single MMA-issuing thread; false when it ran out
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
 {
+#pragma unroll 1
     for (unsigned i = 0; i < WAIT_LIMIT; ++i)
         if (mbar_try_wait(bar, parity)) return true;
     return false;
@@ -40,6 +41,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
 __device__ __forceinline__ bool mbar_wait_relaxed(uint32_t bar, uint32_t parity)
 {
     if (mbar_try_wait(bar, parity)) return true;
+#pragma unroll 1
     for (unsigned i = 0; i < WAIT_LIMIT; ++i) {
         __nanosleep(40);
         if (mbar_try_wait(bar, parity)) return true;
@@ -52,6 +54,7 @@ __device__ __forceinline__ bool mbar_wait_relaxed(uint32_t bar, uint32_t parity)
 __device__ __forceinline__ bool mbar_wait_relaxed(uint32_t bar, uint32_t parity, const volatile int* failed)
 {
     if (mbar_try_wait(bar, parity)) return true;
+#pragma unroll 1
     for (unsigned i = 0; i < WAIT_LIMIT && !*failed; ++i) {
         __nanosleep(40);
         if (mbar_try_wait(bar, parity)) return true;
