@@ -39,14 +39,12 @@ namespace amq {
 
 constexpr int QUANT_MAX_WARPS = 16;
 
-// Shared-memory scratch of one group of NW warps (NW = 1: a single warp, which needs the level scratch only).
+// Shared-memory scratch of one group of NW warps (NW = 1: a single warp, which needs none).
 template <int K, int NW>
 struct __align__(16) QuantScratch {
     static constexpr int V = 1 + K + K * (K - 1) / 2;
     static constexpr int SLOTS = NW > 1 ? ((NW + 3) / 4) * 4 : 4;
     float red[2][V][SLOTS];             // [reduction parity][value][warp]: per-warp partial sums
-    float level[NW][1 << K];            // per-warp scratch of the level sort (k >= 3)
-    int code[NW][1 << K];
 };
 
 // The threads of a group of several warps: the whole CTA, or some consecutive warps of it with a hardware barrier of their own.
@@ -75,6 +73,39 @@ __device__ __forceinline__ void quant_scratch_init(QuantScratch<K, NW>& sc, cons
         if ((idx % SLOTS) >= warps) flat[idx] = 0.0f;
 }
 
+// Sums over the warp of VF floats, every lane gets all of them.  Four values at a time are reduced and scattered over the lanes at
+// once (2 + 1 + 3 shuffles instead of 20) and gathered again; the additions pair the same lanes in the same order as a butterfly
+// over distances 16, 8, 4, 2, 1 on each value, so the result is that butterfly's bit for bit.
+template <int VF>
+__device__ __forceinline__ void warp_sums(float (&f)[VF], int lane, bool gather)
+{
+    constexpr unsigned ALL = 0xffffffffu;
+#pragma unroll
+    for (int i = 0; i + 2 < VF; i += 4) {           // three or four values (a missing one rides along as a copy)
+        const float v0 = f[i], v1 = f[i + 1], v2 = f[i + 2], v3 = i + 3 < VF ? f[i + 3 < VF ? i + 3 : 0] : 0.0f;
+        const bool up16 = (lane & 16) != 0, up8 = (lane & 8) != 0;
+        float a = up16 ? v2 : v0, b = up16 ? v3 : v1;               // kept by this half
+        a += __shfl_xor_sync(ALL, up16 ? v0 : v2, 16);
+        b += __shfl_xor_sync(ALL, up16 ? v1 : v3, 16);
+        float c = up8 ? b : a;
+        c += __shfl_xor_sync(ALL, up8 ? a : b, 8);
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) c += __shfl_xor_sync(ALL, c, off);
+        if (gather) {
+            f[i] = __shfl_sync(ALL, c, 0); f[i + 1] = __shfl_sync(ALL, c, 8); f[i + 2] = __shfl_sync(ALL, c, 16);
+            if (i + 3 < VF) f[i + 3 < VF ? i + 3 : 0] = __shfl_sync(ALL, c, 24);
+        } else {
+            f[i] = c;                               // value i + lane / 8
+        }
+    }
+    constexpr int REST = VF % 4 == 3 ? 0 : VF % 4;
+#pragma unroll
+    for (int i = VF - REST; i < VF; ++i) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) f[i] += __shfl_xor_sync(ALL, f[i], off);
+    }
+}
+
 // Totals over the group of VF floats and VI ints (ints are carried exactly); every thread of the group holds
 // them afterwards.  NW > 1: the group is a team and the call contains exactly one barrier of it; when `flag`
 // is given, that barrier also ORs *flag over the team (every thread gets the result).
@@ -82,47 +113,57 @@ template <int VF, int VI, int K, int NW>
 __device__ __forceinline__ void group_totals(float (&f)[VF], int (&iv)[VI > 0 ? VI : 1], QuantScratch<K, NW>& sc,
                                              int parity, int* flag, const QuantTeam& team)
 {
-#pragma unroll
-    for (int i = 0; i < VF; ++i) {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) f[i] += __shfl_xor_sync(0xffffffffu, f[i], off);
-    }
+    const int lane = threadIdx.x & 31;
+    warp_sums<VF>(f, lane, NW == 1);
 #pragma unroll
     for (int i = 0; i < VI; ++i) iv[i] = __reduce_add_sync(0xffffffffu, iv[i]);
     if (NW == 1) return;
     constexpr int SLOTS = QuantScratch<K, NW>::SLOTS;
-    const int warp = team.warp, lane = threadIdx.x & 31;
+    const int warp = team.warp;
+    constexpr int FULL = VF % 4 == 3 ? VF : VF / 4 * 4;             // values that were reduced in fours
+    if ((lane & 7) == 0) {
+#pragma unroll
+        for (int i = 0; i < FULL; i += 4)
+            if (i + 3 < VF || lane < 24) sc.red[parity][i + (lane >> 3)][warp] = f[i];
+    }
     if (lane == 0) {
 #pragma unroll
-        for (int i = 0; i < VF; ++i) sc.red[parity][i][warp] = f[i];
+        for (int i = FULL; i < VF; ++i) sc.red[parity][i][warp] = f[i];
 #pragma unroll
         for (int i = 0; i < VI; ++i) sc.red[parity][VF + i][warp] = __int_as_float(iv[i]);
     }
     if (flag) *flag = team.sync_or(*flag);
     else team.sync();
-    // every thread: the partials of all warps, added in a fixed tree (slots of absent warps hold zeros)
+    // Every warp adds up the partials of all warps: eight lanes per value, each with the partial of one warp or of two neighbours
+    // (teams of up to sixteen warps), a butterfly over distances 1, 2, 4, and one shuffle per value to hand the total to all lanes.
+    // (Every thread reading every partial itself took 14 to 28 128-bit loads per reduction, most of its 1300 to 2000 clocks.)
+    static_assert(SLOTS <= 16, "two partials per lane");
+    const bool two = team.threads > 256;
+    auto partial = [&](int value) {
+        const float* r = sc.red[parity][value];
+        return two ? *reinterpret_cast<const float2*>(r + 2 * (lane & 7)) : make_float2((lane & 7) < SLOTS ? r[lane & 7] : 0.0f, 0.0f);
+    };
 #pragma unroll
-    for (int i = 0; i < VF; ++i) {
-        float tot = 0.0f;
+    for (int i = 0; i < VF; i += 4) {
+        const int v = i + (lane >> 3) < VF ? i + (lane >> 3) : VF - 1;
+        const float2 q = partial(v);
+        float c = two ? q.x + q.y : q.x;
 #pragma unroll
-        for (int q = 0; q < SLOTS / 4; ++q) {
-            if (q > 0 && 4 * q >= team.threads >> 5) break;         // (slots of warps that a smaller team does not have)
-            const float4 v = *reinterpret_cast<const float4*>(&sc.red[parity][i][4 * q]);
-            const float s = (v.x + v.y) + (v.z + v.w);
-            tot = (q == 0) ? s : tot + s;
-        }
-        f[i] = tot;
+        for (int off = 1; off < 8; off <<= 1) c += __shfl_xor_sync(0xffffffffu, c, off);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (i + k < VF) f[i + k < VF ? i + k : 0] = __shfl_sync(0xffffffffu, c, 8 * k);
     }
 #pragma unroll
-    for (int i = 0; i < VI; ++i) {
-        int tot = 0;
+    for (int i = 0; i < VI; i += 4) {
+        const int v = i + (lane >> 3) < VI ? i + (lane >> 3) : VI - 1;
+        const float2 q = partial(VF + v);
+        int c = __float_as_int(q.x) + (two ? __float_as_int(q.y) : 0);
 #pragma unroll
-        for (int q = 0; q < SLOTS / 4; ++q) {
-            if (q > 0 && 4 * q >= team.threads >> 5) break;
-            const int4 v = *reinterpret_cast<const int4*>(&sc.red[parity][VF + i][4 * q]);
-            tot += (v.x + v.y) + (v.z + v.w);
-        }
-        iv[i] = tot;
+        for (int off = 1; off < 8; off <<= 1) c += __shfl_xor_sync(0xffffffffu, c, off);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (i + k < VI) iv[i + k < VI ? i + k : 0] = __shfl_sync(0xffffffffu, c, 8 * k);
     }
 }
 
@@ -169,7 +210,11 @@ __device__ __forceinline__ bool solve_refit(const float (&c)[K], const int (&gra
         const double tiny = 1e-9 * n_;
         const double pivot2n = fmax(fabs(A22), fabs(A12));          // n x the second pivot
         if (!(pivot2n >= tiny * n_) || !(fabs(det) >= tiny * pivot2n)) return false;
-        const double rd = 1.0 / det;
+        // reciprocal of the determinant (an integer below 2^40 in magnitude): the fp32 one, refined by two Newton steps r (2 - d r) in
+        // fp64, a fifth of the latency of the fp64 division (the solve is on the critical path of every vector)
+        double rd = (double)__fdividef(1.0f, (float)det);
+        rd = fma(rd, fma(-det, rd, 1.0), rd);
+        rd = fma(rd, fma(-det, rd, 1.0), rd);
         const double c0 = (double)c[0], c1 = (double)c[1], c2 = (double)c[2];
         a[0] = (float)((A00 * c0 + A01 * c1 + A02 * c2) * rd);
         a[1] = (float)((A01 * c0 + A11 * c1 + A12 * c2) * rd);
@@ -223,114 +268,91 @@ __device__ __forceinline__ bool solve_refit(const float (&c)[K], const int (&gra
     return true;
 }
 
-// Per-plane bit tables of the sorted code table: bit p of plane[i] = sign (1 = +1) of plane i at level p.
+// Levels that already ascend by code index (K >= 3): the usual case, a_1 > a_2 + a_3 (+ ..) > .. > 0, in which code bit i of an element
+// is the i-th decision of the tree itself and no level has to be ranked.  v and -v are levels together and round alike, so the
+// table is antisymmetric about its middle: the upper half decides, and the midpoints come out as the general table's, bit for bit.
+// Fills the upper midpoints thr[2^(K-1) - 1 ..] and returns whether the levels do ascend.
 template <int K>
-__device__ __forceinline__ void planes_from_table(unsigned long long table, uint32_t (&plane)[K])
-{
-#pragma unroll
-    for (int i = 0; i < K; ++i) plane[i] = 0u;
-#pragma unroll
-    for (int p = 0; p < (1 << K); ++p) {
-        const uint32_t code = (uint32_t)(table >> (4 * p)) & 15u;
-#pragma unroll
-        for (int i = 0; i < K; ++i) plane[i] |= ((code >> (K - 1 - i)) & 1u) << p;
-    }
-}
-
-// Ascending level table of the 2^K values sum_i +-alpha_i, ordered by (value, code index), plane 0 the most
-// significant code bit.  Produces the 2^K - 1 midpoints and, per plane, the signs along the table (bit p of
-// plane[i]: sign, 1 = +1, of plane i at sorted level p).
-// Executed by one full warp (K >= 3 uses its lanes, __syncwarp and the warp's own scratch rows).
-template <int K>
-__device__ __forceinline__ void level_table(const float (&alpha)[K], int lane, float (&thr)[(1 << K) - 1],
-                                            uint32_t (&plane)[K], float* sc_level, int* sc_code)
+__device__ __forceinline__ bool ascending_levels(const float (&alpha)[K], float (&thr)[(1 << K) - 1])
 {
     constexpr int M = 1 << K;
-    unsigned long long table = 0ull;          // codes packed 4 bits per table position (K != 2)
-    if (K == 1) {
-        // levels -a, +a (or swapped when a < 0); the midpoint is 0 either way
-        thr[0] = (-alpha[0] + alpha[0]) * 0.5f;
-        table = (alpha[0] < 0.0f) ? 0x01ull : 0x10ull;
-        planes_from_table<K>(table, plane);
-        return;
+    float v[M / 2];
+#pragma unroll
+    for (int c = 0; c < M / 2; ++c) {
+        float s = alpha[0];
+#pragma unroll
+        for (int i = 1; i < K; ++i) s += ((c >> (K - 1 - i)) & 1) ? alpha[i] : -alpha[i];
+        v[c] = s;
     }
-    if (K == 2) {
-        // The four levels +-a +-b in closed form.  With A = |a|, B = |b| the ascending values are
-        // -(A+B), -|A-B|, +|A-B|, A+B, so the midpoints are -(fl(A+B) + |fl(A-B)|)/2, 0 and its negative
-        // (exactly what sorting the four rounded sums gives).  In terms of the magnitudes the sign patterns
-        // come in the order (-,-) (-,+) (+,-) (+,+) when A > B and (-,-) (+,-) (-,+) (+,+) when A < B; a
-        // negative coefficient flips its own bit of every code.  Equal values are ordered by code index:
-        // A == B ties the two middle levels (the first order is the ascending one unless a < 0); a coefficient
-        // that is zero, or vanishes against the other in fp32, ties the outer pairs, and its bit then ascends.
-        const float a = alpha[0], b = alpha[1];
-        const float A = fabsf(a), B = fabsf(b);
-        const float d = A - B;
-        const float t0 = -0.5f * ((A + B) + fabsf(d));
-        thr[0] = t0; thr[1] = 0.0f; thr[2] = -t0;
-        bool sa = a < 0.0f, sb = b < 0.0f;
-        const bool first = d > 0.0f || (d == 0.0f && !sa);
-        if ((A + B) == fabsf(d)) {            // the smaller coefficient vanishes in the sums: its sign orders nothing
-            if (first) sb = false; else sa = false;
-        }
-        plane[0] = (first ? 0xCu : 0xAu) ^ (sa ? 0xFu : 0u);      // bit p: sign of plane 0 at level p
-        plane[K - 1] = (first ? 0xAu : 0xCu) ^ (sb ? 0xFu : 0u);
-        return;
+    bool up = v[0] >= 0.0f;
+    thr[M / 2 - 1] = 0.0f;
+#pragma unroll
+    for (int c = 0; c + 1 < M / 2; ++c) {
+        up = up && v[c] <= v[c + 1];
+        thr[M / 2 + c] = (v[c] + v[c + 1]) * 0.5f;
     }
-    // K >= 3: lane c < 2^K ranks its own level among all, through shared memory
-    __syncwarp();
-    if (lane < M) {
-        float mine = 0.0f;
-#pragma unroll
-        for (int i = 0; i < K; ++i) mine += ((lane >> (K - 1 - i)) & 1) ? alpha[i] : -alpha[i];
-        int rank = 0;
-#pragma unroll
-        for (int c = 0; c < M; ++c) {
-            float v = 0.0f;
-#pragma unroll
-            for (int i = 0; i < K; ++i) v += ((c >> (K - 1 - i)) & 1) ? alpha[i] : -alpha[i];
-            rank += (v < mine || (v == mine && c < lane)) ? 1 : 0;
-        }
-        sc_level[rank] = mine;
-        sc_code[rank] = lane;
-    }
-    __syncwarp();
-#pragma unroll
-    for (int p = 0; p < M - 1; ++p) thr[p] = (sc_level[p] + sc_level[p + 1]) * 0.5f;
-    // bit p of plane[i] = sign of plane i in the code at sorted position p: lane p holds that code, one ballot per plane
-    // (the same masks as planes_from_table builds from the packed table, in a tenth of the instructions)
-    const int code = lane < M ? sc_code[lane] : 0;
-#pragma unroll
-    for (int i = 0; i < K; ++i) plane[i] = __ballot_sync(0xffffffffu, ((code >> (K - 1 - i)) & 1) != 0);
-    (void)table;
+    return up;
 }
 
-// Algorithm 1 for one element: index of the leaf (sorted level) the descent over the midpoints reaches.
-// The midpoints are non-decreasing; ">=" goes to the upper half.
+// The same for any coefficients, K >= 3: of every pair of levels v, -v the one in the upper half of the table (at v = 0 the one of the
+// larger code index), sorted by (value, code index); its codes and the upper midpoints.
 template <int K>
-__device__ __forceinline__ int bst_leaf(float x, const float (&thr)[(1 << K) - 1])
+__device__ __forceinline__ void upper_levels(const float (&alpha)[K], float (&thr)[(1 << K) - 1], uint32_t (&code)[1 << (K - 1)])
 {
-    if (K == 1) return (x >= thr[0]) ? 1 : 0;
-    if (K == 2) {
-        const bool c1 = x >= thr[1];
-        const bool c2 = x >= (c1 ? thr[2] : thr[0]);
-        return (c1 ? 2 : 0) + (c2 ? 1 : 0);
+    constexpr int M = 1 << K, M2 = M / 2;
+    float v[M2];
+#pragma unroll
+    for (int c = 0; c < M2; ++c) {
+        float s = alpha[0];
+#pragma unroll
+        for (int i = 1; i < K; ++i) s += ((c >> (K - 1 - i)) & 1) ? alpha[i] : -alpha[i];
+        const bool flip = s < 0.0f;                 // (code M2 + c is the larger index of its pair)
+        v[c] = flip ? -s : s;
+        code[c] = flip ? (uint32_t)(M2 - 1 - c) : (uint32_t)(M2 + c);
     }
-    if (K == 3) {
-        const bool c1 = x >= thr[3];
-        const bool c2 = x >= (c1 ? thr[5] : thr[1]);
-        const float hi = c2 ? thr[6] : thr[4], lo = c2 ? thr[2] : thr[0];
-        const bool c3 = x >= (c1 ? hi : lo);
-        return (c1 ? 4 : 0) + (c2 ? 2 : 0) + (c3 ? 1 : 0);
+    auto order = [&](int i, int j) {                // compare and exchange
+        const bool swap = v[i] > v[j] || (v[i] == v[j] && code[i] > code[j]);
+        const float a = v[i], b = v[j];
+        const uint32_t ca = code[i], cb = code[j];
+        v[i] = swap ? b : a; v[j] = swap ? a : b;
+        code[i] = swap ? cb : ca; code[j] = swap ? ca : cb;
+    };
+    // odd-even merge sort of four, or of twice four
+#pragma unroll
+    for (int h = 0; h < M2; h += 4) { order(h, h + 1); order(h + 2, h + 3); order(h, h + 2); order(h + 1, h + 3); order(h + 1, h + 2); }
+    if constexpr (K == 4) {
+        order(0, M2 - 4); order(1, M2 - 3); order(2, M2 - 2); order(3, M2 - 1);
+        order(2, M2 - 4); order(3, M2 - 3);
+        order(1, 2); order(3, M2 - 4); order(M2 - 3, M2 - 2);
     }
-    const bool c1 = x >= thr[7];
-    const bool c2 = x >= (c1 ? thr[11] : thr[3]);
-    const float hi3 = c2 ? thr[13] : thr[9], lo3 = c2 ? thr[5] : thr[1];
-    const bool c3 = x >= (c1 ? hi3 : lo3);
-    const float q3 = c3 ? thr[14] : thr[12], q2 = c3 ? thr[10] : thr[8];
-    const float q1 = c3 ? thr[6] : thr[4], q0 = c3 ? thr[2] : thr[0];
-    const float hi4 = c2 ? q3 : q2, lo4 = c2 ? q1 : q0;
-    const bool c4 = x >= (c1 ? hi4 : lo4);
-    return (c1 ? 8 : 0) + (c2 ? 4 : 0) + (c3 ? 2 : 0) + (c4 ? 1 : 0);
+    thr[M2 - 1] = 0.0f;
+#pragma unroll
+    for (int c = 0; c + 1 < M2; ++c) thr[M2 + c] = (v[c] + v[c + 1]) * 0.5f;
+}
+
+// Algorithm 1 for one element, K >= 3, over an antisymmetric table: decision i compares w with the midpoint of the half, quarter, .. it
+// is in (">=" goes up); d[i] = w minus that midpoint, whose sign bit is the inverted decision, collected in below[i] (i >= 1; decision 0
+// is the sign of w).  The midpoints of the lower half are the negatives of the upper ones.
+template <int K, int EPT>
+__device__ __forceinline__ void tree_decisions(float w, const float (&thr)[(1 << K) - 1], uint32_t (&below)[K], uint32_t* d = nullptr)
+{
+    constexpr int M = 1 << K, M2 = M / 2;
+    constexpr uint32_t SIGN = 0x80000000u;
+    const uint32_t wb = __float_as_uint(w), sw = wb & SIGN;
+    const uint32_t d1 = __float_as_uint(w - __uint_as_float(__float_as_uint(thr[M2 - 1 + M2 / 2]) | sw));
+    const bool out1 = (int)(wb ^ d1) >= 0;          // the decision agrees with the sign: outer part of the half
+    const float t2 = out1 ? thr[M2 - 1 + M2 / 2 + M2 / 4] : thr[M2 - 1 + M2 / 4];
+    const uint32_t d2 = __float_as_uint(w - __uint_as_float(__float_as_uint(t2) | sw));
+    below[1] = __funnelshift_l(d1, below[1], 1);
+    below[2] = __funnelshift_l(d2, below[2], 1);
+    if (d) { d[1] = d1; d[2] = d2; }
+    if constexpr (K == 4) {
+        const bool out2 = (int)(wb ^ d2) >= 0;
+        const float hi = out2 ? thr[M - 2] : thr[M - 4], lo = out2 ? thr[M2 + 2] : thr[M2];
+        const uint32_t d3 = __float_as_uint(w - __uint_as_float(__float_as_uint(out1 ? hi : lo) | sw));
+        below[K - 1] = __funnelshift_l(d3, below[K - 1], 1);
+        if (d) d[K - 1] = d3;
+    }
 }
 
 // Elements past the end of the vector inside the threads that do hold some of it, for the two ownership patterns in
@@ -360,8 +382,6 @@ __device__ __forceinline__ void quantize_group(const float (&w_in)[EPT], uint32_
     constexpr int M = 1 << K;
     constexpr int NG = K * (K - 1) / 2;
     constexpr uint32_t SIGN = 0x80000000u;
-    const int lane = threadIdx.x & 31;
-    const int slot = NW > 1 ? team.warp : 0;
     const int nvalid = __popc(valid);
     const float inv_n = 1.0f / (float)n;
     const float padding = (float)pad_elems;                      // zero elements past the end that are summed along
@@ -373,7 +393,8 @@ __device__ __forceinline__ void quantize_group(const float (&w_in)[EPT], uint32_
     for (int j = 0; j < EPT; ++j) w[j] = w_in[j] + 0.0f;          // -0.0 -> +0.0: from here on "x >= 0" is "sign bit clear"
 
     // ---- greedy initialisation, Eq. 3-4 (and, for T > 0, B^T w of the first refit in the same pass) ----
-    float last_abs = 0.0f, csum[K];
+    float last_abs = 0.0f, csum[K], abs_w = 0.0f;                 // abs_w: this thread's sum |w|
+    uint32_t positive = 0;                                        // bit j: w[j] >= 0
     float rho = 0.0f;                                             // residue of a zero element (the padding)
     {
         float r[EPT];
@@ -388,10 +409,12 @@ __device__ __forceinline__ void quantize_group(const float (&w_in)[EPT], uint32_
                 const uint32_t rb = __float_as_uint(r[j]);
                 part += fabsf(r[j]);
                 neg = __funnelshift_l(rb, neg, 1);                // sign bit of r[j] enters at bit 0
-                cs += __uint_as_float(__float_as_uint(w[j]) ^ (rb & SIGN));        // b_i * w
+                if (i > 0) cs += __uint_as_float(__float_as_uint(w[j]) ^ (rb & SIGN));     // b_i * w (i = 0: |w|)
             }
             bits[i] = ~neg & valid;
-            csum[i] = cs;
+            if (i == 0) positive = ~neg;
+            csum[i] = i > 0 ? cs : part;
+            if (i == 0) abs_w = part;
             part = holds_some ? part : 0.0f;
             if (i == K - 1 && T > 0) { last_abs = part; alpha[i] = 0.0f; break; }
             float tot[1] = {part};
@@ -430,34 +453,111 @@ __device__ __forceinline__ void quantize_group(const float (&w_in)[EPT], uint32_
         flag = nullptr;
         parity ^= 1;
         float thr[M - 1];
-        uint32_t plane[K];
         {
             if (it == 0) alpha[K - 1] = (fsum[0] - padding * fabsf(rho)) * inv_n;   // the last greedy coefficient
             float c[K];
 #pragma unroll
             for (int i = 0; i < K; ++i) c[i] = fsum[1 + i];
             solve_refit<K>(c, gram, n, alpha);
-            level_table<K>(alpha, lane, thr, plane, sc.level[slot], sc.code[slot]);
         }
         last_abs = 0.0f;
-
-        // Algorithm 1 for every element; the sums B^T w of the next refit are taken in the same pass
         const bool more = it + 1 < T;
-        uint32_t pos_bits[K];
+
+        if constexpr (K == 1) {
+            // levels -a, a: the sign plane, or its opposite for a < 0
+            bits[0] = (alpha[0] < 0.0f ? ~positive : positive) & valid;
+            csum[0] = alpha[0] < 0.0f ? -abs_w : abs_w;
+            continue;
+        }
+        if constexpr (K == 2) {
+            // The closed form of level_table, with the tree's two decisions as words of bits: the sign of w, and w against the
+            // midpoint of its half.  Which plane is which decision, and its sign, follow from the coefficients.
+            const float A = fabsf(alpha[0]), B = fabsf(alpha[K - 1]), d = A - B;
+            const uint32_t mid = __float_as_uint(0.5f * ((A + B) + fabsf(d)));         // >= 0
+            bool sa = alpha[0] < 0.0f, sb = alpha[K - 1] < 0.0f;
+            const bool first = d > 0.0f || (d == 0.0f && !sa);
+            if ((A + B) == fabsf(d)) { if (first) sb = false; else sa = false; }
+            uint32_t below = 0;
+            float s1 = 0.0f;
 #pragma unroll
-        for (int i = 0; i < K; ++i) { pos_bits[i] = 0u; csum[i] = 0.0f; }
+            for (int j = EPT - 1; j >= 0; --j) {
+                const uint32_t wb = __float_as_uint(w[j]);
+                const uint32_t db = __float_as_uint(w[j] - __uint_as_float(mid | (wb & SIGN)));
+                below = __funnelshift_l(db, below, 1);
+                if (more) s1 += __uint_as_float(wb ^ (db & SIGN));
+            }
+            const uint32_t c1 = positive, c2 = ~below;
+            bits[0] = ((first ? c1 : c2) ^ (sa ? 0xffffffffu : 0u)) & valid;
+            bits[K - 1] = ((first ? c2 : c1) ^ (sb ? 0xffffffffu : 0u)) & valid;
+            const float sum0 = first ? abs_w : s1, sum1 = first ? s1 : abs_w;
+            csum[0] = sa ? -sum0 : sum0;
+            csum[K - 1] = sb ? -sum1 : sum1;
+            continue;
+        }
+        if constexpr (K >= 3) {
+            // ascending levels: code bit i is decision i of the tree, the sign of w minus the midpoint that decision compares with;
+            // plane 0 is the sign of w, whose sum is known
+            if (ascending_levels<K>(alpha, thr)) {
+                uint32_t below[K];
+                float s[K];
 #pragma unroll
-        for (int j = EPT - 1; j >= 0; --j) {
-            const int sh = 31 - bst_leaf<K>(w[j], thr);
+                for (int i = 0; i < K; ++i) { below[i] = 0u; s[i] = 0.0f; }
 #pragma unroll
-            for (int i = 0; i < K; ++i) {
-                const uint32_t y = plane[i] << sh;                 // sign of plane i at this leaf, in the top bit
-                pos_bits[i] = __funnelshift_l(y, pos_bits[i], 1);
-                if (more) csum[i] += __uint_as_float(__float_as_uint(w[j]) ^ (~y & SIGN));
+                for (int j = EPT - 1; j >= 0; --j) {
+                    uint32_t d[K];
+                    tree_decisions<K, EPT>(w[j], thr, below, d);
+                    if (more) {
+#pragma unroll
+                        for (int i = 1; i < K; ++i) s[i] += __uint_as_float(__float_as_uint(w[j]) ^ (d[i] & SIGN));
+                    }
+                }
+                bits[0] = positive & valid;
+                csum[0] = abs_w;
+#pragma unroll
+                for (int i = 1; i < K; ++i) { bits[i] = ~below[i] & valid; csum[i] = s[i]; }
+                continue;
             }
         }
+        if constexpr (K >= 3) {
+            // Any other order of the levels.  The table is still antisymmetric (v and -v are levels together, of complementary codes, and
+            // ties are ordered alike), so the tree's decisions are the same comparisons with the sorted upper half; a plane is a
+            // function of the leaf, evaluated on whole words of decision bits.
+            constexpr int M2 = M / 2;
+            uint32_t code[M2];
+            upper_levels<K>(alpha, thr, code);
+            uint32_t below[K];
 #pragma unroll
-        for (int i = 0; i < K; ++i) bits[i] = pos_bits[i] & valid;
+            for (int i = 0; i < K; ++i) below[i] = 0u;
+#pragma unroll
+            for (int j = EPT - 1; j >= 0; --j) tree_decisions<K, EPT>(w[j], thr, below);
+            // minterms of the leaf within the half: bit i of the leaf = decision i agrees with the sign of w
+            uint32_t leaf[M2];
+            {
+                const uint32_t u1 = positive ^ below[1], u2 = positive ^ below[2];          // (below: decision bits inverted)
+                const uint32_t q3 = u1 & u2, q2 = u1 & ~u2, q1 = ~u1 & u2, q0 = ~(u1 | u2);
+                if constexpr (K == 3) {
+                    leaf[0] = q0; leaf[1] = q1; leaf[2] = q2; leaf[3] = q3;
+                } else {
+                    const uint32_t u3 = positive ^ below[K - 1];
+                    leaf[0] = q0 & ~u3; leaf[1] = q0 & u3; leaf[2] = q1 & ~u3; leaf[3] = q1 & u3;
+                    leaf[M2 - 4] = q2 & ~u3; leaf[M2 - 3] = q2 & u3; leaf[M2 - 2] = q3 & ~u3; leaf[M2 - 1] = q3 & u3;
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < K; ++i) {
+                uint32_t f = 0u;
+#pragma unroll
+                for (int q = 0; q < M2; ++q) f |= leaf[q] & (0u - ((code[q] >> (K - 1 - i)) & 1u));
+                const uint32_t pb = ~(positive ^ f);        // the lower half has the complementary codes
+                bits[i] = pb & valid;
+                if (more) {
+                    float cs = 0.0f;
+#pragma unroll
+                    for (int j = EPT - 1; j >= 0; --j) cs += __uint_as_float(__float_as_uint(w[j]) ^ (~(pb << (31 - j)) & SIGN));
+                    csum[i] = cs;
+                }
+            }
+        }
     }
     if (parity_io) *parity_io = parity;
 }
