@@ -2,7 +2,8 @@
 
 PyTorch supplies device memory and the current stream; every step of the path runs in the CUDA
 library.  Importing this module loads paper_1802_00150_b200/libamq_b200.so and raises if it is missing:
-there is no CPU fallback.
+there is no CPU fallback.  The calls that enqueue work go through the native binding (csrc/amq_binding.cpp), which
+checks tensors, takes their addresses and adds the current stream; size helpers and status calls go through ctypes.
 """
 import ctypes
 import os
@@ -19,6 +20,10 @@ if not os.path.exists(LIB_PATH):
         "(there is no CPU fallback)" % LIB_PATH)
 
 _lib = ctypes.CDLL(LIB_PATH)
+
+from . import _amq_binding as _native  # noqa: E402  (built beside the library; raises if it is missing)
+
+_native.open(LIB_PATH)
 
 OK = 0
 MAX_K = 4
@@ -99,14 +104,6 @@ def _stream():
     return torch.cuda.current_stream().cuda_stream
 
 
-def _dev(t, dtype, name):
-    if t is None:
-        return None
-    if not (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype == dtype and t.is_contiguous()):
-        raise TypeError("%s must be a contiguous CUDA tensor of dtype %s" % (name, dtype))
-    return t
-
-
 def status_string(status):
     return _lib.amq_status_string(status).decode()
 
@@ -123,8 +120,8 @@ def codes_bytes(rows, n, k):
     return _lib.amq_codes_bytes(rows, n, k)
 
 
-def _new_codes(rows, k, n, device):
-    return torch.empty((rows, k, words_per_row(n)), dtype=torch.int32, device=device)
+def _new_codes(rows, k, n, like):
+    return _native.empty(like, 1, rows, k, 4 * ((n + 127) // 128))
 
 
 def quantize(x, k, T, codes=None, coeffs=None):
@@ -133,66 +130,58 @@ def quantize(x, k, T, codes=None, coeffs=None):
         raise TypeError("x must be a 2-D CUDA fp32 tensor with unit column stride")
     rows, n = x.shape
     ldx = x.stride(0) if rows > 1 else max(n, x.stride(0))
-    codes = _new_codes(rows, k, n, x.device) if codes is None else _dev(codes, torch.int32, "codes")
-    coeffs = torch.empty((rows, k), dtype=torch.float32, device=x.device) if coeffs is None else _dev(coeffs, torch.float32, "coeffs")
-    _check(_lib.amq_quantize(_ptr(x), rows, n, ldx, k, T, _ptr(codes), _ptr(coeffs), _stream()))
+    codes = _new_codes(rows, k, n, x) if codes is None else codes
+    coeffs = _native.empty(x, 0, rows, k) if coeffs is None else coeffs
+    _check(_native.amq_quantize(x.data_ptr(), rows, n, ldx, k, T, codes, coeffs))
     return codes, coeffs
 
 
 def pack(planes):
     """planes (rows, k, n) fp32 (>= 0 -> +1) -> codes (rows, k, wpr) int32."""
-    planes = _dev(planes, torch.float32, "planes")
     rows, k, n = planes.shape
-    codes = _new_codes(rows, k, n, planes.device)
-    _check(_lib.amq_pack(_ptr(planes), rows, n, k, _ptr(codes), _stream()))
+    codes = _new_codes(rows, k, n, planes)
+    _check(_native.amq_pack(planes, rows, n, k, codes))
     return codes
 
 
 def unpack(codes, coeffs, n):
-    codes, coeffs = _dev(codes, torch.int32, "codes"), _dev(coeffs, torch.float32, "coeffs")
     rows, k, _ = codes.shape
-    xhat = torch.empty((rows, n), dtype=torch.float32, device=codes.device)
-    _check(_lib.amq_unpack(_ptr(codes), _ptr(coeffs), rows, n, k, _ptr(xhat), _stream()))
+    xhat = _native.empty(codes, 0, rows, n)
+    _check(_native.amq_unpack(codes, coeffs, rows, n, k, xhat))
     return xhat
 
 
 def binary_dots(Wcodes, xcodes, n):
     """-> D (batch, m, k_w, k_a) int32."""
-    Wcodes, xcodes = _dev(Wcodes, torch.int32, "Wcodes"), _dev(xcodes, torch.int32, "xcodes")
     m, k_w, _ = Wcodes.shape
     batch, k_a, _ = xcodes.shape
-    D = torch.empty((batch, m, k_w, k_a), dtype=torch.int32, device=Wcodes.device)
-    _check(_lib.amq_binary_dots(_ptr(Wcodes), m, n, k_w, _ptr(xcodes), batch, k_a, _ptr(D), _stream()))
+    D = _native.empty(Wcodes, 1, batch, m, k_w, k_a)
+    _check(_native.amq_binary_dots(Wcodes, m, n, k_w, xcodes, batch, k_a, D))
     return D
 
 
 def binary_gemm(Wcodes, Walpha, xcodes, xbeta, n, bias=None, y=None):
     """-> y (batch, m) fp32."""
-    Wcodes, xcodes = _dev(Wcodes, torch.int32, "Wcodes"), _dev(xcodes, torch.int32, "xcodes")
-    Walpha, xbeta = _dev(Walpha, torch.float32, "Walpha"), _dev(xbeta, torch.float32, "xbeta")
-    bias = _dev(bias, torch.float32, "bias")
     m, k_w, _ = Wcodes.shape
     batch, k_a, _ = xcodes.shape
     if y is None:
-        y = torch.empty((batch, m), dtype=torch.float32, device=Wcodes.device)
-    _check(_lib.amq_binary_gemm(_ptr(Wcodes), _ptr(Walpha), m, n, k_w, _ptr(xcodes), _ptr(xbeta), batch, k_a,
-                                _ptr(bias), _ptr(y), y.stride(0) if batch > 1 else max(m, y.stride(0)), _stream()))
+        y = _native.empty(Wcodes, 0, batch, m)
+    _check(_native.amq_binary_gemm(Wcodes, Walpha, m, n, k_w, xcodes, xbeta, batch, k_a,
+                                bias, y.data_ptr(), y.stride(0) if batch > 1 else max(m, y.stride(0))))
     return y
 
 
 def quantized_gemv(Wcodes, Walpha, x, k_a, T, bias=None, y=None, want_codes=False):
     """Table 6's operation in one launch: x (n,) or (1, n) fp32 is quantized on-line (k_a bits, T cycles) inside the
     product kernel.  Returns y (m,), or (y, xcodes (k_a, wpr), xbeta (k_a,)) with want_codes."""
-    Wcodes, Walpha = _dev(Wcodes, torch.int32, "Wcodes"), _dev(Walpha, torch.float32, "Walpha")
-    x = _dev(x, torch.float32, "x")
     m, k_w, wpr = Wcodes.shape
     n = x.numel()
     if y is None:
-        y = torch.empty((m,), dtype=torch.float32, device=x.device)
-    xc = torch.empty((k_a, wpr), dtype=torch.int32, device=x.device) if want_codes else None
-    xb = torch.empty((k_a,), dtype=torch.float32, device=x.device) if want_codes else None
-    _check(_lib.amq_quantized_gemv(_ptr(Wcodes), _ptr(Walpha), m, n, k_w, _ptr(x), k_a, T, _ptr(bias), _ptr(y),
-                                   _ptr(xc), _ptr(xb), _stream()))
+        y = _native.empty(x, 0, m)
+    xc = _native.empty(x, 1, k_a, wpr) if want_codes else None
+    xb = _native.empty(x, 0, k_a) if want_codes else None
+    _check(_native.amq_quantized_gemv(Wcodes, Walpha, m, n, k_w, x, k_a, T, bias, y,
+                                   xc, xb))
     return (y, xc, xb) if want_codes else y
 
 
@@ -218,13 +207,11 @@ def new_host_staging(I, H, batch, steps, device="cuda"):
 
 
 def lstm_step(Wcodes, Walpha, bias, I, H, x, h_in, c_in, k_a, T, workspace, h_out=None, c_out=None):
-    Wcodes, Walpha = _dev(Wcodes, torch.int32, "Wcodes"), _dev(Walpha, torch.float32, "Walpha")
-    x, h_in, c_in = _dev(x, torch.float32, "x"), _dev(h_in, torch.float32, "h_in"), _dev(c_in, torch.float32, "c_in")
     batch, k_w = h_in.shape[0], Wcodes.shape[1]
-    h_out = torch.empty_like(h_in) if h_out is None else h_out
-    c_out = torch.empty_like(c_in) if c_out is None else c_out
-    _check(_lib.amq_lstm_step(_ptr(Wcodes), _ptr(Walpha), _ptr(bias), I, H, k_w, _ptr(x), _ptr(h_in), _ptr(c_in),
-                              batch, k_a, T, _ptr(h_out), _ptr(c_out), _ptr(workspace), workspace.numel(), _stream()))
+    h_out = _native.empty(h_in, 0, *h_in.shape) if h_out is None else h_out
+    c_out = _native.empty(c_in, 0, *c_in.shape) if c_out is None else c_out
+    _check(_native.amq_lstm_step(Wcodes, Walpha, bias, I, H, k_w, x, h_in, c_in,
+                              batch, k_a, T, h_out, c_out, workspace, workspace.numel()))
     return h_out, c_out
 
 
@@ -239,63 +226,51 @@ def lstm_step_static(Wcodes, Walpha, bias, I, H, x, h_in, c_in, k_a, T, h_out, c
     """amq_lstm_step without a workspace: the library's built-in scratch array is used, and neither this
     wrapper nor the call allocates (the caller brings h_out and c_out).  Problems whose scratch exceeds
     STATIC_SCRATCH_BYTES raise AmqError(-4)."""
-    Wcodes, Walpha = _dev(Wcodes, torch.int32, "Wcodes"), _dev(Walpha, torch.float32, "Walpha")
-    x, h_in, c_in = _dev(x, torch.float32, "x"), _dev(h_in, torch.float32, "h_in"), _dev(c_in, torch.float32, "c_in")
-    h_out, c_out = _dev(h_out, torch.float32, "h_out"), _dev(c_out, torch.float32, "c_out")
     batch, k_w = h_in.shape[0], Wcodes.shape[1]
-    _check(_lib.amq_lstm_step_static(_ptr(Wcodes), _ptr(Walpha), _ptr(bias), I, H, k_w, _ptr(x), _ptr(h_in),
-                                     _ptr(c_in), batch, k_a, T, _ptr(h_out), _ptr(c_out), _stream()))
+    _check(_native.amq_lstm_step_static(Wcodes, Walpha, bias, I, H, k_w, x, h_in,
+                                     c_in, batch, k_a, T, h_out, c_out))
     return h_out, c_out
 
 
 def gru_step(Wcodes, Walpha, bias, I, H, x, h_in, k_a, T, workspace, h_out=None):
-    Wcodes, Walpha = _dev(Wcodes, torch.int32, "Wcodes"), _dev(Walpha, torch.float32, "Walpha")
-    x, h_in = _dev(x, torch.float32, "x"), _dev(h_in, torch.float32, "h_in")
     batch, k_w = h_in.shape[0], Wcodes.shape[1]
-    h_out = torch.empty_like(h_in) if h_out is None else h_out
-    _check(_lib.amq_gru_step(_ptr(Wcodes), _ptr(Walpha), _ptr(bias), I, H, k_w, _ptr(x), _ptr(h_in),
-                             batch, k_a, T, _ptr(h_out), _ptr(workspace), workspace.numel(), _stream()))
+    h_out = _native.empty(h_in, 0, *h_in.shape) if h_out is None else h_out
+    _check(_native.amq_gru_step(Wcodes, Walpha, bias, I, H, k_w, x, h_in,
+                             batch, k_a, T, h_out, workspace, workspace.numel()))
     return h_out
 
 
 def lstm_sequence(Wcodes, Walpha, bias, I, H, x_seq, h0, c0, k_a, T, workspace, want_h_seq=False,
                   h_seq=None, h_last=None, c_last=None):
-    Wcodes, Walpha = _dev(Wcodes, torch.int32, "Wcodes"), _dev(Walpha, torch.float32, "Walpha")
-    x_seq, h0, c0 = _dev(x_seq, torch.float32, "x_seq"), _dev(h0, torch.float32, "h0"), _dev(c0, torch.float32, "c0")
     steps, batch, k_w = x_seq.shape[0], h0.shape[0], Wcodes.shape[1]
     if want_h_seq and h_seq is None:
-        h_seq = torch.empty((steps, batch, H), dtype=torch.float32, device=h0.device)
-    h_last = torch.empty_like(h0) if h_last is None else h_last
-    c_last = torch.empty_like(c0) if c_last is None else c_last
-    _check(_lib.amq_lstm_sequence(_ptr(Wcodes), _ptr(Walpha), _ptr(bias), I, H, k_w, _ptr(x_seq), steps, _ptr(h0),
-                                  _ptr(c0), batch, k_a, T, _ptr(h_seq), _ptr(h_last), _ptr(c_last),
-                                  _ptr(workspace), workspace.numel(), _stream()))
+        h_seq = _native.empty(h0, 0, steps, batch, H)
+    h_last = _native.empty(h0, 0, *h0.shape) if h_last is None else h_last
+    c_last = _native.empty(c0, 0, *c0.shape) if c_last is None else c_last
+    _check(_native.amq_lstm_sequence(Wcodes, Walpha, bias, I, H, k_w, x_seq, steps, h0,
+                                  c0, batch, k_a, T, h_seq, h_last, c_last,
+                                  workspace, workspace.numel()))
     return h_seq, h_last, c_last
 
 
 def selftest_sequence_give_up(Wcodes, Walpha, bias, I, H, x_seq, h0, c0, k_a, T, workspace, poll_limit):
     """Test aid: the batch-1 LSTM sequence kernel with waits that run out (see amq.h).  Returns (h_last, c_last),
     which the kernel leaves unwritten; read the outcome with workspace_status."""
-    Wcodes, Walpha = _dev(Wcodes, torch.int32, "Wcodes"), _dev(Walpha, torch.float32, "Walpha")
-    x_seq, h0, c0 = _dev(x_seq, torch.float32, "x_seq"), _dev(h0, torch.float32, "h0"), _dev(c0, torch.float32, "c0")
     h_last, c_last = torch.zeros_like(h0), torch.zeros_like(c0)
-    _check(_lib.amq_selftest_sequence_give_up(_ptr(Wcodes), _ptr(Walpha), _ptr(bias), I, H, Wcodes.shape[1], _ptr(x_seq),
-                                              x_seq.shape[0], _ptr(h0), _ptr(c0), k_a, T, _ptr(h_last), _ptr(c_last),
-                                              _ptr(workspace), workspace.numel(), poll_limit, _stream()))
+    _check(_native.amq_selftest_sequence_give_up(Wcodes, Walpha, bias, I, H, Wcodes.shape[1], x_seq,
+                                              x_seq.shape[0], h0, c0, k_a, T, h_last, c_last,
+                                              workspace, workspace.numel(), poll_limit))
     return h_last, c_last
 
 
 def gru_sequence(Wcodes, Walpha, bias, I, H, x_seq, h0, k_a, T, workspace, want_h_seq=False,
                  h_seq=None, h_last=None):
-    Wcodes, Walpha = _dev(Wcodes, torch.int32, "Wcodes"), _dev(Walpha, torch.float32, "Walpha")
-    x_seq, h0 = _dev(x_seq, torch.float32, "x_seq"), _dev(h0, torch.float32, "h0")
     steps, batch, k_w = x_seq.shape[0], h0.shape[0], Wcodes.shape[1]
     if want_h_seq and h_seq is None:
-        h_seq = torch.empty((steps, batch, H), dtype=torch.float32, device=h0.device)
-    h_last = torch.empty_like(h0) if h_last is None else h_last
-    _check(_lib.amq_gru_sequence(_ptr(Wcodes), _ptr(Walpha), _ptr(bias), I, H, k_w, _ptr(x_seq), steps, _ptr(h0),
-                                 batch, k_a, T, _ptr(h_seq), _ptr(h_last), _ptr(workspace), workspace.numel(),
-                                 _stream()))
+        h_seq = _native.empty(h0, 0, steps, batch, H)
+    h_last = _native.empty(h0, 0, *h0.shape) if h_last is None else h_last
+    _check(_native.amq_gru_sequence(Wcodes, Walpha, bias, I, H, k_w, x_seq, steps, h0,
+                                 batch, k_a, T, h_seq, h_last, workspace, workspace.numel()))
     return h_seq, h_last
 
 
@@ -312,20 +287,20 @@ def lstm_sequence_host(Wcodes, Walpha, bias, I, H, x_seq, h0, c0, k_a, T, worksp
     """x_seq, h0, c0, h_last, c_last, h_seq are HOST tensors (pinned for asynchronous copies)."""
     x_seq, h0, c0 = _host(x_seq, "x_seq"), _host(h0, "h0"), _host(c0, "c0")
     steps, batch, k_w = x_seq.shape[0], h0.shape[0], Wcodes.shape[1]
-    _check(_lib.amq_lstm_sequence_host(_ptr(Wcodes), _ptr(Walpha), _ptr(bias), I, H, k_w, _ptr(x_seq), steps,
+    _check(_native.amq_lstm_sequence_host(Wcodes, Walpha, bias, I, H, k_w, _ptr(x_seq), steps,
                                        _ptr(h0), _ptr(c0), batch, k_a, T, _ptr(_host(h_seq, "h_seq")),
                                        _ptr(_host(h_last, "h_last")), _ptr(_host(c_last, "c_last")),
-                                       _ptr(workspace), workspace.numel(), _ptr(staging), staging.numel(), _stream()))
+                                       workspace, workspace.numel(), staging, staging.numel()))
     return h_seq, h_last, c_last
 
 
 def gru_sequence_host(Wcodes, Walpha, bias, I, H, x_seq, h0, k_a, T, workspace, staging, h_last, h_seq=None):
     x_seq, h0 = _host(x_seq, "x_seq"), _host(h0, "h0")
     steps, batch, k_w = x_seq.shape[0], h0.shape[0], Wcodes.shape[1]
-    _check(_lib.amq_gru_sequence_host(_ptr(Wcodes), _ptr(Walpha), _ptr(bias), I, H, k_w, _ptr(x_seq), steps,
+    _check(_native.amq_gru_sequence_host(Wcodes, Walpha, bias, I, H, k_w, _ptr(x_seq), steps,
                                       _ptr(h0), batch, k_a, T, _ptr(_host(h_seq, "h_seq")),
-                                      _ptr(_host(h_last, "h_last")), _ptr(workspace), workspace.numel(),
-                                      _ptr(staging), staging.numel(), _stream()))
+                                      _ptr(_host(h_last, "h_last")), workspace, workspace.numel(),
+                                      staging, staging.numel()))
     return h_seq, h_last
 
 
@@ -335,13 +310,11 @@ def workspace_status(workspace):
 
 def embedding_rows(We_codes, We_alpha, n, tokens):
     """Rows of the quantized embedding matrix for int32 token ids of any shape -> codes (*shape, k, wpr), coeffs (*shape, k)."""
-    We_codes, We_alpha = _dev(We_codes, torch.int32, "We_codes"), _dev(We_alpha, torch.float32, "We_alpha")
-    tokens = _dev(tokens, torch.int32, "tokens")
     vocab, k, wpr = We_codes.shape
     xcodes = torch.empty(tuple(tokens.shape) + (k, wpr), dtype=torch.int32, device=We_codes.device)
     xbeta = torch.empty(tuple(tokens.shape) + (k,), dtype=torch.float32, device=We_codes.device)
-    _check(_lib.amq_embedding_rows(_ptr(We_codes), _ptr(We_alpha), vocab, n, k, _ptr(tokens), tokens.numel(),
-                                   _ptr(xcodes), _ptr(xbeta), _stream()))
+    _check(_native.amq_embedding_rows(We_codes, We_alpha, vocab, n, k, tokens, tokens.numel(),
+                                   xcodes, xbeta))
     return xcodes, xbeta
 
 
@@ -352,11 +325,11 @@ def new_paper_workspace(H, batch, steps, k_a, device="cuda"):
 def lstm_step_paper(Wi_codes, Wi_alpha, Wh_codes, Wh_alpha, bias, I, H, xcodes, xbeta, h_in, c_in, k_a, T, workspace,
                     h_out=None, c_out=None):
     batch, k_w, k_e = h_in.shape[0], Wi_codes.shape[1], xcodes.shape[-2]
-    h_out = torch.empty_like(h_in) if h_out is None else h_out
-    c_out = torch.empty_like(c_in) if c_out is None else c_out
-    _check(_lib.amq_lstm_step_paper(_ptr(Wi_codes), _ptr(Wi_alpha), _ptr(Wh_codes), _ptr(Wh_alpha), _ptr(bias), I, H, k_w,
-                                    _ptr(xcodes), _ptr(xbeta), k_e, _ptr(h_in), _ptr(c_in), batch, k_a, T,
-                                    _ptr(h_out), _ptr(c_out), _ptr(workspace), workspace.numel(), _stream()))
+    h_out = _native.empty(h_in, 0, *h_in.shape) if h_out is None else h_out
+    c_out = _native.empty(c_in, 0, *c_in.shape) if c_out is None else c_out
+    _check(_native.amq_lstm_step_paper(Wi_codes, Wi_alpha, Wh_codes, Wh_alpha, bias, I, H, k_w,
+                                    xcodes, xbeta, k_e, h_in, c_in, batch, k_a, T,
+                                    h_out, c_out, workspace, workspace.numel()))
     return h_out, c_out
 
 
@@ -364,13 +337,12 @@ def lstm_sequence_paper(Wi_codes, Wi_alpha, Wh_codes, Wh_alpha, bias, I, H, xcod
                         want_h_seq=False, h_last=None, c_last=None):
     steps, batch, k_e = xcodes_seq.shape[0], h0.shape[0], xcodes_seq.shape[-2]
     k_w = Wi_codes.shape[1]
-    h_seq = torch.empty((steps, batch, H), dtype=torch.float32, device=h0.device) if want_h_seq else None
-    h_last = torch.empty_like(h0) if h_last is None else h_last
-    c_last = torch.empty_like(c0) if c_last is None else c_last
-    _check(_lib.amq_lstm_sequence_paper(_ptr(Wi_codes), _ptr(Wi_alpha), _ptr(Wh_codes), _ptr(Wh_alpha), _ptr(bias), I, H, k_w,
-                                        _ptr(xcodes_seq), _ptr(xbeta_seq), k_e, steps, _ptr(h0), _ptr(c0), batch, k_a, T,
-                                        _ptr(h_seq), _ptr(h_last), _ptr(c_last), _ptr(workspace), workspace.numel(),
-                                        _stream()))
+    h_seq = _native.empty(h0, 0, steps, batch, H) if want_h_seq else None
+    h_last = _native.empty(h0, 0, *h0.shape) if h_last is None else h_last
+    c_last = _native.empty(c0, 0, *c0.shape) if c_last is None else c_last
+    _check(_native.amq_lstm_sequence_paper(Wi_codes, Wi_alpha, Wh_codes, Wh_alpha, bias, I, H, k_w,
+                                        xcodes_seq, xbeta_seq, k_e, steps, h0, c0, batch, k_a, T,
+                                        h_seq, h_last, c_last, workspace, workspace.numel()))
     return h_seq, h_last, c_last
 
 
@@ -381,9 +353,9 @@ def log_softmax_argmax(logits, want_logp=True, argmax=None):
         raise TypeError("logits must be a 2-D CUDA float32 tensor with contiguous rows")
     rows, n = logits.shape
     ld = logits.stride(0) if rows > 1 else max(n, logits.stride(0))
-    logp = torch.empty((rows, n), dtype=torch.float32, device=logits.device) if want_logp else None
-    argmax = torch.empty((rows,), dtype=torch.int32, device=logits.device) if argmax is None else argmax
-    _check(_lib.amq_log_softmax_argmax(_ptr(logits), rows, n, ld, _ptr(logp), n, _ptr(argmax), _stream()))
+    logp = _native.empty(logits, 0, rows, n) if want_logp else None
+    argmax = _native.empty(logits, 1, rows) if argmax is None else argmax
+    _check(_native.amq_log_softmax_argmax(logits.data_ptr(), rows, n, ld, logp, n, argmax))
     return logp, argmax
 
 
@@ -397,10 +369,10 @@ def lm_greedy_decode(We_codes, We_alpha, Wi_codes, Wi_alpha, Wh_codes, Wh_alpha,
     vocab, k_e = We_codes.shape[0], We_codes.shape[1]
     k_w, k_s = Wi_codes.shape[1], Ws_codes.shape[1]
     steps = tokens.numel() - 1
-    _check(_lib.amq_lm_greedy_decode(_ptr(We_codes), _ptr(We_alpha), vocab, I, k_e, _ptr(Wi_codes), _ptr(Wi_alpha),
-                                     _ptr(Wh_codes), _ptr(Wh_alpha), _ptr(bias), H, k_w, _ptr(Ws_codes), _ptr(Ws_alpha),
-                                     _ptr(bias_s), k_s, k_a, T, _ptr(tokens), steps, _ptr(h), _ptr(c), _ptr(logp),
-                                     _ptr(workspace), workspace.numel(), _stream()))
+    _check(_native.amq_lm_greedy_decode(We_codes, We_alpha, vocab, I, k_e, Wi_codes, Wi_alpha,
+                                     Wh_codes, Wh_alpha, bias, H, k_w, Ws_codes, Ws_alpha,
+                                     bias_s, k_s, k_a, T, tokens, steps, h, c, logp,
+                                     workspace, workspace.numel()))
     return tokens
 
 
@@ -413,10 +385,9 @@ def quantize_variant(x, k, T, method=METHOD_ALTERNATING, final_refit=False):
         raise TypeError("x must be a 2-D CUDA fp32 tensor with unit column stride")
     rows, n = x.shape
     ldx = x.stride(0) if rows > 1 else max(n, x.stride(0))
-    codes = _new_codes(rows, k, n, x.device)
-    coeffs = torch.empty((rows, k), dtype=torch.float32, device=x.device)
-    _check(_lib.amq_quantize_variant(_ptr(x), rows, n, ldx, k, T, method, int(final_refit), _ptr(codes), _ptr(coeffs),
-                                     _stream()))
+    codes = _new_codes(rows, k, n, x)
+    coeffs = _native.empty(x, 0, rows, k)
+    _check(_native.amq_quantize_variant(x.data_ptr(), rows, n, ldx, k, T, method, int(final_refit), codes, coeffs))
     return codes, coeffs
 
 
@@ -425,7 +396,7 @@ def gru_step_original(Wcodes, Walpha, bias, I, H, x, h_in, k_a, T, workspace=Non
     batch, k_w = h_in.shape[0], Wcodes.shape[1]
     if workspace is None:
         workspace = torch.empty((_lib.amq_gru_original_workspace_bytes(I, H, batch, k_a),), dtype=torch.uint8, device=h_in.device)
-    h_out = torch.empty_like(h_in) if h_out is None else h_out
-    _check(_lib.amq_gru_step_original(_ptr(Wcodes), _ptr(Walpha), _ptr(bias), I, H, k_w, _ptr(x), _ptr(h_in), batch, k_a, T,
-                                      _ptr(h_out), _ptr(workspace), workspace.numel(), _stream()))
+    h_out = _native.empty(h_in, 0, *h_in.shape) if h_out is None else h_out
+    _check(_native.amq_gru_step_original(Wcodes, Walpha, bias, I, H, k_w, x, h_in, batch, k_a, T,
+                                      h_out, workspace, workspace.numel()))
     return h_out

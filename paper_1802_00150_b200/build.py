@@ -1,4 +1,5 @@
-"""Compile the CUDA library for sm_100a with nvcc into paper_1802_00150_b200/libamq_b200.so (in-tree).
+"""Compile the CUDA library for sm_100a with nvcc into paper_1802_00150_b200/libamq_b200.so (in-tree), and the Python
+binding beside it (g++ against the installed torch headers).
 
     python -m paper_1802_00150_b200.build [--force] [-v] [--define NAME ...] [--lib FILE]
 
@@ -11,6 +12,7 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -25,12 +27,38 @@ NVCC_FLAGS = [
 ]
 
 
+BINDING = os.path.join(HERE, "_amq_binding" + sysconfig.get_config_var("EXT_SUFFIX"))
+
+
+def build_binding(force=False):
+    """The CPython extension that marshals arguments (host code only; it opens the CUDA library at import)."""
+    src = os.path.join(CSRC, "amq_binding.cpp")
+    newest = max(os.path.getmtime(p) for p in (src, os.path.join(ROOT, "include", "amq.h")))
+    if not force and os.path.exists(BINDING) and os.path.getmtime(BINDING) >= newest:
+        return BINDING
+    import torch
+    from torch.utils.cpp_extension import include_paths
+    lib_dir = os.path.join(os.path.dirname(torch.__file__), "lib")
+    tmp = BINDING + ".tmp%d" % os.getpid()
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", src, "-o", tmp,
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), "-I", os.path.join(ROOT, "include"),
+           "-I", sysconfig.get_paths()["include"]]
+    for p in include_paths("cuda"):
+        cmd += ["-isystem", p]
+    cmd += ["-L", lib_dir, "-Wl,-rpath," + lib_dir, "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-ldl"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("building the binding failed:\n%s\n%s" % (res.stdout, res.stderr))
+    os.replace(tmp, BINDING)
+    return BINDING
+
+
 def _sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
 def _deps_mtime():
-    paths = glob.glob(os.path.join(CSRC, "*")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
+    paths = glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
     return max(os.path.getmtime(p) for p in paths)
 
 
@@ -39,6 +67,7 @@ def build(force=False, verbose=False, defines=(), lib_name=None):
     lib = LIB if lib_name is None else os.path.join(HERE, lib_name)
     obj_dir = OBJ if lib_name is None else os.path.join(OBJ, os.path.splitext(lib_name)[0])
     flags = NVCC_FLAGS + ["-D" + d for d in defines]
+    build_binding(force)
     if not force and os.path.exists(lib) and os.path.getmtime(lib) >= _deps_mtime():
         return lib
     os.makedirs(obj_dir, exist_ok=True)

@@ -134,6 +134,8 @@ amq_status enqueue_sequence(const CellCall& c, const CellWorkspace& ws, const fl
 amq_status step_entry(const CellCall& c, const CellWorkspace& ws, const float* x, const float* h_in, const float* c_in, float* h_out,
                       float* c_out, cudaStream_t st)
 {
+    // (one sequence: the kernel clears the status word itself, a clear of its own costs as much host time as the launch)
+    if (c.batch == 1 && use_persistent(c)) return enqueue_persistent(c, ws, x, 1, h_in, c_in, nullptr, h_out, c_out, st);
     AMQ_CUDA_TRY(cudaMemsetAsync(ws.status, 0, 256 + ws.counter_bytes, st));
     const BatchedSequence b = batched_call(c, ws, x, 1, h_in, c_in, nullptr, h_out, c_out);
     if (batched_sequence_supported(b)) return launch_batched_sequence(b, st);

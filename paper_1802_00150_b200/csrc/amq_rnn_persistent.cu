@@ -125,6 +125,9 @@ rnn_persistent_kernel(PersistArgs a)
     QuantScratch<KA, NW>* scratch = reinterpret_cast<QuantScratch<KA, NW>*>(
         (reinterpret_cast<uintptr_t>(sC + upc) + 15) & ~uintptr_t(15));
 
+    // a single step waits for nobody, so nobody can have written the status word yet (sequences: the caller has cleared it)
+    if (a.steps <= 1 && blockIdx.x == 0 && tid == 0) a.status[0] = 0u;
+
     // ---- resident weights: local plane-row pr = (ul * GATES + gate) * k_w + i ----
     {
         uint32_t* sWw = reinterpret_cast<uint32_t*>(sW);
