@@ -167,6 +167,24 @@ amq_status tc_status_word(uint32_t** word);       // device address of the statu
 bool gemm_resident_supported(const GemmArgs& a);
 amq_status launch_binary_gemm_resident(const GemmArgs& a, cudaStream_t st);
 
+// Greedy decoding without log-probabilities: all tokens in one cooperative launch.  `exchange` (decode_exchange_bytes, 128-byte
+// aligned): {value, tag} words of h, then {logit, tag}, {index, tag} pairs, [2 parities][copies][..] each.
+constexpr int DECODE_MAX_CTAS = 256;
+inline size_t decode_exchange_bytes(int H)
+{
+    return (size_t)2 * PERSISTENT_EXCHANGE_COPIES * (persistent_exchange_stride(H) * 8 + DECODE_MAX_CTAS * 16);
+}
+struct DecodeSequence {
+    const uint32_t* We; const float* We_alpha; int vocab, I, k_e;
+    const uint32_t* Wi; const float* Wi_alpha; const uint32_t* Wh; const float* Wh_alpha; const float* bias; int H, k_w;
+    const uint32_t* Ws; const float* Ws_alpha; const float* bias_s; int k_s;
+    int k_a, T, steps;
+    int32_t* tokens; float* h; float* c;
+    unsigned long long* exchange;
+};
+bool decode_persistent_supported(const DecodeSequence& d);
+amq_status launch_decode_persistent(const DecodeSequence& d, cudaStream_t st);
+
 // Batched recurrent kernel: all timesteps of a batch of sequences in one cooperative launch.  z = [x ; h] (LSTM, GRU) or h alone with
 // the input projections as `addend` (paper form: I = 0, n = H).  `counters` cleared by the caller.
 struct BatchedSequence {
