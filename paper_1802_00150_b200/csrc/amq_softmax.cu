@@ -15,7 +15,8 @@ __device__ __forceinline__ void max_combine(float& v, int& i, float ov, int oi)
     if (ov > v || (ov == v && oi < i)) { v = ov; i = oi; }
 }
 
-// (value, index) maximum over the CTA; every thread returns the result
+// (value, index) maximum over the CTA of NW warps; every thread returns the result
+template <int NW>
 __device__ __forceinline__ void block_max(float& mv, int& mi, float* s_val, int* s_idx)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -24,12 +25,13 @@ __device__ __forceinline__ void block_max(float& mv, int& mi, float* s_val, int*
         max_combine(mv, mi, __shfl_xor_sync(0xffffffffu, mv, off), __shfl_xor_sync(0xffffffffu, mi, off));
     if (lane == 0) { s_val[warp] = mv; s_idx[warp] = mi; }
     __syncthreads();
-    mv = s_val[lane]; mi = s_idx[lane];
+    mv = s_val[lane & (NW - 1)]; mi = s_idx[lane & (NW - 1)];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1)
+    for (int off = NW / 2; off > 0; off >>= 1)
         max_combine(mv, mi, __shfl_xor_sync(0xffffffffu, mv, off), __shfl_xor_sync(0xffffffffu, mi, off));
 }
 
+template <int NW>
 __device__ __forceinline__ float block_sum(float sum, float* s_sum)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -37,17 +39,18 @@ __device__ __forceinline__ float block_sum(float sum, float* s_sum)
     for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
     if (lane == 0) s_sum[warp] = sum;
     __syncthreads();
-    sum = s_sum[lane];
+    sum = s_sum[lane & (NW - 1)];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+    for (int off = NW / 2; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
     return sum;
 }
 
-// Rows of up to SM_THREADS * 4 * VEC floats whose start is 16-byte aligned: the row is read once, as float4, and
-// stays in registers for the three steps (maximum, sum of exponentials, write).
-constexpr int VEC = 12;
-
-__global__ void __launch_bounds__(SM_THREADS)
+// Rows of up to 4 * THREADS * VEC floats: the row is read once, as float4 from its first 16-byte boundary on, and stays in
+// registers for the three steps (maximum, sum of exponentials, write).  The up to three floats before that boundary and the up to
+// three after the last whole float4 belong to one thread each, so that rows of an odd length or stride keep the wide loads (600
+// rows of 9999: see the dispatch below).
+template <int THREADS, int VEC>
+__global__ void __launch_bounds__(THREADS)
 log_softmax_argmax_resident_kernel(const float* logits, int n, int ld, float* __restrict__ logp, int ldp,
                                    int32_t* __restrict__ arg)
 {
@@ -57,49 +60,52 @@ log_softmax_argmax_resident_kernel(const float* logits, int n, int ld, float* __
     __shared__ float s_sum[32];
     const int tid = threadIdx.x;
     const float* z = logits + (size_t)blockIdx.x * ld;
-    const int n4 = n >> 2;                                          // whole float4 groups; the tail is handled by scalars
+    const int lead = (int)((0u - (unsigned)(reinterpret_cast<uintptr_t>(z) >> 2)) & 3u), head = lead < n ? lead : n;
+    const int n4 = (n - head) >> 2;                                 // whole float4 groups from the boundary on
+    const float* zb = z + head;
     float4 v[VEC];
 #pragma unroll
     for (int q = 0; q < VEC; ++q) {
-        const int t4 = tid + q * SM_THREADS;
-        v[q] = t4 < n4 ? __ldcg(reinterpret_cast<const float4*>(z) + t4) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+        const int t4 = tid + q * THREADS;
+        v[q] = t4 < n4 ? __ldcg(reinterpret_cast<const float4*>(zb) + t4) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
     }
-    const int tail = n4 * 4 + tid;                                  // at most three tail elements, one per thread
-    const float vt = tail < n ? __ldcg(z + tail) : -INFINITY;
+    const int single = tid < head ? tid : n4 * 4 + tid;             // at most six elements outside the groups, one per thread
+    const float vt = single < n ? __ldcg(z + single) : -INFINITY;
 
     float mv = vt;
-    int mi = tail < n ? tail : 0x7fffffff;
+    int mi = single < n ? single : 0x7fffffff;
 #pragma unroll
     for (int q = 0; q < VEC; ++q) {
-        const int base = (tid + q * SM_THREADS) * 4;
+        const int base = head + (tid + q * THREADS) * 4;
         max_combine(mv, mi, v[q].x, base); max_combine(mv, mi, v[q].y, base + 1);
         max_combine(mv, mi, v[q].z, base + 2); max_combine(mv, mi, v[q].w, base + 3);
     }
-    block_max(mv, mi, s_val, s_idx);
+    block_max<THREADS / 32>(mv, mi, s_val, s_idx);
 
-    float sum = tail < n ? __expf(vt - mv) : 0.0f;
+    float sum = single < n ? __expf(vt - mv) : 0.0f;
 #pragma unroll
     for (int q = 0; q < VEC; ++q)                                    // exp(-inf) = 0 for the positions past the end
         sum += (__expf(v[q].x - mv) + __expf(v[q].y - mv)) + (__expf(v[q].z - mv) + __expf(v[q].w - mv));
-    sum = block_sum(sum, s_sum);
+    sum = block_sum<THREADS / 32>(sum, s_sum);
     const float lse = mv + logf(sum);
 
     if (logp) {
-        float* out = logp + (size_t)blockIdx.x * ldp;
-        if ((ldp & 3) == 0 && (reinterpret_cast<uintptr_t>(logp) & 15) == 0) {
+        float* row = logp + (size_t)blockIdx.x * ldp;
+        float* out = row + head;
+        if ((reinterpret_cast<uintptr_t>(out) & 15) == 0) {
 #pragma unroll
             for (int q = 0; q < VEC; ++q) {
-                const int t4 = tid + q * SM_THREADS;
+                const int t4 = tid + q * THREADS;
                 if (t4 < n4) reinterpret_cast<float4*>(out)[t4] = make_float4(v[q].x - lse, v[q].y - lse, v[q].z - lse, v[q].w - lse);
             }
         } else {
 #pragma unroll
             for (int q = 0; q < VEC; ++q) {
-                const int t4 = tid + q * SM_THREADS;
+                const int t4 = tid + q * THREADS;
                 if (t4 < n4) { out[4 * t4] = v[q].x - lse; out[4 * t4 + 1] = v[q].y - lse; out[4 * t4 + 2] = v[q].z - lse; out[4 * t4 + 3] = v[q].w - lse; }
             }
         }
-        if (tail < n) out[tail] = vt - lse;
+        if (single < n) row[single] = vt - lse;
     }
     if (arg && tid == 0) arg[blockIdx.x] = mi;
 }
@@ -153,9 +159,15 @@ log_softmax_argmax_kernel(const float* logits, int n, int ld, float* __restrict_
 amq_status launch_log_softmax_argmax(const float* logits, int rows, int n, int ld, float* logp, int ldp, int32_t* argmax,
                                      cudaStream_t st, bool overlap_with_previous)
 {
-    const bool resident = n <= SM_THREADS * 4 * VEC && (ld & 3) == 0 && (reinterpret_cast<uintptr_t>(logits) & 15) == 0;
-    AMQ_CUDA_TRY(launch_kernel(resident ? log_softmax_argmax_resident_kernel : log_softmax_argmax_kernel, dim3((unsigned)rows),
-                               dim3(SM_THREADS), 0, st, overlap_with_previous, logits, n, ld, logp, ldp, argmax));
+    // The smallest CTA whose registers hold a row (less three leading floats): several rows are then in flight per SM, and no thread
+    // works on positions past the end.
+    auto kernel = log_softmax_argmax_kernel;
+    int threads = SM_THREADS;
+    if (n <= 4 * 128 * 4) { kernel = log_softmax_argmax_resident_kernel<128, 4>; threads = 128; }
+    else if (n <= 4 * 512 * 5) { kernel = log_softmax_argmax_resident_kernel<512, 5>; threads = 512; }
+    else if (n <= 4 * 1024 * 12) kernel = log_softmax_argmax_resident_kernel<1024, 12>;
+    AMQ_CUDA_TRY(launch_kernel(kernel, dim3((unsigned)rows), dim3((unsigned)threads), 0, st, overlap_with_previous, logits, n, ld,
+                               logp, ldp, argmax));
     AMQ_LAUNCH_CHECK();
     return AMQ_OK;
 }
