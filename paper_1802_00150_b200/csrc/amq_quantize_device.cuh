@@ -134,6 +134,21 @@ __device__ __forceinline__ void group_totals(float (&f)[VF], int (&iv)[VI > 0 ? 
     }
     if (flag) *flag = team.sync_or(*flag);
     else team.sync();
+    if constexpr (SLOTS == 4) {
+        // Up to four warps: every thread reads the four partials of a value with one load and adds them in the order of the butterfly
+        // below (a step of 576 units at 3 bits: 4.8 us, 5.4 us with the butterfly, whose shuffles are one after the other).
+#pragma unroll
+        for (int i = 0; i < VF; ++i) {
+            const float4 r = *reinterpret_cast<const float4*>(sc.red[parity][i]);
+            f[i] = (r.x + r.y) + (r.z + r.w);
+        }
+#pragma unroll
+        for (int i = 0; i < VI; ++i) {
+            const int4 r = *reinterpret_cast<const int4*>(sc.red[parity][VF + i]);
+            iv[i] = (r.x + r.y) + (r.z + r.w);
+        }
+        return;
+    }
     // Every warp adds up the partials of all warps: eight lanes per value, each with the partial of one warp or of two neighbours
     // (teams of up to sixteen warps), a butterfly over distances 1, 2, 4, and one shuffle per value to hand the total to all lanes.
     // (Every thread reading every partial itself took 14 to 28 128-bit loads per reduction, most of its 1300 to 2000 clocks.)
