@@ -1,0 +1,149 @@
+"""The kernels that take over whole calls (resident-operand product, batched sequences in one launch, decoding in one launch, the
+bulk quantizer, the output softmax), each at the sizes where its tiling can go wrong, against the CPU oracle or against the
+call-by-call form that the oracle pins."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import parity
+from paper_1802_00150_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def amq():
+    assert torch.cuda.is_available(), "these tests need a CUDA device"
+    from paper_1802_00150_b200 import amq as binding
+    return binding
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).to(torch.float32).cuda()
+
+
+def cdev(c):
+    return torch.from_numpy(np.ascontiguousarray(c).view(np.int32)).cuda()
+
+
+def quantized(shape, std, k, seed, stream):
+    return oracle.quantize_rows(synth.normal(shape, std, seed, stream).astype(np.float64), k, 2)
+
+
+@pytest.mark.parametrize("m,n,kw,ka,batch,offset", [
+    (1, 1, 1, 1, 16, 0),                # one row, one column
+    (127, 255, 2, 2, 31, 0),            # one short of the row tile, of a slot of 256 positions, of a block of vectors
+    (129, 257, 3, 3, 33, 1),            # one past each of them, output rows off every 16-byte boundary
+    (130, 8448, 1, 4, 17, 0),           # the longest rows the operand is kept for
+    (130, 8449, 1, 1, 17, 0),           # one more: the streaming kernel
+    (4000, 512, 4, 1, 2, 3),            # the smallest batch, many rows
+    (300, 1000, 4, 4, 97, 2),
+])
+def test_product_at_the_edges_of_its_tiles(amq, m, n, kw, ka, batch, offset):
+    Wc, Wa = quantized((m, n), 0.03, kw, 200 + m, 1)
+    Xc, Xb = quantized((batch, n), 1.0, ka, 200 + m, 2)
+    bias = synth.normal((m,), 0.1, 200 + m, 3)
+    out = torch.full((batch, m + offset + 2), 7.0, device="cuda")
+    amq.binary_gemm(cdev(Wc), dev(Wa), cdev(Xc), dev(Xb), n, bias=dev(bias), y=out[:, offset:offset + m])
+    ref = oracle.binary_gemm(Wc, Wa, Xc, Xb, n, bias.astype(np.float64))
+    assert np.abs(out[:, offset:offset + m].cpu().numpy() - ref).max() <= 1e-5 * (np.abs(ref).max() + 1)
+    assert torch.all(out[:, :offset] == 7.0) and torch.all(out[:, offset + m:] == 7.0)      # nothing written beside the rows
+    assert amq.device_status() == 0
+
+
+@pytest.mark.parametrize("cell,I,H,kw,ka,batch", [
+    ("lstm", 1, 1, 1, 1, 2),            # the smallest
+    ("lstm", 255, 33, 3, 2, 9),         # one short of a slot, one unit past a tile of 32, one vector past a block of 8
+    ("lstm", 300, 640, 2, 3, 33),
+    ("gru", 257, 129, 2, 2, 31),        # the column split one past a slot, one unit past a tile of 128
+    ("gru", 512, 256, 4, 4, 65),        # the split on a slot
+    ("gru", 2100, 2050, 1, 2, 5),       # rows of more than 4096 positions
+    ("lstm", 70, 1200, 4, 4, 70),
+])
+def test_batched_sequence_at_the_edges_of_its_tiles(amq, cell, I, H, kw, ka, batch):
+    """Three timesteps in one call equal three calls of one timestep bit for bit; the first is held against the oracle."""
+    steps, n, gates = 3, I + H, 4 if cell == "lstm" else 3
+    Wc, Wa = quantized((gates * H, n), 0.05, kw, 300 + H, 1)
+    bias = synth.normal((4 * H,), 0.1, 300 + H, 2)
+    xs = synth.uniform((steps, batch, I), -1, 1, 301, 1)
+    h0, c0 = synth.uniform((batch, H), -1, 1, 301, 2), synth.uniform((batch, H), -1, 1, 301, 3)
+    ws = amq.new_workspace(I, H, batch, ka)
+    args = (cdev(Wc), dev(Wa), dev(bias), I, H)
+    x, h, c = dev(xs), dev(h0), dev(c0)
+    if cell == "lstm":
+        seq, last, c_last = amq.lstm_sequence(*args, x, h, c, ka, 2, ws, want_h_seq=True)
+        ref, c_ref = oracle.lstm_step(Wc, Wa, bias, I, H, xs[0], h0, c0, ka, 2)
+    else:
+        seq, last = amq.gru_sequence(*args, x, h, ka, 2, ws, want_h_seq=True)
+        ref = oracle.gru_step(Wc, Wa, bias, I, H, xs[0], h0, ka, 2)
+    _, beta = oracle.quantize_rows(np.concatenate([xs[0], h0], axis=1).astype(np.float64), ka, 2)
+    assert np.abs(seq[0].cpu().numpy() - ref).max() <= 3.0 * parity.output_tolerance(Wa, beta, n).max() + 1e-6
+    for t in range(steps):
+        if cell == "lstm":
+            _, h, c = amq.lstm_sequence(*args, x[t:t + 1], h, c, ka, 2, ws)
+        else:
+            _, h = amq.gru_sequence(*args, x[t:t + 1], h, ka, 2, ws)
+        assert torch.equal(h, seq[t]), t
+    assert torch.equal(h, last) and (cell == "gru" or torch.equal(c, c_last))
+    assert amq.workspace_status(ws) == 0
+
+
+@pytest.mark.parametrize("V,I,H,ke,kw,ks,ka,steps", [
+    (1, 1, 1, 1, 1, 1, 1, 1),           # one word, one unit
+    (149, 33, 147, 1, 2, 4, 2, 5),      # SMs without units, one word more than SMs
+    (3001, 96, 149, 2, 3, 2, 1, 9),     # an odd number of units per SM, three row planes
+    (5000, 1000, 257, 4, 4, 1, 4, 7),   # three 128-bit chunks of the state
+    (40000, 64, 2048, 3, 1, 3, 3, 4),   # the widest state, output rows that do not all fit a SM
+])
+def test_decoding_in_one_launch_equals_the_chain_of_kernels(amq, V, I, H, ke, kw, ks, ka, steps):
+    """Asked for log-probabilities the call runs kernel by kernel (held against the oracle elsewhere), without them in one launch:
+    the same tokens and the same state bit for bit, called again as well (no word of the first call may be taken for a new one)."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(V)
+    q = lambda shape, std, k: amq.quantize(torch.randn(shape, device="cuda", generator=g) * std, k, 2)
+    We, Wi, Wh, Ws = q((V, I), 1.0, ke), q((4 * H, I), 0.2, kw), q((4 * H, H), 0.1, kw), q((V, H), 0.2, ks)
+    bias, bias_s = torch.randn((4 * H,), device="cuda", generator=g) * 0.1, torch.randn((V,), device="cuda", generator=g) * 0.1
+    ws = amq.new_decode_workspace(V, I, H, ke, ka)
+    runs = []
+    for logp in (torch.empty((steps, V), device="cuda"), None, None):
+        tokens = torch.full((steps + 1,), V // 2, dtype=torch.int32, device="cuda")
+        h, c = torch.full((1, H), 0.25, device="cuda"), torch.zeros((1, H), device="cuda")
+        amq.lm_greedy_decode(*We, *Wi, *Wh, bias, *Ws, bias_s, I, H, ka, 2, tokens, h, c, ws, logp=logp)
+        runs.append((tokens, h, c))
+    for r in runs[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(r, runs[0]))
+    assert amq.device_status() == 0
+
+
+@pytest.mark.parametrize("rows,n,ld,skip", [(3, 2, 5, 3), (5, 2047, 2049, 1), (5, 2049, 2051, 2), (4, 10239, 10241, 3), (3, 10241, 10243, 1),
+                                            (2, 49151, 49157, 1), (2, 49153, 49153, 3)])
+def test_log_softmax_of_rows_off_the_16_byte_boundary(amq, rows, n, ld, skip):
+    z = synth.normal((rows, n), 3.0, 400 + n, 1)
+    z[0, 0] = z[0].max() + 1.0                                     # the maximum before the first boundary
+    z[-1, n - 1] = z[-1].max() + 2.0
+    flat = torch.full((rows * ld + 8,), float("nan"), device="cuda")
+    wide = flat[skip:skip + rows * ld].view(rows, ld)
+    wide[:, :n] = dev(z)
+    logp, arg = amq.log_softmax_argmax(wide[:, :n])
+    ref, rarg = oracle.log_softmax_argmax(z.astype(np.float64))
+    assert np.abs(logp.cpu().numpy() - ref).max() <= 2e-5
+    assert np.array_equal(arg.cpu().numpy(), rarg)
+
+
+@pytest.mark.parametrize("rows,n,k", [(2100, 1023, 3), (2100, 1024, 4), (2100, 65, 4), (1100, 513, 2), (3, 2049, 4)])
+def test_quantizer_with_levels_out_of_order(amq, rows, n, k):
+    """Rows whose refitted coefficients come out negative or not in decreasing order (two clusters and a constant part), so that the
+    levels have to be sorted before the tree decisions; T = 4 cycles, edges of the warp and CTA ownership."""
+    x = synth.normal((rows, n), 1.0, 500 + n, 1)
+    u = synth.uniform01(rows * n, 500 + n, 2).reshape(rows, n)
+    x = np.where(u < 0.5, 1.0 + 0.01 * x, np.where(u < 0.55, -3.0 + 0.2 * x, 0.02 * x)).astype(np.float32)
+    codes, coeffs = amq.quantize(dev(x), k, 4)
+    b = parity.unpack_rows(codes.cpu().numpy(), n)
+    assert parity.pad_bits_zero(codes.cpu().numpy(), n)
+    coeffs = coeffs.cpu().numpy().astype(np.float64)
+    for r in range(0, rows, max(1, rows // 24)):
+        oa, ob = oracle.quantize(x[r].astype(np.float64), k, 4)
+        got = ((x[r] - coeffs[r] @ b[r]) ** 2).sum()
+        want = ((x[r] - oa @ ob) ** 2).sum()
+        assert abs(got - want) <= 1e-3 * max(want, 1e-6 * (x[r].astype(np.float64) ** 2).sum()), r
