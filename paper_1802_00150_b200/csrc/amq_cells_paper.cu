@@ -20,6 +20,7 @@ struct PaperWorkspace {
     float* h[2];        // [batch][H] ping / pong
     float* c;           // [batch][H]
     float* gates;       // [4H] pre-activations of a single sequence (batch 1)
+    uint32_t* counters; // progress counters of the batched sequence kernel (batch > 1)
     size_t bytes;
 };
 
@@ -35,6 +36,7 @@ PaperWorkspace carve(void* base, int H, int batch, int steps, int k_a)
     w.h[1] = reinterpret_cast<float*>(p + off);      off += round_up((size_t)batch * H * 4, 256);
     w.c = reinterpret_cast<float*>(p + off);         off += round_up((size_t)batch * H * 4, 256);
     w.gates = reinterpret_cast<float*>(p + off);     off += round_up((size_t)4 * H * 4, 256);
+    w.counters = reinterpret_cast<uint32_t*>(p + off); off += batched_counter_bytes(batch);
     w.bytes = off;
     return w;
 }
@@ -108,6 +110,20 @@ amq_status recurrent_part(const PaperCall& c, const PaperWorkspace& ws, const fl
     return launch_binary_gemm(a, st);
 }
 
+// The time loop in one launch (batches; a step is a sequence of one, so that steps and sequences give the same bits);
+// AMQ_ERR_UNSUPPORTED: nothing has been enqueued.
+amq_status one_launch(const PaperCall& c, const PaperWorkspace& ws, int steps, const float* h0, const float* c0, float* h_seq, float* h_last,
+                      float* c_last, cudaStream_t st)
+{
+    BatchedSequence b{c.Wh_codes, c.Wh_alpha, nullptr, 0, c.H, c.H, c.k_w, c.k_a, c.T, c.batch, steps, false, nullptr, h0, c0,
+                      h_seq, h_last, c_last, {ws.h[0], ws.h[1]}, ws.c, ws.proj, ws.hcodes, ws.hbeta, ws.counters, nullptr};
+    if (!batched_sequence_supported(b)) return AMQ_ERR_UNSUPPORTED;
+    const amq_status s = tc_status_word(&b.status);         // (reported by amq_device_status, as for the kernels of the chain)
+    if (s != AMQ_OK) return s;
+    AMQ_CUDA_TRY(cudaMemsetAsync(ws.counters, 0, batched_counter_bytes(c.batch), st));
+    return launch_batched_sequence(b, st);
+}
+
 }  // namespace
 }  // namespace amq
 
@@ -135,6 +151,8 @@ amq_status amq_lstm_step_paper(const uint32_t* Wi_codes, const float* Wi_alpha, 
     cudaStream_t st = (cudaStream_t)stream;
     s = amq::input_projection(c, xcodes, xbeta, batch, ws.proj, st);
     if (s != AMQ_OK) return s;
+    s = amq::one_launch(c, ws, 1, h_in, c_in, nullptr, h_out, c_out, st);
+    if (s != AMQ_ERR_UNSUPPORTED) return s;
     return amq::recurrent_part(c, ws, ws.proj, h_in, c_in, h_out, c_out, st);
 }
 
@@ -159,6 +177,8 @@ amq_status amq_lstm_sequence_paper(const uint32_t* Wi_codes, const float* Wi_alp
     if (steps > 0) {
         s = amq::input_projection(c, xcodes_seq, xbeta_seq, steps * batch, ws.proj, st);
         if (s != AMQ_OK) return s;
+        s = amq::one_launch(c, ws, steps, h0, c0, h_seq, h_last, c_last, st);
+        if (s != AMQ_ERR_UNSUPPORTED) return s;
     }
     AMQ_CUDA_TRY(cudaMemcpyAsync(ws.c, c0, state_bytes, cudaMemcpyDeviceToDevice, st));
     const float* h_prev = h0;

@@ -197,6 +197,8 @@ struct BatchedSequence {
     const float* addend;
     uint32_t* zcodes; float* zbeta; uint32_t* counters; uint32_t* status;
 };
+// the form with the weights in tensor memory, where they fit; AMQ_ERR_UNSUPPORTED (nothing enqueued) where they do not
+amq_status launch_resident_sequence(const BatchedSequence& s, cudaStream_t st);
 bool batched_sequence_supported(const BatchedSequence& s);
 amq_status launch_batched_sequence(const BatchedSequence& s, cudaStream_t st);
 

@@ -11,14 +11,13 @@
 // of the activation planes by every tile of weight rows.  What bounds a timestep now: the steps of the weight pipeline (240-300
 // clocks per 256 bit positions of 128 plane-rows), the quantizer's chain of reductions, and the two waits.
 #include "amq_resident.cuh"
-#include "amq_quantize_device.cuh"
+#include "amq_sequence.cuh"
 
 namespace amq {
 
 namespace {
 
 constexpr int SEQ_Y_LD = 132;                   // row stride of the staged pre-activations
-constexpr unsigned SEQ_POLL_LIMIT = 1u << 21;   // looks at a counter before giving up (a second or so)
 using R = ResRoles<2, 8, 3>;                     // (640 threads: 96 registers each; the quantizer and the epilogue spill with 64)
 constexpr int SEQ_QUANT_WARPS = 16;             // warps that quantize: two teams of 8, or one of 16
 constexpr int SEQ_NG = 2;                       // groups of eight vectors per epilogue thread: blocks of up to 32 vectors
@@ -26,35 +25,18 @@ constexpr int SEQ_NG = 2;                       // groups of eight vectors per e
 struct SeqParams {
     ResProblem p;               // units = H
     const float* bias;
-    int H, T, steps, k_a;
-    int xn;                     // elements of z that come from x (0: z = h)
+    int H, steps, k_a;
+    SeqVectors z;
     const float* x_seq; const float* h0; const float* c0;
     float* h_seq; float* h_last; float* c_last;
     float* h[2]; float* c;
     const float* addend;        // [steps][batch][4H] added before the gates, or null
-    uint32_t* zcodes; float* zbeta;
     uint32_t* counters;         // [blocks][64]: word 0 quantized shares, word 32 finished products
     uint32_t* status;
     int P, unit_blocks, b_bytes;
     int team_warps;             // warps per quantized vector
     int unit_steps;             // pipeline steps of a block of units
 };
-
-__device__ __forceinline__ void seq_publish(uint32_t* counter)
-{
-    __threadfence();
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" :: "l"(counter) : "memory");
-}
-
-__device__ __forceinline__ bool seq_wait(const uint32_t* counter, uint32_t target)
-{
-    for (unsigned i = 0; i < SEQ_POLL_LIMIT; ++i) {
-        uint32_t v;
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(counter) : "memory");
-        if (v >= target) return true;
-    }
-    return false;
-}
 
 // shared memory behind the activation operand
 struct __align__(16) SeqShared {
@@ -65,54 +47,6 @@ struct __align__(16) SeqShared {
     uint32_t table[RES_TABLE];
     ResSync sync;
 };
-
-// Quantize one vector with a team of warps, thread g of the team owning the elements EPT g .. EPT g + EPT - 1.
-template <int KA, int EPT>
-__device__ __forceinline__ void seq_quantize(const SeqParams& a, const float* x, const float* h, int vector,
-                                             QuantScratch<KA, SEQ_QUANT_WARPS>& sc, const QuantTeam& team, int& parity)
-{
-    const int n = a.p.n, g = team.warp * 32 + ((int)threadIdx.x & 31), t0 = g * EPT;
-    float w[EPT];
-    uint32_t valid = 0;
-    const float* xr = x + (size_t)vector * a.xn;
-    const float* hr = h + (size_t)vector * a.H - a.xn;
-#pragma unroll
-    for (int q = 0; q < EPT / 4; ++q) {
-        const int t = t0 + 4 * q;
-        const float* p = (t < a.xn ? xr : hr) + t;
-        const bool one_piece = t + 3 < n && (t + 3 < a.xn || t >= a.xn) && (reinterpret_cast<uintptr_t>(p) & 15u) == 0;
-        if (one_piece) {
-            const float4 v = __ldcg(reinterpret_cast<const float4*>(p));        // (h: written by other SMs)
-            w[4 * q] = v.x; w[4 * q + 1] = v.y; w[4 * q + 2] = v.z; w[4 * q + 3] = v.w;
-            valid |= 0xFu << (4 * q);
-        } else {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const bool ok = t + e < n;
-                w[4 * q + e] = ok ? __ldcg((t + e < a.xn ? xr : hr) + t + e) : 0.0f;
-                valid |= (ok ? 1u : 0u) << (4 * q + e);
-            }
-        }
-    }
-    float beta[KA];
-    uint32_t bits[KA];
-    quantize_group<KA, EPT, SEQ_QUANT_WARPS>(w, valid, n, quant_padding_consecutive(n, EPT), a.T, beta, bits, sc, nullptr, &parity, team);
-    const int wpr = a.p.wpr;
-    if (t0 < wpr * 32) {
-#pragma unroll
-        for (int i = 0; i < KA; ++i)
-            if (EPT == 8) reinterpret_cast<uint8_t*>(a.zcodes + ((size_t)vector * KA + i) * wpr)[g] = (uint8_t)bits[i];
-            else reinterpret_cast<uint16_t*>(a.zcodes + ((size_t)vector * KA + i) * wpr)[g] = (uint16_t)bits[i];
-    }
-    if (g < KA) {
-        float b = beta[0];
-#pragma unroll
-        for (int i = 1; i < KA; ++i) b = (g == i) ? beta[i] : b;
-        a.zbeta[(size_t)vector * KA + g] = b;
-    }
-}
-
-__device__ __forceinline__ float seq_logistic(float v) { return 1.0f / (1.0f + __expf(-v)); }
 
 // The state update of one (unit, vector) from its staged pre-activations `yv` (gate g at yv[32 g]) and biases.
 __device__ __forceinline__ void seq_cell(const SeqParams& a, const float* yv, const float (&bias)[4], const float* addend, size_t o,
@@ -189,10 +123,10 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
             if (__syncthreads_or(!ok)) { ok = false; break; }
         }
         if (warp < SEQ_QUANT_WARPS) {
-            const float* x = a.x_seq + (size_t)t * p.batch * a.xn;
+            const float* x = a.x_seq + (size_t)t * p.batch * a.z.xn;
 #pragma unroll 1
             for (int v = part + team * a.P; v < in_block; v += teams * a.P)
-                seq_quantize<KA, EPT>(a, x, h_prev, b0 + v, scratch[team], quant, quant_parity);
+                seq_quantize<KA, EPT, SEQ_QUANT_WARPS>(a.z, x, h_prev, b0 + v, scratch[team], quant, quant_parity);
         }
         __syncthreads();
         if (tid == 0) {
@@ -204,9 +138,9 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
         // ---- 2. the planes of the whole block as the activation operand ----
         if (tid < p.N) {
             const int b = b0 + res_row_vector<KA>(tid), j = res_row_plane<KA>(tid);
-            sh.beta[tid] = tid < p.TB * KA && b < p.batch ? __ldcg(a.zbeta + (size_t)b * KA + j) : 0.0f;
+            sh.beta[tid] = tid < p.TB * KA && b < p.batch ? __ldcg(a.z.zbeta + (size_t)b * KA + j) : 0.0f;
         }
-        res_expand_activations<KA>(p, a.zcodes, b0, sB, sh.sum[0]);
+        res_expand_activations<KA>(p, a.z.zcodes, b0, sB, sh.sum[0]);
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -354,10 +288,11 @@ bool plan(const BatchedSequence& s, SeqPlan* out)
     if (best == 0.0) return false;
     const int blocks = (s.batch + a.p.TB - 1) / a.p.TB;
     a.b_bytes = a.p.NS * a.p.N * 128;
-    a.bias = s.bias; a.H = s.H; a.T = s.T; a.steps = s.steps; a.k_a = s.k_a; a.xn = s.n - s.H;
+    a.bias = s.bias; a.H = s.H; a.steps = s.steps; a.k_a = s.k_a;
+    a.z = SeqVectors{s.n, a.p.wpr, s.H, s.n - s.H, s.T, s.zcodes, s.zbeta, (size_t)a.p.wpr * 4, 16};
     a.x_seq = s.x_seq; a.h0 = s.h0; a.c0 = s.c0; a.h_seq = s.h_seq; a.h_last = s.h_last; a.c_last = s.c_last;
     a.h[0] = s.h[0]; a.h[1] = s.h[1]; a.c = s.c; a.addend = s.addend;
-    a.zcodes = s.zcodes; a.zbeta = s.zbeta; a.counters = s.counters; a.status = s.status;
+    a.counters = s.counters; a.status = s.status;
     out->grid = blocks * a.P;
     out->smem = (size_t)a.b_bytes + seq_more_smem(a.p);
     out->a = a;
@@ -386,6 +321,8 @@ bool batched_sequence_supported(const BatchedSequence& s)
 
 amq_status launch_batched_sequence(const BatchedSequence& s, cudaStream_t st)
 {
+    const amq_status r = launch_resident_sequence(s, st);
+    if (r != AMQ_ERR_UNSUPPORTED) return r;
     SeqPlan pl;
     if (!plan(s, &pl)) return AMQ_ERR_UNSUPPORTED;
     switch (s.k_a) {
