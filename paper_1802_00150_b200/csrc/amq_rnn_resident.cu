@@ -24,7 +24,9 @@ namespace amq {
 
 namespace {
 
-constexpr int RS_WARPS = 16, RS_WORKERS = 32 * RS_WARPS, RS_THREADS = RS_WORKERS + 32;      // the last warp issues the MMAs
+// Sixteen warps (128 registers a thread: the quantizer and the folding spill with the 96 that a seventeenth leaves); while the others expand
+// operand rows the last one issues the MMAs.
+constexpr int RS_WARPS = 16, RS_THREADS = 32 * RS_WARPS, RS_MMA_WARP = RS_WARPS - 1, RS_FEEDERS = 32 * RS_MMA_WARP;
 constexpr int RS_CHUNKS = 4;                    // (row, slot) pairs per thread and pass: shared memory holds 1800
 constexpr int RS_TMEM_COLS = 512, RS_SF_COLS = 16;
 constexpr int RS_SMEM_LIMIT = 226 * 1024, RS_SMEM_MIN = 116 * 1024;       // (more than half an SM's: one CTA per SM)
@@ -98,8 +100,6 @@ __device__ __forceinline__ void rs_expand_row(uint32_t addr, const uint4& v, int
                      ((v.w << (3 - s)) & 0x88888888u) | 0x22222222u);
 }
 
-__device__ __forceinline__ void rs_worker_bar() { asm volatile("bar.sync 1, %0;" :: "n"(RS_WORKERS) : "memory"); }
-
 template <int KA, int NW>
 __global__ void __launch_bounds__(RS_THREADS, 1)
 rnn_resident_kernel(const __grid_constant__ RsParams a)
@@ -122,11 +122,11 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
 
     if (tid == 0) {
 #pragma unroll
-        for (int q = 0; q < RS_CHUNKS; ++q) mbar_init(smem_u32(&sh.chunk[q]), RS_WARPS);
+        for (int q = 0; q < RS_CHUNKS; ++q) mbar_init(smem_u32(&sh.chunk[q]), RS_MMA_WARP);
         mbar_init(smem_u32(&sh.done), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == RS_WARPS) {
+    if (warp == RS_MMA_WARP) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      :: "r"(smem_u32(&sh.tmem_slot)), "r"((uint32_t)RS_TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -149,7 +149,7 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = __shfl_sync(0xffffffffu, sh.tmem_slot, 0), sf = tmem + (uint32_t)(a.tiles * a.N), a0 = sf + RS_SF_COLS;
     if (warp < 4) write_unit_scales(tmem, a.tiles * a.N, warp);
-    if (warp < RS_WARPS) rs_expand_weights(a, a0, u0, warp, lane);      // (made visible to the MMAs by the barriers of the first timestep)
+    rs_expand_weights(a, a0, u0, warp, lane);      // (made visible to the MMAs by the barriers of the first timestep)
 
     const QuantTeam quant{warp % NW, 8 + warp / NW, NW * 32};
     int quant_parity = 0;
@@ -157,7 +157,7 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
     // every CTA takes the slots from another one on: they all read the same planes at the same time
     const int first_slot = part % a.NS;
     int rows_now = 0, slot_0 = 0, row_0 = 0, d_slot = 0, d_row = 0;     // this thread's first (slot, row) of a pass, and the step to the next
-    const int v_0 = tid / units, ul_0 = tid - v_0 * units, d_v = RS_WORKERS / units, d_ul = RS_WORKERS - d_v * units;    // the same of (vector, unit)
+    const int v_0 = tid / units, ul_0 = tid - v_0 * units, d_v = RS_THREADS / units, d_ul = RS_THREADS - d_v * units;    // the same of (vector, unit)
     bool ok = true;
 
 #pragma unroll 1
@@ -171,16 +171,14 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
                 if (tid == 0) ok = seq_wait(counter + 32, (uint32_t)(t * a.P));
                 if (__syncthreads_or(!ok)) { ok = false; break; }
             }
-            if (warp < RS_WARPS) {
-                const float* x = a.x_seq + (size_t)t * a.batch * a.z.xn;
+            const float* x = a.x_seq + (size_t)t * a.batch * a.z.xn;
 #pragma unroll 1
-                for (int v = part + warp / NW * a.P; v < in_block; v += RS_WARPS / NW * a.P) {
-                    seq_quantize<KA, 8, NW>(a.z, x, h_prev, b0 + v, scratch[warp / NW], quant, quant_parity);
-                    // the next timestep's inputs on their way into L2
-                    const int e = (quant.warp * 32 + lane) * 8;
-                    if (!last && e < a.z.xn)
-                        asm volatile("prefetch.global.L2 [%0];" :: "l"(x + (size_t)(a.batch + b0 + v) * a.z.xn + e));
-                }
+            for (int v = part + warp / NW * a.P; v < in_block; v += RS_WARPS / NW * a.P) {
+                seq_quantize<KA, 8, NW>(a.z, x, h_prev, b0 + v, scratch[warp / NW], quant, quant_parity);
+                // the next timestep's inputs on their way into L2
+                const int e = (quant.warp * 32 + lane) * 8;
+                if (!last && e < a.z.xn)
+                    asm volatile("prefetch.global.L2 [%0];" :: "l"(x + (size_t)(a.batch + b0 + v) * a.z.xn + e));
             }
             __syncthreads();
             if (tid == 0) seq_publish(counter);
@@ -195,25 +193,33 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
 #pragma unroll 1
         for (int v0 = 0; v0 < in_block; v0 += a.TB, phase ^= 1u) {
             const int nv = in_block - v0 < a.TB ? in_block - v0 : a.TB, rows = nv * KA;
-            if (warp == RS_WARPS) {
+            if (warp == RS_MMA_WARP) {
+                if (v0 > 0) __syncthreads();
                 // ---- 2. MMAs of a slot as soon as its operand rows are there ----
                 const bool issues = elect_one();
                 const uint32_t idesc = (1u << 7) | (1u << 10) | ((uint32_t)(a.N >> 3) << 17) | (1u << 23) | (8u << 24);     // E2M1, E8M0, M 128
                 const uint64_t desc = smem_desc(sB);
                 const uint32_t lo = (uint32_t)desc, hi = (uint32_t)(desc >> 32);
-                int have = 0, slot = first_slot;
+                int s = 0;
+                uint32_t b = lo + (uint32_t)(first_slot * a.N * 8), w = a0 + (uint32_t)(first_slot * 32), wrap = (uint32_t)(a.NS - first_slot);
 #pragma unroll 1
-                for (int s = 0; s < a.NS && ok; ++s) {
-                    for (const int need = ((s + 1) * rows - 1) / RS_WORKERS + 1; have < need && ok; ++have)
-                        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&sh.chunk[have]), phase));
-                    if (!ok) break;
+                for (int have = 1; s < a.NS && ok; ++have) {
+                    ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&sh.chunk[have - 1]), phase));
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    // the slots whose rows the chunks so far cover, without a look at anything in between
+                    int end = have * RS_FEEDERS / rows;
+                    if (end > a.NS) end = a.NS;
 #pragma unroll 1
-                    for (int tile = 0; tile < a.tiles; ++tile)
-                        if (issues)
-                            mma_mxf4_stage_ta(tmem + (uint32_t)(tile * a.N), a0 + (uint32_t)((tile * a.NS + slot) * 32), lo + (uint32_t)(slot * a.N * 8), hi,
-                                              idesc, s != 0 ? 1u : 0u, sf);
-                    if (++slot == a.NS) slot = 0;
+                    for (; s < end; ++s) {
+                        if (s == (int)wrap) { b = lo; w = a0; }
+                        uint32_t wt = w, acc = tmem;
+#pragma unroll 1
+                        for (int tile = 0; tile < a.tiles; ++tile) {
+                            if (issues) mma_mxf4_stage_ta(acc, wt, b, hi, idesc, s != 0 ? 1u : 0u, sf);
+                            wt += (uint32_t)(a.NS * 32); acc += (uint32_t)a.N;
+                        }
+                        b += (uint32_t)(a.N * 8); w += 32;
+                    }
                 }
                 if (issues && ok) mma_commit(smem_u32(&sh.done));
                 __syncwarp();
@@ -221,7 +227,7 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
                 const size_t row0 = (size_t)(b0 + v0) * KA, half = (size_t)a.batch * KA;
                 if (rows != rows_now) {
                     rows_now = rows;
-                    slot_0 = tid / rows; row_0 = tid - slot_0 * rows; d_slot = RS_WORKERS / rows; d_row = RS_WORKERS - d_slot * rows;
+                    slot_0 = tid / rows; row_0 = tid - slot_0 * rows; d_slot = RS_FEEDERS / rows; d_row = RS_FEEDERS - d_slot * rows;
                 }
                 uint4 lo[RS_CHUNKS], hi[RS_CHUNKS];
                 uint32_t addr[RS_CHUNKS];           // 0: no such pair
@@ -239,7 +245,7 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
                     slot += d_slot; row += d_row;
                     if (row >= rows) { row -= rows; ++slot; }
                 }
-                if (v0 > 0) rs_worker_bar();        // the folded rows of the pass before have been read
+                if (v0 > 0) __syncthreads();        // the folded rows of the pass before have been read
                 if (tid < rows) sh.beta[tid] = __ldcg(a.z.zbeta + row0 + tid);
 #pragma unroll
                 for (int q = 0; q < RS_CHUNKS; ++q) {
@@ -251,86 +257,92 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
                     __syncwarp();
                     if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(&sh.chunk[q])) : "memory");
                 }
+            }
 
-                // the first addends of this thread on their way
-                float ahead[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-                if (a.addend && v_0 < nv) {
+            // the first addends of this thread on their way
+            float ahead[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+            if (a.addend && v_0 < nv) {
 #pragma unroll
-                    for (int g = 0; g < 4; ++g)
-                        ahead[g] = __ldcg(a.addend + (((size_t)t * a.batch + b0 + v0 + v_0) * 4 + g) * H + u0 + ul_0);
-                }
+                for (int g = 0; g < 4; ++g)
+                    ahead[g] = __ldcg(a.addend + (((size_t)t * a.batch + b0 + v0 + v_0) * 4 + g) * H + u0 + ul_0);
+            }
 
-                // ---- 3. accumulators: sum over the activation planes of every plane-row ----
-                rs_worker_bar();                    // (the coefficients)
-                if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&sh.done), phase))) ok = false;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const int r = (warp & 3) * 32 + lane;
+            // ---- 3. accumulators: sum over the activation planes of every plane-row ----
+            __syncthreads();                        // (the coefficients)
+            if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&sh.done), phase))) ok = false;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const int r = (warp & 3) * 32 + lane;
 #pragma unroll 1
-                for (int tile = 0; tile < a.tiles && ok; ++tile) {
-                    const int in_tile = all_rows - tile * rows_per_tile < rows_per_tile ? all_rows - tile * rows_per_tile : rows_per_tile;
-                    if ((warp & 3) * 32 >= in_tile) break;          // (uniform over the warp)
-                    const uint32_t acc = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(tile * a.N);
+            for (int tile = 0; tile < a.tiles && ok; ++tile) {
+                const int in_tile = all_rows - tile * rows_per_tile < rows_per_tile ? all_rows - tile * rows_per_tile : rows_per_tile;
+                if ((warp & 3) * 32 >= in_tile) break;          // (uniform over the warp)
+                const uint32_t acc = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(tile * a.N);
 #pragma unroll 1
-                    for (int g = (warp >> 2) * 8; g < nv; g += RS_WARPS / 4 * 8) {
-                        int d[KA][8];
+                for (int g = (warp >> 2) * 8; g < nv; g += RS_WARPS / 4 * 8) {
+                    int d[KA][8];
+                    float beta[8 * KA];
 #pragma unroll
-                        for (int q = 0; q < KA; ++q) tmem_ld8(acc + (uint32_t)(g * KA + 8 * q), d[q]);
-                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    for (int q = 0; q < KA; ++q) tmem_ld8(acc + (uint32_t)(g * KA + 8 * q), d[q]);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                        for (int q = 0; q < KA; ++q)
-                            asm volatile("" : "+r"(d[q][0]), "+r"(d[q][1]), "+r"(d[q][2]), "+r"(d[q][3]), "+r"(d[q][4]), "+r"(d[q][5]),
-                                              "+r"(d[q][6]), "+r"(d[q][7]));
+                    for (int q = 0; q < KA; ++q)
+                        asm volatile("" : "+r"(d[q][0]), "+r"(d[q][1]), "+r"(d[q][2]), "+r"(d[q][3]), "+r"(d[q][4]), "+r"(d[q][5]),
+                                          "+r"(d[q][6]), "+r"(d[q][7]));
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            float s = sh.beta[(g + e) * KA] * __int_as_float(d[e * KA / 8][e * KA % 8]);
+                    for (int q = 0; q < 2 * KA; ++q) {
+                        const float4 v = *reinterpret_cast<const float4*>(sh.beta + g * KA + 4 * q);
+                        beta[4 * q] = v.x; beta[4 * q + 1] = v.y; beta[4 * q + 2] = v.z; beta[4 * q + 3] = v.w;
+                    }
 #pragma unroll
-                            for (int j = 1; j < KA; ++j)
-                                s = fmaf(sh.beta[(g + e) * KA + j], __int_as_float(d[(e * KA + j) / 8][(e * KA + j) % 8]), s);
-                            if (g + e < nv && r < in_tile) sS[(g + e) * LD + tile * rows_per_tile + r] = s;
-                        }
+                    for (int e = 0; e < 8; ++e) {
+                        float s = beta[e * KA] * __int_as_float(d[e * KA / 8][e * KA % 8]);
+#pragma unroll
+                        for (int j = 1; j < KA; ++j)
+                            s = fmaf(beta[e * KA + j], __int_as_float(d[(e * KA + j) / 8][(e * KA + j) % 8]), s);
+                        if (g + e < nv && r < in_tile) sS[(g + e) * LD + tile * rows_per_tile + r] = s;
                     }
                 }
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                rs_worker_bar();
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncthreads();
 
-                // ---- 4. sum over the weight planes, gates ----
-                int v = v_0, ul = ul_0;
+            // ---- 4. sum over the weight planes, gates ----
+            int v = v_0, ul = ul_0;
 #pragma unroll 1
-                for (; v < nv && ok; v += d_v, ul += d_ul) {
-                    if (ul >= units) {
-                        ul -= units;
-                        if (++v >= nv) break;
-                    }
-                    const size_t o = (size_t)(b0 + v0 + v) * H + u0 + ul;
-                    const float* add = a.addend ? a.addend + ((size_t)t * a.batch + b0 + v0 + v) * 4 * H + u0 + ul : nullptr;
-                    const float* ss = sS + v * LD + ul * 4 * k_w;
-                    const float* al = sAlpha + ul * 4 * k_w;
-                    float* state = sState + (v0 + v) * a.upc + ul;
-                    float g4[4];
-#pragma unroll
-                    for (int g = 0; g < 4; ++g) {
-                        float y = 0.0f;
-#pragma unroll
-                        for (int i = 0; i < AMQ_MAX_K; ++i)
-                            if (i < k_w) y = fmaf(al[g * k_w + i], ss[g * k_w + i], y);
-                        g4[g] = y + sBias[4 * ul + g];
-                        if (add) g4[g] += v == v_0 ? ahead[g] : __ldcg(add + (size_t)g * H);
-                    }
-                    float h;
-                    if (!a.gru) {
-                        const float ig = seq_logistic(g4[0]), fg = seq_logistic(g4[1]), og = seq_logistic(g4[2]);
-                        const float c = fg * *state + ig * tanhf(g4[3]);
-                        *state = c;
-                        if (last) a.c_last[o] = c;
-                        h = og * tanhf(c);
-                    } else {
-                        const float rg = seq_logistic(g4[0]), zg = seq_logistic(g4[1]), cand = tanhf(g4[2] + rg * g4[3]);
-                        h = (1.0f - zg) * cand + zg * *state;
-                        *state = h;
-                    }
-                    h_next[o] = h;
-                    if (h_also) h_also[o] = h;
+            for (; v < nv && ok; v += d_v, ul += d_ul) {
+                if (ul >= units) {
+                    ul -= units;
+                    if (++v >= nv) break;
                 }
+                const size_t o = (size_t)(b0 + v0 + v) * H + u0 + ul;
+                const float* add = a.addend ? a.addend + ((size_t)t * a.batch + b0 + v0 + v) * 4 * H + u0 + ul : nullptr;
+                const float* ss = sS + v * LD + ul * 4 * k_w;
+                const float* al = sAlpha + ul * 4 * k_w;
+                float* state = sState + (v0 + v) * a.upc + ul;
+                float g4[4];
+#pragma unroll
+                for (int g = 0; g < 4; ++g) {
+                    float y = 0.0f;
+#pragma unroll
+                    for (int i = 0; i < AMQ_MAX_K; ++i)
+                        if (i < k_w) y = fmaf(al[g * k_w + i], ss[g * k_w + i], y);
+                    g4[g] = y + sBias[4 * ul + g];
+                    if (add) g4[g] += v == v_0 ? ahead[g] : __ldcg(add + (size_t)g * H);
+                }
+                float h;
+                if (!a.gru) {
+                    const float ig = seq_logistic(g4[0]), fg = seq_logistic(g4[1]), og = seq_logistic(g4[2]);
+                    const float c = fg * *state + ig * tanhf(g4[3]);
+                    *state = c;
+                    if (last) a.c_last[o] = c;
+                    h = og * tanhf(c);
+                } else {
+                    const float rg = seq_logistic(g4[0]), zg = seq_logistic(g4[1]), cand = tanhf(g4[2] + rg * g4[3]);
+                    h = (1.0f - zg) * cand + zg * *state;
+                    *state = h;
+                }
+                h_next[o] = h;
+                if (h_also) h_also[o] = h;
             }
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -346,7 +358,7 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
         __nanosleep(1000000);
         __syncthreads();
     }
-    if (warp == RS_WARPS)
+    if (warp == RS_MMA_WARP)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"((uint32_t)RS_TMEM_COLS) : "memory");
 }
 
@@ -369,7 +381,7 @@ bool plan(const BatchedSequence& s, RsPlan* out)
         P = (s.H + upc - 1) / upc;
         for (int passes = 1; passes <= 64 && passes <= block; ++passes) {
             const int TB = (block + passes - 1) / passes, N = (TB * s.k_a + 15) / 16 * 16;
-            if (N > 256 || tiles * (32 * NS + N) + RS_SF_COLS > RS_TMEM_COLS || TB * s.k_a * NS > RS_CHUNKS * RS_WORKERS) continue;
+            if (N > 256 || tiles * (32 * NS + N) + RS_SF_COLS > RS_TMEM_COLS || TB * s.k_a * NS > RS_CHUNKS * RS_FEEDERS) continue;
             size_t b = (size_t)NS * N * 128;
             const size_t folded = (size_t)TB * (all_rows | 1) * 4, scratch = RS_WARPS / NW * sizeof(QuantScratch<4, 16>);
             if (folded > b) b = folded;
@@ -380,7 +392,7 @@ bool plan(const BatchedSequence& s, RsPlan* out)
             // clocks of a timestep: the quantizer's rounds; per pass the slower of expansion and tensor pipe, the folding, the gates
             const int teams = RS_WARPS / NW, vectors = (block + P - 1) / P;
             const double expand = 2.2 * TB * s.k_a * NS, mma = 4.0 * NS * tiles * (N > 92 ? 0.5 * N : 46.0);
-            const double fold = 5.0 * tiles * TB * s.k_a, gates = 500.0 * ((TB * upc + RS_WORKERS - 1) / RS_WORKERS);
+            const double fold = 5.0 * tiles * TB * s.k_a, gates = 500.0 * ((TB * upc + RS_THREADS - 1) / RS_THREADS);
             const double t = (vectors + teams - 1) / teams * (s.k_a >= 3 ? 4500.0 : 3500.0) + passes * ((expand > mma ? expand : mma) + fold + gates + 1500.0);
             if (best == 0.0 || t < best) {
                 best = t;
