@@ -3,6 +3,8 @@
 // epilogue.  No step returns to the host; a sequence is enqueued as one chain on the caller's stream.
 #include "amq_common.cuh"
 
+#include <mutex>
+
 namespace amq {
 
 namespace {
@@ -59,7 +61,7 @@ BatchedSequence batched_call(const CellCall& c, const CellWorkspace& ws, const f
                              float* h_seq, float* h_last, float* c_last)
 {
     return BatchedSequence{c.Wcodes, c.Walpha, c.bias, c.I, c.H, c.I + c.H, c.k_w, c.k_a, c.T, c.batch, steps, c.gru, x_seq, h0, c0,
-                           h_seq, h_last, c_last, {ws.h[0], ws.h[1]}, ws.c, nullptr, ws.zcodes, ws.zbeta, ws.counters, ws.status};
+                           h_seq, h_last, c_last, {ws.h[0], ws.h[1]}, ws.c, nullptr, ws.zcodes, ws.zbeta, ws.counters, ws.status, 0};
 }
 
 // quantize z = [x ; h_in] into the workspace, then product + gates
@@ -91,6 +93,45 @@ struct Chunks {
     cudaEvent_t ready[MAX_CHUNKS + 1];      // (one more, for the start of the copy stream)
 };
 
+// Copy stream and events of one host call.  Creating and destroying them cost 100 us a call, so up to LANES of them wait for the next call
+// (of any thread: a lane belongs to one call at a time); a lane more than that is destroyed when its call ends.
+constexpr int LANES = 4;
+struct CopyLane { int device; cudaStream_t stream; cudaEvent_t event[MAX_CHUNKS + 1]; };
+std::mutex g_lanes_mutex;
+CopyLane g_lanes[LANES];
+int g_lane_count = 0;
+
+void destroy_lane(CopyLane& l)
+{
+    for (cudaEvent_t& e : l.event) if (e) { cudaEventDestroy(e); e = nullptr; }
+    if (l.stream) { cudaStreamDestroy(l.stream); l.stream = nullptr; }
+}
+
+cudaError_t take_lane(CopyLane* out)
+{
+    CopyLane l{};
+    cudaError_t e = cudaGetDevice(&l.device);
+    if (e != cudaSuccess) return e;
+    {
+        std::lock_guard<std::mutex> lock(g_lanes_mutex);
+        for (int q = 0; q < g_lane_count; ++q)
+            if (g_lanes[q].device == l.device) { *out = g_lanes[q]; g_lanes[q] = g_lanes[--g_lane_count]; return cudaSuccess; }
+    }
+    e = cudaStreamCreateWithFlags(&l.stream, cudaStreamNonBlocking);
+    for (int q = 0; q <= MAX_CHUNKS && e == cudaSuccess; ++q) e = cudaEventCreateWithFlags(&l.event[q], cudaEventDisableTiming);
+    *out = l;
+    return e;
+}
+
+void give_lane(CopyLane& l)
+{
+    {
+        std::lock_guard<std::mutex> lock(g_lanes_mutex);
+        if (g_lane_count < LANES) { g_lanes[g_lane_count++] = l; l = CopyLane{}; return; }
+    }
+    destroy_lane(l);
+}
+
 // `chunks` (may be NULL): the stream waits for a chunk's event before the first kernel that reads it (batched calls only).
 amq_status enqueue_sequence(const CellCall& c, const CellWorkspace& ws, const float* x_seq, int steps,
                             const float* h0, const float* c0, float* h_seq, float* h_last, float* c_last,
@@ -107,10 +148,10 @@ amq_status enqueue_sequence(const CellCall& c, const CellWorkspace& ws, const fl
         for (int q = 0; q < (chunks ? chunks->count : 1); ++q) {
             const int s0 = chunks ? chunks->begin[q] : 0, s1 = chunks ? chunks->begin[q + 1] : steps;
             if (chunks) AMQ_CUDA_TRY(cudaStreamWaitEvent(st, chunks->ready[q], 0));
-            if (q > 0) AMQ_CUDA_TRY(cudaMemsetAsync(ws.counters, 0, ws.counter_bytes, st));
-            const amq_status r = launch_batched_sequence(
-                batched_call(c, ws, x_seq + (size_t)s0 * c.batch * c.I, s1 - s0, q ? h_last : h0, q ? c_last : c0,
-                             h_seq ? h_seq + (size_t)s0 * state : nullptr, h_last, c_last), st);
+            BatchedSequence b = batched_call(c, ws, x_seq + (size_t)s0 * c.batch * c.I, s1 - s0, q ? h_last : h0, q ? c_last : c0,
+                                             h_seq ? h_seq + (size_t)s0 * state : nullptr, h_last, c_last);
+            b.counted = s0;
+            const amq_status r = launch_batched_sequence(b, st);
             if (r != AMQ_OK) return r;
         }
         return AMQ_OK;
@@ -196,15 +237,11 @@ amq_status sequence_host_entry(const CellCall& c, const float* x_seq_host, int s
     const size_t x_bytes = (size_t)steps * c.batch * c.I * sizeof(float);
     // Large inputs of a batched call travel in chunks of timesteps on a stream of their own, so that the copy of the later
     // timesteps runs beside the kernels of the earlier ones (C4: 73 MB of inputs); the kernels wait for a chunk's event before
-    // its first step.  The copy stream and the events live for the duration of the call.  Chunks grow from a twelfth of the
-    // sequence by 1.6 to a quarter: nothing runs during the first copy, and every chunk is a launch.
+    // its first step.  Chunks grow from a twelfth of the sequence by 1.6 to a quarter (a remainder below half a chunk joins the last):
+    // nothing runs during the first copy, and every chunk is a launch.
     const bool chunked = x_bytes >= ((size_t)4 << 20) && steps >= 2 && !(steps > 0 && use_persistent(c));
-    cudaStream_t copy_stream = nullptr;
     Chunks chunks{};
-    auto release = [&]() {
-        for (cudaEvent_t e : chunks.ready) if (e) cudaEventDestroy(e);
-        if (copy_stream) cudaStreamDestroy(copy_stream);
-    };
+    CopyLane lane{};
     // the small copies of the initial state go first: host-to-device copies are served in the order they were submitted,
     // whatever their stream, and the chain's first kernel needs them
     cudaError_t e = cudaMemcpyAsync(hs.h0, h0_host, state_bytes, cudaMemcpyHostToDevice, st);
@@ -213,37 +250,36 @@ amq_status sequence_host_entry(const CellCall& c, const float* x_seq_host, int s
     if (chunked) {
         for (int done = 0, size = (steps + 11) / 12; done < steps; ++chunks.count) {
             chunks.begin[chunks.count] = done;
-            done = chunks.count == MAX_CHUNKS - 1 || done + size > steps ? steps : done + size;
+            done = chunks.count == MAX_CHUNKS - 1 || done + size + size / 2 > steps ? steps : done + size;
             chunks.begin[chunks.count + 1] = done;
             size = (size * 8 + 4) / 5;
             if (size > (steps + 3) / 4) size = (steps + 3) / 4;
         }
-        e = cudaStreamCreateWithFlags(&copy_stream, cudaStreamNonBlocking);
-        for (int q = 0; q <= chunks.count && e == cudaSuccess; ++q) e = cudaEventCreateWithFlags(&chunks.ready[q], cudaEventDisableTiming);
+        e = take_lane(&lane);
+        for (int q = 0; q <= MAX_CHUNKS; ++q) chunks.ready[q] = lane.event[q];
         // the copy stream starts after what the caller's stream holds so far (the staging buffer may still be in use there)
         if (e == cudaSuccess) e = cudaEventRecord(chunks.ready[chunks.count], st);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(copy_stream, chunks.ready[chunks.count], 0);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(lane.stream, chunks.ready[chunks.count], 0);
         const size_t step_bytes = (size_t)c.batch * c.I * sizeof(float);
         for (int q = 0; q < chunks.count && e == cudaSuccess; ++q) {
             const int s0 = chunks.begin[q], s1 = chunks.begin[q + 1];
             e = cudaMemcpyAsync(reinterpret_cast<char*>(hs.x_seq) + s0 * step_bytes,
                                 reinterpret_cast<const char*>(x_seq_host) + s0 * step_bytes, (size_t)(s1 - s0) * step_bytes,
-                                cudaMemcpyHostToDevice, copy_stream);
-            if (e == cudaSuccess) e = cudaEventRecord(chunks.ready[q], copy_stream);
+                                cudaMemcpyHostToDevice, lane.stream);
+            if (e == cudaSuccess) e = cudaEventRecord(chunks.ready[q], lane.stream);
         }
-        if (e != cudaSuccess) { cudaStreamSynchronize(copy_stream); release(); return AMQ_ERR_CUDA; }
+        if (e != cudaSuccess) { if (lane.stream) cudaStreamSynchronize(lane.stream); destroy_lane(lane); return AMQ_ERR_CUDA; }
     } else if (x_bytes) {
         AMQ_CUDA_TRY(cudaMemcpyAsync(hs.x_seq, x_seq_host, x_bytes, cudaMemcpyHostToDevice, st));
     }
     s = enqueue_sequence(c, ws, hs.x_seq, steps, hs.h0, hs.c0, h_seq_host ? hs.h_seq : nullptr, hs.h_last, hs.c_last, st,
                          chunked ? &chunks : nullptr);
-    if (chunked) {
-        // the events and the stream may go once both streams have drained
-        cudaStreamSynchronize(copy_stream);
-        if (s != AMQ_OK) cudaStreamSynchronize(st);
-    }
-    if (s != AMQ_OK) { release(); return s; }
-    struct Releaser { decltype(release)& r; ~Releaser() { r(); } } releaser{release};
+    // the lane goes back, and its next user may record its events again, once the caller's stream has passed every wait for them
+    struct Return {
+        CopyLane& lane; cudaStream_t st;
+        ~Return() { if (lane.stream) { cudaStreamSynchronize(lane.stream); cudaStreamSynchronize(st); give_lane(lane); } }
+    } give_back{lane, st};
+    if (s != AMQ_OK) return s;
     if (h_seq_host && steps > 0)
         AMQ_CUDA_TRY(cudaMemcpyAsync(h_seq_host, hs.h_seq, (size_t)steps * state_bytes, cudaMemcpyDeviceToHost, st));
     AMQ_CUDA_TRY(cudaMemcpyAsync(h_last_host, hs.h_last, state_bytes, cudaMemcpyDeviceToHost, st));

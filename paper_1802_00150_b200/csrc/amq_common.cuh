@@ -196,6 +196,7 @@ struct BatchedSequence {
     float* h[2]; float* c;
     const float* addend;
     uint32_t* zcodes; float* zbeta; uint32_t* counters; uint32_t* status;
+    int counted;                // timesteps that earlier launches have added to the counters since they were cleared
 };
 // the form with the weights in tensor memory, where they fit; AMQ_ERR_UNSUPPORTED (nothing enqueued) where they do not
 amq_status launch_resident_sequence(const BatchedSequence& s, cudaStream_t st);

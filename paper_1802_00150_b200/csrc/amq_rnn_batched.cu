@@ -33,6 +33,7 @@ struct SeqParams {
     const float* addend;        // [steps][batch][4H] added before the gates, or null
     uint32_t* counters;         // [blocks][64]: word 0 quantized shares, word 32 finished products
     uint32_t* status;
+    int counted;                // timesteps in the counters at the start
     int P, unit_blocks, b_bytes;
     int team_warps;             // warps per quantized vector
     int unit_steps;             // pipeline steps of a block of units
@@ -119,7 +120,7 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
 
         // ---- 1. this CTA's share of the block's vectors ----
         if (t > 0) {
-            if (tid == 0) ok = seq_wait(counter + 32, (uint32_t)(t * a.P));
+            if (tid == 0) ok = seq_wait(counter + 32, (uint32_t)((a.counted + t) * a.P));
             if (__syncthreads_or(!ok)) { ok = false; break; }
         }
         if (warp < SEQ_QUANT_WARPS) {
@@ -131,7 +132,7 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
         __syncthreads();
         if (tid == 0) {
             seq_publish(counter);
-            ok = seq_wait(counter, (uint32_t)((t + 1) * a.P));
+            ok = seq_wait(counter, (uint32_t)((a.counted + t + 1) * a.P));
         }
         if (__syncthreads_or(!ok)) { ok = false; break; }
 
@@ -226,7 +227,7 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
         }
         first_step = (first_step + my_blocks * a.unit_steps) & (R::GROUPS - 1);
         if (__syncthreads_or(!ok)) { ok = false; break; }
-        if (tid == 0 && !last) seq_publish(counter + 32);
+        if (tid == 0) seq_publish(counter + 32);
     }
 
     __syncwarp();
@@ -292,7 +293,7 @@ bool plan(const BatchedSequence& s, SeqPlan* out)
     a.z = SeqVectors{s.n, a.p.wpr, s.H, s.n - s.H, s.T, s.zcodes, s.zbeta, (size_t)a.p.wpr * 4, 16};
     a.x_seq = s.x_seq; a.h0 = s.h0; a.c0 = s.c0; a.h_seq = s.h_seq; a.h_last = s.h_last; a.c_last = s.c_last;
     a.h[0] = s.h[0]; a.h[1] = s.h[1]; a.c = s.c; a.addend = s.addend;
-    a.counters = s.counters; a.status = s.status;
+    a.counters = s.counters; a.counted = s.counted; a.status = s.status;
     out->grid = blocks * a.P;
     out->smem = (size_t)a.b_bytes + seq_more_smem(a.p);
     out->a = a;

@@ -41,6 +41,7 @@ struct RsParams {
     const float* addend;        // [steps][batch][4H] added before the gates, or null
     uint32_t* counters;         // [blocks][64]: word 0 quantized shares, word 32 finished products
     uint32_t* status;
+    int counted;                // timesteps in the counters at the start
     int P, block;               // CTAs and vectors of a block
     int upc, upt, tiles;        // units per CTA, per tile of 128 lanes
     int TB, N, NS;              // vectors and operand rows of a pass, slots of 256 positions
@@ -100,6 +101,28 @@ __device__ __forceinline__ void rs_expand_row(uint32_t addr, const uint4& v, int
                      ((v.w << (3 - s)) & 0x88888888u) | 0x22222222u);
 }
 
+// Folded rows of a vector: whole 16-byte pieces, an odd number of them (neighbouring vectors in different banks).
+__host__ __device__ inline int rs_folded_stride(int rows) { return (rows >> 2 | 1) << 2; }
+
+// The four gates of a unit from its 4 KW folded plane-rows, planes added in order.
+template <int KW>
+__device__ __forceinline__ void rs_unit_sums(const float* folded, const float* alpha, float (&g4)[4])
+{
+    float s[4 * KW], al[4 * KW];
+#pragma unroll
+    for (int q = 0; q < KW; ++q) {
+        const float4 v = reinterpret_cast<const float4*>(folded)[q], w = reinterpret_cast<const float4*>(alpha)[q];
+        s[4 * q] = v.x; s[4 * q + 1] = v.y; s[4 * q + 2] = v.z; s[4 * q + 3] = v.w;
+        al[4 * q] = w.x; al[4 * q + 1] = w.y; al[4 * q + 2] = w.z; al[4 * q + 3] = w.w;
+    }
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+        g4[g] = 0.0f;
+#pragma unroll
+        for (int i = 0; i < KW; ++i) g4[g] = fmaf(al[g * KW + i], s[g * KW + i], g4[g]);
+    }
+}
+
 template <int KA, int NW>
 __global__ void __launch_bounds__(RS_THREADS, 1)
 rnn_resident_kernel(const __grid_constant__ RsParams a)
@@ -109,7 +132,7 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
     const int bb = (int)blockIdx.x / a.P, part = (int)blockIdx.x - bb * a.P, b0 = bb * a.block;
     const int in_block = a.batch - b0 < a.block ? a.batch - b0 : a.block, quantizers = in_block < a.P ? in_block : a.P;
     const int u0 = part * a.upc, units = u0 < H ? (H - u0 < a.upc ? H - u0 : a.upc) : 0;
-    const int rows_per_tile = a.upt * 4 * k_w, all_rows = a.upc * 4 * k_w, LD = all_rows | 1;
+    const int rows_per_tile = a.upt * 4 * k_w, all_rows = a.upc * 4 * k_w, LD = rs_folded_stride(all_rows);
     RsShared& sh = *reinterpret_cast<RsShared*>(smem_raw + a.b_bytes);
     float* sAlpha = reinterpret_cast<float*>(&sh + 1);              // [all_rows]
     float* sBias = sAlpha + all_rows;                               // [upc][4]
@@ -147,7 +170,9 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = __shfl_sync(0xffffffffu, sh.tmem_slot, 0), sf = tmem + (uint32_t)(a.tiles * a.N), a0 = sf + RS_SF_COLS;
+    // All 512 columns start at column 0.  (As a constant the address keeps the operands of the MMAs in uniform registers.)
+    constexpr uint32_t tmem = 0;
+    const uint32_t sf = tmem + (uint32_t)(a.tiles * a.N), a0 = sf + RS_SF_COLS;
     if (warp < 4) write_unit_scales(tmem, a.tiles * a.N, warp);
     rs_expand_weights(a, a0, u0, warp, lane);      // (made visible to the MMAs by the barriers of the first timestep)
 
@@ -158,17 +183,17 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
     const int first_slot = part % a.NS;
     int rows_now = 0, slot_0 = 0, row_0 = 0, d_slot = 0, d_row = 0;     // this thread's first (slot, row) of a pass, and the step to the next
     const int v_0 = tid / units, ul_0 = tid - v_0 * units, d_v = RS_THREADS / units, d_ul = RS_THREADS - d_v * units;    // the same of (vector, unit)
-    bool ok = true;
+    bool ok = sh.tmem_slot == tmem;
 
 #pragma unroll 1
-    for (int t = 0; t < a.steps; ++t) {
+    for (int t = 0; ok && t < a.steps; ++t) {
         const bool last = t + 1 == a.steps;
         const float* h_prev = t == 0 ? a.h0 : (a.h_seq ? a.h_seq + (size_t)(t - 1) * a.batch * H : a.h[(t - 1) & 1]);
 
         // ---- 1. this CTA's share of the block's vectors ----
         if (part < quantizers) {                    // (uniform over the CTA)
             if (t > 0) {
-                if (tid == 0) ok = seq_wait(counter + 32, (uint32_t)(t * a.P));
+                if (tid == 0) ok = seq_wait(counter + 32, (uint32_t)((a.counted + t) * a.P));
                 if (__syncthreads_or(!ok)) { ok = false; break; }
             }
             const float* x = a.x_seq + (size_t)t * a.batch * a.z.xn;
@@ -183,7 +208,7 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
             __syncthreads();
             if (tid == 0) seq_publish(counter);
         }
-        if (tid == 0) ok = seq_wait(counter, (uint32_t)((t + 1) * quantizers));
+        if (tid == 0) ok = seq_wait(counter, (uint32_t)((a.counted + t + 1) * quantizers));
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         if (__syncthreads_or(!ok)) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -320,14 +345,15 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
                 const float* al = sAlpha + ul * 4 * k_w;
                 float* state = sState + (v0 + v) * a.upc + ul;
                 float g4[4];
+                if (k_w == 1) rs_unit_sums<1>(ss, al, g4);
+                else if (k_w == 2) rs_unit_sums<2>(ss, al, g4);
+                else if (k_w == 3) rs_unit_sums<3>(ss, al, g4);
+                else rs_unit_sums<4>(ss, al, g4);
+                const float4 bias = *reinterpret_cast<const float4*>(sBias + 4 * ul);
+                g4[0] += bias.x; g4[1] += bias.y; g4[2] += bias.z; g4[3] += bias.w;
+                if (add) {
 #pragma unroll
-                for (int g = 0; g < 4; ++g) {
-                    float y = 0.0f;
-#pragma unroll
-                    for (int i = 0; i < AMQ_MAX_K; ++i)
-                        if (i < k_w) y = fmaf(al[g * k_w + i], ss[g * k_w + i], y);
-                    g4[g] = y + sBias[4 * ul + g];
-                    if (add) g4[g] += v == v_0 ? ahead[g] : __ldcg(add + (size_t)g * H);
+                    for (int g = 0; g < 4; ++g) g4[g] += v == v_0 ? ahead[g] : __ldcg(add + (size_t)g * H);
                 }
                 float h;
                 if (!a.gru) {
@@ -347,7 +373,7 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         if (__syncthreads_or(!ok)) { ok = false; break; }
-        if (tid == 0 && !last) seq_publish(counter + 32);
+        if (tid == 0) seq_publish(counter + 32);
     }
 
     __syncwarp();
@@ -359,7 +385,7 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
         __syncthreads();
     }
     if (warp == RS_MMA_WARP)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"((uint32_t)RS_TMEM_COLS) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(sh.tmem_slot), "r"((uint32_t)RS_TMEM_COLS) : "memory");
 }
 
 struct RsPlan { RsParams a; int grid, warps; size_t smem; };
@@ -383,7 +409,7 @@ bool plan(const BatchedSequence& s, RsPlan* out)
             const int TB = (block + passes - 1) / passes, N = (TB * s.k_a + 15) / 16 * 16;
             if (N > 256 || tiles * (32 * NS + N) + RS_SF_COLS > RS_TMEM_COLS || TB * s.k_a * NS > RS_CHUNKS * RS_FEEDERS) continue;
             size_t b = (size_t)NS * N * 128;
-            const size_t folded = (size_t)TB * (all_rows | 1) * 4, scratch = RS_WARPS / NW * sizeof(QuantScratch<4, 16>);
+            const size_t folded = (size_t)TB * rs_folded_stride(all_rows) * 4, scratch = RS_WARPS / NW * sizeof(QuantScratch<4, 16>);
             if (folded > b) b = folded;
             if (scratch > b) b = scratch;
             b = round_up(b, 1024);
@@ -409,7 +435,7 @@ bool plan(const BatchedSequence& s, RsPlan* out)
     a.z = SeqVectors{s.n, words_per_row(s.n), s.H, s.n - s.H, s.T, s.zcodes, s.zbeta, 16, (size_t)s.batch * s.k_a * 16};
     a.I = s.I; a.k_w = s.k_w; a.gru = s.gru; a.steps = s.steps; a.batch = s.batch;
     a.x_seq = s.x_seq; a.h0 = s.h0; a.c0 = s.c0; a.h_seq = s.h_seq; a.h_last = s.h_last; a.c_last = s.c_last;
-    a.h[0] = s.h[0]; a.h[1] = s.h[1]; a.addend = s.addend; a.counters = s.counters; a.status = s.status;
+    a.h[0] = s.h[0]; a.h[1] = s.h[1]; a.addend = s.addend; a.counters = s.counters; a.counted = s.counted; a.status = s.status;
     *out = p;
     return true;
 }
