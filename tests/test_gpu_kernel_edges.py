@@ -59,7 +59,10 @@ def test_product_at_the_edges_of_its_tiles(amq, m, n, kw, ka, batch, offset):
     ("gru", 257, 129, 2, 2, 31),        # the column split one past a slot, one unit past a tile of 128
     ("gru", 512, 256, 4, 4, 65),        # the split on a slot
     ("gru", 2100, 2050, 1, 2, 5),       # rows of more than 4096 positions
-    ("lstm", 70, 1200, 4, 4, 70),
+    ("lstm", 70, 1200, 4, 4, 70),       # two tiles of plane-rows, several passes over the vectors
+    ("lstm", 1030, 500, 3, 2, 130),
+    ("gru", 1700, 1900, 1, 2, 3),       # fifteen slots: nearly all of tensor memory
+    ("lstm", 4000, 200, 2, 2, 17),      # weights that do not stay in tensor memory
 ])
 def test_batched_sequence_at_the_edges_of_its_tiles(amq, cell, I, H, kw, ka, batch):
     """Three timesteps in one call equal three calls of one timestep bit for bit; the first is held against the oracle."""
