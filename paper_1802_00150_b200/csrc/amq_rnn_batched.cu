@@ -6,6 +6,8 @@
 // gate rows (amq_resident.cuh) with the gates in the epilogue, wait for the other CTAs' h.  The two waits are counters in the
 // workspace, one pair per block of vectors: blocks never wait for one another.
 //
+// This is the form for weights that do not fit tensor memory (amq_rnn_resident.cu takes those that do).
+//
 // Against a quantizer launch and a product launch per timestep this takes out two launches (some 6 us of host time each on this
 // machine, which had become longer than the kernels), the set-up of tensor memory and barriers, and the repeated expansion
 // of the activation planes by every tile of weight rows.  What bounds a timestep now: the steps of the weight pipeline (240-300
@@ -288,6 +290,9 @@ bool plan(const BatchedSequence& s, SeqPlan* out)
         }
     if (best == 0.0) return false;
     const int blocks = (s.batch + a.p.TB - 1) / a.p.TB;
+    // several vectors per CTA: two teams take one each, sixteen elements a thread; their chains of reductions overlap
+    // (GRU 2048, 256 sequences, 35 steps: 1551 us with one team of sixteen warps, 1457 us)
+    if (s.n <= 4096 && a.p.TB > a.P) a.team_warps = 8;
     a.b_bytes = a.p.NS * a.p.N * 128;
     a.bias = s.bias; a.H = s.H; a.steps = s.steps; a.k_a = s.k_a;
     a.z = SeqVectors{s.n, a.p.wpr, s.H, s.n - s.H, s.T, s.zcodes, s.zbeta, (size_t)a.p.wpr * 4, 16};
@@ -303,7 +308,7 @@ bool plan(const BatchedSequence& s, SeqPlan* out)
 template <int KA>
 amq_status launch(const SeqPlan& pl, cudaStream_t st)
 {
-    auto kernel = pl.a.p.n <= 4096 ? rnn_batched_kernel<KA, 8> : rnn_batched_kernel<KA, 16>;
+    auto kernel = pl.a.p.n <= pl.a.team_warps * 256 ? rnn_batched_kernel<KA, 8> : rnn_batched_kernel<KA, 16>;
     AMQ_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem));
     SeqParams args = pl.a;
     void* params[] = {&args};
