@@ -156,8 +156,8 @@ AMQ_API amq_status amq_quantized_gemv(const uint32_t* Wcodes, const float* Walph
  * Synchronises `stream`, then reads and clears the library's device-side status word of the current
  * device: AMQ_OK, or AMQ_ERR_TIMEOUT if a bounded wait inside a product kernel ran out since the last
  * read (the outputs of that call are then undefined).  Covers amq_binary_dots, amq_binary_gemm and the
- * product inside the cell calls (amq_lstm_step_static included); the sequence kernels report through
- * amq_workspace_status as well.  The word belongs to the device, not to a stream: a failure on any stream of the
+ * product inside the cell calls (amq_lstm_step_static included), paper-form sequences and greedy decoding; the other
+ * sequence kernels report through amq_workspace_status.  The word belongs to the device, not to a stream: a failure on any stream of the
  * device is reported to whoever reads next (the read is one atomic swap enqueued on `stream`), and two host threads
  * reading at the same time must be serialised by the caller.
  */
@@ -337,8 +337,8 @@ AMQ_API amq_status amq_lm_greedy_decode(const uint32_t* We_codes, const float* W
  * (pinned memory makes the copies asynchronous) into `staging`, the sequence runs, and h_last / c_last
  * (and h_seq when not NULL) are copied back to host memory; the call returns after the stream has
  * drained.  Weights, bias, workspace and staging (amq_cell_host_staging_bytes) stay DEVICE pointers.
- * Inputs of 4 MiB and more of a batched sequence are copied in up to eight chunks of timesteps on a stream that
- * the call creates and destroys, so that the copy of later timesteps runs beside the kernels of earlier ones;
+ * Inputs of 4 MiB and more of a batched sequence are copied in up to eight chunks of timesteps on a stream of
+ * the library's (a few are kept between calls, each used by one call at a time), so that the copy of later timesteps runs beside the kernels of earlier ones;
  * the results do not depend on it.
  */
 AMQ_API amq_status amq_lstm_sequence_host(const uint32_t* Wcodes, const float* Walpha, const float* bias,
