@@ -233,42 +233,58 @@ decode_persistent_kernel(const __grid_constant__ DecodeArgs a)
             for (int j = 0; j < KA; ++j) xr[j] = has ? sH[j * CHH + sub] : make_uint4(0, 0, 0, 0);
             float mv = -INFINITY;
             int mi = 0x7fffffff;
-            auto load = [&](int r, uint4 (&v)[KS]) {
-                const uint4* src = r < res_rows ? sWs + (size_t)r * KS * CHH : a.Ws + ((size_t)r0 + r) * KS * CHH;
+            auto load = [&](int r, uint4 (&v)[KS]) {        // (two loads, not one through a pointer to either: that would be a generic load)
+                const size_t at = (size_t)r * KS * CHH + sub;
 #pragma unroll
-                for (int i = 0; i < KS; ++i) v[i] = (has && r < rows) ? src[i * CHH + sub] : make_uint4(0, 0, 0, 0);
-            };
-            uint4 cur[KS], nxt[KS];
-            int r = warp * per_warp + lane / SEG;
-            load(r, cur);
-            for (; r - lane / SEG < rows; r += DEC_WARPS * per_warp) {
-                load(r + DEC_WARPS * per_warp, nxt);
-                // counts of differing bits: at most 2048, two to a register
-                uint32_t d[(KS * KA + 1) / 2];
+                for (int i = 0; i < KS; ++i) v[i] = make_uint4(0, 0, 0, 0);
+                if (has && r < res_rows) {
 #pragma unroll
-                for (int q = 0; q < (KS * KA + 1) / 2; ++q) {
-                    d[q] = (uint32_t)dec_popc(cur[(2 * q) / KA], xr[(2 * q) % KA]);
-                    if (2 * q + 1 < KS * KA) d[q] |= (uint32_t)dec_popc(cur[(2 * q + 1) / KA % KS], xr[(2 * q + 1) % KA]) << 16;
+                    for (int i = 0; i < KS; ++i) v[i] = sWs[at + i * CHH];
+                } else if (has && r < rows) {
+#pragma unroll
+                    for (int i = 0; i < KS; ++i) v[i] = __ldg(a.Ws + (size_t)r0 * KS * CHH + at + i * CHH);
                 }
+            };
+            // Two rows per lane segment at a time, so that one's shuffles run beside the other's bit counts (284 rows of two planes per SM:
+            // 7200 clocks of a token before, 6600 now; the bit counts alone need 2300).
+            constexpr int PAIRS = (KS * KA + 1) / 2;
+            const int stride = DEC_WARPS * per_warp;
+            for (int r = warp * per_warp + lane / SEG; r - lane / SEG < rows; r += 2 * stride) {
+                uint4 v[2][KS];
+                load(r, v[0]);
+                load(r + stride, v[1]);
+                // counts of differing bits: at most 2048, two to a register
+                uint32_t d[2][PAIRS];
+#pragma unroll
+                for (int p = 0; p < 2; ++p)
+#pragma unroll
+                    for (int q = 0; q < PAIRS; ++q) {
+                        d[p][q] = (uint32_t)dec_popc(v[p][(2 * q) / KA], xr[(2 * q) % KA]);
+                        if (2 * q + 1 < KS * KA) d[p][q] |= (uint32_t)dec_popc(v[p][(2 * q + 1) / KA % KS], xr[(2 * q + 1) % KA]) << 16;
+                    }
                 for (int off = SEG >> 1; off > 0; off >>= 1) {
 #pragma unroll
-                    for (int q = 0; q < (KS * KA + 1) / 2; ++q) d[q] += __shfl_xor_sync(0xffffffffu, d[q], off);
+                    for (int p = 0; p < 2; ++p)
+#pragma unroll
+                        for (int q = 0; q < PAIRS; ++q) d[p][q] += __shfl_xor_sync(0xffffffffu, d[p][q], off);
                 }
-                if (r < rows) {
-                    float y = 0.0f;
 #pragma unroll
-                    for (int i = 0; i < KS; ++i) {
-                        const float al = sWsA[r * KS + i];
+                for (int p = 0; p < 2; ++p) {
+                    const int row = r + p * stride;
+                    if (row < rows) {
+                        float y = 0.0f;
 #pragma unroll
-                        for (int j = 0; j < KA; ++j) {
-                            const int q = i * KA + j, n = (int)((d[q >> 1] >> (16 * (q & 1))) & 0xffffu);
-                            y += al * beta[j] * (float)(H - 2 * n);
+                        for (int i = 0; i < KS; ++i) {
+                            const float al = sWsA[row * KS + i];
+#pragma unroll
+                            for (int j = 0; j < KA; ++j) {
+                                const int q = i * KA + j, n = (int)((d[p][q >> 1] >> (16 * (q & 1))) & 0xffffu);
+                                y += al * beta[j] * (float)(H - 2 * n);
+                            }
                         }
+                        dec_max(mv, mi, y + sBs[row], r0 + row);
                     }
-                    dec_max(mv, mi, y + sBs[r], r0 + r);
                 }
-#pragma unroll
-                for (int i = 0; i < KS; ++i) cur[i] = nxt[i];
             }
             dec_warp_max(mv, mi);
             if (lane == 0) { sMaxV[warp] = mv; sMaxI[warp] = mi; }
