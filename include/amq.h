@@ -374,6 +374,29 @@ AMQ_API amq_status amq_selftest_sequence_give_up(const uint32_t* Wcodes, const f
                                          void* workspace, size_t workspace_bytes, unsigned poll_limit, void* stream);
 
 /*
+ * Test aid for the batched sequences: amq_lstm_sequence (gru = 0) or amq_gru_sequence (gru = 1; c0 and c_last are not read) with batch >= 2
+ * and steps >= 1, run in the given form whatever the library would choose: AMQ_FORM_CHAIN (launches per timestep),
+ * AMQ_FORM_STREAMING (one launch, weights streamed) or AMQ_FORM_RESIDENT (one launch, weights in tensor memory).  The progress
+ * counters of the one-launch forms start as `counted` (0 .. 2^31 - 1 - steps) earlier timesteps would have left them.  Results are
+ * those of the ordinary call in that form, whatever `counted` is.  AMQ_ERR_UNSUPPORTED where the form does not take the problem.
+ */
+#define AMQ_FORM_CHAIN 0
+#define AMQ_FORM_STREAMING 1
+#define AMQ_FORM_RESIDENT 2
+/*
+ * Test aid: how a batched sequence would run on a device of `sm_count` SMs (0: the current device's; any other value needs no device).
+ * *form (HOST): one of the forms, or -1 for the one the library chooses, which is then stored there.  *ctas (HOST): CTAs that share a block
+ * of vectors; *clocks (HOST): the estimate for a timestep that the forms and their splits are chosen by (0, 0 for the chain).
+ */
+AMQ_API amq_status amq_selftest_sequence_plan(int gru, int I, int H, int k_w, int k_a, int batch, int sm_count,
+                                      int* form, int* ctas, double* clocks);
+
+AMQ_API amq_status amq_selftest_batched_sequence(const uint32_t* Wcodes, const float* Walpha, const float* bias, int I, int H, int k_w,
+                                         int gru, const float* x_seq, int steps, const float* h0, const float* c0,
+                                         int batch, int k_a, int T, float* h_seq, float* h_last, float* c_last,
+                                         void* workspace, size_t workspace_bytes, int form, int counted, void* stream);
+
+/*
  * Synchronises `stream`, then reads the status word at the start of a cell workspace: AMQ_OK, or
  * AMQ_ERR_TIMEOUT if a bounded device-side wait gave up during a call that used this workspace.
  * The word is cleared by the next cell call.

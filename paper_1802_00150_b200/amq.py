@@ -61,6 +61,10 @@ EXPORTS = {
     "amq_workspace_status": (_int, [_vp, _vp]),
     "amq_selftest_sequence_give_up": (_int, [_vp, _vp, _vp, _int, _int, _int, _vp, _int, _vp, _vp, _int, _int,
                                              _vp, _vp, _vp, _sz, ctypes.c_uint, _vp]),
+    "amq_selftest_sequence_plan": (_int, [_int, _int, _int, _int, _int, _int, _int, ctypes.POINTER(_int), ctypes.POINTER(_int),
+                                          ctypes.POINTER(ctypes.c_double)]),
+    "amq_selftest_batched_sequence": (_int, [_vp, _vp, _vp, _int, _int, _int, _int, _vp, _int, _vp, _vp, _int, _int, _int,
+                                             _vp, _vp, _vp, _vp, _sz, _int, _int, _vp]),
     "amq_gru_original_workspace_bytes": (_sz, [_int, _int, _int, _int]),
     "amq_gru_step_original": (_int, [_vp, _vp, _vp, _int, _int, _int, _vp, _vp, _int, _int, _int, _vp, _vp, _sz, _vp]),
     "amq_quantize_variant": (_int, [_vp, _int, _int, _int, _int, _int, _int, _int, _vp, _vp, _vp]),
@@ -261,6 +265,27 @@ def selftest_sequence_give_up(Wcodes, Walpha, bias, I, H, x_seq, h0, c0, k_a, T,
                                               x_seq.shape[0], h0, c0, k_a, T, h_last, c_last,
                                               workspace, workspace.numel(), poll_limit))
     return h_last, c_last
+
+
+FORM_CHAIN, FORM_STREAMING, FORM_RESIDENT = 0, 1, 2
+
+
+def selftest_sequence_plan(gru, I, H, k_w, k_a, batch, sm_count=0, form=-1):
+    """How a batched sequence would run (see amq.h): (form, CTAs of a block of vectors, estimated clocks of a timestep)."""
+    f, ctas, clocks = _int(form), _int(0), ctypes.c_double(0.0)
+    _check(_lib.amq_selftest_sequence_plan(int(gru), I, H, k_w, k_a, batch, sm_count, ctypes.byref(f), ctypes.byref(ctas), ctypes.byref(clocks)))
+    return f.value, ctas.value, clocks.value
+
+
+def selftest_batched_sequence(Wcodes, Walpha, bias, I, H, x_seq, h0, c0, k_a, T, workspace, form, counted=0):
+    """Test aid: a batched sequence (LSTM, or GRU when c0 is None) in a given form, its progress counters starting as after `counted`
+    timesteps (see amq.h).  Returns (h_seq, h_last, c_last or None)."""
+    steps, batch, k_w, gru = x_seq.shape[0], h0.shape[0], Wcodes.shape[1], c0 is None
+    h_seq = _native.empty(h0, 0, steps, batch, H)
+    h_last, c_last = torch.zeros_like(h0), None if gru else torch.zeros_like(c0)
+    _check(_native.amq_selftest_batched_sequence(Wcodes, Walpha, bias, I, H, k_w, int(gru), x_seq, steps, h0, c0, batch, k_a, T,
+                                                 h_seq, h_last, c_last, workspace, workspace.numel(), form, counted))
+    return h_seq, h_last, c_last
 
 
 def gru_sequence(Wcodes, Walpha, bias, I, H, x_seq, h0, k_a, T, workspace, want_h_seq=False,

@@ -132,10 +132,27 @@ void give_lane(CopyLane& l)
     destroy_lane(l);
 }
 
-// `chunks` (may be NULL): the stream waits for a chunk's event before the first kernel that reads it (batched calls only).
+// The counters as they stand after `counted` timesteps (self-test).
+amq_status start_counters(const BatchedSequence& s, SequenceForm form, int counted, cudaStream_t st)
+{
+    SequenceShape shape;
+    if (!(form == SEQ_RESIDENT ? resident_sequence_shape(s, 0, &shape) : streaming_sequence_shape(s, 0, &shape))) return AMQ_ERR_UNSUPPORTED;
+    for (int b = 0; b < shape.blocks; ++b) {
+        const int in_block = s.batch - b * shape.block < shape.block ? s.batch - b * shape.block : shape.block;
+        const int quantizers = form == SEQ_RESIDENT && in_block < shape.ctas ? in_block : shape.ctas;
+        const uint32_t word[2] = {(uint32_t)counted * (uint32_t)quantizers, (uint32_t)counted * (uint32_t)shape.ctas};
+        for (int q = 0; q < 2; ++q)
+            AMQ_CUDA_TRY(cudaMemcpyAsync(s.counters + (size_t)b * 64 + 32 * q, &word[q], 4, cudaMemcpyHostToDevice, st));
+    }
+    AMQ_CUDA_TRY(cudaStreamSynchronize(st));            // (the words are on this stack)
+    return AMQ_OK;
+}
+
+// `chunks` (may be NULL): the stream waits for a chunk's event before the first kernel that reads it (batched calls only).  `form` and
+// `counted` (timesteps the counters start with) are the self-test's.
 amq_status enqueue_sequence(const CellCall& c, const CellWorkspace& ws, const float* x_seq, int steps,
                             const float* h0, const float* c0, float* h_seq, float* h_last, float* c_last,
-                            cudaStream_t st, const Chunks* chunks = nullptr)
+                            cudaStream_t st, const Chunks* chunks = nullptr, SequenceForm form = SEQ_ANY, int counted = 0)
 {
     const size_t state = (size_t)c.batch * c.H, state_bytes = state * sizeof(float);
     const bool persistent = steps > 0 && use_persistent(c);
@@ -143,15 +160,21 @@ amq_status enqueue_sequence(const CellCall& c, const CellWorkspace& ws, const fl
     AMQ_CUDA_TRY(cudaMemsetAsync(ws.status, 0, 256 + ((persistent && steps > 1) ? ws.hx_bytes : 0) + ws.counter_bytes, st));
     if (persistent)
         return enqueue_persistent(c, ws, x_seq, steps, h0, c0, h_seq, h_last, c_last, st);
-    if (steps > 0 && batched_sequence_supported(batched_call(c, ws, x_seq, steps, h0, c0, h_seq, h_last, c_last))) {
+    const BatchedSequence whole = batched_call(c, ws, x_seq, steps, h0, c0, h_seq, h_last, c_last);
+    if (form == SEQ_ANY) form = batched_sequence_form(whole);
+    if (steps > 0 && form != SEQ_CHAIN) {
+        if (counted > 0) {
+            const amq_status r = start_counters(whole, form, counted, st);
+            if (r != AMQ_OK) return r;
+        }
         // one launch for all steps, or one per chunk, the state handed on in the caller's h_last / c_last
         for (int q = 0; q < (chunks ? chunks->count : 1); ++q) {
             const int s0 = chunks ? chunks->begin[q] : 0, s1 = chunks ? chunks->begin[q + 1] : steps;
             if (chunks) AMQ_CUDA_TRY(cudaStreamWaitEvent(st, chunks->ready[q], 0));
             BatchedSequence b = batched_call(c, ws, x_seq + (size_t)s0 * c.batch * c.I, s1 - s0, q ? h_last : h0, q ? c_last : c0,
                                              h_seq ? h_seq + (size_t)s0 * state : nullptr, h_last, c_last);
-            b.counted = s0;
-            const amq_status r = launch_batched_sequence(b, st);
+            b.counted = counted + s0;
+            const amq_status r = launch_batched_sequence(b, form, st);
             if (r != AMQ_OK) return r;
         }
         return AMQ_OK;
@@ -179,7 +202,8 @@ amq_status step_entry(const CellCall& c, const CellWorkspace& ws, const float* x
     if (c.batch == 1 && use_persistent(c)) return enqueue_persistent(c, ws, x, 1, h_in, c_in, nullptr, h_out, c_out, st);
     AMQ_CUDA_TRY(cudaMemsetAsync(ws.status, 0, 256 + ws.counter_bytes, st));
     const BatchedSequence b = batched_call(c, ws, x, 1, h_in, c_in, nullptr, h_out, c_out);
-    if (batched_sequence_supported(b)) return launch_batched_sequence(b, st);
+    const SequenceForm form = batched_sequence_form(b);
+    if (form != SEQ_CHAIN) return launch_batched_sequence(b, form, st);
     return enqueue_step(c, ws, x, h_in, c_in, h_out, c_out, st);
 }
 
@@ -402,6 +426,40 @@ amq_status amq_selftest_sequence_give_up(const uint32_t* Wcodes, const float* Wa
     // expected tags are offset by 2^30: the tags the CTAs publish (1 .. steps) never match
     return amq::enqueue_persistent(c, ws, x_seq, steps, h0, c0, nullptr, h_last, c_last, (cudaStream_t)stream,
                                    poll_limit, 1u << 30);
+}
+
+amq_status amq_selftest_batched_sequence(const uint32_t* Wcodes, const float* Walpha, const float* bias, int I, int H, int k_w, int gru,
+                                         const float* x_seq, int steps, const float* h0, const float* c0, int batch, int k_a, int T,
+                                         float* h_seq, float* h_last, float* c_last, void* workspace, size_t workspace_bytes,
+                                         int form, int counted, void* stream)
+{
+    amq::CellCall c{Wcodes, Walpha, bias, I, H, k_w, batch, k_a, T, gru != 0};
+    amq_status s = amq::validate(c, workspace, workspace_bytes);
+    if (s != AMQ_OK) return s;
+    if (steps < 1 || !h0 || !h_last || (!c.gru && (!c0 || !c_last)) || (I > 0 && !x_seq) || h_last == h0 || (!c.gru && c_last == c0))
+        return AMQ_ERR_INVALID_ARG;
+    if (form < AMQ_FORM_CHAIN || form > AMQ_FORM_RESIDENT || counted < 0 || counted > 0x7fffffff - steps) return AMQ_ERR_INVALID_ARG;
+    if (batch < 2) return AMQ_ERR_UNSUPPORTED;
+    amq::CellWorkspace ws = amq::carve_cell_workspace(workspace, I, H, batch, k_a);
+    return amq::enqueue_sequence(c, ws, x_seq, steps, h0, c0, h_seq, h_last, c_last, (cudaStream_t)stream, nullptr,
+                                 (amq::SequenceForm)form, counted);
+}
+
+amq_status amq_selftest_sequence_plan(int gru, int I, int H, int k_w, int k_a, int batch, int sm_count, int* form, int* ctas, double* clocks)
+{
+    if (I < 0 || H < 1 || batch < 1 || sm_count < 0 || !form || !ctas || !clocks || *form < -1 || *form > AMQ_FORM_RESIDENT)
+        return AMQ_ERR_INVALID_ARG;
+    if (!amq::valid_k(k_w) || !amq::valid_k(k_a) || I + H > AMQ_MAX_N) return AMQ_ERR_UNSUPPORTED;
+    amq::BatchedSequence s{};
+    s.I = I; s.H = H; s.n = I + H; s.k_w = k_w; s.k_a = k_a; s.T = 2; s.batch = batch; s.steps = 1; s.gru = gru != 0;
+    if (*form < 0) *form = amq::batched_sequence_form(s, sm_count);
+    amq::SequenceShape shape{};
+    if (*form != AMQ_FORM_CHAIN &&
+        !(*form == AMQ_FORM_RESIDENT ? amq::resident_sequence_shape(s, sm_count, &shape) : amq::streaming_sequence_shape(s, sm_count, &shape)))
+        return AMQ_ERR_UNSUPPORTED;
+    *ctas = shape.ctas;
+    *clocks = shape.clocks;
+    return AMQ_OK;
 }
 
 amq_status amq_workspace_status(const void* workspace, void* stream)

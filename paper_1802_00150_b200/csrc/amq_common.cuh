@@ -198,10 +198,20 @@ struct BatchedSequence {
     uint32_t* zcodes; float* zbeta; uint32_t* counters; uint32_t* status;
     int counted;                // timesteps that earlier launches have added to the counters since they were cleared
 };
-// the form with the weights in tensor memory, where they fit; AMQ_ERR_UNSUPPORTED (nothing enqueued) where they do not
+// The ways to run one: a chain of launches per timestep, or one launch with the weights streamed past the activations (amq_rnn_batched.cu)
+// or held in tensor memory (amq_rnn_resident.cu).
+enum SequenceForm { SEQ_ANY = -1, SEQ_CHAIN = 0, SEQ_STREAMING = 1, SEQ_RESIDENT = 2 };
+// How a one-launch form splits a problem over `sms` SMs (0: those of the current device): `blocks` of up to `block` vectors, `ctas` CTAs
+// each; `clocks`: the estimate for a timestep that the split was chosen by.  False where the form does not take the problem.
+struct SequenceShape { int blocks, block, ctas; double clocks; };
+bool streaming_sequence_shape(const BatchedSequence& s, int sms, SequenceShape* out);
+bool resident_sequence_shape(const BatchedSequence& s, int sms, SequenceShape* out);
+// AMQ_ERR_UNSUPPORTED: nothing has been enqueued
+amq_status launch_streaming_sequence(const BatchedSequence& s, cudaStream_t st);
 amq_status launch_resident_sequence(const BatchedSequence& s, cudaStream_t st);
-bool batched_sequence_supported(const BatchedSequence& s);
-amq_status launch_batched_sequence(const BatchedSequence& s, cudaStream_t st);
+// the form the library takes (SEQ_CHAIN where neither of the one-launch forms does), and its launch
+SequenceForm batched_sequence_form(const BatchedSequence& s, int sms = 0);
+amq_status launch_batched_sequence(const BatchedSequence& s, SequenceForm form, cudaStream_t st);
 
 // Persistent batch-1 recurrent kernel: whether it covers a problem (sizes, shared memory), and its launch.
 bool persistent_supported(int I, int H, int batch, int k_w, int k_a, bool gru, int* grid_out, int* upc_out,

@@ -122,7 +122,7 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
 
         // ---- 1. this CTA's share of the block's vectors ----
         if (t > 0) {
-            if (tid == 0) ok = seq_wait(counter + 32, (uint32_t)((a.counted + t) * a.P));
+            if (tid == 0) ok = seq_wait(counter + 32, seq_target(a.counted + t, a.P));
             if (__syncthreads_or(!ok)) { ok = false; break; }
         }
         if (warp < SEQ_QUANT_WARPS) {
@@ -134,7 +134,7 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
         __syncthreads();
         if (tid == 0) {
             seq_publish(counter);
-            ok = seq_wait(counter, (uint32_t)((a.counted + t + 1) * a.P));
+            ok = seq_wait(counter, seq_target(a.counted + t + 1, a.P));
         }
         if (__syncthreads_or(!ok)) { ok = false; break; }
 
@@ -244,7 +244,7 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"((uint32_t)RES_TMEM_COLS) : "memory");
 }
 
-struct SeqPlan { SeqParams a; int grid; size_t smem; };
+struct SeqPlan { SeqParams a; int grid; size_t smem; double clocks; };
 
 size_t seq_more_smem(const ResProblem& p)
 {
@@ -254,10 +254,10 @@ size_t seq_more_smem(const ResProblem& p)
     return sizeof(SeqShared) + (y > scratch ? y : scratch);
 }
 
-bool plan(const BatchedSequence& s, SeqPlan* out)
+bool plan(const BatchedSequence& s, int sms, SeqPlan* out)
 {
     if (s.batch < 2 || s.H < 1 || s.n > AMQ_MAX_N || (s.gru && s.I < 1)) return false;
-    const int sms = res_sm_count();
+    if (sms < 1) sms = res_sm_count();
     SeqParams a{};
     a.team_warps = s.n <= 2048 ? 8 : 16;
     ResProblem p{};
@@ -302,6 +302,7 @@ bool plan(const BatchedSequence& s, SeqPlan* out)
     out->grid = blocks * a.P;
     out->smem = (size_t)a.b_bytes + seq_more_smem(a.p);
     out->a = a;
+    out->clocks = best;
     return true;
 }
 
@@ -319,18 +320,18 @@ amq_status launch(const SeqPlan& pl, cudaStream_t st)
 
 }  // namespace
 
-bool batched_sequence_supported(const BatchedSequence& s)
+bool streaming_sequence_shape(const BatchedSequence& s, int sms, SequenceShape* out)
 {
     SeqPlan pl;
-    return plan(s, &pl);
+    if (!plan(s, sms, &pl)) return false;
+    *out = SequenceShape{pl.grid / pl.a.P, pl.a.p.TB, pl.a.P, pl.clocks};
+    return true;
 }
 
-amq_status launch_batched_sequence(const BatchedSequence& s, cudaStream_t st)
+amq_status launch_streaming_sequence(const BatchedSequence& s, cudaStream_t st)
 {
-    const amq_status r = launch_resident_sequence(s, st);
-    if (r != AMQ_ERR_UNSUPPORTED) return r;
     SeqPlan pl;
-    if (!plan(s, &pl)) return AMQ_ERR_UNSUPPORTED;
+    if (!plan(s, 0, &pl)) return AMQ_ERR_UNSUPPORTED;
     switch (s.k_a) {
         case 1: return launch<1>(pl, st);
         case 2: return launch<2>(pl, st);
@@ -338,6 +339,17 @@ amq_status launch_batched_sequence(const BatchedSequence& s, cudaStream_t st)
         case 4: return launch<4>(pl, st);
     }
     return AMQ_ERR_UNSUPPORTED;
+}
+
+SequenceForm batched_sequence_form(const BatchedSequence& s, int sms)
+{
+    SequenceShape shape;
+    return resident_sequence_shape(s, sms, &shape) ? SEQ_RESIDENT : streaming_sequence_shape(s, sms, &shape) ? SEQ_STREAMING : SEQ_CHAIN;
+}
+
+amq_status launch_batched_sequence(const BatchedSequence& s, SequenceForm form, cudaStream_t st)
+{
+    return form == SEQ_RESIDENT ? launch_resident_sequence(s, st) : form == SEQ_STREAMING ? launch_streaming_sequence(s, st) : AMQ_ERR_UNSUPPORTED;
 }
 
 }  // namespace amq

@@ -197,7 +197,7 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
         // ---- 1. this CTA's share of the block's vectors ----
         if (part < quantizers) {                    // (uniform over the CTA)
             if (t > 0) {
-                if (tid == 0) ok = seq_wait(counter + 32, (uint32_t)((a.counted + t) * a.P));
+                if (tid == 0) ok = seq_wait(counter + 32, seq_target(a.counted + t, a.P));
                 if (__syncthreads_or(!ok)) { ok = false; break; }
             }
             const float* x = a.x_seq + (size_t)t * a.batch * a.z.xn;
@@ -212,7 +212,7 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
             __syncthreads();
             if (tid == 0) seq_publish(counter);
         }
-        if (tid == 0) ok = seq_wait(counter, (uint32_t)((a.counted + t + 1) * quantizers));
+        if (tid == 0) ok = seq_wait(counter, seq_target(a.counted + t + 1, quantizers));
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         if (__syncthreads_or(!ok)) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -392,14 +392,14 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(sh.tmem_slot), "r"((uint32_t)RS_TMEM_COLS) : "memory");
 }
 
-struct RsPlan { RsParams a; int grid, warps; size_t smem; };
+struct RsPlan { RsParams a; int grid, warps; size_t smem; double clocks; };
 
 // Block of vectors x vectors per pass with the least estimated time per timestep; false when the weights do not fit tensor memory.
-bool plan(const BatchedSequence& s, RsPlan* out)
+bool plan(const BatchedSequence& s, int sms, RsPlan* out)
 {
     if (s.batch < 2 || s.H < 1 || s.n > 4096 || (s.gru && s.I < 1)) return false;
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
+    int dev = 0;
+    if (sms < 1 && (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)) return false;
     const int NS = (s.n + 255) / 256, upt = 32 / s.k_w, NW = s.n <= 1024 ? 4 : s.n <= 2048 ? 8 : 16;
     double best = 0.0;
     RsPlan p{};
@@ -434,6 +434,7 @@ bool plan(const BatchedSequence& s, RsPlan* out)
         }
     }
     if (best == 0.0) return false;
+    p.clocks = best;
     RsParams& a = p.a;
     a.W = s.Wcodes; a.Walpha = s.Walpha; a.bias = s.bias;
     a.z = SeqVectors{s.n, words_per_row(s.n), s.H, s.n - s.H, s.T, s.zcodes, s.zbeta, 16, (size_t)s.batch * s.k_a * 16};
@@ -464,10 +465,18 @@ amq_status launch_warps(const RsPlan& pl, cudaStream_t st)
 
 }  // namespace
 
+bool resident_sequence_shape(const BatchedSequence& s, int sms, SequenceShape* out)
+{
+    RsPlan pl;
+    if (!plan(s, sms, &pl)) return false;
+    *out = SequenceShape{pl.grid / pl.a.P, pl.a.block, pl.a.P, pl.clocks};
+    return true;
+}
+
 amq_status launch_resident_sequence(const BatchedSequence& s, cudaStream_t st)
 {
     RsPlan pl;
-    if (!plan(s, &pl)) return AMQ_ERR_UNSUPPORTED;
+    if (!plan(s, 0, &pl)) return AMQ_ERR_UNSUPPORTED;
     switch (s.k_a) {
         case 1: return launch_warps<1>(pl, st);
         case 2: return launch_warps<2>(pl, st);

@@ -15,12 +15,17 @@ __device__ __forceinline__ void seq_publish(uint32_t* counter)
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" :: "l"(counter) : "memory");
 }
 
+// What a counter reads once `ctas` CTAs have published `timesteps` times since it was cleared, modulo 2^32: with 148 CTAs a counter wraps
+// after 29 million timesteps (and the product leaves the range of int after half of that).
+__device__ __forceinline__ uint32_t seq_target(int timesteps, int ctas) { return (uint32_t)timesteps * (uint32_t)ctas; }
+
+// A counter is never more than a timestep's CTAs away from what is waited for, so the sign of the difference tells across a wrap.
 __device__ __forceinline__ bool seq_wait(const uint32_t* counter, uint32_t target)
 {
     for (unsigned i = 0; i < SEQ_POLL_LIMIT; ++i) {
         uint32_t v;
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(counter) : "memory");
-        if (v >= target) return true;
+        if ((int32_t)(v - target) >= 0) return true;
     }
     return false;
 }

@@ -76,3 +76,25 @@ def test_give_up_selftest_rejects_what_it_cannot_run(amq):
     with pytest.raises(amq.AmqError) as e:      # a single step waits for nothing: refused
         amq.selftest_sequence_give_up(Wcodes, Walpha, None, I, H, xs[:1], h0, h0.clone(), ka, 2, ws, 100)
     assert e.value.status == -1
+
+
+@pytest.mark.parametrize("form,cell,I,H,batch,kw,ka", [
+    (2, "lstm", 64, 48, 9, 2, 2), (2, "gru", 300, 650, 20, 3, 2),      # one block of vectors; more CTAs than quantize
+    (1, "lstm", 64, 200, 40, 2, 2), (1, "gru", 300, 650, 70, 1, 3),    # several blocks
+])
+def test_progress_counters_may_wrap(amq, form, cell, I, H, batch, kw, ka):
+    """The counters of a one-launch sequence count CTAs times timesteps: past 2^31 (the sign of an int) and across 2^32 the results stay those
+    of a run that starts at zero."""
+    steps, gru = 4, cell == "gru"
+    Wcodes, Walpha = amq.quantize(dev(synth.normal(((3 if gru else 4) * H, I + H), 0.08, 84, 1)), kw, 2)
+    xs = dev(synth.normal((steps, batch, I), 1.0, 84, 2))
+    h0, c0 = dev(synth.uniform((batch, H), -1, 1, 84, 3)), None if gru else dev(synth.uniform((batch, H), -1, 1, 84, 4))
+    ws = amq.new_workspace(I, H, batch, ka)
+    ctas = amq.selftest_sequence_plan(gru, I, H, kw, ka, batch, form=form)[1]
+    want = amq.selftest_batched_sequence(Wcodes, Walpha, None, I, H, xs, h0, c0, ka, 2, ws, form)
+    assert amq.workspace_status(ws) == 0
+    for wrap in (31, 32):
+        counted = min((1 << wrap) // ctas - 2, (1 << 31) - 1 - steps)      # reached within the four timesteps
+        got = amq.selftest_batched_sequence(Wcodes, Walpha, None, I, H, xs, h0, c0, ka, 2, ws, form, counted)
+        assert amq.workspace_status(ws) == 0
+        assert all(torch.equal(g, w) for g, w in zip(got, want) if w is not None), wrap
