@@ -385,11 +385,12 @@ AMQ_API amq_status amq_selftest_sequence_give_up(const uint32_t* Wcodes, const f
 #define AMQ_FORM_RESIDENT 2
 /*
  * Test aid: how a batched sequence would run on a device of `sm_count` SMs (0: the current device's; any other value needs no device).
- * *form (HOST): one of the forms, or -1 for the one the library chooses, which is then stored there.  *ctas (HOST): CTAs that share a block
- * of vectors; *clocks (HOST): the estimate for a timestep that the forms and their splits are chosen by (0, 0 for the chain).
+ * *form (HOST): one of the forms, or -1 for the one the library chooses, which is then stored there.  split (HOST, 3 ints): CTAs that
+ * share a block of vectors, vectors of a block, warps that quantize a vector (zeros for the chain); *clocks (HOST): the estimate for a
+ * timestep that the split was chosen by.
  */
 AMQ_API amq_status amq_selftest_sequence_plan(int gru, int I, int H, int k_w, int k_a, int batch, int sm_count,
-                                      int* form, int* ctas, double* clocks);
+                                      int* form, int* split, double* clocks);
 
 AMQ_API amq_status amq_selftest_batched_sequence(const uint32_t* Wcodes, const float* Walpha, const float* bias, int I, int H, int k_w,
                                          int gru, const float* x_seq, int steps, const float* h0, const float* c0,

@@ -271,10 +271,11 @@ FORM_CHAIN, FORM_STREAMING, FORM_RESIDENT = 0, 1, 2
 
 
 def selftest_sequence_plan(gru, I, H, k_w, k_a, batch, sm_count=0, form=-1):
-    """How a batched sequence would run (see amq.h): (form, CTAs of a block of vectors, estimated clocks of a timestep)."""
-    f, ctas, clocks = _int(form), _int(0), ctypes.c_double(0.0)
-    _check(_lib.amq_selftest_sequence_plan(int(gru), I, H, k_w, k_a, batch, sm_count, ctypes.byref(f), ctypes.byref(ctas), ctypes.byref(clocks)))
-    return f.value, ctas.value, clocks.value
+    """How a batched sequence would run (see amq.h): (form, (CTAs and vectors of a block, warps per quantized vector), estimated clocks of a
+    timestep)."""
+    f, split, clocks = _int(form), (_int * 3)(), ctypes.c_double(0.0)
+    _check(_lib.amq_selftest_sequence_plan(int(gru), I, H, k_w, k_a, batch, sm_count, ctypes.byref(f), split, ctypes.byref(clocks)))
+    return f.value, tuple(split), clocks.value
 
 
 def selftest_batched_sequence(Wcodes, Walpha, bias, I, H, x_seq, h0, c0, k_a, T, workspace, form, counted=0):

@@ -445,9 +445,9 @@ amq_status amq_selftest_batched_sequence(const uint32_t* Wcodes, const float* Wa
                                  (amq::SequenceForm)form, counted);
 }
 
-amq_status amq_selftest_sequence_plan(int gru, int I, int H, int k_w, int k_a, int batch, int sm_count, int* form, int* ctas, double* clocks)
+amq_status amq_selftest_sequence_plan(int gru, int I, int H, int k_w, int k_a, int batch, int sm_count, int* form, int* split, double* clocks)
 {
-    if (I < 0 || H < 1 || batch < 1 || sm_count < 0 || !form || !ctas || !clocks || *form < -1 || *form > AMQ_FORM_RESIDENT)
+    if (I < 0 || H < 1 || batch < 1 || sm_count < 0 || !form || !split || !clocks || *form < -1 || *form > AMQ_FORM_RESIDENT)
         return AMQ_ERR_INVALID_ARG;
     if (!amq::valid_k(k_w) || !amq::valid_k(k_a) || I + H > AMQ_MAX_N) return AMQ_ERR_UNSUPPORTED;
     amq::BatchedSequence s{};
@@ -457,7 +457,7 @@ amq_status amq_selftest_sequence_plan(int gru, int I, int H, int k_w, int k_a, i
     if (*form != AMQ_FORM_CHAIN &&
         !(*form == AMQ_FORM_RESIDENT ? amq::resident_sequence_shape(s, sm_count, &shape) : amq::streaming_sequence_shape(s, sm_count, &shape)))
         return AMQ_ERR_UNSUPPORTED;
-    *ctas = shape.ctas;
+    split[0] = shape.ctas; split[1] = shape.block; split[2] = shape.warps;
     *clocks = shape.clocks;
     return AMQ_OK;
 }

@@ -202,8 +202,8 @@ struct BatchedSequence {
 // or held in tensor memory (amq_rnn_resident.cu).
 enum SequenceForm { SEQ_ANY = -1, SEQ_CHAIN = 0, SEQ_STREAMING = 1, SEQ_RESIDENT = 2 };
 // How a one-launch form splits a problem over `sms` SMs (0: those of the current device): `blocks` of up to `block` vectors, `ctas` CTAs
-// each; `clocks`: the estimate for a timestep that the split was chosen by.  False where the form does not take the problem.
-struct SequenceShape { int blocks, block, ctas; double clocks; };
+// each, `warps` to quantize a vector; `clocks`: the estimate for a timestep that the split was chosen by.  False where the form does not take the problem.
+struct SequenceShape { int blocks, block, ctas, warps; double clocks; };
 bool streaming_sequence_shape(const BatchedSequence& s, int sms, SequenceShape* out);
 bool resident_sequence_shape(const BatchedSequence& s, int sms, SequenceShape* out);
 // AMQ_ERR_UNSUPPORTED: nothing has been enqueued

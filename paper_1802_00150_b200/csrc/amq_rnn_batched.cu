@@ -290,9 +290,10 @@ bool plan(const BatchedSequence& s, int sms, SeqPlan* out)
         }
     if (best == 0.0) return false;
     const int blocks = (s.batch + a.p.TB - 1) / a.p.TB;
-    // several vectors per CTA: two teams take one each, sixteen elements a thread; their chains of reductions overlap
-    // (GRU 2048, 256 sequences, 35 steps: 1551 us with one team of sixteen warps, 1457 us)
-    if (s.n <= 4096 && a.p.TB > a.P) a.team_warps = 8;
+    // Several vectors per CTA: two teams take one each, sixteen elements a thread; their chains of reductions overlap (35 steps of GRU 2048, 256
+    // sequences, 3-bit activations: 1561 us with one team of sixteen warps, 1496 us; 4 to 27 % less over 24 problems with 1 to 3
+    // bits).  Not at four bits, where sixteen elements do not fit the registers (LSTM 2000/2000, 200 sequences: 2153 us against 2660).
+    if (s.n <= 4096 && a.p.TB > a.P && s.k_a <= 3) a.team_warps = 8;
     a.b_bytes = a.p.NS * a.p.N * 128;
     a.bias = s.bias; a.H = s.H; a.steps = s.steps; a.k_a = s.k_a;
     a.z = SeqVectors{s.n, a.p.wpr, s.H, s.n - s.H, s.T, s.zcodes, s.zbeta, (size_t)a.p.wpr * 4, 16};
@@ -324,7 +325,7 @@ bool streaming_sequence_shape(const BatchedSequence& s, int sms, SequenceShape* 
 {
     SeqPlan pl;
     if (!plan(s, sms, &pl)) return false;
-    *out = SequenceShape{pl.grid / pl.a.P, pl.a.p.TB, pl.a.P, pl.clocks};
+    *out = SequenceShape{pl.grid / pl.a.P, pl.a.p.TB, pl.a.P, pl.a.team_warps, pl.clocks};
     return true;
 }
 

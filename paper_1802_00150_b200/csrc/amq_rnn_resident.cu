@@ -469,7 +469,7 @@ bool resident_sequence_shape(const BatchedSequence& s, int sms, SequenceShape* o
 {
     RsPlan pl;
     if (!plan(s, sms, &pl)) return false;
-    *out = SequenceShape{pl.grid / pl.a.P, pl.a.block, pl.a.P, pl.clocks};
+    *out = SequenceShape{pl.grid / pl.a.P, pl.a.block, pl.a.P, pl.warps, pl.clocks};
     return true;
 }
 

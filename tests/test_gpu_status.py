@@ -90,7 +90,7 @@ def test_progress_counters_may_wrap(amq, form, cell, I, H, batch, kw, ka):
     xs = dev(synth.normal((steps, batch, I), 1.0, 84, 2))
     h0, c0 = dev(synth.uniform((batch, H), -1, 1, 84, 3)), None if gru else dev(synth.uniform((batch, H), -1, 1, 84, 4))
     ws = amq.new_workspace(I, H, batch, ka)
-    ctas = amq.selftest_sequence_plan(gru, I, H, kw, ka, batch, form=form)[1]
+    ctas = amq.selftest_sequence_plan(gru, I, H, kw, ka, batch, form=form)[1][0]
     want = amq.selftest_batched_sequence(Wcodes, Walpha, None, I, H, xs, h0, c0, ka, 2, ws, form)
     assert amq.workspace_status(ws) == 0
     for wrap in (31, 32):
