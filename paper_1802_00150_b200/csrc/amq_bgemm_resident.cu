@@ -3,7 +3,7 @@
 // equal contiguous shares, so that a CTA expands the activation operand once or twice and streams weight tiles past it.
 //
 // What bounds it: the pace of the pipeline steps (240-265 clocks per 256 bit positions of 128 plane-rows) times the number of
-// blocks the batch is cut into; outputs leave as 128-byte stores of consecutive rows from registers.
+// blocks the batch is cut into; outputs leave through shared memory as 128-byte stores of consecutive rows.
 #include "amq_resident.cuh"
 
 namespace amq {
@@ -221,7 +221,7 @@ bool plan(const GemmArgs& g, ResGemmPlan* out)
     ResProblem& p = a.p;
     p.W = g.Wcodes; p.Walpha = g.Walpha; p.k_w = g.k_w; p.wpr = words_per_row(g.n);
     p.vec32 = p.wpr % 8 == 0 && (reinterpret_cast<uintptr_t>(g.Wcodes) & 31) == 0;
-    p.cell = RES_PLAIN; p.units = g.m; p.ut = 128; p.tpu = 1;
+    p.cell = RES_PLAIN; p.units = g.m;
     p.n = g.n; p.NS = (g.n + 255) / 256; p.batch = g.batch;
     a.mtiles = (g.m + 127) / 128;
     // block of vectors: the size with the least estimated time (shares of tiles x steps, plus the expansion of the operand,
@@ -241,7 +241,7 @@ bool plan(const GemmArgs& g, ResGemmPlan* out)
     a.xcodes = g.xcodes; a.xbeta = g.xbeta; a.bias = g.bias; a.y = g.y; a.ldy = g.ldy;
     const long long total = (long long)a.blocks * a.mtiles;
     out->grid = (int)(total < sms ? total : sms);
-    out->smem = res_smem_bytes(a.p, g.k_a) + (size_t)a.p.TB * Y_LD * 4;
+    out->smem = res_smem_bytes(a.p) + (size_t)a.p.TB * Y_LD * 4;
     a.vec_out = (reinterpret_cast<uintptr_t>(g.y) & 15) == 0 && g.ldy % 4 == 0;
     out->a = a;
     return true;

@@ -59,10 +59,7 @@ struct ResProblem {
     const uint32_t* W; const float* Walpha; int k_w, wpr;
     int vec32;          // every plane-row is whole 32-byte pieces (256-bit loads)
     int cell;           // ResCell
-    int units;          // rows of a plain product, hidden units of a cell
-    int ut;             // units per block: 128 (lane = unit; a cell's gates are four tiles one after the other), or 32 (a
-                        // cell only: lane quarter = gate)
-    int tpu;            // tiles per block of units: 1, or 4
+    int units;          // rows of a plain product (a tile is 128 of them), hidden units of a cell (a tile is 32: lane quarter = gate)
     int n, I;           // vector length; first column of the h part (GRU)
     int NS, nx, xw;     // slots; slots of the x part (0: no split); whole x slots before the doubled one
     int TB, N, ring;    // activation vectors per CTA, operand rows (TB * k_a rounded up to 16), accumulator buffers
@@ -70,34 +67,15 @@ struct ResProblem {
     int batch;
 };
 
-// gate order of the four tiles of a 128-unit block, chosen so that an epilogue thread keeps one value per (unit, vector) alive:
-// LSTM i, g, f, o; GRU r, nh, nx, z
-__device__ __forceinline__ int res_gate_of_tile(int cell, int tt)
-{
-    return cell == RES_LSTM ? (tt == 0 ? 0 : tt == 1 ? 3 : tt == 2 ? 1 : 2) : (tt == 0 ? 0 : tt == 3 ? 1 : 2);
-}
-
-__device__ __forceinline__ void res_tile_slots(const ResProblem& p, int tt, int& s0, int& s1)
-{
-    s0 = 0; s1 = p.NS;
-    if (p.cell == RES_GRU && p.tpu == 4) {
-        if (tt == 1) s0 = p.nx;
-        if (tt == 2) s1 = p.nx;
-    }
-}
-
 __device__ __forceinline__ int res_slot_word(const ResProblem& p, int s) { return 8 * (s < p.nx ? s : p.xw + s - p.nx); }
 
-// weight row of lane r of tile tt of unit block ub; -1: none
-__device__ __forceinline__ int res_row(const ResProblem& p, int ub, int tt, int r)
+// weight row of lane r of tile `tile`; -1: none.  The lane quarters of a GRU's tile are r, z and the candidate's x and h parts.
+template <int CELL>
+__device__ __forceinline__ int res_row(const ResProblem& p, int tile, int r)
 {
-    if (p.ut == 32) {
-        const int u = ub * 32 + (r & 31), q = r >> 5;
-        return u < p.units ? ((p.cell == RES_GRU && q == 3) ? 2 : q) * p.units + u : -1;
-    }
-    const int u = ub * 128 + r;
-    if (u >= p.units) return -1;
-    return p.cell == RES_PLAIN ? u : res_gate_of_tile(p.cell, tt) * p.units + u;
+    if (CELL == RES_PLAIN) { const int u = tile * 128 + r; return u < p.units ? u : -1; }
+    const int u = tile * 32 + (r & 31), q = r >> 5;
+    return u < p.units ? ((p.cell == RES_GRU && q == 3) ? 2 : q) * p.units + u : -1;
 }
 
 // Synchronisation block in shared memory.
@@ -232,16 +210,8 @@ __device__ __forceinline__ void res_row_constants(const ResProblem& p, int* sSum
 
 // The steps of a tile (two consecutive slots of one plane each) as a table in shared memory, two words per step: word offset in
 // the row's planes, bit 29: no such slot, bit 30: the slot has only 16 bytes of the row, bit 31: it belongs to the h part of a split.
-constexpr int RES_KIND = AMQ_MAX_K * 34;            // entries of one kind of tile: AMQ_MAX_N / 256 + 1 slots, in pairs
-constexpr int RES_TABLE = 4 * RES_KIND;             // up to four kinds (a GRU block of 128 units)
+constexpr int RES_TABLE = AMQ_MAX_K * 34;           // AMQ_MAX_N / 256 + 1 slots, in pairs
 constexpr uint32_t RES_STEP_NONE = 1u << 29, RES_STEP_HALF = 1u << 30, RES_STEP_H = 1u << 31;
-
-__device__ __forceinline__ int res_tile_steps(const ResProblem& p, int tt)
-{
-    int s0, s1;
-    res_tile_slots(p, tt, s0, s1);
-    return p.k_w * ((s1 - s0 + 1) >> 1);
-}
 
 // One group's share of the CTA's steps: the steps of all tiles in order are dealt to the groups in turn.  Thread = plane-row.  The
 // packed words of a step are fetched one of the group's steps ahead.  (Every instruction counts here: the expander warps
@@ -250,25 +220,22 @@ template <typename R, int CELL>
 struct ResFeeder {
     const uint32_t* row;            // plane 0 of this thread's row in the cursor's tile (a lane without a weight row takes the last one:
                                     // its accumulators are read by nobody)
-    int i, n;                       // the cursor's step in its tile, steps of the tile
+    int i, n;                       // the cursor's step in its tile, steps of a tile
     int it, nitems;                 // tile counter of the CTA
-    int base;                       // the tile kind's part of the table
-    int ub0, ub_step;
+    int tile0, tile_step;
     uint4 v[2][2];                  // the next step's packed words, and its table entries
     uint2 e;
     bool live;                      // there is a next step
 
     __device__ __forceinline__ void tile(const ResProblem& p, int r)
     {
-        const int ub = ub0 + (CELL != RES_PLAIN && p.tpu == 4 ? it >> 2 : it) * ub_step, tt = CELL != RES_PLAIN && p.tpu == 4 ? it & 3 : 0;
-        const int wr = CELL == RES_PLAIN ? ub * 128 + r : res_row(p, ub, tt, r);
-        row = p.W + (size_t)(wr < 0 || (CELL == RES_PLAIN && wr >= p.units) ? p.units - 1 : wr) * (p.k_w * p.wpr);
-        if (CELL != RES_PLAIN && p.tpu == 4) { n = res_tile_steps(p, tt); base = tt * RES_KIND; }
+        const int wr = res_row<CELL>(p, tile0 + it * tile_step, r);
+        row = p.W + (size_t)(wr < 0 ? p.units - 1 : wr) * (p.k_w * p.wpr);
     }
-    // position on the first own step of a pass over tiles ub0, ub0 + ub_step, ..; `skip` steps of other groups come first
-    __device__ __forceinline__ void start(const ResProblem& p, const uint32_t* table, int first_block, int block_step, int tiles, int r, int skip)
+    // position on the first own step of a pass over `tiles` tiles first, first + step, ..; `skip` steps of other groups come first
+    __device__ __forceinline__ void start(const ResProblem& p, const uint32_t* table, int first, int step, int tiles, int r, int skip)
     {
-        it = 0; nitems = tiles; ub0 = first_block; ub_step = block_step; base = 0;
+        it = 0; nitems = tiles; tile0 = first; tile_step = step;
         n = p.k_w * ((p.NS + 1) >> 1); i = skip;
         if (nitems > 0) tile(p, r);
         next_tile(p, r);
@@ -282,17 +249,17 @@ struct ResFeeder {
             if (++it < nitems) tile(p, r);
         }
     }
-    // whether this lane's row is zero in the slot of table entry `entry` (candidate rows of a 32-unit GRU block)
+    // whether this lane's row is zero in the slot of table entry `entry` (a GRU's candidate rows)
     __device__ __forceinline__ static bool zero_row(const ResProblem& p, uint32_t entry, int r)
     {
-        return CELL != RES_PLAIN && p.cell == RES_GRU && p.ut == 32 && (r >> 5) == ((entry & RES_STEP_H) ? 2 : 3);
+        return CELL != RES_PLAIN && p.cell == RES_GRU && (r >> 5) == ((entry & RES_STEP_H) ? 2 : 3);
     }
     // packed words of the cursor's step, and on to the group's next step
     __device__ __forceinline__ void fetch(const ResProblem& p, const uint32_t* table, int r)
     {
         live = it < nitems;
         if (!live) return;
-        e = *reinterpret_cast<const uint2*>(table + base + 2 * i);
+        e = *reinterpret_cast<const uint2*>(table + 2 * i);
         const uint4* src0 = reinterpret_cast<const uint4*>(row + (e.x & (RES_STEP_NONE - 1)));
         const uint4* src1 = reinterpret_cast<const uint4*>(row + (e.y & (RES_STEP_NONE - 1)));
         if (p.vec32) {
@@ -316,18 +283,12 @@ struct ResFeeder {
 // fill the table (all threads; a CTA barrier follows)
 __device__ __forceinline__ void res_fill_table(const ResProblem& p, uint32_t* table)
 {
-    const int kinds = p.cell == RES_GRU && p.tpu == 4 ? 4 : 1;
+    const int per_plane = (p.NS + 1) & ~1;
 #pragma unroll 1
-    for (int tt = 0; tt < kinds; ++tt) {
-        int s0, s1;
-        res_tile_slots(p, tt, s0, s1);
-        const int per_plane = (s1 - s0 + 1) & ~1;
-#pragma unroll 1
-        for (int q = threadIdx.x; q < p.k_w * per_plane; q += blockDim.x) {
-            const int plane = q / per_plane, s = s0 + q - plane * per_plane, w0 = res_slot_word(p, s);
-            table[tt * RES_KIND + q] = s >= s1 ? RES_STEP_NONE | RES_STEP_HALF          // (offset 0: loads what is there, used by nobody)
-                : (uint32_t)(plane * p.wpr + w0) | (w0 + 8 > p.wpr ? RES_STEP_HALF : 0u) | (p.nx > 0 && s >= p.nx ? RES_STEP_H : 0u);
-        }
+    for (int q = threadIdx.x; q < p.k_w * per_plane; q += blockDim.x) {
+        const int plane = q / per_plane, s = q - plane * per_plane, w0 = res_slot_word(p, s);
+        table[q] = s >= p.NS ? RES_STEP_NONE | RES_STEP_HALF          // (offset 0: loads what is there, used by nobody)
+            : (uint32_t)(plane * p.wpr + w0) | (w0 + 8 > p.wpr ? RES_STEP_HALF : 0u) | (p.nx > 0 && s >= p.nx ? RES_STEP_H : 0u);
     }
 }
 
@@ -421,23 +382,21 @@ __device__ __forceinline__ bool res_issue(const ResProblem& p, ResSync& sy, int 
     bool ready = false;
 #pragma unroll 1
     for (int it = 0; it < nitems; ++it) {
-        int s0, s1;
-        res_tile_slots(p, p.tpu == 4 ? it & 3 : 0, s0, s1);
 #pragma unroll 1
         for (int plane = 0; plane < p.k_w; ++plane) {
             if (!mbar_wait(smem_u32(&sy.tempty[st.ring]), st.ring_parity)) { *(volatile int*)&sy.failed = 1; return false; }
             const uint32_t acc = tmem + (uint32_t)(st.ring * p.N);
-            uint32_t b = lo + (uint32_t)s0 * slot_units;
+            uint32_t b = lo;
 #pragma unroll 1
-            for (int s = s0; s < s1; s += 2) {
+            for (int s = 0; s < p.NS; s += 2) {
                 if (!ready && !mbar_wait(full0 + 8 * st.stage, st.full_parity)) { *(volatile int*)&sy.failed = 1; return false; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t a = a0 + (uint32_t)(st.stage * RES_STAGE_COLS), empty = empty0 + 8 * st.stage;
-                if (issues) mma_mxf4_slot(acc, a, b, hi, idesc, s != s0 ? 1u : 0u, sfa, sf);
+                if (issues) mma_mxf4_slot(acc, a, b, hi, idesc, s != 0 ? 1u : 0u, sfa, sf);
                 if (++st.stage == p.stages) { st.stage = 0; st.full_parity ^= 1u; }
                 ready = mbar_test(full0 + 8 * st.stage, st.full_parity);
                 if (issues) {
-                    if (s + 1 < s1) mma_mxf4_slot(acc, a + 32, b + slot_units, hi, idesc, 1u, sfa, sf);
+                    if (s + 1 < p.NS) mma_mxf4_slot(acc, a + 32, b + slot_units, hi, idesc, 1u, sfa, sf);
                     mma_commit(empty);
                 }
                 b += 2 * slot_units;
@@ -520,9 +479,8 @@ inline int res_sm_count()
 }
 
 // shared memory: operand, coefficients, synchronisation block, and what the caller adds behind them
-inline size_t res_smem_bytes(const ResProblem& p, int k_a)
+inline size_t res_smem_bytes(const ResProblem& p)
 {
-    (void)k_a;
     return (size_t)p.NS * p.N * 128 + RES_ROW_BYTES + RES_ALPHA_BYTES + RES_TABLE * 4 + sizeof(ResSync);
 }
 
@@ -537,7 +495,7 @@ inline bool res_set_block(ResProblem& p, int TB, int k_a, size_t more_smem = 0)
     p.ring = (RES_TMEM_COLS - 16 - 2 * p.N) / RES_STAGE_COLS >= R::GROUPS ? 2 : 1;
     const int stages = (RES_TMEM_COLS - 16 - p.ring * p.N) / RES_STAGE_COLS;
     p.stages = stages < RES_MAX_STAGES ? stages : RES_MAX_STAGES;
-    return res_smem_bytes(p, k_a) + more_smem <= (size_t)RES_SMEM_LIMIT;
+    return res_smem_bytes(p) + more_smem <= (size_t)RES_SMEM_LIMIT;
 }
 
 // estimated clocks per slot of 128 plane-rows (measured: 240 up to N = 96, 265 at N = 128, then the tensor pipe's own pace); with

@@ -81,10 +81,14 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     const ResProblem& p = a.p;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, H = a.H;
+    // The warp's number in a uniform register leaves one more to the quantizer, which spills otherwise (35 steps of LSTM 1728/1024, 48 sequences,
+    // 3-bit weights and activations: 641 us, 602 us so).  At four bits, and at two with sixteen elements a thread, it is that which
+    // makes the compiler spill (up to 7 % slower).
+    constexpr bool UNIFORM = KA != 4 && !(KA == 2 && EPT == 16);
+    const int tid = threadIdx.x, warp = UNIFORM ? __shfl_sync(0xffffffffu, tid >> 5, 0) : tid >> 5, lane = tid & 31, H = a.H;
     const int bb = (int)blockIdx.x / a.P, part = (int)blockIdx.x - bb * a.P, b0 = bb * p.TB;
     const int in_block = p.batch - b0 < p.TB ? p.batch - b0 : p.TB;         // vectors of this block
-    const int my_blocks = (a.unit_blocks - part + a.P - 1) / a.P, tiles = my_blocks * p.tpu;
+    const int tiles = (a.unit_blocks - part + a.P - 1) / a.P;              // blocks of 32 units
     SeqShared& sh = *reinterpret_cast<SeqShared*>(smem_raw + a.b_bytes);
     float* sY = reinterpret_cast<float*>(&sh + 1);                          // [TB][SEQ_Y_LD] pre-activations of a tile
     QuantScratch<KA, SEQ_QUANT_WARPS>* scratch = reinterpret_cast<QuantScratch<KA, SEQ_QUANT_WARPS>*>(&sh + 1);    // (they are dead then)
@@ -106,12 +110,10 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
     const uint32_t tmem = __shfl_sync(0xffffffffu, sh.sync.tmem_slot, 0);
     if (warp < 4) res_write_scales(p, tmem, warp);
 
-    int first_step = 0;                             // pipeline steps so far, mod the number of groups
-    ResFeedState feed_state{warp >> 2, 1u};
-    ResIssueState issue{0, 0, 0, 1};
-    ResDrainState drain{0, 0};
-    const int team = warp / a.team_warps, teams = SEQ_QUANT_WARPS / a.team_warps;
-    const QuantTeam quant{warp - team * a.team_warps, 8 + team, a.team_warps * 32};
+    ResIssueState issue{0, 0, 0, 1};                // (apart and from constants: it stays in uniform registers)
+    // stage of an expander or accumulator of an epilogue warp, and its parity: the same two registers, the quantizer needs the others
+    int at = warp < R::EXP_WARPS ? warp >> 2 : 0;
+    uint32_t at_parity = warp < R::EXP_WARPS ? 1u : 0u;
     int quant_parity = 0;
     bool ok = true;
 
@@ -127,6 +129,8 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
         }
         if (warp < SEQ_QUANT_WARPS) {
             const float* x = a.x_seq + (size_t)t * p.batch * a.z.xn;
+            const int teams = a.team_warps == 8 ? 2 : 1, team = teams == 2 ? warp >> 3 : 0;
+            const QuantTeam quant{warp - 8 * team, 8 + team, a.team_warps * 32};
 #pragma unroll 1
             for (int v = part + team * a.P; v < in_block; v += teams * a.P)
                 seq_quantize<KA, EPT, SEQ_QUANT_WARPS>(a.z, x, h_prev, b0 + v, scratch[team], quant, quant_parity);
@@ -151,8 +155,12 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
         // ---- 3. product, gates ----
         if (warp < R::EXP_WARPS) {
             ResFeeder<R, RES_GRU> feed;
-            feed.start(p, sh.table, part, a.P, tiles, tid & 127, ((warp >> 2) - first_step) & (R::GROUPS - 1));
-            ok = res_feed(p, sh.sync, sh.table, feed, tmem, feed_state);
+            // (steps of earlier timesteps: the groups take turns without a break)
+            const uint32_t skip = (uint32_t)(warp >> 2) - (uint32_t)t * (uint32_t)(tiles * a.unit_steps);
+            feed.start(p, sh.table, part, a.P, tiles, tid & 127, (int)(skip & (R::GROUPS - 1)));
+            ResFeedState state{at, at_parity};
+            ok = res_feed(p, sh.sync, sh.table, feed, tmem, state);
+            at = state.stage; at_parity = state.parity;
         } else if (warp == R::MMA_WARP) {
             ok = res_issue(p, sh.sync, tiles, tmem, sB, issue);
         } else if (warp < R::MMA_WARP) {
@@ -161,14 +169,14 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
             float* h_also = last && a.h_seq ? a.h_seq + (size_t)t * p.batch * H : nullptr;
             const float* c_prev = t == 0 ? a.c0 : a.c;
             float* c_next = last ? a.c_last : a.c;
+            ResDrainState drain{at, at_parity};
             res_row_constants<R>(p, sh.sum[0], sh.row[0]);
-            float keep[16];                         // 128-unit blocks: one value per (unit, vector) of this thread, from gate to gate
 #pragma unroll 1
             for (int it = 0; it < tiles && ok; ++it) {
-                const int tt = p.tpu == 4 ? it & 3 : 0, ub = part + (p.tpu == 4 ? it >> 2 : it) * a.P;
+                const int ub = part + it * a.P;
                 float* sa = sh.alpha[it & 1];
                 {
-                    const int wr = res_row(p, ub, tt, te & 127);
+                    const int wr = res_row<RES_GRU>(p, ub, te & 127);
 #pragma unroll
                     for (int q = 0; q < 2; ++q) {
                         const int plane = (te >> 7) + 2 * q;
@@ -176,7 +184,7 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
                     }
                 }
                 res_epi_bar<R>(false);              // (also: everybody is past the tile before last, whose buffer this is)
-                const int kind = p.cell != RES_GRU ? 0 : p.tpu == 4 ? (tt == 1 ? 2 : tt == 2 ? 1 : 0) : quarter >= 2 ? quarter - 1 : 0;
+                const int kind = p.cell == RES_GRU && quarter >= 2 ? quarter - 1 : 0;
                 f32x2 y[SEQ_NG][4];
                 ok = res_drain_tile<R, KA, SEQ_NG>(p, sh.sync, sa, quarter, sub, tmem, sh.beta, sh.row[kind], drain, y);
 #pragma unroll
@@ -191,43 +199,23 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
                         sY[(e + 1) * SEQ_Y_LD + rl + 8 * i] = y1;
                     }
                 }
-                if (p.tpu == 1) {                   // lane quarter = gate: lane = unit, one vector per warp
-                    const int u = ub * 32 + lane;
-                    float bias[4];
+                // lane quarter = gate: lane = unit, one vector per warp
+                const int u = ub * 32 + lane;
+                float bias[4];
 #pragma unroll
-                    for (int g = 0; g < 4; ++g) bias[g] = (a.bias && u < H) ? __ldg(a.bias + g * H + u) : 0.0f;
-                    res_epi_bar<R>(false);
-                    const float* addend = a.addend ? a.addend + ((size_t)t * p.batch + b0) * 4 * H + u : nullptr;
-                    if (u < H) {
+                for (int g = 0; g < 4; ++g) bias[g] = (a.bias && u < H) ? __ldg(a.bias + g * H + u) : 0.0f;
+                res_epi_bar<R>(false);
+                const float* addend = a.addend ? a.addend + ((size_t)t * p.batch + b0) * 4 * H + u : nullptr;
+                if (u < H) {
 #pragma unroll 1
-                        for (int e = te >> 5; e < in_block; e += R::EPI_WARPS)
-                            seq_cell(a, sY + e * SEQ_Y_LD + lane, bias, addend ? addend + (size_t)e * 4 * H : nullptr, (size_t)(b0 + e) * H + u,
-                                     h_prev, c_prev, h_next, h_also, c_next);
-                    }
-                } else {                            // the gates r, n (h part), n (x part), z of 128 units one after the other
-                    const int u = ub * 128 + (te & 127), bias_row = (tt == 0 ? 0 : tt == 1 ? 3 : tt == 2 ? 2 : 1) * H;
-                    const float bias = (a.bias && u < H) ? __ldg(a.bias + bias_row + u) : 0.0f;
-                    res_epi_bar<R>(false);
-#pragma unroll 1
-                    for (int e = te >> 7; e < in_block; e += 2) {
-                        const float s = sY[e * SEQ_Y_LD + (te & 127)] + bias;
-                        float k = keep[e >> 1];
-                        if (tt == 0) k = seq_logistic(s);
-                        else if (tt == 1) k *= s;
-                        else if (tt == 2) k = tanhf(s + k);
-                        else if (u < H) {
-                            const size_t o = (size_t)(b0 + e) * H + u;
-                            const float zg = seq_logistic(s), h = (1.0f - zg) * k + zg * __ldcg(h_prev + o);
-                            h_next[o] = h;
-                            if (h_also) h_also[o] = h;
-                        }
-                        keep[e >> 1] = k;
-                    }
+                    for (int e = te >> 5; e < in_block; e += R::EPI_WARPS)
+                        seq_cell(a, sY + e * SEQ_Y_LD + lane, bias, addend ? addend + (size_t)e * 4 * H : nullptr, (size_t)(b0 + e) * H + u,
+                                 h_prev, c_prev, h_next, h_also, c_next);
                 }
                 __syncwarp();                       // (the next tile's values are staged behind the barrier inside its drain)
             }
+            at = drain.ring; at_parity = drain.parity;
         }
-        first_step = (first_step + my_blocks * a.unit_steps) & (R::GROUPS - 1);
         if (__syncthreads_or(!ok)) { ok = false; break; }
         if (tid == 0) seq_publish(counter + 32);
     }
@@ -270,24 +258,22 @@ bool plan(const BatchedSequence& s, int sms, SeqPlan* out)
     } else {
         p.NS = (s.n + 255) / 256;
     }
-    // Block of vectors x block of units with the least estimated time per timestep.  128-unit blocks (GRU only) save the quarter of
-    // the weight steps that 32-unit blocks spend on the zero halves of the candidate rows, 32-unit blocks divide more finely.
+    // block of vectors with the least estimated time per timestep
     double best = 0.0;
-    for (int wide = 0; wide <= (s.gru ? 1 : 0); ++wide)
-        for (int TB = 8; TB <= 8 * SEQ_NG * R::SPLIT; TB += 8) {
-            ResProblem q = p;
-            q.ut = wide ? 128 : 32; q.tpu = wide ? 4 : 1; q.TB = TB;
-            if (!res_set_block<R>(q, TB, s.k_a, seq_more_smem(q))) break;
-            const int blocks = (s.batch + TB - 1) / TB, ub = (s.H + q.ut - 1) / q.ut;
-            if (blocks > sms) continue;
-            const int P = ub < sms / blocks ? ub : sms / blocks, per_cta = (ub + P - 1) / P;
-            const int steps = q.k_w * (wide ? 2 * ((q.NS + 1) / 2) + (q.nx + 1) / 2 + (q.NS - q.nx + 1) / 2 : (q.NS + 1) / 2);
-            const int vectors = (TB + P - 1) / P, teams = SEQ_QUANT_WARPS / a.team_warps;
-            const double t = per_cta * (steps * 2 * res_slot_clocks(q) + 1500.0 * q.tpu) + (double)q.N * q.NS * 128 / 60.0 +
-                             (vectors + teams - 1) / teams * (s.k_a >= 3 ? 4500.0 : 3500.0);
-            if (best == 0.0 || t < best) { best = t; a.p = q; a.P = P; a.unit_blocks = ub; a.unit_steps = steps; }
-            if (TB >= s.batch) break;
-        }
+    const int ub = (s.H + 31) / 32, steps = p.k_w * ((p.NS + 1) / 2);
+    for (int TB = 8; TB <= 8 * SEQ_NG * R::SPLIT; TB += 8) {
+        ResProblem q = p;
+        q.TB = TB;
+        if (!res_set_block<R>(q, TB, s.k_a, seq_more_smem(q))) break;
+        const int blocks = (s.batch + TB - 1) / TB;
+        if (blocks > sms) continue;
+        const int P = ub < sms / blocks ? ub : sms / blocks, per_cta = (ub + P - 1) / P;
+        const int vectors = (TB + P - 1) / P, teams = SEQ_QUANT_WARPS / a.team_warps;
+        const double t = per_cta * (steps * 2 * res_slot_clocks(q) + 1500.0) + (double)q.N * q.NS * 128 / 60.0 +
+                         (vectors + teams - 1) / teams * (s.k_a >= 3 ? 4500.0 : 3500.0);
+        if (best == 0.0 || t < best) { best = t; a.p = q; a.P = P; a.unit_blocks = ub; a.unit_steps = steps; }
+        if (TB >= s.batch) break;
+    }
     if (best == 0.0) return false;
     const int blocks = (s.batch + a.p.TB - 1) / a.p.TB;
     // Several vectors per CTA: two teams take one each, sixteen elements a thread; their chains of reductions overlap (35 steps of GRU 2048, 256
