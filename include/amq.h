@@ -387,7 +387,7 @@ AMQ_API amq_status amq_selftest_sequence_give_up(const uint32_t* Wcodes, const f
  * Test aid: how a batched sequence would run on a device of `sm_count` SMs (0: the current device's; any other value needs no device).
  * *form (HOST): one of the forms, or -1 for the one the library chooses, which is then stored there.  split (HOST, 3 ints): CTAs that
  * share a block of vectors, vectors of a block, warps that quantize a vector (zeros for the chain); *clocks (HOST): the estimate for a
- * timestep that the split was chosen by.
+ * timestep that the form is chosen by (0 for a chain whose product runs on the CUDA cores).
  */
 AMQ_API amq_status amq_selftest_sequence_plan(int gru, int I, int H, int k_w, int k_a, int batch, int sm_count,
                                       int* form, int* split, double* clocks);

@@ -1104,12 +1104,11 @@ int sm_count()
 
 // The persistent form: one M tile per CTA step, dedicated epilogue warps, two accumulator buffers when they fit tensor
 // memory.  Possible when there are more tiles than SMs (otherwise nothing could overlap).
-bool plan_persistent(const TcParams& base, int mtiles, int btiles, TcPlan* out)
+bool plan_persistent(const TcParams& base, int mtiles, int btiles, int sms, TcPlan* out)
 {
     TcParams p = base;
     p.MT = 1;
     p.mgroups = mtiles;
-    const int sms = sm_count();
     if (mtiles > 0x7fffffff / btiles) return false;
     p.ntiles = mtiles * btiles;
     if (p.ntiles <= sms) return false;
@@ -1160,8 +1159,9 @@ bool plan_persistent(const TcParams& base, int mtiles, int btiles, TcPlan* out)
     return out->smem <= 227 * 1024;
 }
 
-bool plan(const GemmArgs& a, TcPlan* out)
+bool plan(const GemmArgs& a, TcPlan* out, int sms = 0)
 {
+    if (sms < 1) sms = sm_count();
     TcParams p{};
     p.a = a;
     p.wpr = words_per_row(a.n);
@@ -1185,13 +1185,13 @@ bool plan(const GemmArgs& a, TcPlan* out)
     for (int sft = 0; sft < 8; ++sft) p.mul[sft] = 1u << (7 - sft);
     p.mask_sign = 0x80808080u;
     p.mask_half = 0x40404040u;
-    p.MT = (2 * p.nseg * p.n_mma <= 512 && (long long)(mtiles / 2) * btiles >= 2 * sm_count()) ? 2 : 1;
+    p.MT = (2 * p.nseg * p.n_mma <= 512 && (long long)(mtiles / 2) * btiles >= 2 * sms) ? 2 : 1;
     // with one M tile per CTA and more tiles than SMs, the persistent form hides the epilogues; with two M tiles
     // per CTA the plain form's lower shared-memory traffic per MMA counts for more (measured), unless their accumulators
     // leave no room for the scale factors of the 4-bit form and one M tile per CTA does (C5: 142 us plain with int8
     // operands, 123 us persistent with 4-bit ones)
     const bool two_tiles_4bit = 2 * p.nseg * p.n_mma + 16 <= 512 && (p.nseg == 1 || a.I % 256 == 0);
-    if ((p.MT == 1 || !two_tiles_4bit) && plan_persistent(p, mtiles, btiles, out) && (p.MT == 1 || out->p.fp4)) return true;
+    if ((p.MT == 1 || !two_tiles_4bit) && plan_persistent(p, mtiles, btiles, sms, out) && (p.MT == 1 || out->p.fp4)) return true;
     // 4-bit operands where the scale factors' 16 tensor-memory columns fit beside the accumulators and a GRU's column
     // split falls on a pipeline step (256 bit positions)
     const int acc_cols = p.MT * p.nseg * p.n_mma;
@@ -1258,6 +1258,21 @@ bool gemm_tc_supported(const GemmArgs& a)
     TcPlan pl;
     const bool big = (long long)a.m * a.k_w * words_per_row(a.n) >= (1ll << 17);
     return (a.batch >= 16 || (a.batch >= 2 && big)) && plan(a, &pl);
+}
+
+double chain_clocks(const BatchedSequence& s, int sms)
+{
+    if (sms < 1) sms = sm_count();
+    GemmArgs a{};
+    a.m = (s.gru ? 3 : 4) * s.H; a.n = s.n; a.k_w = s.k_w; a.batch = s.batch; a.k_a = s.k_a;
+    a.epilogue = s.gru ? EPI_GRU : EPI_LSTM;
+    a.I = s.I; a.H = s.H;
+    TcPlan pl;
+    if (s.batch < 16 || !plan(a, &pl, sms)) return 0.0;
+    const long long tiles = pl.persistent ? pl.p.ntiles : (long long)pl.grid.x * pl.grid.y, waves = (tiles + sms - 1) / sms * pl.p.MT;
+    const double elements = (double)s.batch * s.n / sms;
+    return 17600.0 + waves * (11000.0 + 685.0 * pl.p.steps + (s.gru ? 22.0 * pl.p.TB : 0.0)) +
+           elements * (s.k_a <= 2 ? 1.15 : s.k_a == 3 ? 1.22 : 4.0);
 }
 
 bool gemm_tc_single_wave(const GemmArgs& a)

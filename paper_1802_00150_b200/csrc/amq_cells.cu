@@ -133,10 +133,8 @@ void give_lane(CopyLane& l)
 }
 
 // The counters as they stand after `counted` timesteps (self-test).
-amq_status start_counters(const BatchedSequence& s, SequenceForm form, int counted, cudaStream_t st)
+amq_status start_counters(const BatchedSequence& s, SequenceForm form, const SequenceShape& shape, int counted, cudaStream_t st)
 {
-    SequenceShape shape;
-    if (!(form == SEQ_RESIDENT ? resident_sequence_shape(s, 0, &shape) : streaming_sequence_shape(s, 0, &shape))) return AMQ_ERR_UNSUPPORTED;
     for (int b = 0; b < shape.blocks; ++b) {
         const int in_block = s.batch - b * shape.block < shape.block ? s.batch - b * shape.block : shape.block;
         const int quantizers = form == SEQ_RESIDENT && in_block < shape.ctas ? in_block : shape.ctas;
@@ -161,10 +159,12 @@ amq_status enqueue_sequence(const CellCall& c, const CellWorkspace& ws, const fl
     if (persistent)
         return enqueue_persistent(c, ws, x_seq, steps, h0, c0, h_seq, h_last, c_last, st);
     const BatchedSequence whole = batched_call(c, ws, x_seq, steps, h0, c0, h_seq, h_last, c_last);
-    if (form == SEQ_ANY) form = batched_sequence_form(whole);
+    SequenceShape shape{};
+    if (form == SEQ_ANY) form = batched_sequence_form(whole, 0, &shape);
+    else if (form != SEQ_CHAIN && !sequence_shape(whole, form, 0, &shape)) return AMQ_ERR_UNSUPPORTED;
     if (steps > 0 && form != SEQ_CHAIN) {
         if (counted > 0) {
-            const amq_status r = start_counters(whole, form, counted, st);
+            const amq_status r = start_counters(whole, form, shape, counted, st);
             if (r != AMQ_OK) return r;
         }
         // one launch for all steps, or one per chunk, the state handed on in the caller's h_last / c_last
@@ -174,7 +174,7 @@ amq_status enqueue_sequence(const CellCall& c, const CellWorkspace& ws, const fl
             BatchedSequence b = batched_call(c, ws, x_seq + (size_t)s0 * c.batch * c.I, s1 - s0, q ? h_last : h0, q ? c_last : c0,
                                              h_seq ? h_seq + (size_t)s0 * state : nullptr, h_last, c_last);
             b.counted = counted + s0;
-            const amq_status r = launch_batched_sequence(b, form, st);
+            const amq_status r = launch_batched_sequence(b, form, shape, st);
             if (r != AMQ_OK) return r;
         }
         return AMQ_OK;
@@ -202,8 +202,9 @@ amq_status step_entry(const CellCall& c, const CellWorkspace& ws, const float* x
     if (c.batch == 1 && use_persistent(c)) return enqueue_persistent(c, ws, x, 1, h_in, c_in, nullptr, h_out, c_out, st);
     AMQ_CUDA_TRY(cudaMemsetAsync(ws.status, 0, 256 + ws.counter_bytes, st));
     const BatchedSequence b = batched_call(c, ws, x, 1, h_in, c_in, nullptr, h_out, c_out);
-    const SequenceForm form = batched_sequence_form(b);
-    if (form != SEQ_CHAIN) return launch_batched_sequence(b, form, st);
+    SequenceShape shape;
+    const SequenceForm form = batched_sequence_form(b, 0, &shape);
+    if (form != SEQ_CHAIN) return launch_batched_sequence(b, form, shape, st);
     return enqueue_step(c, ws, x, h_in, c_in, h_out, c_out, st);
 }
 
@@ -452,11 +453,10 @@ amq_status amq_selftest_sequence_plan(int gru, int I, int H, int k_w, int k_a, i
     if (!amq::valid_k(k_w) || !amq::valid_k(k_a) || I + H > AMQ_MAX_N) return AMQ_ERR_UNSUPPORTED;
     amq::BatchedSequence s{};
     s.I = I; s.H = H; s.n = I + H; s.k_w = k_w; s.k_a = k_a; s.T = 2; s.batch = batch; s.steps = 1; s.gru = gru != 0;
-    if (*form < 0) *form = amq::batched_sequence_form(s, sm_count);
     amq::SequenceShape shape{};
-    if (*form != AMQ_FORM_CHAIN &&
-        !(*form == AMQ_FORM_RESIDENT ? amq::resident_sequence_shape(s, sm_count, &shape) : amq::streaming_sequence_shape(s, sm_count, &shape)))
-        return AMQ_ERR_UNSUPPORTED;
+    if (*form < 0) *form = amq::batched_sequence_form(s, sm_count, &shape);
+    else if (*form != AMQ_FORM_CHAIN && !amq::sequence_shape(s, (amq::SequenceForm)*form, sm_count, &shape)) return AMQ_ERR_UNSUPPORTED;
+    if (*form == AMQ_FORM_CHAIN) { shape = amq::SequenceShape{}; shape.clocks = amq::chain_clocks(s, sm_count); }
     split[0] = shape.ctas; split[1] = shape.block; split[2] = shape.warps;
     *clocks = shape.clocks;
     return AMQ_OK;

@@ -117,12 +117,13 @@ amq_status one_launch(const PaperCall& c, const PaperWorkspace& ws, int steps, c
 {
     BatchedSequence b{c.Wh_codes, c.Wh_alpha, nullptr, 0, c.H, c.H, c.k_w, c.k_a, c.T, c.batch, steps, false, nullptr, h0, c0,
                       h_seq, h_last, c_last, {ws.h[0], ws.h[1]}, ws.c, ws.proj, ws.hcodes, ws.hbeta, ws.counters, nullptr, 0};
-    const SequenceForm form = batched_sequence_form(b);
+    SequenceShape shape;
+    const SequenceForm form = batched_sequence_form(b, 0, &shape);
     if (form == SEQ_CHAIN) return AMQ_ERR_UNSUPPORTED;
     const amq_status s = tc_status_word(&b.status);         // (reported by amq_device_status, as for the kernels of the chain)
     if (s != AMQ_OK) return s;
     AMQ_CUDA_TRY(cudaMemsetAsync(ws.counters, 0, batched_counter_bytes(c.batch), st));
-    return launch_batched_sequence(b, form, st);
+    return launch_batched_sequence(b, form, shape, st);
 }
 
 }  // namespace

@@ -82,8 +82,8 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     const ResProblem& p = a.p;
     // The warp's number in a uniform register leaves one more to the quantizer, which spills otherwise (35 steps of LSTM 1728/1024, 48 sequences,
-    // 3-bit weights and activations: 641 us, 602 us so).  At four bits, and at two with sixteen elements a thread, it is that which
-    // makes the compiler spill (up to 7 % slower).
+    // 3-bit weights and activations: 641 us, 602 us so).  At four bits, and at two with sixteen elements a thread, the registers come
+    // out the worse for it (2 to 7 % slower).
     constexpr bool UNIFORM = KA != 4 && !(KA == 2 && EPT == 16);
     const int tid = threadIdx.x, warp = UNIFORM ? __shfl_sync(0xffffffffu, tid >> 5, 0) : tid >> 5, lane = tid & 31, H = a.H;
     const int bb = (int)blockIdx.x / a.P, part = (int)blockIdx.x - bb * a.P, b0 = bb * p.TB;
@@ -242,12 +242,22 @@ size_t seq_more_smem(const ResProblem& p)
     return sizeof(SeqShared) + (y > scratch ? y : scratch);
 }
 
-bool plan(const BatchedSequence& s, int sms, SeqPlan* out)
+// Estimated clocks of a timestep: quantizer rounds (by activation bits), steps and epilogues of a CTA's blocks of units, expansion of the
+// activations, waits.  Fitted to 415 problems (LSTM and GRU, 1 to 4 bits, 2 to 5000 sequences, widths 64 to 2048) on a B200, within 6 %
+// (standard deviation; 19 % at worst).
+double streaming_clocks(const ResProblem& p, int k_a, int P, int unit_blocks, int unit_steps, int team_warps)
+{
+    const int teams = SEQ_QUANT_WARPS / team_warps, vectors = (p.TB + P - 1) / P, per_cta = (unit_blocks + P - 1) / P;
+    const double quantizer = (k_a <= 2 ? 6000.0 : k_a == 3 ? 8000.0 : 16800.0) * (p.n > team_warps * 256 ? 1.3 : 1.0);
+    return 6200.0 + (vectors + teams - 1) / teams * quantizer + per_cta * (1.5 * unit_steps * res_slot_clocks(p) + 3000.0 + 14.0 * p.N * p.k_w) +
+           11.0 * p.N * p.NS;
+}
+
+// `only`: blocks of that many vectors (0: the best)
+bool plan(const BatchedSequence& s, int sms, int only, SeqPlan* out)
 {
     if (s.batch < 2 || s.H < 1 || s.n > AMQ_MAX_N || (s.gru && s.I < 1)) return false;
-    if (sms < 1) sms = res_sm_count();
     SeqParams a{};
-    a.team_warps = s.n <= 2048 ? 8 : 16;
     ResProblem p{};
     p.W = s.Wcodes; p.Walpha = s.Walpha; p.k_w = s.k_w; p.wpr = words_per_row(s.n);
     p.vec32 = p.wpr % 8 == 0 && (reinterpret_cast<uintptr_t>(s.Wcodes) & 31) == 0;
@@ -262,24 +272,24 @@ bool plan(const BatchedSequence& s, int sms, SeqPlan* out)
     double best = 0.0;
     const int ub = (s.H + 31) / 32, steps = p.k_w * ((p.NS + 1) / 2);
     for (int TB = 8; TB <= 8 * SEQ_NG * R::SPLIT; TB += 8) {
+        if (only && TB != only) continue;
         ResProblem q = p;
         q.TB = TB;
         if (!res_set_block<R>(q, TB, s.k_a, seq_more_smem(q))) break;
         const int blocks = (s.batch + TB - 1) / TB;
         if (blocks > sms) continue;
-        const int P = ub < sms / blocks ? ub : sms / blocks, per_cta = (ub + P - 1) / P;
-        const int vectors = (TB + P - 1) / P, teams = SEQ_QUANT_WARPS / a.team_warps;
-        const double t = per_cta * (steps * 2 * res_slot_clocks(q) + 1500.0) + (double)q.N * q.NS * 128 / 60.0 +
-                         (vectors + teams - 1) / teams * (s.k_a >= 3 ? 4500.0 : 3500.0);
-        if (best == 0.0 || t < best) { best = t; a.p = q; a.P = P; a.unit_blocks = ub; a.unit_steps = steps; }
+        const int P = ub < sms / blocks ? ub : sms / blocks;
+        // Several vectors per CTA: two teams take one each, sixteen elements a thread; their chains of reductions overlap (35 steps of GRU
+        // 2048, 256 sequences, 3-bit activations: 1561 us with one team of sixteen warps, 1496 us; 4 to 27 % less over 24 problems with
+        // 1 to 3 bits).  Not at four bits, where sixteen elements do not fit the registers (LSTM 2000/2000, 200 sequences: 2153 us
+        // against 2660).
+        const int team_warps = s.n <= 2048 || (s.n <= 4096 && TB > P && s.k_a <= 3) ? 8 : 16;
+        const double t = streaming_clocks(q, s.k_a, P, ub, steps, team_warps);
+        if (best == 0.0 || t < best) { best = t; a.p = q; a.P = P; a.unit_blocks = ub; a.unit_steps = steps; a.team_warps = team_warps; }
         if (TB >= s.batch) break;
     }
     if (best == 0.0) return false;
     const int blocks = (s.batch + a.p.TB - 1) / a.p.TB;
-    // Several vectors per CTA: two teams take one each, sixteen elements a thread; their chains of reductions overlap (35 steps of GRU 2048, 256
-    // sequences, 3-bit activations: 1561 us with one team of sixteen warps, 1496 us; 4 to 27 % less over 24 problems with 1 to 3
-    // bits).  Not at four bits, where sixteen elements do not fit the registers (LSTM 2000/2000, 200 sequences: 2153 us against 2660).
-    if (s.n <= 4096 && a.p.TB > a.P && s.k_a <= 3) a.team_warps = 8;
     a.b_bytes = a.p.NS * a.p.N * 128;
     a.bias = s.bias; a.H = s.H; a.steps = s.steps; a.k_a = s.k_a;
     a.z = SeqVectors{s.n, a.p.wpr, s.H, s.n - s.H, s.T, s.zcodes, s.zbeta, (size_t)a.p.wpr * 4, 16};
@@ -310,15 +320,16 @@ amq_status launch(const SeqPlan& pl, cudaStream_t st)
 bool streaming_sequence_shape(const BatchedSequence& s, int sms, SequenceShape* out)
 {
     SeqPlan pl;
-    if (!plan(s, sms, &pl)) return false;
-    *out = SequenceShape{pl.grid / pl.a.P, pl.a.p.TB, pl.a.P, pl.a.team_warps, pl.clocks};
+    if (sms < 1) sms = res_sm_count();
+    if (!plan(s, sms, 0, &pl)) return false;
+    *out = SequenceShape{sms, pl.grid / pl.a.P, pl.a.p.TB, pl.a.P, pl.a.team_warps, pl.clocks};
     return true;
 }
 
-amq_status launch_streaming_sequence(const BatchedSequence& s, cudaStream_t st)
+amq_status launch_streaming_sequence(const BatchedSequence& s, const SequenceShape& shape, cudaStream_t st)
 {
     SeqPlan pl;
-    if (!plan(s, 0, &pl)) return AMQ_ERR_UNSUPPORTED;
+    if (!plan(s, shape.sms, shape.block, &pl)) return AMQ_ERR_UNSUPPORTED;
     switch (s.k_a) {
         case 1: return launch<1>(pl, st);
         case 2: return launch<2>(pl, st);
@@ -328,15 +339,26 @@ amq_status launch_streaming_sequence(const BatchedSequence& s, cudaStream_t st)
     return AMQ_ERR_UNSUPPORTED;
 }
 
-SequenceForm batched_sequence_form(const BatchedSequence& s, int sms)
+SequenceForm batched_sequence_form(const BatchedSequence& s, int sms, SequenceShape* out)
 {
+    // The least estimated time.  The weights are worth keeping in tensor memory while the vectors of a block need few passes over them: 35
+    // timesteps of LSTM 1024/1024, 64 sequences, 3/3 bits take 394 us resident, 517 streamed; of GRU 1900/1900, 256 sequences, 2/3 bits
+    // (52 passes of five vectors) 7301 us resident, 1486 streamed.  Over 420 problems the choice costs 0.2 % on average against the
+    // best form of each, 12 % at worst (always the resident form: 8 %, and five times the time at worst).
+    if (sms < 1) sms = res_sm_count();
     SequenceShape shape;
-    return resident_sequence_shape(s, sms, &shape) ? SEQ_RESIDENT : streaming_sequence_shape(s, sms, &shape) ? SEQ_STREAMING : SEQ_CHAIN;
-}
-
-amq_status launch_batched_sequence(const BatchedSequence& s, SequenceForm form, cudaStream_t st)
-{
-    return form == SEQ_RESIDENT ? launch_resident_sequence(s, st) : form == SEQ_STREAMING ? launch_streaming_sequence(s, st) : AMQ_ERR_UNSUPPORTED;
+    SequenceForm form = SEQ_CHAIN;
+    double best = 0.0;
+    if (resident_sequence_shape(s, sms, &shape)) { form = SEQ_RESIDENT; best = shape.clocks; *out = shape; }
+    if (streaming_sequence_shape(s, sms, &shape) && (best == 0.0 || shape.clocks < best)) { form = SEQ_STREAMING; best = shape.clocks; *out = shape; }
+    // From eight tiles of 256 operand rows on the product of the chain fills the machine for longer than its launches take (GRU 1024/1024,
+    // 4096 sequences, 2/3 bits: 6976 us, streamed 7274, resident 10877); below, a one-launch form was at most 12 % behind it, and up
+    // to 27 times faster where the chain's product has to run on the CUDA cores.
+    if (best > 0.0 && (long long)s.batch * s.k_a >= 2048) {
+        const double chain = chain_clocks(s, sms);
+        if (chain > 0.0 && chain < best) form = SEQ_CHAIN;
+    }
+    return form;
 }
 
 }  // namespace amq
