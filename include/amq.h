@@ -338,7 +338,8 @@ AMQ_API amq_status amq_lm_greedy_decode(const uint32_t* We_codes, const float* W
  * (and h_seq when not NULL) are copied back to host memory; the call returns after the stream has
  * drained.  Weights, bias, workspace and staging (amq_cell_host_staging_bytes) stay DEVICE pointers.
  * Inputs of 4 MiB and more of a batched sequence are copied in up to eight chunks of timesteps on a stream of
- * the library's (a few are kept between calls, each used by one call at a time), so that the copy of later timesteps runs beside the kernels of earlier ones;
+ * the library's (up to four per device are kept between calls, each used by one call at a time; they belong to the device's primary
+ * context and are forgotten when it is reset; calls in other contexts make their own), so that the copy of later timesteps runs beside the kernels of earlier ones;
  * the results do not depend on it.
  */
 AMQ_API amq_status amq_lstm_sequence_host(const uint32_t* Wcodes, const float* Walpha, const float* bias,

@@ -3,6 +3,9 @@
 // epilogue.  No step returns to the host; a sequence is enqueued as one chain on the caller's stream.
 #include "amq_common.cuh"
 
+#include <cuda.h>
+#include <cudaTypedefs.h>
+
 #include <mutex>
 
 namespace amq {
@@ -93,13 +96,58 @@ struct Chunks {
     cudaEvent_t ready[MAX_CHUNKS + 1];      // (one more, for the start of the copy stream)
 };
 
-// Copy stream and events of one host call.  Creating and destroying them cost 100 us a call, so up to LANES of them wait for the next call
-// (of any thread: a lane belongs to one call at a time); a lane more than that is destroyed when its call ends.
-constexpr int LANES = 4;
-struct CopyLane { int device; cudaStream_t stream; cudaEvent_t event[MAX_CHUNKS + 1]; };
+// Copy stream and events of one host call.  Creating and destroying them cost 100 us a call, so up to LANES of a device wait for the next
+// call (of any thread: a lane belongs to one call at a time); a lane more than that is destroyed when its call ends.
+//
+// Streams and events belong to a context and go with it, so lanes are kept for a device's primary context only, under its id (unique in
+// the process: a device reset makes another).  A call that finds lanes of another id forgets them: they went with their context.  In a
+// context that the application made with the driver API a call creates and destroys its own.
+constexpr int LANES = 4, LANE_DEVICES = 16;
+struct CopyLane { int device; unsigned long long context; cudaStream_t stream; cudaEvent_t event[MAX_CHUNKS + 1]; };     // context 0: not kept
+struct KeptLanes { unsigned long long context; int count; CopyLane lane[LANES]; };
 std::mutex g_lanes_mutex;
-CopyLane g_lanes[LANES];
-int g_lane_count = 0;
+KeptLanes g_lanes[LANE_DEVICES];
+
+// Id of the current context when it is the primary context of its device, else (or when the driver does not tell) 0.
+unsigned long long primary_context_id()
+{
+    struct Driver {
+        PFN_cuCtxGetCurrent_v4000 current = nullptr;
+        PFN_cuCtxGetDevice_v2000 device = nullptr;
+        PFN_cuDevicePrimaryCtxGetState_v7000 state = nullptr;
+        PFN_cuDevicePrimaryCtxRetain_v7000 retain = nullptr;
+        PFN_cuDevicePrimaryCtxRelease_v11000 release = nullptr;
+        PFN_cuCtxGetId_v12000 id = nullptr;
+        bool all = false;
+        Driver()
+        {
+            auto get = [](const char* name, unsigned version) {
+                void* f = nullptr;
+                cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+                return cudaGetDriverEntryPointByVersion(name, &f, version, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess ? f : nullptr;
+            };
+            current = reinterpret_cast<PFN_cuCtxGetCurrent_v4000>(get("cuCtxGetCurrent", 4000));
+            device = reinterpret_cast<PFN_cuCtxGetDevice_v2000>(get("cuCtxGetDevice", 2000));
+            state = reinterpret_cast<PFN_cuDevicePrimaryCtxGetState_v7000>(get("cuDevicePrimaryCtxGetState", 7000));
+            retain = reinterpret_cast<PFN_cuDevicePrimaryCtxRetain_v7000>(get("cuDevicePrimaryCtxRetain", 7000));
+            release = reinterpret_cast<PFN_cuDevicePrimaryCtxRelease_v11000>(get("cuDevicePrimaryCtxRelease", 11000));
+            id = reinterpret_cast<PFN_cuCtxGetId_v12000>(get("cuCtxGetId", 12000));
+            all = current && device && state && retain && release && id;
+        }
+    };
+    static const Driver d;
+    CUcontext current = nullptr, primary = nullptr;
+    CUdevice device;
+    unsigned long long id = 0;
+    unsigned flags;
+    int active = 0;
+    if (!d.all || d.current(&current) != CUDA_SUCCESS || !current || d.device(&device) != CUDA_SUCCESS ||
+        d.state(device, &flags, &active) != CUDA_SUCCESS || !active || d.retain(&primary, device) != CUDA_SUCCESS)
+        return 0;
+    if (primary != current || d.id(current, &id) != CUDA_SUCCESS) id = 0;
+    d.release(device);
+    return id;
+}
 
 void destroy_lane(CopyLane& l)
 {
@@ -112,10 +160,12 @@ cudaError_t take_lane(CopyLane* out)
     CopyLane l{};
     cudaError_t e = cudaGetDevice(&l.device);
     if (e != cudaSuccess) return e;
-    {
+    if (l.device < LANE_DEVICES) l.context = primary_context_id();
+    if (l.context) {
         std::lock_guard<std::mutex> lock(g_lanes_mutex);
-        for (int q = 0; q < g_lane_count; ++q)
-            if (g_lanes[q].device == l.device) { *out = g_lanes[q]; g_lanes[q] = g_lanes[--g_lane_count]; return cudaSuccess; }
+        KeptLanes& kept = g_lanes[l.device];
+        if (kept.context != l.context) { kept.context = l.context; kept.count = 0; }
+        if (kept.count > 0) { *out = kept.lane[--kept.count]; return cudaSuccess; }
     }
     e = cudaStreamCreateWithFlags(&l.stream, cudaStreamNonBlocking);
     for (int q = 0; q <= MAX_CHUNKS && e == cudaSuccess; ++q) e = cudaEventCreateWithFlags(&l.event[q], cudaEventDisableTiming);
@@ -125,9 +175,10 @@ cudaError_t take_lane(CopyLane* out)
 
 void give_lane(CopyLane& l)
 {
-    {
+    if (l.context) {
         std::lock_guard<std::mutex> lock(g_lanes_mutex);
-        if (g_lane_count < LANES) { g_lanes[g_lane_count++] = l; l = CopyLane{}; return; }
+        KeptLanes& kept = g_lanes[l.device];
+        if (kept.context == l.context && kept.count < LANES) { kept.lane[kept.count++] = l; l = CopyLane{}; return; }
     }
     destroy_lane(l);
 }
