@@ -322,7 +322,7 @@ amq_status sequence_host_entry(const CellCall& c, const float* x_seq_host, int s
     // whatever their stream, and the chain's first kernel needs them
     cudaError_t e = cudaMemcpyAsync(hs.h0, h0_host, state_bytes, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && !c.gru) e = cudaMemcpyAsync(hs.c0, c0_host, state_bytes, cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) return AMQ_ERR_CUDA;
+    if (e != cudaSuccess) return cuda_fail(e);
     if (chunked) {
         for (int done = 0, size = (steps + 11) / 12; done < steps; ++chunks.count) {
             chunks.begin[chunks.count] = done;
@@ -344,7 +344,7 @@ amq_status sequence_host_entry(const CellCall& c, const float* x_seq_host, int s
                                 cudaMemcpyHostToDevice, lane.stream);
             if (e == cudaSuccess) e = cudaEventRecord(chunks.ready[q], lane.stream);
         }
-        if (e != cudaSuccess) { if (lane.stream) cudaStreamSynchronize(lane.stream); destroy_lane(lane); return AMQ_ERR_CUDA; }
+        if (e != cudaSuccess) { if (lane.stream) cudaStreamSynchronize(lane.stream); destroy_lane(lane); return cuda_fail(e); }
     } else if (x_bytes) {
         AMQ_CUDA_TRY(cudaMemcpyAsync(hs.x_seq, x_seq_host, x_bytes, cudaMemcpyHostToDevice, st));
     }

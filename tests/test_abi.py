@@ -197,3 +197,20 @@ def test_paper_table6_fixture_is_the_one_the_benchmark_reads():
             rows[(int(f[0]), int(f[2]))] = float(f[4])
     assert rows[(4096, 2)] == 0.35 and rows[(4096, 3)] == 0.72 and rows[(42000, 2)] == 3.17 and rows[(42000, 3)] == 6.46
     assert rows[(4096, 0)] == 1.95 and rows[(42000, 0)] == 19.10       # the full-precision baseline of the same table
+
+
+def test_a_failing_copy_of_a_host_call_is_reported(lib):
+    """Without a device the first copy fails: AMQ_ERR_CUDA, and amq_last_cuda_error tells which error it was."""
+    import torch
+    if torch.cuda.is_available():
+        pytest.skip("needs a machine without a device (the pointers are made up)")
+    vp, ci, sz = ctypes.c_void_p, ctypes.c_int, ctypes.c_size_t
+    lib.amq_cell_workspace_bytes.restype = lib.amq_cell_host_staging_bytes.restype = sz
+    host = (ctypes.c_float * 1024)()
+    p = ctypes.cast(host, vp)
+    need, staging = lib.amq_cell_workspace_bytes(8, 8, 2, 2), lib.amq_cell_host_staging_bytes(8, 8, 2, 3)
+    f = lib.amq_gru_sequence_host
+    f.argtypes = [vp, vp, vp, ci, ci, ci, vp, ci, vp, ci, ci, ci, vp, vp, vp, sz, vp, sz, vp]
+    fake = vp(0x1000)
+    assert f(fake, fake, None, 8, 8, 2, p, 3, p, 2, 2, 2, None, p, fake, need, fake, staging, None) == -5
+    assert lib.amq_last_cuda_error() != 0
