@@ -159,13 +159,25 @@ log_softmax_argmax_kernel(const float* logits, int n, int ld, float* __restrict_
 amq_status launch_log_softmax_argmax(const float* logits, int rows, int n, int ld, float* logp, int ldp, int32_t* argmax,
                                      cudaStream_t st, bool overlap_with_previous)
 {
-    // The smallest CTA whose registers hold a row (less three leading floats): several rows are then in flight per SM, and no thread
-    // works on positions past the end.
-    auto kernel = log_softmax_argmax_kernel;
+    // The tightest of these that holds a row (its up to three leading floats apart), so that several rows are in flight per SM and few registers
+    // lie past the end (of a row above 2048 floats at most a half, above 4096 three eighths).  2240 rows, with steps at 2048, 10240
+    // and 49152 only and now: 3000 floats 24.8 -> 12.5 us, 8000 31.0 -> 26.8, 12288 112.8 -> 43.8, 20001 122.6 -> 60.0 (three
+    // passes over L2: 111), 30000 136.7 -> 119.1.  (Up to 10240 floats <256, 10> takes 11.0 us against 12.6 for 600 rows of 9999, but
+    // 6.3 against 4.6 for one.)
+    struct Size { int n; decltype(&log_softmax_argmax_kernel) kernel; int threads; };
+    static constexpr Size sizes[] = {
+        {4 * 128 * 4, log_softmax_argmax_resident_kernel<128, 4>, 128},     {4 * 256 * 4, log_softmax_argmax_resident_kernel<256, 4>, 256},
+        {4 * 256 * 5, log_softmax_argmax_resident_kernel<256, 5>, 256},     {4 * 512 * 3, log_softmax_argmax_resident_kernel<512, 3>, 512},
+        {4 * 512 * 4, log_softmax_argmax_resident_kernel<512, 4>, 512},
+        {4 * 512 * 5, log_softmax_argmax_resident_kernel<512, 5>, 512},     {4 * 512 * 8, log_softmax_argmax_resident_kernel<512, 8>, 512},
+        {4 * 512 * 10, log_softmax_argmax_resident_kernel<512, 10>, 512},   {4 * 512 * 12, log_softmax_argmax_resident_kernel<512, 12>, 512},
+        {4 * 1024 * 8, log_softmax_argmax_resident_kernel<1024, 8>, 1024},  {4 * 1024 * 10, log_softmax_argmax_resident_kernel<1024, 10>, 1024},
+        {4 * 1024 * 12, log_softmax_argmax_resident_kernel<1024, 12>, 1024},
+    };
+    auto kernel = &log_softmax_argmax_kernel;
     int threads = SM_THREADS;
-    if (n <= 4 * 128 * 4) { kernel = log_softmax_argmax_resident_kernel<128, 4>; threads = 128; }
-    else if (n <= 4 * 512 * 5) { kernel = log_softmax_argmax_resident_kernel<512, 5>; threads = 512; }
-    else if (n <= 4 * 1024 * 12) kernel = log_softmax_argmax_resident_kernel<1024, 12>;
+    for (const Size& s : sizes)
+        if (n <= s.n) { kernel = s.kernel; threads = s.threads; break; }
     AMQ_CUDA_TRY(launch_kernel(kernel, dim3((unsigned)rows), dim3((unsigned)threads), 0, st, overlap_with_previous, logits, n, ld,
                                logp, ldp, argmax));
     AMQ_LAUNCH_CHECK();

@@ -134,6 +134,20 @@ def test_log_softmax_of_rows_off_the_16_byte_boundary(amq, rows, n, ld, skip):
     assert np.array_equal(arg.cpu().numpy(), rarg)
 
 
+@pytest.mark.parametrize("n", [2048, 4096, 5120, 6144, 8192, 10240, 16384, 20480, 24576, 32768, 40960, 49152])
+@pytest.mark.parametrize("past", [0, 1])
+def test_log_softmax_at_the_edges_of_its_sizes(amq, n, past):
+    """Every length at which another CTA size takes over, and one more; the first row starts on a 16-byte boundary, the next do not where the
+    length is odd.  Tolerance: fp32 sum of up to 49153 exponentials, its logarithm and one subtraction (logits within +-17)."""
+    n += past
+    z = synth.normal((3, n), 3.0, 450 + n, 1)
+    z[1, n - 1] = z[1].max() + 1.0
+    logp, arg = amq.log_softmax_argmax(dev(z))
+    ref, rarg = oracle.log_softmax_argmax(z.astype(np.float64))
+    assert np.abs(logp.cpu().numpy() - ref).max() <= 2e-5
+    assert np.array_equal(arg.cpu().numpy(), rarg)
+
+
 @pytest.mark.parametrize("rows,n,k", [(2100, 1023, 3), (2100, 1024, 4), (2100, 65, 4), (1100, 513, 2), (3, 2049, 4)])
 def test_quantizer_with_levels_out_of_order(amq, rows, n, k):
     """Rows whose refitted coefficients come out negative or not in decreasing order (two clusters and a constant part), so that the
