@@ -333,6 +333,19 @@ AMQ_API amq_status amq_lm_greedy_decode(const uint32_t* We_codes, const float* W
                                 void* workspace, size_t workspace_bytes, void* stream);
 
 /*
+ * Test aid for the give-up path of decoding in one launch: amq_lm_greedy_decode without log-probabilities, its CTAs looking for the words
+ * of the state (late = 1) or of the shares' maxima (late = 2) where none of them writes.  In the first step every wait runs out (about a
+ * second: the ordinary limit), every CTA records that in the device status word (amq_device_status) and returns; tokens, h and c are
+ * left as they were.  AMQ_ERR_UNSUPPORTED where the call would not run in one launch.
+ */
+AMQ_API amq_status amq_selftest_decode_give_up(const uint32_t* We_codes, const float* We_alpha, int vocab, int I, int k_e,
+                                const uint32_t* Wi_codes, const float* Wi_alpha,
+                                const uint32_t* Wh_codes, const float* Wh_alpha, const float* bias, int H, int k_w,
+                                const uint32_t* Ws_codes, const float* Ws_alpha, const float* bias_s, int k_s,
+                                int k_a, int T, int32_t* tokens, int steps, float* h, float* c,
+                                void* workspace, size_t workspace_bytes, int late, void* stream);
+
+/*
  * The sequence calls with HOST activations and results: x_seq, h0, c0 are read from host memory
  * (pinned memory makes the copies asynchronous) into `staging`, the sequence runs, and h_last / c_last
  * (and h_seq when not NULL) are copied back to host memory; the call returns after the stream has
@@ -380,6 +393,9 @@ AMQ_API amq_status amq_selftest_sequence_give_up(const uint32_t* Wcodes, const f
  * AMQ_FORM_STREAMING (one launch, weights streamed) or AMQ_FORM_RESIDENT (one launch, weights in tensor memory).  The progress
  * counters of the one-launch forms start as `counted` (0 .. 2^31 - 1 - steps) earlier timesteps would have left them.  Results are
  * those of the ordinary call in that form, whatever `counted` is.  AMQ_ERR_UNSUPPORTED where the form does not take the problem.
+ *   late = 1 or 2 (one-launch forms, counted = 0; 0: none): the CTAs look for the counts of quantized vectors (from step 0 on) or of finished
+ *   products (from step 1 on: steps >= 2) where none of them counts.  Every wait runs out (a second or two: the ordinary limit),
+ *   every CTA records that in the workspace status word, gives its tensor memory back and returns; h_last and c_last are left unwritten.
  */
 #define AMQ_FORM_CHAIN 0
 #define AMQ_FORM_STREAMING 1
@@ -396,7 +412,7 @@ AMQ_API amq_status amq_selftest_sequence_plan(int gru, int I, int H, int k_w, in
 AMQ_API amq_status amq_selftest_batched_sequence(const uint32_t* Wcodes, const float* Walpha, const float* bias, int I, int H, int k_w,
                                          int gru, const float* x_seq, int steps, const float* h0, const float* c0,
                                          int batch, int k_a, int T, float* h_seq, float* h_last, float* c_last,
-                                         void* workspace, size_t workspace_bytes, int form, int counted, void* stream);
+                                         void* workspace, size_t workspace_bytes, int form, int counted, int late, void* stream);
 
 /*
  * Synchronises `stream`, then reads the status word at the start of a cell workspace: AMQ_OK, or

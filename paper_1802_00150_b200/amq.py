@@ -64,7 +64,9 @@ EXPORTS = {
     "amq_selftest_sequence_plan": (_int, [_int, _int, _int, _int, _int, _int, _int, ctypes.POINTER(_int), ctypes.POINTER(_int),
                                           ctypes.POINTER(ctypes.c_double)]),
     "amq_selftest_batched_sequence": (_int, [_vp, _vp, _vp, _int, _int, _int, _int, _vp, _int, _vp, _vp, _int, _int, _int,
-                                             _vp, _vp, _vp, _vp, _sz, _int, _int, _vp]),
+                                             _vp, _vp, _vp, _vp, _sz, _int, _int, _int, _vp]),
+    "amq_selftest_decode_give_up": (_int, [_vp, _vp, _int, _int, _int, _vp, _vp, _vp, _vp, _vp, _int, _int, _vp, _vp, _vp, _int,
+                                           _int, _int, _vp, _int, _vp, _vp, _vp, _sz, _int, _vp]),
     "amq_gru_original_workspace_bytes": (_sz, [_int, _int, _int, _int]),
     "amq_gru_step_original": (_int, [_vp, _vp, _vp, _int, _int, _int, _vp, _vp, _int, _int, _int, _vp, _vp, _sz, _vp]),
     "amq_quantize_variant": (_int, [_vp, _int, _int, _int, _int, _int, _int, _int, _vp, _vp, _vp]),
@@ -278,14 +280,14 @@ def selftest_sequence_plan(gru, I, H, k_w, k_a, batch, sm_count=0, form=-1):
     return f.value, tuple(split), clocks.value
 
 
-def selftest_batched_sequence(Wcodes, Walpha, bias, I, H, x_seq, h0, c0, k_a, T, workspace, form, counted=0):
+def selftest_batched_sequence(Wcodes, Walpha, bias, I, H, x_seq, h0, c0, k_a, T, workspace, form, counted=0, late=0):
     """Test aid: a batched sequence (LSTM, or GRU when c0 is None) in a given form, its progress counters starting as after `counted`
-    timesteps (see amq.h).  Returns (h_seq, h_last, c_last or None)."""
+    timesteps, its waits running out with `late` (see amq.h).  Returns (h_seq, h_last, c_last or None)."""
     steps, batch, k_w, gru = x_seq.shape[0], h0.shape[0], Wcodes.shape[1], c0 is None
     h_seq = _native.empty(h0, 0, steps, batch, H)
     h_last, c_last = torch.zeros_like(h0), None if gru else torch.zeros_like(c0)
     _check(_native.amq_selftest_batched_sequence(Wcodes, Walpha, bias, I, H, k_w, int(gru), x_seq, steps, h0, c0, batch, k_a, T,
-                                                 h_seq, h_last, c_last, workspace, workspace.numel(), form, counted))
+                                                 h_seq, h_last, c_last, workspace, workspace.numel(), form, counted, late))
     return h_seq, h_last, c_last
 
 
@@ -400,6 +402,15 @@ def lm_greedy_decode(We_codes, We_alpha, Wi_codes, Wi_alpha, Wh_codes, Wh_alpha,
                                      bias_s, k_s, k_a, T, tokens, steps, h, c, logp,
                                      workspace, workspace.numel()))
     return tokens
+
+
+def selftest_decode_give_up(We_codes, We_alpha, Wi_codes, Wi_alpha, Wh_codes, Wh_alpha, bias, Ws_codes, Ws_alpha, bias_s, I, H,
+                            k_a, T, tokens, h, c, workspace, late):
+    """Test aid: lm_greedy_decode in one launch with waits that run out (see amq.h); read the outcome with device_status."""
+    _check(_native.amq_selftest_decode_give_up(We_codes, We_alpha, We_codes.shape[0], I, We_codes.shape[1], Wi_codes, Wi_alpha,
+                                               Wh_codes, Wh_alpha, bias, H, Wi_codes.shape[1], Ws_codes, Ws_alpha, bias_s,
+                                               Ws_codes.shape[1], k_a, T, tokens, tokens.numel() - 1, h, c, workspace,
+                                               workspace.numel(), late))
 
 
 METHOD_ALTERNATING, METHOD_REFINED_GREEDY = 0, 1

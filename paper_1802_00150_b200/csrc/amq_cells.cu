@@ -64,7 +64,7 @@ BatchedSequence batched_call(const CellCall& c, const CellWorkspace& ws, const f
                              float* h_seq, float* h_last, float* c_last)
 {
     return BatchedSequence{c.Wcodes, c.Walpha, c.bias, c.I, c.H, c.I + c.H, c.k_w, c.k_a, c.T, c.batch, steps, c.gru, x_seq, h0, c0,
-                           h_seq, h_last, c_last, {ws.h[0], ws.h[1]}, ws.c, nullptr, ws.zcodes, ws.zbeta, ws.counters, ws.status, 0};
+                           h_seq, h_last, c_last, {ws.h[0], ws.h[1]}, ws.c, nullptr, ws.zcodes, ws.zbeta, ws.counters, ws.status, 0, 0};
 }
 
 // quantize z = [x ; h_in] into the workspace, then product + gates
@@ -197,11 +197,13 @@ amq_status start_counters(const BatchedSequence& s, SequenceForm form, const Seq
     return AMQ_OK;
 }
 
-// `chunks` (may be NULL): the stream waits for a chunk's event before the first kernel that reads it (batched calls only).  `form` and
-// `counted` (timesteps the counters start with) are the self-test's.
+// What the self-test asks for: a form, timesteps the counters start with, waits that run out.
+struct Forced { SequenceForm form; int counted, late; };
+
+// `chunks` (may be NULL): the stream waits for a chunk's event before the first kernel that reads it (batched calls only).
 amq_status enqueue_sequence(const CellCall& c, const CellWorkspace& ws, const float* x_seq, int steps,
                             const float* h0, const float* c0, float* h_seq, float* h_last, float* c_last,
-                            cudaStream_t st, const Chunks* chunks = nullptr, SequenceForm form = SEQ_ANY, int counted = 0)
+                            cudaStream_t st, const Chunks* chunks = nullptr, const Forced* forced = nullptr)
 {
     const size_t state = (size_t)c.batch * c.H, state_bytes = state * sizeof(float);
     const bool persistent = steps > 0 && use_persistent(c);
@@ -211,11 +213,11 @@ amq_status enqueue_sequence(const CellCall& c, const CellWorkspace& ws, const fl
         return enqueue_persistent(c, ws, x_seq, steps, h0, c0, h_seq, h_last, c_last, st);
     const BatchedSequence whole = batched_call(c, ws, x_seq, steps, h0, c0, h_seq, h_last, c_last);
     SequenceShape shape{};
-    if (form == SEQ_ANY) form = batched_sequence_form(whole, 0, &shape);
-    else if (form != SEQ_CHAIN && !sequence_shape(whole, form, 0, &shape)) return AMQ_ERR_UNSUPPORTED;
+    const SequenceForm form = forced ? forced->form : batched_sequence_form(whole, 0, &shape);
+    if (forced && form != SEQ_CHAIN && !sequence_shape(whole, form, 0, &shape)) return AMQ_ERR_UNSUPPORTED;
     if (steps > 0 && form != SEQ_CHAIN) {
-        if (counted > 0) {
-            const amq_status r = start_counters(whole, form, shape, counted, st);
+        if (forced && forced->counted > 0) {
+            const amq_status r = start_counters(whole, form, shape, forced->counted, st);
             if (r != AMQ_OK) return r;
         }
         // one launch for all steps, or one per chunk, the state handed on in the caller's h_last / c_last
@@ -224,7 +226,8 @@ amq_status enqueue_sequence(const CellCall& c, const CellWorkspace& ws, const fl
             if (chunks) AMQ_CUDA_TRY(cudaStreamWaitEvent(st, chunks->ready[q], 0));
             BatchedSequence b = batched_call(c, ws, x_seq + (size_t)s0 * c.batch * c.I, s1 - s0, q ? h_last : h0, q ? c_last : c0,
                                              h_seq ? h_seq + (size_t)s0 * state : nullptr, h_last, c_last);
-            b.counted = counted + s0;
+            b.counted = s0;
+            if (forced) { b.counted += forced->counted; b.late = forced->late; }
             const amq_status r = launch_batched_sequence(b, form, shape, st);
             if (r != AMQ_OK) return r;
         }
@@ -483,7 +486,7 @@ amq_status amq_selftest_sequence_give_up(const uint32_t* Wcodes, const float* Wa
 amq_status amq_selftest_batched_sequence(const uint32_t* Wcodes, const float* Walpha, const float* bias, int I, int H, int k_w, int gru,
                                          const float* x_seq, int steps, const float* h0, const float* c0, int batch, int k_a, int T,
                                          float* h_seq, float* h_last, float* c_last, void* workspace, size_t workspace_bytes,
-                                         int form, int counted, void* stream)
+                                         int form, int counted, int late, void* stream)
 {
     amq::CellCall c{Wcodes, Walpha, bias, I, H, k_w, batch, k_a, T, gru != 0};
     amq_status s = amq::validate(c, workspace, workspace_bytes);
@@ -491,10 +494,12 @@ amq_status amq_selftest_batched_sequence(const uint32_t* Wcodes, const float* Wa
     if (steps < 1 || !h0 || !h_last || (!c.gru && (!c0 || !c_last)) || (I > 0 && !x_seq) || h_last == h0 || (!c.gru && c_last == c0))
         return AMQ_ERR_INVALID_ARG;
     if (form < AMQ_FORM_CHAIN || form > AMQ_FORM_RESIDENT || counted < 0 || counted > 0x7fffffff - steps) return AMQ_ERR_INVALID_ARG;
+    if (late < 0 || late > 2 || (late > 0 && (form == AMQ_FORM_CHAIN || counted > 0)) || (late == 2 && steps < 2))
+        return AMQ_ERR_INVALID_ARG;
     if (batch < 2) return AMQ_ERR_UNSUPPORTED;
     amq::CellWorkspace ws = amq::carve_cell_workspace(workspace, I, H, batch, k_a);
-    return amq::enqueue_sequence(c, ws, x_seq, steps, h0, c0, h_seq, h_last, c_last, (cudaStream_t)stream, nullptr,
-                                 (amq::SequenceForm)form, counted);
+    const amq::Forced forced{(amq::SequenceForm)form, counted, late};
+    return amq::enqueue_sequence(c, ws, x_seq, steps, h0, c0, h_seq, h_last, c_last, (cudaStream_t)stream, nullptr, &forced);
 }
 
 amq_status amq_selftest_sequence_plan(int gru, int I, int H, int k_w, int k_a, int batch, int sm_count, int* form, int* split, double* clocks)

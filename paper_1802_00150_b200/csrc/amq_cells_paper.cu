@@ -116,7 +116,7 @@ amq_status one_launch(const PaperCall& c, const PaperWorkspace& ws, int steps, c
                       float* c_last, cudaStream_t st)
 {
     BatchedSequence b{c.Wh_codes, c.Wh_alpha, nullptr, 0, c.H, c.H, c.k_w, c.k_a, c.T, c.batch, steps, false, nullptr, h0, c0,
-                      h_seq, h_last, c_last, {ws.h[0], ws.h[1]}, ws.c, ws.proj, ws.hcodes, ws.hbeta, ws.counters, nullptr, 0};
+                      h_seq, h_last, c_last, {ws.h[0], ws.h[1]}, ws.c, ws.proj, ws.hcodes, ws.hbeta, ws.counters, nullptr, 0, 0};
     SequenceShape shape;
     const SequenceForm form = batched_sequence_form(b, 0, &shape);
     if (form == SEQ_CHAIN) return AMQ_ERR_UNSUPPORTED;

@@ -181,6 +181,7 @@ struct DecodeSequence {
     int k_a, T, steps;
     int32_t* tokens; float* h; float* c;
     unsigned long long* exchange;
+    int late;                   // self-test of the waits: the CTAs look for h (1) or for the maxima (2) where nobody writes them; 0: none
 };
 bool decode_persistent_supported(const DecodeSequence& d);
 amq_status launch_decode_persistent(const DecodeSequence& d, cudaStream_t st);
@@ -197,10 +198,12 @@ struct BatchedSequence {
     const float* addend;
     uint32_t* zcodes; float* zbeta; uint32_t* counters; uint32_t* status;
     int counted;                // timesteps that earlier launches have added to the counters since they were cleared
+    int late;                   // self-test of the waits: the CTAs look for the counts of quantized shares (1) or of finished products (2) where
+                                // nobody counts; 0: none
 };
 // The ways to run one: a chain of launches per timestep, or one launch with the weights streamed past the activations (amq_rnn_batched.cu)
 // or held in tensor memory (amq_rnn_resident.cu).
-enum SequenceForm { SEQ_ANY = -1, SEQ_CHAIN = 0, SEQ_STREAMING = 1, SEQ_RESIDENT = 2 };
+enum SequenceForm { SEQ_CHAIN = 0, SEQ_STREAMING = 1, SEQ_RESIDENT = 2 };
 // How a one-launch form splits a problem over `sms` SMs (0: those of the current device): `blocks` of up to `block` vectors, `ctas` CTAs
 // each, `warps` to quantize a vector; `clocks`: the estimate for a timestep that the split was chosen by.  False where the form does not take the problem.
 struct SequenceShape { int sms, blocks, block, ctas, warps; double clocks; };

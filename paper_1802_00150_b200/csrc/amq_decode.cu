@@ -40,6 +40,19 @@ DecodeWorkspace carve(void* base, int vocab, int I, int H, int k_e, int k_a)
     return w;
 }
 
+amq_status validate(const DecodeSequence& d, const void* workspace, size_t workspace_bytes)
+{
+    if (!d.We || !d.We_alpha || !d.Wi || !d.Wi_alpha || !d.Wh || !d.Wh_alpha || !d.Ws || !d.Ws_alpha || d.vocab < 1 || d.I < 1 || d.H < 1 ||
+        d.steps < 0)
+        return AMQ_ERR_INVALID_ARG;
+    if (!valid_k(d.k_e) || !valid_k(d.k_w) || !valid_k(d.k_s) || !valid_k(d.k_a) || d.T < 0 || d.I > AMQ_MAX_N || d.H > AMQ_MAX_N)
+        return AMQ_ERR_UNSUPPORTED;
+    if (!workspace || workspace_bytes < amq_lm_decode_workspace_bytes(d.vocab, d.I, d.H, d.k_e, d.k_a)) return AMQ_ERR_WORKSPACE;
+    if (!aligned16(workspace) || !aligned16(d.We) || !aligned16(d.Wi) || !aligned16(d.Wh) || !aligned16(d.Ws)) return AMQ_ERR_ALIGNMENT;
+    if (d.steps > 0 && (!d.tokens || !d.h || !d.c)) return AMQ_ERR_INVALID_ARG;
+    return AMQ_OK;
+}
+
 }  // namespace
 }  // namespace amq
 
@@ -58,25 +71,14 @@ amq_status amq_lm_greedy_decode(const uint32_t* We_codes, const float* We_alpha,
                                 int k_a, int T, int32_t* tokens, int steps, float* h, float* c, float* logp,
                                 void* workspace, size_t workspace_bytes, void* stream)
 {
-    if (!We_codes || !We_alpha || !Wi_codes || !Wi_alpha || !Wh_codes || !Wh_alpha || !Ws_codes || !Ws_alpha || vocab < 1 ||
-        I < 1 || H < 1 || steps < 0)
-        return AMQ_ERR_INVALID_ARG;
-    if (!amq::valid_k(k_e) || !amq::valid_k(k_w) || !amq::valid_k(k_s) || !amq::valid_k(k_a) || T < 0 || I > AMQ_MAX_N ||
-        H > AMQ_MAX_N)
-        return AMQ_ERR_UNSUPPORTED;
-    if (!workspace || workspace_bytes < amq_lm_decode_workspace_bytes(vocab, I, H, k_e, k_a)) return AMQ_ERR_WORKSPACE;
-    if (!amq::aligned16(workspace) || !amq::aligned16(We_codes) || !amq::aligned16(Wi_codes) || !amq::aligned16(Wh_codes) ||
-        !amq::aligned16(Ws_codes))
-        return AMQ_ERR_ALIGNMENT;
-    if (steps == 0) return AMQ_OK;
-    if (!tokens || !h || !c) return AMQ_ERR_INVALID_ARG;
+    amq::DecodeSequence d{We_codes, We_alpha, vocab, I, k_e, Wi_codes, Wi_alpha, Wh_codes, Wh_alpha, bias, H, k_w,
+                          Ws_codes, Ws_alpha, bias_s, k_s, k_a, T, steps, tokens, h, c, nullptr, 0};
+    const amq_status valid = amq::validate(d, workspace, workspace_bytes);
+    if (valid != AMQ_OK || steps == 0) return valid;
     const amq::DecodeWorkspace ws = amq::carve(workspace, vocab, I, H, k_e, k_a);
     cudaStream_t st = (cudaStream_t)stream;
-    if (!logp) {
-        const amq::DecodeSequence d{We_codes, We_alpha, vocab, I, k_e, Wi_codes, Wi_alpha, Wh_codes, Wh_alpha, bias, H, k_w,
-                                    Ws_codes, Ws_alpha, bias_s, k_s, k_a, T, steps, tokens, h, c, ws.exchange};
-        if (amq::decode_persistent_supported(d)) return amq::launch_decode_persistent(d, st);
-    }
+    d.exchange = ws.exchange;
+    if (!logp && amq::decode_persistent_supported(d)) return amq::launch_decode_persistent(d, st);
     // every launch after the first is a programmatic dependent of its predecessor (each kernel waits for it first
     // thing), which takes most of the gaps between these short kernels out of the chain
     auto product = [&](const uint32_t* Wc, const float* Wa, int m, int n, int kw, const uint32_t* xc, const float* xb, int ka,
@@ -113,6 +115,23 @@ amq_status amq_lm_greedy_decode(const uint32_t* We_codes, const float* We_alpha,
                                            tokens + t + 1, st, true);
     }
     return s;
+}
+
+amq_status amq_selftest_decode_give_up(const uint32_t* We_codes, const float* We_alpha, int vocab, int I, int k_e,
+                                       const uint32_t* Wi_codes, const float* Wi_alpha, const uint32_t* Wh_codes, const float* Wh_alpha,
+                                       const float* bias, int H, int k_w,
+                                       const uint32_t* Ws_codes, const float* Ws_alpha, const float* bias_s, int k_s,
+                                       int k_a, int T, int32_t* tokens, int steps, float* h, float* c,
+                                       void* workspace, size_t workspace_bytes, int late, void* stream)
+{
+    amq::DecodeSequence d{We_codes, We_alpha, vocab, I, k_e, Wi_codes, Wi_alpha, Wh_codes, Wh_alpha, bias, H, k_w,
+                          Ws_codes, Ws_alpha, bias_s, k_s, k_a, T, steps, tokens, h, c, nullptr, late};
+    const amq_status s = amq::validate(d, workspace, workspace_bytes);
+    if (s != AMQ_OK) return s;
+    if (steps < 1 || late < 1 || late > 2) return AMQ_ERR_INVALID_ARG;
+    if (!amq::decode_persistent_supported(d)) return AMQ_ERR_UNSUPPORTED;
+    d.exchange = amq::carve(workspace, vocab, I, H, k_e, k_a).exchange;
+    return amq::launch_decode_persistent(d, (cudaStream_t)stream);
 }
 
 }  // extern "C"

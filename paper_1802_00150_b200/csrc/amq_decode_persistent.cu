@@ -32,6 +32,8 @@ struct DecodeArgs {
     int32_t* tokens; float* h; float* c;
     unsigned long long* hx; size_t hx_stride;       // [2][copies][stride]: {h value, tag}
     ulonglong2* best;                               // [2][copies][grid]: {logit, tag}, {index, tag}
+    const unsigned long long* hx_polled;            // where the CTAs look for them: hx and best (the self-test of the waits: half an area
+    const ulonglong2* best_polled;                  // further, where step 0 writes nothing)
     uint32_t* status;
     int CHI, CHH;                                   // 128-bit chunks of a plane of x, of h
     int upc, rpc, resident;                         // hidden units, vocabulary rows per CTA, how many of those rows stay in shared memory
@@ -199,7 +201,7 @@ decode_persistent_kernel(const __grid_constant__ DecodeArgs a)
         uint32_t pending = t >= 0 ? valid : 0u;
 #pragma unroll
         for (int j = 0; j < DEC_EPT; ++j) w[j] = (t < 0 && (valid >> j) & 1u) ? __ldcg(a.h + e0 + j) : 0.0f;
-        const unsigned long long* hx = a.hx + ((size_t)(t & 1) * DEC_COPIES + my_copy) * a.hx_stride;
+        const unsigned long long* hx = a.hx_polled + ((size_t)(t & 1) * DEC_COPIES + my_copy) * a.hx_stride;
         for (unsigned spins = 0; pending && spins < DEC_POLL_LIMIT; ++spins) {
             unsigned long long v[DEC_EPT];
 #pragma unroll
@@ -312,7 +314,7 @@ decode_persistent_kernel(const __grid_constant__ DecodeArgs a)
             float mv = -INFINITY;
             int mi = 0x7fffffff;
             for (int q = tid; q < (int)gridDim.x; q += DEC_THREADS) {
-                const ulonglong2* in = a.best + ((size_t)(t & 1) * DEC_COPIES + my_copy) * gridDim.x + q;
+                const ulonglong2* in = a.best_polled + ((size_t)(t & 1) * DEC_COPIES + my_copy) * gridDim.x + q;
                 ulonglong2 v = make_ulonglong2(0, 0);
                 bool there = false;                 // (each half is validated by its own tag)
                 for (unsigned spins = 0; !there && spins < DEC_POLL_LIMIT; ++spins) {
@@ -411,6 +413,8 @@ amq_status launch_decode_persistent(const DecodeSequence& d, cudaStream_t st)
     a.T = d.T; a.steps = d.steps; a.tokens = d.tokens; a.h = d.h; a.c = d.c;
     a.hx = d.exchange; a.hx_stride = persistent_exchange_stride(d.H);
     a.best = reinterpret_cast<ulonglong2*>(d.exchange + 2 * DEC_COPIES * a.hx_stride);
+    a.hx_polled = a.hx + (d.late == 1 ? DEC_COPIES * a.hx_stride : 0);
+    a.best_polled = a.best + (d.late == 2 ? DEC_COPIES * p.grid : 0);
     a.status = status;
     a.CHI = words_per_row(d.I) / 4; a.CHH = words_per_row(d.H) / 4;
     a.upc = p.upc; a.rpc = p.rpc; a.resident = p.resident;

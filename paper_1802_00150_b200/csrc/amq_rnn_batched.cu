@@ -34,6 +34,7 @@ struct SeqParams {
     float* h[2]; float* c;
     const float* addend;        // [steps][batch][4H] added before the gates, or null
     uint32_t* counters;         // [blocks][64]: word 0 quantized shares, word 32 finished products
+    int planes_word, h_word;    // where a block's CTAs look for them: 0 and 32 (the self-test of the waits: the next word, which stays 0)
     uint32_t* status;
     int counted;                // timesteps in the counters at the start
     int P, unit_blocks, b_bytes;
@@ -124,7 +125,7 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
 
         // ---- 1. this CTA's share of the block's vectors ----
         if (t > 0) {
-            if (tid == 0) ok = seq_wait(counter + 32, seq_target(a.counted + t, a.P));
+            if (tid == 0) ok = seq_wait(counter + a.h_word, seq_target(a.counted + t, a.P));
             if (__syncthreads_or(!ok)) { ok = false; break; }
         }
         if (warp < SEQ_QUANT_WARPS) {
@@ -138,7 +139,7 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
         __syncthreads();
         if (tid == 0) {
             seq_publish(counter);
-            ok = seq_wait(counter, seq_target(a.counted + t + 1, a.P));
+            ok = seq_wait(counter + a.planes_word, seq_target(a.counted + t + 1, a.P));
         }
         if (__syncthreads_or(!ok)) { ok = false; break; }
 
@@ -296,6 +297,7 @@ bool plan(const BatchedSequence& s, int sms, int only, SeqPlan* out)
     a.x_seq = s.x_seq; a.h0 = s.h0; a.c0 = s.c0; a.h_seq = s.h_seq; a.h_last = s.h_last; a.c_last = s.c_last;
     a.h[0] = s.h[0]; a.h[1] = s.h[1]; a.c = s.c; a.addend = s.addend;
     a.counters = s.counters; a.counted = s.counted; a.status = s.status;
+    a.planes_word = s.late == 1 ? 1 : 0; a.h_word = s.late == 2 ? 33 : 32;
     out->grid = blocks * a.P;
     out->smem = (size_t)a.b_bytes + seq_more_smem(a.p);
     out->a = a;

@@ -44,6 +44,7 @@ struct RsParams {
     float* h[2];
     const float* addend;        // [steps][batch][4H] added before the gates, or null
     uint32_t* counters;         // [blocks][64]: word 0 quantized shares, word 32 finished products
+    int planes_word, h_word;    // where a block's CTAs look for them: 0 and 32 (the self-test of the waits: the next word, which stays 0)
     uint32_t* status;
     int counted;                // timesteps in the counters at the start
     int P, block;               // CTAs and vectors of a block
@@ -197,7 +198,7 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
         // ---- 1. this CTA's share of the block's vectors ----
         if (part < quantizers) {                    // (uniform over the CTA)
             if (t > 0) {
-                if (tid == 0) ok = seq_wait(counter + 32, seq_target(a.counted + t, a.P));
+                if (tid == 0) ok = seq_wait(counter + a.h_word, seq_target(a.counted + t, a.P));
                 if (__syncthreads_or(!ok)) { ok = false; break; }
             }
             const float* x = a.x_seq + (size_t)t * a.batch * a.z.xn;
@@ -212,7 +213,7 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
             __syncthreads();
             if (tid == 0) seq_publish(counter);
         }
-        if (tid == 0) ok = seq_wait(counter, seq_target(a.counted + t + 1, quantizers));
+        if (tid == 0) ok = seq_wait(counter + a.planes_word, seq_target(a.counted + t + 1, quantizers));
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         if (__syncthreads_or(!ok)) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -454,6 +455,7 @@ bool plan(const BatchedSequence& s, int sms, int only, RsPlan* out)
     a.I = s.I; a.k_w = s.k_w; a.gru = s.gru; a.steps = s.steps; a.batch = s.batch;
     a.x_seq = s.x_seq; a.h0 = s.h0; a.c0 = s.c0; a.h_seq = s.h_seq; a.h_last = s.h_last; a.c_last = s.c_last;
     a.h[0] = s.h[0]; a.h[1] = s.h[1]; a.addend = s.addend; a.counters = s.counters; a.counted = s.counted; a.status = s.status;
+    a.planes_word = s.late == 1 ? 1 : 0; a.h_word = s.late == 2 ? 33 : 32;
     *out = p;
     return true;
 }

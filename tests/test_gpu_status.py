@@ -1,6 +1,7 @@
 """The give-up path of bounded device-side waits, exercised without hurting the GPU: a status word written from
-the host, and the batch-1 sequence kernel run with waits that are made to run out (a smaller bound on the same
-bounded polls, expecting step tags nobody publishes).  Nothing here faults, traps or spins without a limit."""
+the host, and the kernels whose CTAs wait for one another (batch-1 and batched sequences, decoding) run with waits that are made to
+run out (a smaller bound on the same bounded polls, or the ordinary one, for tags and counts nobody publishes).  Nothing here faults, traps or spins
+without a limit."""
 import numpy as np
 import pytest
 import torch
@@ -31,7 +32,7 @@ def small_model(amq, I, H, k_w=2, seed=80):
 def test_status_word_written_from_the_host_is_reported_and_cleared_by_the_next_call(amq):
     I, H, ka = 64, 48, 2
     Wcodes, Walpha = small_model(amq, I, H)
-    for batch in (1, 5):                       # the persistent kernel and the two-kernel chain share the status word
+    for batch in (1, 5):                       # the batch-1 kernel and a batched one-launch kernel
         ws = amq.new_workspace(I, H, batch, ka)
         assert amq.workspace_status(ws) == 0
         ws[:4] = torch.tensor([1, 0, 0, 0], dtype=torch.uint8, device="cuda")
@@ -41,6 +42,11 @@ def test_status_word_written_from_the_host_is_reported_and_cleared_by_the_next_c
         h = dev(synth.uniform((batch, H), -1, 1, 81, 2))
         c = dev(synth.uniform((batch, H), -1, 1, 81, 3))
         amq.lstm_step(Wcodes, Walpha, None, I, H, x, h, c, ka, 2, ws)
+        assert amq.workspace_status(ws) == 0
+    for form in (amq.FORM_CHAIN, amq.FORM_STREAMING, amq.FORM_RESIDENT):        # every form of the last, batched call
+        ws[:4] = torch.tensor([1, 0, 0, 0], dtype=torch.uint8, device="cuda")
+        assert amq.workspace_status(ws) == TIMEOUT
+        amq.selftest_batched_sequence(Wcodes, Walpha, None, I, H, x[None], h, c, ka, 2, ws, form)
         assert amq.workspace_status(ws) == 0
 
 
@@ -63,6 +69,59 @@ def test_waits_that_run_out_set_the_status_and_leave_the_context_usable(amq, I, 
         assert torch.equal(g, w)
 
 
+@pytest.mark.parametrize("late", [1, 2])
+@pytest.mark.parametrize("form,cell,I,H,batch,kw,ka", [
+    (2, "lstm", 64, 48, 9, 2, 2),           # one block of vectors, more CTAs than quantize
+    (2, "gru", 300, 650, 150, 3, 2),       # several vectors per CTA
+    (2, "lstm", 1024, 1024, 64, 3, 3),
+    (1, "lstm", 64, 200, 40, 2, 2),         # several blocks
+    (1, "gru", 2048, 2048, 256, 2, 3),
+])
+def test_batched_waits_that_run_out_set_the_status_and_leave_the_context_usable(amq, form, cell, I, H, batch, kw, ka, late):
+    """late 1: nobody sees enough quantized vectors in step 0; late 2: nobody sees enough finished products in step 1."""
+    steps, gru = 3, cell == "gru"
+    Wcodes, Walpha = amq.quantize(dev(synth.normal(((3 if gru else 4) * H, I + H), 0.08, 85, 1)), kw, 2)
+    xs = dev(synth.normal((steps, batch, I), 1.0, 85, 2))
+    h0, c0 = dev(synth.uniform((batch, H), -1, 1, 85, 3)), None if gru else dev(synth.uniform((batch, H), -1, 1, 85, 4))
+    args = (Wcodes, Walpha, None, I, H, xs, h0, c0, ka, 2)
+    ws = amq.new_workspace(I, H, batch, ka)
+    want = amq.selftest_batched_sequence(*args, amq.new_workspace(I, H, batch, ka), form)
+    h_seq, h_last, c_last = amq.selftest_batched_sequence(*args, ws, form, late=late)
+    assert amq.workspace_status(ws) == TIMEOUT
+    assert torch.all(h_last == 0) and (gru or torch.all(c_last == 0))       # outputs untouched
+    if late == 2:
+        assert torch.equal(h_seq[0], want[0][0])                            # step 0 waits for nothing that is late
+    # the same workspace, the same stream, the next call: status cleared, results as from a fresh workspace (the tensor memory is free again)
+    got = amq.selftest_batched_sequence(*args, ws, form)
+    assert amq.workspace_status(ws) == 0
+    assert all(torch.equal(g, w) for g, w in zip(got, want) if w is not None)
+
+
+@pytest.mark.parametrize("late", [1, 2])
+@pytest.mark.parametrize("V,I,H", [(149, 33, 147), (3001, 96, 149), (42000, 1024, 1024)])
+def test_decoding_waits_that_run_out_set_the_status_and_leave_the_context_usable(amq, V, I, H, late):
+    steps, ka = 4, 2
+    q = lambda shape, std, seed: amq.quantize(dev(synth.normal(shape, std, 86, seed)), 2, 2)
+    We, Wi, Wh, Ws = q((V, I), 1.0, 1), q((4 * H, I), 0.2, 2), q((4 * H, H), 0.1, 3), q((V, H), 0.2, 4)
+    ws = amq.new_decode_workspace(V, I, H, 2, ka)
+
+    def start():
+        tokens = torch.full((steps + 1,), -7, dtype=torch.int32, device="cuda")
+        tokens[0] = V // 2
+        return tokens, torch.full((1, H), 0.25, device="cuda"), torch.zeros((1, H), device="cuda")
+
+    want, got, left = start(), start(), start()
+    call = lambda f, r, *more: f(*We, *Wi, *Wh, None, *Ws, None, I, H, ka, 2, *r, ws, *more)
+    call(amq.lm_greedy_decode, want)
+    assert amq.device_status() == 0
+    call(amq.selftest_decode_give_up, left, late)
+    assert amq.device_status() == TIMEOUT and amq.device_status() == 0      # (the read clears it)
+    assert all(torch.equal(a, b) for a, b in zip(left, start()))            # tokens and state as they were
+    call(amq.lm_greedy_decode, got)
+    assert amq.device_status() == 0
+    assert all(torch.equal(a, b) for a, b in zip(got, want))
+
+
 def test_give_up_selftest_rejects_what_it_cannot_run(amq):
     I, H, ka = 64, 48, 2
     Wcodes, Walpha = small_model(amq, I, H)
@@ -72,6 +131,12 @@ def test_give_up_selftest_rejects_what_it_cannot_run(amq):
     for bad_limit in (0, 1 << 20):
         with pytest.raises(amq.AmqError) as e:
             amq.selftest_sequence_give_up(Wcodes, Walpha, None, I, H, xs, h0, h0.clone(), ka, 2, ws, bad_limit)
+        assert e.value.status == -1
+    h1 = torch.zeros((9, H), device="cuda")
+    for form, late, counted, steps in ((0, 1, 0, 3), (1, 3, 0, 3), (2, 1, 5, 3), (2, 2, 0, 1)):
+        with pytest.raises(amq.AmqError) as e:
+            amq.selftest_batched_sequence(Wcodes, Walpha, None, I, H, torch.zeros((steps, 9, I), device="cuda"), h1, h1.clone(), ka, 2,
+                                          amq.new_workspace(I, H, 9, ka), form, counted, late)
         assert e.value.status == -1
     with pytest.raises(amq.AmqError) as e:      # a single step waits for nothing: refused
         amq.selftest_sequence_give_up(Wcodes, Walpha, None, I, H, xs[:1], h0, h0.clone(), ka, 2, ws, 100)
