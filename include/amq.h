@@ -333,6 +333,17 @@ AMQ_API amq_status amq_lm_greedy_decode(const uint32_t* We_codes, const float* W
                                 void* workspace, size_t workspace_bytes, void* stream);
 
 /*
+ * Test aid: which kernel amq_binary_gemm runs for batch >= 2 vectors on a device of `sm_count` SMs (0: the current device's; any other
+ * value needs no device): *form (HOST) 0 = CUDA cores, 1 = tensor cores with both operands streamed, 2 = tensor cores with the
+ * activations resident; clocks[0], clocks[1] (HOST): the estimates of forms 1 and 2 (0 where a form does not take the problem).
+ */
+AMQ_API amq_status amq_selftest_product_plan(int m, int n, int k_w, int k_a, int batch, int ldy, int sm_count, int* form, double* clocks);
+/* Test aid: amq_binary_gemm in form 1 or 2 whatever the library would choose; AMQ_ERR_UNSUPPORTED where it does not take the problem. */
+AMQ_API amq_status amq_selftest_binary_gemm(const uint32_t* Wcodes, const float* Walpha, int m, int n, int k_w,
+                                    const uint32_t* xcodes, const float* xbeta, int batch, int k_a,
+                                    const float* bias, float* y, int ldy, int form, void* stream);
+
+/*
  * Test aid for the give-up path of decoding in one launch: amq_lm_greedy_decode without log-probabilities, its CTAs looking for the words
  * of the state (late = 1) or of the shares' maxima (late = 2) where none of them writes.  In the first step every wait runs out (about a
  * second: the ordinary limit), every CTA records that in the device status word (amq_device_status) and returns; tokens, h and c are

@@ -65,6 +65,8 @@ EXPORTS = {
                                           ctypes.POINTER(ctypes.c_double)]),
     "amq_selftest_batched_sequence": (_int, [_vp, _vp, _vp, _int, _int, _int, _int, _vp, _int, _vp, _vp, _int, _int, _int,
                                              _vp, _vp, _vp, _vp, _sz, _int, _int, _int, _vp]),
+    "amq_selftest_product_plan": (_int, [_int, _int, _int, _int, _int, _int, _int, ctypes.POINTER(_int), ctypes.POINTER(ctypes.c_double)]),
+    "amq_selftest_binary_gemm": (_int, [_vp, _vp, _int, _int, _int, _vp, _vp, _int, _int, _vp, _vp, _int, _int, _vp]),
     "amq_selftest_decode_give_up": (_int, [_vp, _vp, _int, _int, _int, _vp, _vp, _vp, _vp, _vp, _int, _int, _vp, _vp, _vp, _int,
                                            _int, _int, _vp, _int, _vp, _vp, _vp, _sz, _int, _vp]),
     "amq_gru_original_workspace_bytes": (_sz, [_int, _int, _int, _int]),
@@ -278,6 +280,26 @@ def selftest_sequence_plan(gru, I, H, k_w, k_a, batch, sm_count=0, form=-1):
     f, split, clocks = _int(form), (_int * 3)(), ctypes.c_double(0.0)
     _check(_lib.amq_selftest_sequence_plan(int(gru), I, H, k_w, k_a, batch, sm_count, ctypes.byref(f), split, ctypes.byref(clocks)))
     return f.value, tuple(split), clocks.value
+
+
+def selftest_product_plan(m, n, k_w, k_a, batch, sm_count=0, ldy=None):
+    """Which kernel a product runs on (see amq.h): (form, (estimates of the streaming and of the resident form))."""
+    f, clocks = _int(0), (ctypes.c_double * 2)()
+    _check(_lib.amq_selftest_product_plan(m, n, k_w, k_a, batch, m if ldy is None else ldy, sm_count, ctypes.byref(f), clocks))
+    return f.value, tuple(clocks)
+
+
+PRODUCT_CUDA_CORES, PRODUCT_STREAMING, PRODUCT_RESIDENT = 0, 1, 2
+
+
+def selftest_binary_gemm(Wcodes, Walpha, xcodes, xbeta, n, form, bias=None, y=None):
+    """Test aid: binary_gemm on a given kernel (see amq.h)."""
+    m, k_w, _ = Wcodes.shape
+    batch, k_a, _ = xcodes.shape
+    y = _native.empty(Wcodes, 0, batch, m) if y is None else y
+    _check(_native.amq_selftest_binary_gemm(Wcodes, Walpha, m, n, k_w, xcodes, xbeta, batch, k_a, bias, y.data_ptr(),
+                                            y.stride(0) if batch > 1 else max(m, y.stride(0)), form))
+    return y
 
 
 def selftest_batched_sequence(Wcodes, Walpha, bias, I, H, x_seq, h0, c0, k_a, T, workspace, form, counted=0, late=0):

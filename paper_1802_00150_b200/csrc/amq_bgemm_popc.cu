@@ -201,11 +201,28 @@ bgemm_popc_kernel(PopcParams p)
 
 }  // namespace
 
+// Which product runs a call that the matrix-vector kernel does not take.  The resident form spends 9000 clocks more before its first
+// result (it expands whole vectors first) and less on every tile after: 4096 x 2048 at 2/2 bits, 64 vectors, 12.9 us against 10.9 in
+// the streaming form, 2752 columns and 13 vectors 16.9 against 8.7, 32768 x 1024 at 3/2 bits, 512 vectors, 61 against 111.  (Chosen
+// by the estimates the 376 products they were fitted to take 0.4 % longer than the better form of each, 23 % at worst; always the
+// resident form 15 %, 93 % at worst.  The factor is what ties were measured to be decided best by.)
+ProductForm gemm_form(const GemmArgs& a, int sms)
+{
+    const double resident = gemm_resident_clocks(a, sms);
+    if (resident > 0.0 && a.same_for_any_batch) return PRODUCT_RESIDENT;
+    const double streaming = gemm_tc_clocks(a, sms);
+    if (resident > 0.0 && (streaming == 0.0 || resident < 1.06 * streaming)) return PRODUCT_RESIDENT;
+    return streaming > 0.0 ? PRODUCT_STREAMING : PRODUCT_CUDA_CORES;
+}
+
 amq_status launch_binary_gemm(const GemmArgs& a, cudaStream_t st)
 {
     if (gemv_supported(a)) return launch_binary_gemv(a, st);
-    if (gemm_resident_supported(a)) return launch_binary_gemm_resident(a, st);
-    if (gemm_tc_supported(a)) return launch_binary_gemm_tc(a, st);
+    switch (gemm_form(a, 0)) {
+        case PRODUCT_RESIDENT: return launch_binary_gemm_resident(a, st);
+        case PRODUCT_STREAMING: return launch_binary_gemm_tc(a, st);
+        case PRODUCT_CUDA_CORES: break;
+    }
     PopcParams p;
     p.a = a;
     p.wpr = words_per_row(a.n);
@@ -227,6 +244,23 @@ amq_status launch_binary_gemm(const GemmArgs& a, cudaStream_t st)
     return AMQ_OK;
 }
 
+namespace {
+
+amq_status product_call(const uint32_t* Wcodes, const float* Walpha, int m, int n, int k_w, const uint32_t* xcodes, const float* xbeta,
+                        int batch, int k_a, const float* bias, float* y, int ldy, GemmArgs* out)
+{
+    if (!Wcodes || !Walpha || !xcodes || !xbeta || !y || m < 0 || batch < 0 || n < 1 || ldy < m) return AMQ_ERR_INVALID_ARG;
+    if (!valid_k(k_w) || !valid_k(k_a)) return AMQ_ERR_UNSUPPORTED;
+    if (!aligned16(Wcodes) || !aligned16(xcodes)) return AMQ_ERR_ALIGNMENT;
+    GemmArgs a{};
+    a.Wcodes = Wcodes; a.Walpha = Walpha; a.m = m; a.n = n; a.k_w = k_w;
+    a.xcodes = xcodes; a.xbeta = xbeta; a.batch = batch; a.k_a = k_a;
+    a.bias = bias; a.epilogue = EPI_Y; a.y = y; a.ldy = ldy;
+    *out = a;
+    return AMQ_OK;
+}
+
+}  // namespace
 }  // namespace amq
 
 extern "C" {
@@ -249,16 +283,35 @@ amq_status amq_binary_gemm(const uint32_t* Wcodes, const float* Walpha, int m, i
                            const uint32_t* xcodes, const float* xbeta, int batch, int k_a,
                            const float* bias, float* y, int ldy, void* stream)
 {
-    if (!Wcodes || !Walpha || !xcodes || !xbeta || !y || m < 0 || batch < 0 || n < 1 || ldy < m)
-        return AMQ_ERR_INVALID_ARG;
-    if (!amq::valid_k(k_w) || !amq::valid_k(k_a)) return AMQ_ERR_UNSUPPORTED;
-    if (!amq::aligned16(Wcodes) || !amq::aligned16(xcodes)) return AMQ_ERR_ALIGNMENT;
-    if (m == 0 || batch == 0) return AMQ_OK;
     amq::GemmArgs a{};
-    a.Wcodes = Wcodes; a.Walpha = Walpha; a.m = m; a.n = n; a.k_w = k_w;
-    a.xcodes = xcodes; a.xbeta = xbeta; a.batch = batch; a.k_a = k_a;
-    a.bias = bias; a.epilogue = amq::EPI_Y; a.y = y; a.ldy = ldy;
+    const amq_status s = amq::product_call(Wcodes, Walpha, m, n, k_w, xcodes, xbeta, batch, k_a, bias, y, ldy, &a);
+    if (s != AMQ_OK || m == 0 || batch == 0) return s;
     return amq::launch_binary_gemm(a, (cudaStream_t)stream);
+}
+
+amq_status amq_selftest_binary_gemm(const uint32_t* Wcodes, const float* Walpha, int m, int n, int k_w,
+                                    const uint32_t* xcodes, const float* xbeta, int batch, int k_a,
+                                    const float* bias, float* y, int ldy, int form, void* stream)
+{
+    amq::GemmArgs a{};
+    const amq_status s = amq::product_call(Wcodes, Walpha, m, n, k_w, xcodes, xbeta, batch, k_a, bias, y, ldy, &a);
+    if (s != AMQ_OK) return s;
+    if (form != amq::PRODUCT_STREAMING && form != amq::PRODUCT_RESIDENT) return AMQ_ERR_INVALID_ARG;
+    if (m == 0 || batch == 0) return AMQ_OK;
+    if ((form == amq::PRODUCT_RESIDENT ? amq::gemm_resident_clocks(a, 0) : amq::gemm_tc_clocks(a, 0)) == 0.0) return AMQ_ERR_UNSUPPORTED;
+    return form == amq::PRODUCT_RESIDENT ? amq::launch_binary_gemm_resident(a, (cudaStream_t)stream) : amq::launch_binary_gemm_tc(a, (cudaStream_t)stream);
+}
+
+amq_status amq_selftest_product_plan(int m, int n, int k_w, int k_a, int batch, int ldy, int sm_count, int* form, double* clocks)
+{
+    if (m < 1 || n < 1 || batch < 1 || ldy < m || sm_count < 0 || !form || !clocks) return AMQ_ERR_INVALID_ARG;
+    if (!amq::valid_k(k_w) || !amq::valid_k(k_a)) return AMQ_ERR_UNSUPPORTED;
+    amq::GemmArgs a{};
+    a.m = m; a.n = n; a.k_w = k_w; a.batch = batch; a.k_a = k_a; a.epilogue = amq::EPI_Y; a.ldy = ldy;
+    *form = amq::gemm_form(a, sm_count);
+    clocks[0] = amq::gemm_tc_clocks(a, sm_count);
+    clocks[1] = amq::gemm_resident_clocks(a, sm_count);
+    return AMQ_OK;
 }
 
 amq_status amq_device_status(void* stream)

@@ -213,10 +213,9 @@ bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
 
 struct ResGemmPlan { ResGemmParams a; int grid; size_t smem; };
 
-bool plan(const GemmArgs& g, ResGemmPlan* out)
+bool plan(const GemmArgs& g, int sms, ResGemmPlan* out)
 {
     if (g.epilogue != EPI_Y) return false;
-    const int sms = res_sm_count();
     ResGemmParams a{};
     ResProblem& p = a.p;
     p.W = g.Wcodes; p.Walpha = g.Walpha; p.k_w = g.k_w; p.wpr = words_per_row(g.n);
@@ -259,19 +258,24 @@ amq_status launch(const ResGemmPlan& pl, bool overlap, cudaStream_t st)
 
 }  // namespace
 
-bool gemm_resident_supported(const GemmArgs& g)
+double gemm_resident_clocks(const GemmArgs& g, int sms)
 {
     // from 16 vectors on always; for 2..15 vectors when the weight matrix is large enough that the CUDA-core kernel's tile loop
     // costs more than this kernel's set-up
+    if (sms < 1) sms = res_sm_count();
     ResGemmPlan pl;
     const bool big = (long long)g.m * g.k_w * words_per_row(g.n) >= (1ll << 17);
-    return (g.batch >= 16 || (g.batch >= 2 && big)) && plan(g, &pl);
+    if (!(g.batch >= 16 || (g.batch >= 2 && big)) || !plan(g, sms, &pl)) return 0.0;
+    const ResProblem& p = pl.a.p;
+    const double tiles = (double)(((long long)pl.a.blocks * pl.a.mtiles + sms - 1) / sms), passes = 1.0 + (tiles - 1.0) / pl.a.mtiles;
+    return passes * (16300.0 + 8.6 * p.N * p.NS) + 7.2 * p.k_w * p.NS +
+           tiles * (p.k_w * (0.96 * p.NS * res_slot_clocks(p) + 1.9 * p.N + 536.0) + (pl.a.vec_out ? 36.0 : 44.0) * p.TB);
 }
 
 amq_status launch_binary_gemm_resident(const GemmArgs& g, cudaStream_t st)
 {
     ResGemmPlan pl;
-    if (!plan(g, &pl)) return AMQ_ERR_UNSUPPORTED;
+    if (!plan(g, res_sm_count(), &pl)) return AMQ_ERR_UNSUPPORTED;
     amq_status s = tc_status_word(&pl.a.status);
     if (s != AMQ_OK) return s;
     switch (g.k_a) {

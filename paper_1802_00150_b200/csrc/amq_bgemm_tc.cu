@@ -1251,13 +1251,24 @@ amq_status launch_ka(const TcPlan& pl, cudaStream_t st)
 
 }  // namespace
 
-bool gemm_tc_supported(const GemmArgs& a)
+bool gemm_tc_supported(const GemmArgs& a, int sms)
 {
     // from 16 vectors on always; for 2..15 vectors (one padded tile of 16) when the weight matrix is large
     // enough that the CUDA-core kernel's tile loop costs more than this kernel's fixed ~10 us
     TcPlan pl;
     const bool big = (long long)a.m * a.k_w * words_per_row(a.n) >= (1ll << 17);
-    return (a.batch >= 16 || (a.batch >= 2 && big)) && plan(a, &pl);
+    return (a.batch >= 16 || (a.batch >= 2 && big)) && plan(a, &pl, sms);
+}
+
+double gemm_tc_clocks(const GemmArgs& a, int sms)
+{
+    if (sms < 1) sms = sm_count();
+    TcPlan pl;
+    if (!gemm_tc_supported(a, sms) || !plan(a, &pl, sms)) return 0.0;
+    const long long tiles = pl.persistent ? pl.p.ntiles : (long long)pl.grid.x * pl.grid.y, waves = (tiles + sms - 1) / sms * pl.p.MT;
+    const double N = pl.p.n_mma, steps = pl.p.steps;
+    return 7650.0 + waves * (3400.0 + steps * (360.0 + 1.5 * N) + (pl.persistent && pl.p.nbuf == 1 ? 9.1 : 7.6) * N + 13.6 * pl.p.TB) +
+           (pl.persistent ? 1790.0 + 466.0 * steps : 0.0) + 172.0 * steps + 7.4 * N;
 }
 
 double chain_clocks(const BatchedSequence& s, int sms)

@@ -95,7 +95,7 @@ PyObject* call(amq_status (*f)(A...), PyObject* const* args, Py_ssize_t nargs)
 #define AMQ_ENTRIES(X)                                                                                                          \
     X(amq_quantize) X(amq_pack) X(amq_unpack) X(amq_binary_dots) X(amq_binary_gemm) X(amq_quantized_gemv) X(amq_lstm_step)      \
     X(amq_lstm_step_static) X(amq_gru_step) X(amq_lstm_sequence) X(amq_gru_sequence) X(amq_lstm_sequence_host)                  \
-    X(amq_gru_sequence_host) X(amq_selftest_sequence_give_up) X(amq_selftest_batched_sequence) X(amq_selftest_decode_give_up)      \
+    X(amq_gru_sequence_host) X(amq_selftest_sequence_give_up) X(amq_selftest_batched_sequence) X(amq_selftest_decode_give_up) X(amq_selftest_binary_gemm) \
     X(amq_gru_step_original) X(amq_quantize_variant) X(amq_lm_greedy_decode) X(amq_log_softmax_argmax) X(amq_embedding_rows) X(amq_lstm_step_paper) X(amq_lstm_sequence_paper)
 
 #define AMQ_WRAP(name)                                                                          \

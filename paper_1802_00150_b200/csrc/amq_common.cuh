@@ -109,6 +109,9 @@ struct GemmArgs {
     // the launch may start while the previous kernel of the stream (the on-line quantizer that produces xcodes / xbeta)
     // still runs: the kernel sets itself up, fetches weights, and waits for that kernel before it reads anything else
     bool overlap_with_previous;
+    // EPI_Y: the result of a vector may not depend on how many others are in the call (the two tensor-core products differ in the order of
+    // their sums): the resident form wherever it covers the problem
+    bool same_for_any_batch;
 };
 
 // programmatic dependent launch (sm_90+): a kernel launched with the programmatic-serialization attribute may have its
@@ -158,13 +161,19 @@ amq_status launch_quantized_gemv(const uint32_t* Wcodes, const float* Walpha, in
 
 // Tensor-core kernel (tcgen05, batch >= 16): whether it covers a problem, its launch, and its status word
 // (nonzero after a bounded device-side wait ran out; cleared by the read).
-bool gemm_tc_supported(const GemmArgs& a);
+bool gemm_tc_supported(const GemmArgs& a, int sms = 0);
+// Estimated clocks of the two tensor-core products on `sms` SMs (0: those of the current device), 0 where one does not cover the problem:
+// fixed part, steps, epilogues.  Fitted to 376 products (1 to 4 bits, 2 to 2240 vectors, 64 to 65536 rows, lengths 64 to 8192) on a
+// B200, within 6 and 5 % (standard deviation; 21 and 19 % at worst).
+double gemm_resident_clocks(const GemmArgs& a, int sms);
+double gemm_tc_clocks(const GemmArgs& a, int sms);
+enum ProductForm { PRODUCT_CUDA_CORES = 0, PRODUCT_STREAMING = 1, PRODUCT_RESIDENT = 2 };
+ProductForm gemm_form(const GemmArgs& a, int sms);
 amq_status launch_binary_gemm_tc(const GemmArgs& a, cudaStream_t st);
 amq_status read_tc_status(cudaStream_t st, uint32_t* out);
 amq_status tc_status_word(uint32_t** word);       // device address of the status word, for kernels of other files
 
-// Tensor-core product with a resident activation operand (EPI_Y): whether it covers a problem, and its launch.
-bool gemm_resident_supported(const GemmArgs& a);
+// Tensor-core product with a resident activation operand (EPI_Y), and its launch.
 amq_status launch_binary_gemm_resident(const GemmArgs& a, cudaStream_t st);
 
 // Greedy decoding without log-probabilities: all tokens in one cooperative launch.  `exchange` (decode_exchange_bytes, 128-byte

@@ -52,6 +52,25 @@ def test_product_at_the_edges_of_its_tiles(amq, m, n, kw, ka, batch, offset):
     assert amq.device_status() == 0
 
 
+@pytest.mark.parametrize("m,n,kw,ka,batch,offset", [
+    (1, 1, 1, 1, 16, 0), (127, 255, 2, 2, 31, 0), (129, 257, 3, 3, 33, 1), (130, 8448, 1, 4, 17, 0), (4000, 512, 4, 1, 2, 3),
+    (300, 1000, 4, 4, 97, 2), (128, 256, 1, 2, 64, 0), (43, 1024, 3, 2, 128, 0), (20000, 130, 2, 2, 129, 0),
+])
+def test_both_tensor_core_products_at_the_edges_of_their_tiles(amq, m, n, kw, ka, batch, offset):
+    """The sizes above and those where the streaming form's tiles end, on either kernel, whichever the library takes.  Tolerance: k_w k_a
+    products of exact integers and fp32 coefficients, summed in fp32."""
+    Wc, Wa = quantized((m, n), 0.03, kw, 210 + m, 1)
+    Xc, Xb = quantized((batch, n), 1.0, ka, 210 + m, 2)
+    bias = synth.normal((m,), 0.1, 210 + m, 3)
+    ref = oracle.binary_gemm(Wc, Wa, Xc, Xb, n, bias.astype(np.float64))
+    for form in (amq.PRODUCT_STREAMING, amq.PRODUCT_RESIDENT):
+        out = torch.full((batch, m + offset + 2), 7.0, device="cuda")
+        amq.selftest_binary_gemm(cdev(Wc), dev(Wa), cdev(Xc), dev(Xb), n, form, bias=dev(bias), y=out[:, offset:offset + m])
+        assert np.abs(out[:, offset:offset + m].cpu().numpy() - ref).max() <= 1e-5 * (np.abs(ref).max() + 1), form
+        assert torch.all(out[:, :offset] == 7.0) and torch.all(out[:, offset + m:] == 7.0)
+    assert amq.device_status() == 0
+
+
 @pytest.mark.parametrize("cell,I,H,kw,ka,batch", [
     ("lstm", 1, 1, 1, 1, 2),            # the smallest
     ("lstm", 255, 33, 3, 2, 9),         # one short of a slot, one unit past a tile of 32, one vector past a block of 8

@@ -1,5 +1,5 @@
-"""How a batched sequence is cut up and which form of it runs, as the library decides it on the host (148 SMs, no device needed).  The times
-quoted were measured on a B200 for 35 timesteps."""
+"""How a batched sequence is cut up, which form of it and which product runs, as the library decides it on the host (148 SMs, no device
+needed).  The times quoted were measured on a B200, of sequences for 35 timesteps."""
 import pytest
 
 from paper_1802_00150_b200 import amq
@@ -80,3 +80,29 @@ def test_a_split_covers_the_problem_and_the_counters_cover_the_split():
         blocks = -(-batch // block)
         assert blocks * ctas <= sms and blocks <= -(-batch // 8) and warps in (4, 8, 16) and clocks > 0
         assert amq.selftest_sequence_plan(gru, I, H, kw, ka, batch, sms, form)[1:] == (split, clocks)
+
+
+@pytest.mark.parametrize("m,n,kw,ka,batch,streaming,resident", [
+    (4096, 2048, 3, 3, 64, 11.0, 14.9),
+    (6144, 4096, 2, 3, 256, 37.4, 37.5),
+    (32768, 1024, 3, 2, 512, 109.3, 60.1),
+    (9999, 650, 2, 2, 600, 33.3, 29.2),
+    (4096, 1024, 2, 2, 64, 8.3, 11.0),
+    (4096, 2048, 2, 2, 64, 9.8, 12.6),
+    (62364, 320, 3, 3, 3, 33.4, 14.9),
+    (61767, 1536, 3, 4, 815, 756.3, 334.6),
+    (42773, 192, 3, 4, 753, 364.7, 135.8),
+    (4275, 2096, 2, 3, 157, 12.9, 21.2),
+    (666, 128, 3, 2, 18, 6.7, 9.5),
+    (16078, 128, 4, 4, 469, 116.3, 48.1),
+    (768, 2752, 4, 2, 13, 8.7, 16.9),
+    (551, 7487, 4, 2, 15, 14.9, 27.1),
+    (1813, 7744, 4, 3, 26, 16.9, 29.2),
+])
+def test_the_product_taken_is_the_faster_measured_one_or_close_to_it(m, n, kw, ka, batch, streaming, resident):
+    """Times in us of the tensor-core product with both operands streamed and with resident activations."""
+    form, clocks = amq.selftest_product_plan(m, n, kw, ka, batch, SMS)
+    times = {amq.PRODUCT_STREAMING: streaming, amq.PRODUCT_RESIDENT: resident}
+    assert times[form] <= 1.06 * min(streaming, resident)
+    for c, t in zip(clocks, (streaming, resident)):
+        assert abs(c / 1965 - t) <= 0.21 * t                # (the worst of the fits)
