@@ -34,15 +34,15 @@ FALLBACK_HBM_GBS = 6650.0
 # DRAM bytes per launch of the dominant kernel from one ncu capture (dram__bytes_read.sum +
 # dram__bytes_write.sum), keyed by workload; the summaries are under profiles/.  None = not captured for the
 # kernel as it stands.
-NCU_TRAFFIC_BYTES = {"lstm1024_b1": 2422016 + 51968}    # rnn_persistent_kernel, profiles/rnn_persistent_kernel_lstm1024_b1.txt
-# the batched workloads time a chain of kernels; for their dominant kernel (the tensor-core product) the cold-cache ncu
-# captures under profiles/ give these DRAM bytes per launch (inside a sequence the packed weights stay in L2)
+NCU_TRAFFIC_BYTES = {
+    "lstm1024_b1": 2436096 + 30976,         # rnn_persistent_kernel, profiles/rnn_persistent_kernel_lstm1024_b1.txt
+    "lstm1024_b64": 12977920 + 18944,       # rnn_resident_kernel, profiles/rnn_resident_kernel_lstm1024_b64.txt (35 timesteps)
+    "gru2048_b256": 81945856 + 40538880,    # rnn_batched_kernel, profiles/rnn_batched_kernel_gru2048_b256.txt (35 timesteps)
+}
+# a pass of proj32768_b512 is three kernels; of the product, the cold-cache capture under profiles/ gives these bytes
 NCU_TRAFFIC_DOMINANT_KERNEL = {
-    "lstm1024_b64": {"kernel": "bgemm_tc_kernel", "bytes": 3586816, "summary": "profiles/bgemm_tc_kernel_lstm1024_b64.txt"},
-    "gru2048_b256": {"kernel": "bgemm_tc_persistent_kernel", "bytes": 8923136,
-                     "summary": "profiles/bgemm_tc_persistent_kernel_gru2048_b256.txt"},
-    "proj32768_b512": {"kernel": "bgemm_tc_persistent_kernel", "bytes": 13188352 + 10061568,
-                       "summary": "profiles/bgemm_tc_persistent_kernel_proj32768_b512.txt"},
+    "proj32768_b512": {"kernel": "bgemm_resident_kernel", "bytes": 14171904 + 12469248,
+                       "summary": "profiles/bgemm_resident_kernel_proj32768_b512.txt"},
 }
 # the same for the cold matrix-vector kernel on 131072 x 8192 at 2/2 bits (profiles/bgemv_kernel_131072x8192_k2k2.txt)
 NCU_TRAFFIC_GEMV_COLD_BYTES = 269500000
@@ -403,8 +403,11 @@ def run_ours(args, wl):
             kernel_name = "bulk quantize + binary GEMM (whole step)"
         else:
             alg_bytes = algorithmic_bytes_per_timestep(wl) * wl.steps
-            kernel_name = ("rnn_persistent_kernel (one launch = the whole sequence)" if wl.batch == 1
-                           else "chain of quantize_kernel + bgemm_tc_kernel per timestep")
+            kernel_name = "rnn_persistent_kernel (one launch = the whole sequence)"
+            if wl.batch > 1:
+                kernel_name = ("chain of quantize_kernel + bgemm_tc_kernel per timestep", "rnn_batched_kernel (one launch = the whole sequence)",
+                               "rnn_resident_kernel (one launch = the whole sequence)")[
+                    amq.selftest_sequence_plan(wl.cell == "gru", wl.I, wl.H, wl.k_w, wl.k_a, wl.batch)[0]]
         achieved = alg_bytes / (step_ms * 1e-3) / 1e9
         line = {
             "metric": METRIC, "value": value, "unit": unit, "n_gpus": world, "steps": args.steps,
@@ -756,8 +759,8 @@ def quality_line(amq, torch, dev):
 
 def greedy_decoding_line(amq, torch, dev):
     """Language-model decoding at the scale of the paper's largest vocabulary (42000 words, hidden 1024, 2/2 bits),
-    one sequence, the arg-max fed back on the device: amq_lm_greedy_decode enqueues, per token, embedding row ->
-    paper-form cell -> output product with the on-line quantizer of h inside -> log-softmax / arg-max (six launches)."""
+    one sequence, the arg-max fed back on the device: amq_lm_greedy_decode runs embedding row -> paper-form cell ->
+    quantizer of h -> output product -> arg-max for all tokens in one launch (decode_persistent_kernel)."""
     I = H = 1024
     V, k, ntok = 42000, 2, 64
     g = torch.Generator(device=dev)
@@ -780,7 +783,7 @@ def greedy_decoding_line(amq, torch, dev):
     ms = _burst_ms(torch, run, 5)
     extra = {}
     try:
-        # the same chain (7 launches per token) captured once in a CUDA graph and replayed
+        # the same call captured once in a CUDA graph and replayed
         side = torch.cuda.Stream()
         side.wait_stream(torch.cuda.current_stream())
         graph = torch.cuda.CUDAGraph()
@@ -794,7 +797,7 @@ def greedy_decoding_line(amq, torch, dev):
     except Exception as exc:
         extra = {"graph_replay_error": str(exc)[:120]}
     return {**extra, "workload": "greedy decoding, vocabulary %d, I=H=%d, 2/2 bits, one sequence, %d tokens per call (embedding row, "
-                        "paper-form cell, quantize(h), output product, log-softmax/arg-max; token fed back on the device)" % (
+                        "paper-form cell, quantize(h), output product, arg-max; token fed back on the device; one launch per call)" % (
                             V, H, ntok),
             "ms": ms, "bound": "latency", "us_per_token": 1e3 * ms / ntok, "tokens_per_s": ntok * 1e3 / ms,
             "distinct_tokens": int(torch.unique(tokens).numel())}
