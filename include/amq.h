@@ -125,7 +125,8 @@ AMQ_API amq_status amq_binary_dots(const uint32_t* Wcodes, int m, int n, int k_w
  * form of Fig. 3, right, for batch > 1):
  *   y[b][r] = sum_i sum_j Walpha[r][i] * xbeta[b][j] * D[b][r][i][j] + bias[r].
  * Walpha [m][k_w], xbeta [batch][k_a], bias [m] or NULL, y [batch][ldy] fp32 out, ldy >= m.
- * The integer partials are exact; the combination is fp32.
+ * The integer partials are exact; the combination is fp32, in an order that depends on the kernel, which is chosen by the sizes
+ * (batch included): results repeat bit for bit for the same sizes, and agree to fp32 rounding between different batches.
  * Wcodes and xcodes must be 16-byte aligned (AMQ_ERR_ALIGNMENT otherwise).  From 16 vectors on the product runs on
  * the tensor cores; its kernels fetch 32 bytes of a packed row at a time where the row starts on a 32-byte boundary
  * (a 32-byte aligned base with an even number of 128-element chunks per row, as torch allocations give for
@@ -229,6 +230,11 @@ AMQ_API amq_status amq_gru_step(const uint32_t* Wcodes, const float* Walpha, con
  * `steps` consecutive steps without returning to the host (step t+1 consumes h_t, so a sequence is one
  * dependency chain: Sec. 1).  x_seq [steps][batch][I]; h0, c0 [batch][H];
  * h_seq [steps][batch][H] out or NULL; h_last, c_last [batch][H] out.  Outputs must not alias inputs.
+ *
+ * How a batch runs (one launch with the weights in tensor memory, one launch with the weights streamed, or launches per step) and how many
+ * threads quantize a vector follow from the sizes, batch and bits, not from `steps`: results repeat bit for bit, and a sequence, its
+ * steps one by one and the *_host calls give the same bits for the same batch.  A sequence that runs in another batch size may
+ * differ in the last bits of the quantizer's fp32 sums, and so an element that lies on a decision boundary may take the other code.
  */
 AMQ_API amq_status amq_lstm_sequence(const uint32_t* Wcodes, const float* Walpha, const float* bias,
                              int I, int H, int k_w,
@@ -312,8 +318,9 @@ AMQ_API amq_status amq_log_softmax_argmax(const float* logits, int rows, int n, 
                                   float* logp, int ldp, int32_t* argmax, void* stream);
 
 /*
- * Greedy decoding with the language model of Eq. 6, one sequence, enqueued as one chain on `stream` (six or seven kernel
- * launches per token, no host round trip).  For t = 0 .. steps-1:
+ * Greedy decoding with the language model of Eq. 6, one sequence, no host round trip: one kernel launch for all tokens when no
+ * log-probabilities are asked for, H <= 2048 and the gate rows fit shared memory, else a chain of six or seven launches per
+ * token (the same tokens and states, bit for bit).  For t = 0 .. steps-1:
  *   x_t = row tokens[t] of the quantized embedding (We_codes [vocab][k_e][wpr(I)], We_alpha [vocab][k_e]);
  *   (h, c) <- LSTM step in the paper's own form (W_i [4H x I], W_h [4H x H], k_w bits, bias [4H] or NULL; h quantized
  *   on-line with k_a bits and T alternating rounds);
