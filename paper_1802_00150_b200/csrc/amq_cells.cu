@@ -1,6 +1,7 @@
-// Quantized LSTM / GRU steps and sequences (Eq. 6; on-line quantization of the activation, Sec. 4):
-// each step is the row quantizer on z = [x ; h] followed by the binary product with the fused gate
-// epilogue.  No step returns to the host; a sequence is enqueued as one chain on the caller's stream.
+// Quantized LSTM / GRU steps and sequences (Eq. 6; on-line quantization of the activation, Sec. 4): each step is the row
+// quantizer on z = [x ; h] followed by the binary product with the gates behind it.  No step returns to the host.  One sequence
+// runs in one launch (amq_rnn_persistent.cu), a batch in one launch (amq_rnn_resident.cu, amq_rnn_batched.cu) or as a chain of two
+// launches per step on the caller's stream.
 #include "amq_common.cuh"
 
 #include <cuda.h>

@@ -5,8 +5,9 @@
 //
 // Because x_t does not depend on the recurrent state, the input projections W_i x_t + b of ALL timesteps of
 // a sequence are one batched binary product (steps * batch vectors) done before the time loop; a timestep
-// is then the on-line quantizer on h (H columns instead of I + H) and the product with W_h, whose epilogue
-// adds the precomputed projection and applies the gates.
+// is then the on-line quantizer on h (H columns instead of I + H) and the product with W_h, behind which the
+// precomputed projection is added and the gates are applied: a batch in one launch for all timesteps or as a chain
+// of two launches per step, as for the stacked form; one sequence as a chain.
 #include "amq_common.cuh"
 
 namespace amq {

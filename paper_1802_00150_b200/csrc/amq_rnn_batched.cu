@@ -6,12 +6,15 @@
 // gate rows (amq_resident.cuh) with the gates in the epilogue, wait for the other CTAs' h.  The two waits are counters in the
 // workspace, one pair per block of vectors: blocks never wait for one another.
 //
-// This is the form for weights that do not fit tensor memory (amq_rnn_resident.cu takes those that do).
+// This is the form for weights that do not fit tensor memory, and for those that do where amq_rnn_resident.cu would need many passes of a few
+// vectors over them; the two and the chain of launches compete on their estimated time (batched_sequence_form below).
 //
 // Against a quantizer launch and a product launch per timestep this takes out two launches (some 6 us of host time each on this
 // machine, which had become longer than the kernels), the set-up of tensor memory and barriers, and the repeated expansion
 // of the activation planes by every tile of weight rows.  What bounds a timestep now: the steps of the weight pipeline (240-300
-// clocks per 256 bit positions of 128 plane-rows), the quantizer's chain of reductions, and the two waits.
+// clocks per 256 bit positions of 128 plane-rows), the quantizer's chain of reductions, and the two waits (GRU 2048, 256 sequences,
+// 2/3 bits, clocks of a timestep: wait for h 1650, quantizer 12200, publish and wait for planes 2700, expansion of the activations
+// 8700, weights 42900, last epilogue 4500, publish 1650).
 #include "amq_resident.cuh"
 #include "amq_sequence.cuh"
 
