@@ -1,8 +1,18 @@
 """How a batched sequence is cut up, which form of it and which product runs, as the library decides it on the host (148 SMs, no device
 needed).  The times quoted were measured on a B200, of sequences for 35 timesteps."""
+import os
+import shutil
+
 import pytest
 
-from paper_1802_00150_b200 import amq
+from paper_1802_00150_b200 import build
+
+if not (os.path.exists(build.LIB) and os.path.exists(build.BINDING)):
+    if shutil.which("nvcc") is None:
+        pytest.skip("library not built and nvcc not available", allow_module_level=True)
+    build.build()
+
+from paper_1802_00150_b200 import amq  # noqa: E402
 
 SMS = 148
 
