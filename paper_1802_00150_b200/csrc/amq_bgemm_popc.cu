@@ -201,17 +201,16 @@ bgemm_popc_kernel(PopcParams p)
 
 }  // namespace
 
-// Which product runs a call that the matrix-vector kernel does not take.  The resident form spends 9000 clocks more before its first
-// result (it expands whole vectors first) and less on every tile after: 4096 x 2048 at 2/2 bits, 64 vectors, 12.9 us against 10.9 in
-// the streaming form, 2752 columns and 13 vectors 16.9 against 8.7, 32768 x 1024 at 3/2 bits, 512 vectors, 61 against 111.  (Chosen
-// by the estimates the 376 products they were fitted to take 0.4 % longer than the better form of each, 23 % at worst; always the
-// resident form 15 %, 93 % at worst.  The factor is what ties were measured to be decided best by.)
+// Which product runs a call that the matrix-vector kernel does not take.  The resident form spends some 9000 clocks more before its first
+// result (it expands whole vectors first) and less on every tile after: 2048 x 256 at 2/2 bits, 1024 vectors, 14.7 us against 14.1 in
+// the streaming form, 32768 x 1024 at 3/2 bits, 512 vectors, 53.5 against 109.  (Chosen by the estimates the 376 products they
+// were fitted to take 0.1 % longer than the better form of each, 10 % at worst; always the resident form 14 %, 97 % at worst.)
 ProductForm gemm_form(const GemmArgs& a, int sms)
 {
     const double resident = gemm_resident_clocks(a, sms);
     if (resident > 0.0 && a.same_for_any_batch) return PRODUCT_RESIDENT;
     const double streaming = gemm_tc_clocks(a, sms);
-    if (resident > 0.0 && (streaming == 0.0 || resident < 1.06 * streaming)) return PRODUCT_RESIDENT;
+    if (resident > 0.0 && (streaming == 0.0 || resident < 1.02 * streaming)) return PRODUCT_RESIDENT;
     return streaming > 0.0 ? PRODUCT_STREAMING : PRODUCT_CUDA_CORES;
 }
 

@@ -2,8 +2,11 @@
 // (amq_resident.cuh).  One CTA per SM; the work is the list of (block of vectors, tile of 128 weight rows) pairs, dealt out in
 // equal contiguous shares, so that a CTA expands the activation operand once or twice and streams weight tiles past it.
 //
-// What bounds it: the pace of the pipeline steps (240-265 clocks per 256 bit positions of 128 plane-rows) times the number of
-// blocks the batch is cut into; outputs leave through shared memory as 128-byte stores of consecutive rows.
+// What bounds it: per tile of 128 rows (32768 x 1024, 512 vectors, 3/2 bits: some 5500 clocks, 3080 of them the tensor pipe's) the chain
+// commit - poll - barrier - read - release of every accumulator, and the issue slots that the roles share with the warp that issues the
+// MMAs.  That product took 59.8 us with a constant of every operand row added back in the epilogue (twice the instructions, and its
+// loads kept the load/store unit busy) and the polling warp on the issuing warp's scheduler; 53.5 us now.  Outputs leave through shared
+// memory as 16-byte pieces.
 #include "amq_resident.cuh"
 
 namespace amq {
@@ -16,7 +19,6 @@ struct ResGemmParams {
     float* y; int ldy;
     int mtiles, blocks;         // tiles of 128 rows, blocks of TB vectors
     int b_bytes;                // expanded activation operand
-    int vec_out;                // rows of y start on 16 bytes
     uint32_t* status;           // set when a bounded wait ran out
 };
 
@@ -27,7 +29,10 @@ __host__ __device__ constexpr int res_ng(int k_a) { return k_a <= 2 ? 2 : 1; }
 
 using R = ResRoles<3, 16, 3>;
 
-template <int KA>
+// VEC: every row of the result starts on 16 bytes.  (Two kernels, not two paths in one: the registers and instructions of all the roles of a
+// kernel of 1024 threads count for each role.  Without VEC a thread stores its four rows one by one; contiguous 128-byte stores, or
+// 16-byte pieces shifted against the rows, were slower at most sizes: up to 35 % for rows of 2000 and more.)
+template <int KA, bool VEC>
 __global__ void __launch_bounds__(R::THREADS, 1)
 bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
 {
@@ -36,9 +41,7 @@ bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
     constexpr int NG = res_ng(KA);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     float* sBeta = reinterpret_cast<float*>(smem_raw + a.b_bytes);                  // [256] per operand row
-    float* sRow = sBeta + 256;                                                      // [3][256]
-    int* sSum = reinterpret_cast<int*>(sRow + 3 * 256);                             // [2][256]
-    float* sAlpha = reinterpret_cast<float*>(sSum + 2 * 256);                       // [2][k_w][128]
+    float* sAlpha = sBeta + 256;                                                    // [2][4][128]
     uint32_t* table = reinterpret_cast<uint32_t*>(sAlpha + 2 * AMQ_MAX_K * 128);
     float* sY = reinterpret_cast<float*>(table + RES_TABLE);                        // [TB][Y_LD] results of a tile
     ResSync& sy = *reinterpret_cast<ResSync*>(sY + p.TB * Y_LD);
@@ -63,9 +66,8 @@ bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = __shfl_sync(0xffffffffu, sy.tmem_slot, 0);
-    if (warp < 4) res_write_scales(p, tmem, warp);
+    if (warp < 4) write_unit_scales(tmem, p.ring * p.N, warp);
 
-    for (int q = tid; q < 512; q += R::THREADS) sSum[q] = 0;
     res_fill_table(p, table);
     __syncthreads();
 
@@ -76,7 +78,7 @@ bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
             const int b = b0 + res_row_vector<KA>(q), j = res_row_plane<KA>(q);
             sBeta[q] = q < p.TB * KA && b < p.batch ? __ldcg(a.xbeta + (size_t)b * KA + j) : 0.0f;
         }
-        res_expand_activations<KA>(p, a.xcodes, b0, sB, sSum);
+        res_expand_activations<KA, 1>(p, a.xcodes, b0, sB);
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -125,20 +127,21 @@ bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
         };
         grid_dependency_wait();
         while (w < w_end) {
-            const int bb = (int)(w / a.mtiles), tile0 = (int)(w % a.mtiles), tiles = pass_tiles(w);
+            const int bb = (int)(w / a.mtiles), b0 = bb * p.TB, tile0 = (int)(w % a.mtiles), tiles = pass_tiles(w);
             float next_alpha = alpha_of(tile0);
             load_block(bb);
-            res_row_constants<R>(p, sSum, sRow);
+            f32x2 beta[NG][KA];
+            res_load_beta<R, KA, NG>(p, sBeta, sub, beta);
             for (int t = 0; t < tiles; ++t) {
                 float* sa = sAlpha + (t & 1) * AMQ_MAX_K * 128;
                 sa[te] = next_alpha;
                 if (res_epi_bar<R>(!ok)) { ok = false; break; }        // (also: everybody is past the tile before last, whose buffer this is)
                 if (t + 1 < tiles) next_alpha = alpha_of(tile0 + t + 1);
                 f32x2 y[NG][4];
-                ok = res_drain_tile<R, KA, NG>(p, sy, sa, quarter, sub, tmem, sBeta, sRow, drain, y);
+                ok = res_drain_tile<R, KA, NG>(p, sy, sa, quarter, sub, tmem, beta, drain, y);
                 // Results leave through shared memory and three warps of their own: in this layout a store from the registers is four
                 // 32-byte pieces, and stores from the epilogue warps held them up for longer than a tile's MMAs take.
-                ok = ok && res_group_wait(sy, smem_u32(&sy.yempty), y_parity, warp == R::EXP_WARPS, 1, 32 * R::EPI_WARPS);
+                if (ok && !__all_sync(0xffffffffu, mbar_wait(smem_u32(&sy.yempty), y_parity))) { *(volatile int*)&sy.failed = 1; ok = false; }
                 y_parity ^= 1u;
 #pragma unroll
                 for (int g = 0; g < NG; ++g) {
@@ -177,7 +180,7 @@ bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
                 ok = __all_sync(0xffffffffu, mbar_wait_relaxed(smem_u32(&sy.yfull), y_parity, &sy.failed));
                 y_parity ^= 1u;
                 if (!ok) { *(volatile int*)&sy.failed = 1; break; }
-                const bool vec = a.vec_out && row + 3 < p.units;
+                const bool vec = VEC && row + 3 < p.units;
 #pragma unroll 4
                 for (int e = warp - R::MMA_WARP - 1; e < last; e += R::OUT_WARPS) {
                     float4 v = *reinterpret_cast<const float4*>(sY + e * Y_LD + 4 * lane);
@@ -211,7 +214,7 @@ bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"((uint32_t)RES_TMEM_COLS) : "memory");
 }
 
-struct ResGemmPlan { ResGemmParams a; int grid; size_t smem; };
+struct ResGemmPlan { ResGemmParams a; int grid; size_t smem; bool vec_out; };
 
 bool plan(const GemmArgs& g, int sms, ResGemmPlan* out)
 {
@@ -241,7 +244,7 @@ bool plan(const GemmArgs& g, int sms, ResGemmPlan* out)
     const long long total = (long long)a.blocks * a.mtiles;
     out->grid = (int)(total < sms ? total : sms);
     out->smem = res_smem_bytes(a.p) + (size_t)a.p.TB * Y_LD * 4;
-    a.vec_out = (reinterpret_cast<uintptr_t>(g.y) & 15) == 0 && g.ldy % 4 == 0;
+    out->vec_out = (reinterpret_cast<uintptr_t>(g.y) & 15) == 0 && g.ldy % 4 == 0;
     out->a = a;
     return true;
 }
@@ -249,7 +252,7 @@ bool plan(const GemmArgs& g, int sms, ResGemmPlan* out)
 template <int KA>
 amq_status launch(const ResGemmPlan& pl, bool overlap, cudaStream_t st)
 {
-    auto kernel = bgemm_resident_kernel<KA>;
+    auto kernel = pl.vec_out ? bgemm_resident_kernel<KA, true> : bgemm_resident_kernel<KA, false>;
     AMQ_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem));
     AMQ_CUDA_TRY(launch_kernel(kernel, dim3((unsigned)pl.grid), dim3(R::THREADS), pl.smem, st, overlap, pl.a));
     AMQ_LAUNCH_CHECK();
@@ -268,8 +271,8 @@ double gemm_resident_clocks(const GemmArgs& g, int sms)
     if (!(g.batch >= 16 || (g.batch >= 2 && big)) || !plan(g, sms, &pl)) return 0.0;
     const ResProblem& p = pl.a.p;
     const double tiles = (double)(((long long)pl.a.blocks * pl.a.mtiles + sms - 1) / sms), passes = 1.0 + (tiles - 1.0) / pl.a.mtiles;
-    return passes * (16300.0 + 8.6 * p.N * p.NS) + 7.2 * p.k_w * p.NS +
-           tiles * (p.k_w * (0.96 * p.NS * res_slot_clocks(p) + 1.9 * p.N + 536.0) + (pl.a.vec_out ? 36.0 : 44.0) * p.TB);
+    return passes * (15600.0 + 7.4 * p.N * p.NS) + 23.8 * p.k_w * p.NS +
+           tiles * (p.k_w * (1.11 * p.NS * res_slot_clocks(p) + 0.3 * p.N + 607.0) + 31.0 * p.TB);
 }
 
 amq_status launch_binary_gemm_resident(const GemmArgs& g, cudaStream_t st)

@@ -13,12 +13,10 @@
 // and lanes store consecutive rows.  (The former layout, k_w plane-rows side by side, needed a pass through shared memory per
 // tile that took longer than the tile's MMAs.)
 //
-// Nibbles.  Output word s of a packed word keeps its bits s, s + 4, .., s + 28.  With bit 1 = -1 on both operands (a dot
-// product of +-1 vectors does not see the common sign), a weight bit needs no shift at all: nibble 0x1, 0x2 or 0x4 for s = 0, 1,
-// 2 is {0, 0.5}, {0, 1} or {0, 2}, which the block scales 4, 2, 1 (32 elements of one s) make {0, 2}; for s = 3 the bit is the
-// sign of 1.0.  The activation operand is b = +-1 for s = 3 and -b for s < 3, so the accumulator is the +-1 dot product minus
-// sum_{s < 3} b, a constant of the operand row that the epilogue adds back before anything is rounded.  Four logic
-// operations per packed word instead of seven: the expanders share the issue slots with the epilogue.
+// Nibbles.  Output word s of a packed word keeps its bits s, s + 4, .., s + 28, as the sign of 1.0 on both operands (bit 1 = -1: a dot
+// product of +-1 vectors does not see the common sign).  A shift and one logic operation per word.  (Weight nibbles that keep the bits
+// in place, {0, 2} by block scales, save the shifts but make the accumulator the dot product less a constant of the operand row: the
+// epilogue, which is the busiest role, had to add it back, and the expansion of the activations to count it.)
 //
 // Along K the vector is cut into slots of 256 positions (128 bytes of every expanded row, 128-byte swizzle: eight rows per 1024
 // bytes).  For the GRU, whose candidate keeps the columns [0, I) and [I, n) apart, the slot that holds column I exists twice,
@@ -39,17 +37,18 @@
 namespace amq {
 
 // Roles of a CTA: groups of four expander warps (which take the pipeline steps in turn), epilogue warps (lane quarter = warp mod 4,
-// SPLIT warps per quarter, groups of eight vectors in turn), one warp that issues the MMAs, others.
+// SPLIT warps per quarter, groups of eight vectors in turn), one warp that issues the MMAs, others.  The epilogue warp
+// that polls for its group is on another scheduler than the issuing warp.
 template <int GROUPS_, int EPI_WARPS_, int OUT_WARPS_>
 struct ResRoles {
     static constexpr int GROUPS = GROUPS_, EXP_WARPS = 4 * GROUPS_, EPI_WARPS = EPI_WARPS_, SPLIT = EPI_WARPS_ / 4,
-                         MMA_WARP = EXP_WARPS + EPI_WARPS, OUT_WARPS = OUT_WARPS_, THREADS = 32 * (MMA_WARP + 1 + OUT_WARPS_);
+                         MMA_WARP = EXP_WARPS + EPI_WARPS, POLL_WARP = EXP_WARPS + 1, OUT_WARPS = OUT_WARPS_, THREADS = 32 * (MMA_WARP + 1 + OUT_WARPS_);
 };
 constexpr int RES_STAGE_COLS = 64;                  // tensor-memory columns of a stage: two slots of the weight operand
 constexpr int RES_MAX_STAGES = 4;
 constexpr int RES_MAX_RING = 2;                     // accumulator buffers
 constexpr int RES_TMEM_COLS = 512;
-constexpr int RES_ROW_BYTES = (256 + 3 * 256 + 2 * 256) * 4;    // per operand row: coefficient, constants as fp32, as they are summed up
+constexpr int RES_ROW_BYTES = 256 * 4;              // coefficient of an operand row
 constexpr int RES_ALPHA_BYTES = 2 * AMQ_MAX_K * 128 * 4;         // weight coefficients of a tile, double-buffered
 constexpr int RES_SMEM_LIMIT = 225 * 1024;
 
@@ -127,12 +126,23 @@ __device__ __forceinline__ bool res_group_wait(ResSync& sy, uint32_t bar, uint32
 // bits n .. 31 (all of them for n <= 0, none for n >= 32)
 __device__ __forceinline__ uint32_t upper_bits(int n) { return n >= 32 ? 0u : 0xffffffffu << (n < 0 ? 0 : n); }
 
-// 256 bit positions of one packed row -> the 128 nibble bytes of operand row `row` in one slot.  `lo`, `hi`: valid element range.
-// Returns sum of b over the valid positions with s < 3 (bit 1 = -1).
-__device__ __forceinline__ int res_expand_row(uint32_t slot_addr, int row, const uint32_t (&w)[8], int first, int lo, int hi)
+// 256 bit positions of one packed row -> the 128 nibble bytes of operand row `row` in one slot.  `lo`, `hi`: valid element range; whole
+// slots inside it need no masks.
+__device__ __forceinline__ void res_expand_row(uint32_t slot_addr, int row, const uint32_t (&w)[8], int first, int lo, int hi)
 {
     const uint32_t base = slot_addr + (uint32_t)row * 128u;
-    int sum = 0;
+    if (lo <= first && first + 256 <= hi) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                uint32_t y[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) y[q] = ((w[4 * h + q] << (3 - s)) & 0x88888888u) | 0x22222222u;
+                st_shared_v4(base + (uint32_t)(((4 * h + s) ^ (row & 7)) << 4), y[0], y[1], y[2], y[3]);
+            }
+        return;
+    }
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         uint32_t vm[4];
@@ -141,69 +151,61 @@ __device__ __forceinline__ int res_expand_row(uint32_t slot_addr, int row, const
             const int e = first + 32 * (4 * h + q);
             // bits of the word inside [lo, hi): everything from lo - e up, less everything from hi - e up
             vm[q] = upper_bits(lo - e) & ~upper_bits(hi - e);
-            const uint32_t m3 = vm[q] & 0x77777777u;
-            sum += __popc(m3) - 2 * __popc(w[4 * h + q] & m3);
         }
 #pragma unroll 1
         for (int s = 0; s < 4; ++s) {
-            const uint32_t flip = s < 3 ? 0xAAAAAAAAu : 0x22222222u;        // s < 3: -b (bit 1 -> +1); s = 3: b
             uint32_t y[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q)
-                y[q] = (((w[4 * h + q] << (3 - s)) & 0x88888888u) ^ flip) & (((vm[q] >> s) & 0x11111111u) * 15u);      // nibble i: bit 4 i + s
+                y[q] = (((w[4 * h + q] << (3 - s)) & 0x88888888u) | 0x22222222u) & (((vm[q] >> s) & 0x11111111u) * 15u);       // nibble i: bit 4 i + s
             st_shared_v4(base + (uint32_t)(((4 * h + s) ^ (row & 7)) << 4), y[0], y[1], y[2], y[3]);
         }
     }
-    return sum;
 }
 
 // operand row -> (vector of the block, plane): rows of a group of eight vectors are plane-major
 template <int KA> __device__ __forceinline__ int res_row_vector(int row) { return row / (8 * KA) * 8 + (row & 7); }
 template <int KA> __device__ __forceinline__ int res_row_plane(int row) { return row / 8 % KA; }
 
-// Expand the planes of vectors b0 .. b0 + TB - 1 (all threads of the CTA; rows past the batch are zero nibbles), add up the
-// constants of the rows (sSum[part][row], zeroed by the caller; part 1: the h part of a GRU's split).  The caller makes the stores
-// visible to the MMAs: every thread executes the proxy fence at the end, then a CTA barrier.
-template <int KA>
-__device__ __forceinline__ void res_expand_activations(const ResProblem& p, const uint32_t* xcodes, int b0, uint32_t sB, int* sSum)
+// Expand the planes of vectors b0 .. b0 + TB - 1 (all threads of the CTA; rows past the batch are zero nibbles).  The caller makes the
+// stores visible to the MMAs: every thread executes the proxy fence at the end, then a CTA barrier.  AHEAD (row, slot) pairs at a time:
+// their loads overlap.
+template <int KA, int AHEAD>
+__device__ __forceinline__ void res_expand_activations(const ResProblem& p, const uint32_t* xcodes, int b0, uint32_t sB)
 {
     const int N = p.N;
     int row = (int)threadIdx.x % N, slot = (int)threadIdx.x / N;
     const int drow = (int)blockDim.x % N, dslot = (int)blockDim.x / N;
 #pragma unroll 1
     while (slot < p.NS) {
-        const int b = b0 + res_row_vector<KA>(row), j = res_row_plane<KA>(row);
-        const int w0 = res_slot_word(p, slot);
-        const bool in_x = slot < p.nx;
-        uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        const bool live = row < p.TB * KA && b < p.batch;
-        if (live) {
-            const uint4* src = reinterpret_cast<const uint4*>(xcodes + ((size_t)b * KA + j) * p.wpr + w0);
-            const uint4 v0 = __ldcg(src);               // (other SMs wrote the planes: not through the read-only path)
-            w[0] = v0.x; w[1] = v0.y; w[2] = v0.z; w[3] = v0.w;
-            if (w0 + 4 < p.wpr) { const uint4 v1 = __ldcg(src + 1); w[4] = v1.x; w[5] = v1.y; w[6] = v1.z; w[7] = v1.w; }
+        uint32_t w[AHEAD][8];
+        int rows[AHEAD], slots[AHEAD];
+        bool live[AHEAD];
+#pragma unroll
+        for (int a = 0; a < AHEAD; ++a) {
+            const int b = b0 + res_row_vector<KA>(row), j = res_row_plane<KA>(row), w0 = res_slot_word(p, slot < p.NS ? slot : 0);
+            rows[a] = row; slots[a] = slot;
+            live[a] = slot < p.NS && row < p.TB * KA && b < p.batch;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) w[a][q] = 0;
+            if (live[a]) {
+                const uint4* src = reinterpret_cast<const uint4*>(xcodes + ((size_t)b * KA + j) * p.wpr + w0);
+                const uint4 v0 = __ldcg(src);               // (other SMs wrote the planes: not through the read-only path)
+                w[a][0] = v0.x; w[a][1] = v0.y; w[a][2] = v0.z; w[a][3] = v0.w;
+                if (w0 + 4 < p.wpr) { const uint4 v1 = __ldcg(src + 1); w[a][4] = v1.x; w[a][5] = v1.y; w[a][6] = v1.z; w[a][7] = v1.w; }
+            }
+            row += drow; slot += dslot;
+            if (row >= N) { row -= N; ++slot; }
         }
-        const int lo = (p.nx > 0 && !in_x) ? p.I : 0, hi = !live ? 0 : (in_x ? p.I : p.n);
-        const int sum = res_expand_row(sB + (uint32_t)(slot * N * 128), row, w, w0 * 32, live ? lo : 0, hi);
-        if (live) atomicAdd(&sSum[(p.nx > 0 && !in_x ? 256 : 0) + row], sum);
-        row += drow; slot += dslot;
-        if (row >= N) { row -= N; ++slot; }
+#pragma unroll
+        for (int a = 0; a < AHEAD; ++a) {
+            if (slots[a] >= p.NS) break;
+            const bool in_x = slots[a] < p.nx;
+            const int lo = (p.nx > 0 && !in_x) ? p.I : 0, hi = !live[a] ? 0 : (in_x ? p.I : p.n);
+            res_expand_row(sB + (uint32_t)(slots[a] * N * 128), rows[a], w[a], res_slot_word(p, slots[a]) * 32, live[a] ? lo : 0, hi);
+        }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
-// Epilogue warps, after the barrier that completes sSum: the constants as fp32, sRow[0] of the whole vector, and of the x and the h
-// part, sRow[1], sRow[2], where the columns are split; clears sSum for the next block.
-template <typename R>
-__device__ __forceinline__ void res_row_constants(const ResProblem& p, int* sSum, float* sRow)
-{
-#pragma unroll 1
-    for (int i = (int)threadIdx.x - 32 * R::EXP_WARPS; i < p.N; i += 32 * R::EPI_WARPS) {
-        const int x = sSum[i], h = p.nx > 0 ? sSum[256 + i] : 0;
-        sSum[i] = 0; sSum[256 + i] = 0;
-        sRow[i] = (float)(x + h);
-        if (p.nx > 0) { sRow[256 + i] = (float)x; sRow[512 + i] = (float)h; }
-    }
 }
 
 // ---- weight operand -------------------------------------------------------------------------------------------------------
@@ -303,12 +305,9 @@ __device__ __forceinline__ void res_store_slot(uint32_t taddr, const uint4& a, c
         for (int q = 0; q < 4; ++q) w[q] &= keep;                   // (all ones where no row can be zero: nothing is executed)
         uint32_t y[16];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            y[q] = w[q] & 0x11111111u;
-            y[4 + q] = w[q] & 0x22222222u;
-            y[8 + q] = w[q] & 0x44444444u;
-            y[12 + q] = (w[q] & 0x88888888u) | one;
-        }
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int t = 0; t < 4; ++t) y[4 * t + q] = ((w[q] << (3 - t)) & 0x88888888u) | one;
         asm volatile(
             "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
             :: "r"(taddr + 16 * h), "r"(y[0]), "r"(y[1]), "r"(y[2]), "r"(y[3]), "r"(y[4]), "r"(y[5]), "r"(y[6]), "r"(y[7]),
@@ -356,18 +355,6 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
     return done != 0;
 }
 
-// Scale factors: eight columns of ones (both operands), eight of the pair (4, 2) for weight blocks s = 0, 1; every lane and word
-// alike.  Four warps, one per lane quarter.
-__device__ __forceinline__ void res_write_scales(const ResProblem& p, uint32_t tmem, int warp)
-{
-    const uint32_t t = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(p.ring * p.N);
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1, %2, %2, %2, %2, %2, %2, %2, %2};"
-        :: "r"(t), "r"(0x7F7F7F7Fu), "r"(0x80818081u) : "memory");
-    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-
 // The issuing warp's part of one pass over `nitems` tiles (whole warp, one elected lane issues).
 __device__ __forceinline__ bool res_issue(const ResProblem& p, ResSync& sy, int nitems, uint32_t tmem, uint32_t sB, ResIssueState& st)
 {
@@ -375,7 +362,7 @@ __device__ __forceinline__ bool res_issue(const ResProblem& p, ResSync& sy, int 
     const uint32_t idesc = (1u << 7) | (1u << 10) | ((uint32_t)(p.N >> 3) << 17) | (1u << 23) | (8u << 24);     // E2M1, E8M0, M 128
     const uint64_t desc = smem_desc(sB);
     const uint32_t lo = (uint32_t)desc, hi = (uint32_t)(desc >> 32), slot_units = (uint32_t)(p.N * 8);      // N * 128 bytes / 16
-    const uint32_t sf = tmem + (uint32_t)(p.ring * p.N), sfa = sf + 8, a0 = sf + 16;
+    const uint32_t sf = tmem + (uint32_t)(p.ring * p.N), a0 = sf + 16;
     const uint32_t full0 = smem_u32(&sy.full[0]), empty0 = smem_u32(&sy.empty[0]);
     // The next step's barrier is looked at between the two halves of a step, while the MMAs of the first half are in the queue: with the
     // look after the last MMA the tensor pipe ran dry for 250-400 clocks between steps.
@@ -392,11 +379,11 @@ __device__ __forceinline__ bool res_issue(const ResProblem& p, ResSync& sy, int 
                 if (!ready && !mbar_wait(full0 + 8 * st.stage, st.full_parity)) { *(volatile int*)&sy.failed = 1; return false; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t a = a0 + (uint32_t)(st.stage * RES_STAGE_COLS), empty = empty0 + 8 * st.stage;
-                if (issues) mma_mxf4_slot(acc, a, b, hi, idesc, s != 0 ? 1u : 0u, sfa, sf);
+                if (issues) mma_mxf4_stage_ta(acc, a, b, hi, idesc, s != 0 ? 1u : 0u, sf);
                 if (++st.stage == p.stages) { st.stage = 0; st.full_parity ^= 1u; }
                 ready = mbar_test(full0 + 8 * st.stage, st.full_parity);
                 if (issues) {
-                    if (s + 1 < p.NS) mma_mxf4_slot(acc, a + 32, b + slot_units, hi, idesc, 1u, sfa, sf);
+                    if (s + 1 < p.NS) mma_mxf4_stage_ta(acc, a + 32, b + slot_units, hi, idesc, 1u, sf);
                     mma_commit(empty);
                 }
                 b += 2 * slot_units;
@@ -412,17 +399,29 @@ __device__ __forceinline__ bool res_issue(const ResProblem& p, ResSync& sy, int 
 // ---- accumulators ---------------------------------------------------------------------------------------------------------
 //
 // An epilogue warp reads its 32 rows in the m16n8 layout: a thread then holds, of every group of eight vectors, the two vectors
-// 2 (lane mod 4) + {0, 1} for the four rows lane / 4 + 8 i.  A pair of vectors shares every instruction, and four rows every load
-// of the activation coefficients and row constants.
+// 2 (lane mod 4) + {0, 1} for the four rows lane / 4 + 8 i.  A pair of vectors shares every instruction, and the coefficients of its
+// vectors stay in registers for a whole pass.
 
 struct ResDrainState { int ring; uint32_t parity; };        // start: {0, 0}
 
+// Activation coefficients of this thread's vectors.
+template <typename R, int KA, int NG>
+__device__ __forceinline__ void res_load_beta(const ResProblem& p, const float* sBeta, int sub, f32x2 (&beta)[NG][KA])
+{
+#pragma unroll
+    for (int g = 0; g < NG; ++g)
+#pragma unroll
+        for (int j = 0; j < KA; ++j) {
+            const int c = (R::SPLIT * g + sub) * 8 * KA + 8 * j + 2 * ((int)threadIdx.x & 3);
+            beta[g][j] = c < p.N ? *reinterpret_cast<const f32x2*>(sBeta + c) : 0ull;
+        }
+}
+
 // One tile: the k_w accumulators of this warp's 32 rows, y[g][i] = sum over planes of alpha * sum_j beta_j D_j for row lane / 4 + 8 i
-// and the two vectors, D_j = accumulator + row constant (exact integers).  `sAlpha`: coefficients [plane][128] of the tile; `sRow`: the
-// row constants that go with the lane's slots.
+// and the two vectors, D_j = the accumulators (exact integers).  `sAlpha`: coefficients [plane][128] of the tile.
 template <typename R, int KA, int NG>
 __device__ __forceinline__ bool res_drain_tile(const ResProblem& p, ResSync& sy, const float* sAlpha, int quarter, int sub, uint32_t tmem,
-                                               const float* sBeta, const float* sRow, ResDrainState& st, f32x2 (&y)[NG][4])
+                                               const f32x2 (&beta)[NG][KA], ResDrainState& st, f32x2 (&y)[NG][4])
 {
     const int lane = (int)threadIdx.x & 31;
 #pragma unroll
@@ -437,26 +436,20 @@ __device__ __forceinline__ bool res_drain_tile(const ResProblem& p, ResSync& sy,
             const float v = sAlpha[plane * 128 + quarter * 32 + (lane >> 2) + 8 * i];
             al[i] = pack2(v, v);
         }
-        if (!res_group_wait(sy, smem_u32(&sy.tfull[st.ring]), st.parity, threadIdx.x >> 5 == R::EXP_WARPS, 1, 32 * R::EPI_WARPS)) return false;
+        if (!res_group_wait(sy, smem_u32(&sy.tfull[st.ring]), st.parity, threadIdx.x >> 5 == R::POLL_WARP, 1, 32 * R::EPI_WARPS)) return false;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(st.ring * p.N);
 #pragma unroll
         for (int g = 0; g < NG; ++g) {
             const int gg = R::SPLIT * g + sub;
             if (gg * 8 >= p.TB) break;
-            f32x2 v[4][KA], beta[KA], row[KA];
-            const int c0 = gg * 8 * KA + 2 * (lane & 3);
-#pragma unroll
-            for (int j = 0; j < KA; ++j) {
-                beta[j] = *reinterpret_cast<const f32x2*>(sBeta + c0 + 8 * j);
-                row[j] = *reinterpret_cast<const f32x2*>(sRow + c0 + 8 * j);
-            }
+            f32x2 v[4][KA];
             tmem_ld_pairs<KA>(acc + (uint32_t)(gg * 8 * KA), v);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                f32x2 s = mul2(beta[0], add2(v[i][0], row[0]));
+                f32x2 s = mul2(beta[g][0], v[i][0]);
 #pragma unroll
-                for (int j = 1; j < KA; ++j) s = fma2(beta[j], add2(v[i][j], row[j]), s);
+                for (int j = 1; j < KA; ++j) s = fma2(beta[g][j], v[i][j], s);
                 y[g][i] = fma2(al[i], s, y[g][i]);
             }
         }

@@ -48,8 +48,6 @@ struct SeqParams {
 // shared memory behind the activation operand
 struct __align__(16) SeqShared {
     float beta[256];
-    float row[3][256];
-    int sum[2][256];
     float alpha[2][AMQ_MAX_K * 128];
     uint32_t table[RES_TABLE];
     ResSync sync;
@@ -99,8 +97,6 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
     const uint32_t sB = smem_u32(smem_raw);
     uint32_t* counter = a.counters + (size_t)bb * 64;
 
-#pragma unroll 1
-    for (int q = tid; q < 512; q += R::THREADS) sh.sum[0][q] = 0;
     res_fill_table(p, sh.table);
     if (tid == 0) res_sync_init<R>(sh.sync);
     if (warp == R::MMA_WARP) {
@@ -112,7 +108,7 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = __shfl_sync(0xffffffffu, sh.sync.tmem_slot, 0);
-    if (warp < 4) res_write_scales(p, tmem, warp);
+    if (warp < 4) write_unit_scales(tmem, p.ring * p.N, warp);
 
     ResIssueState issue{0, 0, 0, 1};                // (apart and from constants: it stays in uniform registers)
     // stage of an expander or accumulator of an epilogue warp, and its parity: the same two registers, the quantizer needs the others
@@ -151,7 +147,7 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
             const int b = b0 + res_row_vector<KA>(tid), j = res_row_plane<KA>(tid);
             sh.beta[tid] = tid < p.TB * KA && b < p.batch ? __ldcg(a.z.zbeta + (size_t)b * KA + j) : 0.0f;
         }
-        res_expand_activations<KA>(p, a.z.zcodes, b0, sB, sh.sum[0]);
+        res_expand_activations<KA, 2>(p, a.z.zcodes, b0, sB);
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -174,7 +170,8 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
             const float* c_prev = t == 0 ? a.c0 : a.c;
             float* c_next = last ? a.c_last : a.c;
             ResDrainState drain{at, at_parity};
-            res_row_constants<R>(p, sh.sum[0], sh.row[0]);
+            f32x2 beta[SEQ_NG][KA];
+            res_load_beta<R, KA, SEQ_NG>(p, sh.beta, sub, beta);
 #pragma unroll 1
             for (int it = 0; it < tiles && ok; ++it) {
                 const int ub = part + it * a.P;
@@ -188,9 +185,8 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
                     }
                 }
                 res_epi_bar<R>(false);              // (also: everybody is past the tile before last, whose buffer this is)
-                const int kind = p.cell == RES_GRU && quarter >= 2 ? quarter - 1 : 0;
                 f32x2 y[SEQ_NG][4];
-                ok = res_drain_tile<R, KA, SEQ_NG>(p, sh.sync, sa, quarter, sub, tmem, sh.beta, sh.row[kind], drain, y);
+                ok = res_drain_tile<R, KA, SEQ_NG>(p, sh.sync, sa, quarter, sub, tmem, beta, drain, y);
 #pragma unroll
                 for (int g = 0; g < SEQ_NG; ++g) {
                     const int e = (R::SPLIT * g + sub) * 8 + 2 * (lane & 3);

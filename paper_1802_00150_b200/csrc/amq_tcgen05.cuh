@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "amq_pairs.cuh"
+
 namespace amq {
 
 constexpr unsigned WAIT_LIMIT = 1u << 20;   // attempts on an mbarrier before giving up
@@ -93,19 +95,6 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, int (&v)[8])
         : "r"(taddr) : "memory");
 }
 
-// Pairs of fp32 in one 64-bit register, for the two-wide instructions (each half rounded as the scalar instruction rounds).
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float x, float y)
-{
-    f32x2 d;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
-    return d;
-}
-__device__ __forceinline__ void unpack2(f32x2 v, float& x, float& y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v)); }
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) { f32x2 d; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d; }
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) { f32x2 d; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d; }
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) { f32x2 d; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c)); return d; }
-
 // 32 lanes x 8 NUM columns of tensor memory in the layout of an m16n8 accumulator, complete on return: v[i][c] = the columns
 // 8 c + 2 (l mod 4) + {0, 1} of lane l / 4 + 8 i.  (The loads, the wait and the packing are one block: nothing that uses the
 // values can be moved above the wait.)
@@ -188,36 +177,6 @@ __device__ __forceinline__ void mma_mxf4_stage_ta(uint32_t d_tmem, uint32_t a_tm
         "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.block32 [%0], [al], db, %4, [%6], [%6], q;\n\t"
         "}"
         :: "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(acc_first), "r"(sf_tmem) : "memory");
-}
-
-// The four MMAs of 256 bit positions, weight operand in tensor memory, with one scale address for the weight blocks of the first
-// and third MMA (`sfa`) and another for everything else (`sf_one`).
-__device__ __forceinline__ void mma_mxf4_slot(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc,
-                                              uint32_t acc_first, uint32_t sfa, uint32_t sf_one)
-{
-    asm volatile(
-        "{\n\t"
-        ".reg .pred p, q;\n\t"
-        ".reg .b64 db;\n\t"
-        ".reg .b32 al, bl;\n\t"
-        "setp.ne.b32 p, %5, 0;\n\t"
-        "setp.eq.b32 q, %5, %5;\n\t"
-        "mov.b64 db, {%2, %3};\n\t"
-        "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.block32 [%0], [%1], db, %4, [%6], [%7], p;\n\t"
-        "add.u32 al, %1, 8;\n\t"
-        "add.u32 bl, %2, 2;\n\t"
-        "mov.b64 db, {bl, %3};\n\t"
-        "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.block32 [%0], [al], db, %4, [%7], [%7], q;\n\t"
-        "add.u32 al, %1, 16;\n\t"
-        "add.u32 bl, %2, 4;\n\t"
-        "mov.b64 db, {bl, %3};\n\t"
-        "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.block32 [%0], [al], db, %4, [%6], [%7], q;\n\t"
-        "add.u32 al, %1, 24;\n\t"
-        "add.u32 bl, %2, 6;\n\t"
-        "mov.b64 db, {bl, %3};\n\t"
-        "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.block32 [%0], [al], db, %4, [%7], [%7], q;\n\t"
-        "}"
-        :: "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(acc_first), "r"(sfa), "r"(sf_one) : "memory");
 }
 
 // Scale factors of the 4-bit form: 16 tensor-memory columns, every byte 0x7F (2^0 in E8M0), written by four warps (one per
