@@ -14,6 +14,12 @@
 // greedy step can produce, so a sign plane is gathered with one funnel shift per element, a residue is
 // updated as r - copysign(alpha, r) with one logic operation and one add, and +-w for the refit sums is one
 // logic operation; the refit sums of a cycle are accumulated in the same pass that assigns the codes.
+// A warp of its own (bulk quantization) is bound by the integer pipe, 64 lanes a clock, and by issue slots, while the fp32 pipe has 128
+// lanes and two-wide instructions: there one logic operation makes s = +-1 of a sign bit, a residue is r - a s, |r| is s r and
+// the refit sums add s w, multiply-adds for two elements at a time (the products are exact: rounded as the plain sums), and a word of
+// sign bits is the exact sum of s 2^j over sixteen elements.  32768 x 1024 at 3 bits 78 -> 62 us, at 2 bits 58 -> 39.  A team's
+// quantizer is a chain of dependent operations, which the multiply-adds make longer: LSTM sequence 1024, one sequence, 154 -> 159 us,
+// decoding 674 -> 730; there it stays as it was.
 // Elements past the end of the vector are zeros that take part in every loop unmasked: their bits are
 // cleared at the end, they add nothing to B^T w, the Gram matrix is counted on masked words, and their known
 // contribution to the greedy |r| sums (all of them follow the trajectory of a zero element) is subtracted.
@@ -36,6 +42,8 @@
 
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include "amq_pairs.cuh"
 
 namespace amq {
 
@@ -429,10 +437,342 @@ __device__ __forceinline__ int bst_leaf(float x, const float (&thr)[(1 << K) - 1
     return (c1 ? 8 : 0) + (c2 ? 4 : 0) + (c3 ? 2 : 0) + (c4 ? 1 : 0);
 }
 
+// +1.0 or -1.0 with the sign of x
+__device__ __forceinline__ float unit_sign(float x) { return __uint_as_float((__float_as_uint(x) & 0x80000000u) | 0x3f800000u); }
+
+__device__ __forceinline__ float pair_sum(f32x2 v)
+{
+    float x, y;
+    unpack2(v, x, y);
+    return x + y;
+}
+
+// Signs s = +-1 of a thread's elements gathered as a word (bit j: s_j = +1).  Up to sixteen terms s_j 2^j plus 2^16 - 1 are twice that
+// word, exactly; halved and added to 2^23 it stands in the low bits of the sum.
+template <int EPT>
+struct SignWord {
+    static constexpr int PER = EPT < 16 ? EPT : 16, PARTS = (EPT + 15) / 16;
+    float acc[PARTS];
+    __device__ __forceinline__ SignWord()
+    {
+#pragma unroll
+        for (int i = 0; i < PARTS; ++i) acc[i] = (float)((1 << PER) - 1);
+    }
+    __device__ __forceinline__ void add(int j, float s) { acc[j / 16] = fmaf(s, (float)(1 << (j % 16)), acc[j / 16]); }
+    __device__ __forceinline__ uint32_t word() const
+    {
+        const uint32_t lo = __float_as_uint(fmaf(acc[0], 0.5f, 8388608.0f));
+        if (PARTS == 1) return lo & ((1u << PER) - 1u);
+        return __byte_perm(lo, __float_as_uint(fmaf(acc[PARTS - 1], 0.5f, 8388608.0f)), 0x5410);
+    }
+};
+
+// Codes of a thread's elements for levels that ascend by code index, K >= 3: plane i is decision i of the tree, the sign of w less the
+// midpoint it compares with (the midpoints of the lower half are the negatives of the upper ones, `thr`).  SUMS: also csum[i] = sum of
+// b_i w, for which an element's own midpoints are chosen; without them every decision of a level is gathered as a word of bits and the
+// words are chosen from, which takes fewer instructions.
+template <int K, int EPT, bool SUMS>
+__device__ __forceinline__ void ascending_pass(const float (&w)[EPT], const f32x2 (&w2)[EPT / 2], const float (&thr)[(1 << K) - 1],
+                                               uint32_t positive, float abs_w, uint32_t valid, uint32_t (&bits)[K], float (&csum)[K])
+{
+    constexpr int M = 1 << K, M2 = M / 2;
+    const float t1 = thr[M2 - 1 + M2 / 2], t2o = thr[M2 - 1 + M2 / 2 + M2 / 4], t2i = thr[M2 - 1 + M2 / 4];
+    bits[0] = positive & valid;
+    csum[0] = abs_w;
+    if constexpr (SUMS) {
+        f32x2 s2[K];
+        SignWord<EPT> plane[K];
+#pragma unroll
+        for (int i = 1; i < K; ++i) s2[i] = 0ull;
+#pragma unroll
+        for (int p = 0; p < EPT / 2; ++p) {
+            const f32x2 sw = pack2(unit_sign(w[2 * p]), unit_sign(w[2 * p + 1]));
+            const f32x2 d1 = fma2(sw, pack2(-t1, -t1), w2[p]);
+            float ea, eb, da, db;
+            unpack2(mul2(sw, d1), ea, eb);          // sign clear: the decision agrees with the sign of w, outer part of the half
+            unpack2(d1, da, db);
+            const bool oa = (int)__float_as_uint(ea) >= 0, ob = (int)__float_as_uint(eb) >= 0;
+            {
+                const float sa = unit_sign(da), sb = unit_sign(db);
+                s2[1] = fma2(pack2(sa, sb), w2[p], s2[1]);
+                plane[1].add(2 * p, sa);
+                plane[1].add(2 * p + 1, sb);
+            }
+            const f32x2 d2 = fma2(sw, pack2(oa ? -t2o : -t2i, ob ? -t2o : -t2i), w2[p]);
+            unpack2(d2, da, db);
+            {
+                const float sa = unit_sign(da), sb = unit_sign(db);
+                s2[2] = fma2(pack2(sa, sb), w2[p], s2[2]);
+                plane[2].add(2 * p, sa);
+                plane[2].add(2 * p + 1, sb);
+            }
+            if constexpr (K == 4) {
+                unpack2(mul2(sw, d2), ea, eb);
+                const bool pa = (int)__float_as_uint(ea) >= 0, pb = (int)__float_as_uint(eb) >= 0;
+                const float ta = oa ? (pa ? thr[M - 2] : thr[M - 4]) : (pa ? thr[M2 + 2] : thr[M2]);
+                const float tb = ob ? (pb ? thr[M - 2] : thr[M - 4]) : (pb ? thr[M2 + 2] : thr[M2]);
+                unpack2(fma2(sw, pack2(-ta, -tb), w2[p]), da, db);
+                const float sa = unit_sign(da), sb = unit_sign(db);
+                s2[K - 1] = fma2(pack2(sa, sb), w2[p], s2[K - 1]);
+                plane[K - 1].add(2 * p, sa);
+                plane[K - 1].add(2 * p + 1, sb);
+            }
+        }
+#pragma unroll
+        for (int i = 1; i < K; ++i) {
+            csum[i] = pair_sum(s2[i]);
+            bits[i] = plane[i].word() & valid;
+        }
+    } else {
+        constexpr int WORDS = M2 - 1;               // midpoints of the upper half
+        uint32_t below[WORDS];
+#pragma unroll
+        for (int c = 0; c < WORDS; ++c) below[c] = 0u;
+#pragma unroll
+        for (int p = EPT / 2 - 1; p >= 0; --p) {
+            const f32x2 sw = pack2(unit_sign(w[2 * p]), unit_sign(w[2 * p + 1]));
+#pragma unroll
+            for (int c = 0; c < WORDS; ++c) {
+                float da, db;
+                unpack2(fma2(sw, pack2(-thr[M2 + c], -thr[M2 + c]), w2[p]), da, db);
+                below[c] = __funnelshift_l(__float_as_uint(db), below[c], 1);
+                below[c] = __funnelshift_l(__float_as_uint(da), below[c], 1);
+            }
+        }
+        // decision i agrees with the sign of w: the outer part
+        const uint32_t b1 = below[M2 / 2 - 1], o1 = positive ^ b1;
+        const uint32_t b2 = (o1 & below[M2 / 2 + M2 / 4 - 1]) | (~o1 & below[M2 / 4 - 1]);
+        bits[1] = ~b1 & valid;
+        bits[2] = ~b2 & valid;
+        if constexpr (K == 4) {
+            const uint32_t o2 = positive ^ b2;
+            const uint32_t outer = (o2 & below[WORDS - 1]) | (~o2 & below[WORDS - 3]), inner = (o2 & below[2]) | (~o2 & below[0]);
+            bits[K - 1] = ~((o1 & outer) | (~o1 & inner)) & valid;
+        }
+#pragma unroll
+        for (int i = 1; i < K; ++i) csum[i] = 0.0f;
+    }
+}
+
 // Elements past the end of the vector inside the threads that do hold some of it, for the two ownership patterns in
 // use: thread g owns the EPT consecutive elements from g * EPT; lane l of a warp owns the elements j * 32 + l.
 __host__ __device__ inline int quant_padding_consecutive(int n, int ept) { return (n + ept - 1) / ept * ept - n; }
 __host__ __device__ inline int quant_padding_strided32(int n, int ept) { return (n >= 32 ? 32 : n) * ept - n; }
+
+// The sorted table of two bits in closed form.  The tree's two decisions are the sign of w and w against the midpoint of its half; which
+// plane is which decision, and its sign, follow from the coefficients.
+struct TwoLevels {
+    float mid;                      // >= 0
+    bool first, sa, sb;
+    __device__ __forceinline__ TwoLevels(float a0, float a1)
+    {
+        const float A = fabsf(a0), B = fabsf(a1), d = A - B;
+        mid = 0.5f * ((A + B) + fabsf(d));
+        sa = a0 < 0.0f; sb = a1 < 0.0f;
+        first = d > 0.0f || (d == 0.0f && !sa);
+        if ((A + B) == fabsf(d)) { if (first) sb = false; else sa = false; }
+    }
+    // c1, c2: words of the two decisions; abs_w, s1: their sums with w
+    __device__ __forceinline__ void planes(uint32_t c1, uint32_t c2, uint32_t valid, float abs_w, float s1, uint32_t (&bits)[2], float (&csum)[2]) const
+    {
+        bits[0] = ((first ? c1 : c2) ^ (sa ? 0xffffffffu : 0u)) & valid;
+        bits[1] = ((first ? c2 : c1) ^ (sb ? 0xffffffffu : 0u)) & valid;
+        const float sum0 = first ? abs_w : s1, sum1 = first ? s1 : abs_w;
+        csum[0] = sa ? -sum0 : sum0;
+        csum[1] = sb ? -sum1 : sum1;
+    }
+};
+
+// Codes for levels in any order, K >= 3.  The table is still antisymmetric (v and -v are levels together, of complementary codes, and
+// ties are ordered alike), so the tree's decisions are the same comparisons with the sorted upper half; a plane is a function of the
+// leaf, evaluated on whole words of decision bits.  `sums`: also csum[i] = sum of b_i w.
+template <int K, int EPT>
+__device__ __forceinline__ void sorted_pass(const float (&w)[EPT], const float (&alpha)[K], uint32_t positive, uint32_t valid, bool sums,
+                                            float (&thr)[(1 << K) - 1], uint32_t (&bits)[K], float (&csum)[K])
+{
+    constexpr uint32_t SIGN = 0x80000000u;
+    constexpr int M2 = 1 << (K - 1);
+                uint32_t code[M2];
+                upper_levels<K>(alpha, thr, code);
+                uint32_t below[K];
+#pragma unroll
+                for (int i = 0; i < K; ++i) below[i] = 0u;
+#pragma unroll
+                for (int j = EPT - 1; j >= 0; --j) tree_decisions<K, EPT>(w[j], thr, below);
+                // minterms of the leaf within the half: bit i of the leaf = decision i agrees with the sign of w
+                uint32_t leaf[M2];
+                {
+                    const uint32_t u1 = positive ^ below[1], u2 = positive ^ below[2];          // (below: decision bits inverted)
+                    const uint32_t q3 = u1 & u2, q2 = u1 & ~u2, q1 = ~u1 & u2, q0 = ~(u1 | u2);
+                    if constexpr (K == 3) {
+                        leaf[0] = q0; leaf[1] = q1; leaf[2] = q2; leaf[3] = q3;
+                    } else {
+                        const uint32_t u3 = positive ^ below[K - 1];
+                        leaf[0] = q0 & ~u3; leaf[1] = q0 & u3; leaf[2] = q1 & ~u3; leaf[3] = q1 & u3;
+                        leaf[M2 - 4] = q2 & ~u3; leaf[M2 - 3] = q2 & u3; leaf[M2 - 2] = q3 & ~u3; leaf[M2 - 1] = q3 & u3;
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < K; ++i) {
+                    uint32_t f = 0u;
+#pragma unroll
+                    for (int q = 0; q < M2; ++q) f |= leaf[q] & (0u - ((code[q] >> (K - 1 - i)) & 1u));
+                    const uint32_t pb = ~(positive ^ f);        // the lower half has the complementary codes
+                    bits[i] = pb & valid;
+                    if (sums) {
+                        float cs = 0.0f;
+#pragma unroll
+                        for (int j = EPT - 1; j >= 0; --j) cs += __uint_as_float(__float_as_uint(w[j]) ^ (~(pb << (31 - j)) & SIGN));
+                        csum[i] = cs;
+                    }
+                }
+}
+
+// quantize_group of a warp of its own: the same steps with two-wide multiply-adds (see above).
+template <int K, int EPT>
+__device__ __forceinline__ void quantize_warp(const float (&w_in)[EPT], uint32_t valid, int n, int pad_elems, int T, float (&alpha)[K],
+                                              uint32_t (&bits)[K], QuantScratch<K, 1>& sc)
+{
+    constexpr int NG = K * (K - 1) / 2;
+    static_assert(EPT % 2 == 0 && EPT <= 32, "");
+    const QuantTeam none_team{0, 0, 32};
+    const int nvalid = __popc(valid);
+    const float inv_n = 1.0f / (float)n;
+    const float padding = (float)pad_elems;
+    const bool holds_some = valid != 0;
+    float w[EPT];
+    f32x2 w2[EPT / 2];
+#pragma unroll
+    for (int p = 0; p < EPT / 2; ++p) {
+        w2[p] = add2(pack2(w_in[2 * p], w_in[2 * p + 1]), 0ull);  // -0.0 -> +0.0
+        unpack2(w2[p], w[2 * p], w[2 * p + 1]);
+    }
+
+    float last_abs = 0.0f, csum[K], abs_w = 0.0f;
+    uint32_t positive = 0;
+    float rho = 0.0f;
+    {
+        f32x2 r2[EPT / 2];
+#pragma unroll
+        for (int p = 0; p < EPT / 2; ++p) r2[p] = w2[p];
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+            float part = 0.0f;
+            if (i == 0) {                                         // (|w| is an operand modifier, the word a funnel shift per element)
+                uint32_t neg = 0;
+#pragma unroll
+                for (int j = EPT - 1; j >= 0; --j) {
+                    part += fabsf(w[j]);
+                    neg = __funnelshift_l(__float_as_uint(w[j]), neg, 1);
+                }
+                positive = ~neg;
+                bits[0] = positive & valid;
+                csum[0] = abs_w = part;
+            } else {
+                f32x2 part2 = 0ull, cs2 = 0ull;
+                SignWord<EPT> plane;
+#pragma unroll
+                for (int p = 0; p < EPT / 2; ++p) {
+                    float ra, rb;
+                    unpack2(r2[p], ra, rb);
+                    const float sa = unit_sign(ra), sb = unit_sign(rb);
+                    const f32x2 s = pack2(sa, sb);
+                    part2 = fma2(s, r2[p], part2);                // |r|
+                    cs2 = fma2(s, w2[p], cs2);                    // b_i w
+                    plane.add(2 * p, sa);
+                    plane.add(2 * p + 1, sb);
+                }
+                bits[i] = plane.word() & valid;
+                csum[i] = pair_sum(cs2);
+                part = pair_sum(part2);
+            }
+            part = holds_some ? part : 0.0f;
+            if (i == K - 1 && T > 0) { last_abs = part; alpha[i] = 0.0f; break; }
+            float tot[1] = {part};
+            int none[1] = {0};
+            group_totals<1, 0, K, 1>(tot, none, sc, 0, nullptr, none_team);
+            const float a = (tot[0] - padding * fabsf(rho)) * inv_n;
+            alpha[i] = a;
+            const f32x2 minus = pack2(-a, -a);
+            rho = fmaf(unit_sign(rho), -a, rho);
+            if (i == K - 1) break;                                // (T = 0: no residue is needed any more)
+#pragma unroll
+            for (int p = 0; p < EPT / 2; ++p) {                   // r - a sign(r)
+                float ra, rb;
+                unpack2(r2[p], ra, rb);
+                r2[p] = fma2(pack2(unit_sign(ra), unit_sign(rb)), minus, r2[p]);
+            }
+        }
+    }
+
+    for (int it = 0; it < T; ++it) {
+        float fsum[1 + K];
+        int gram[NG > 0 ? NG : 1];
+        fsum[0] = last_abs;
+#pragma unroll
+        for (int i = 0; i < K; ++i) fsum[1 + i] = csum[i];
+        {
+            int q = 0;
+#pragma unroll
+            for (int i = 0; i < K; ++i)
+#pragma unroll
+                for (int j = i + 1; j < K; ++j)
+                    gram[q++] = nvalid - 2 * __popc((bits[i] ^ bits[j]) & valid);
+            if (NG == 0) gram[0] = 0;
+        }
+        group_totals<1 + K, NG, K, 1>(fsum, gram, sc, 0, nullptr, none_team);
+        if (it == 0) alpha[K - 1] = (fsum[0] - padding * fabsf(rho)) * inv_n;
+        {
+            float c[K];
+#pragma unroll
+            for (int i = 0; i < K; ++i) c[i] = fsum[1 + i];
+            solve_refit<K>(c, gram, n, alpha);
+        }
+        last_abs = 0.0f;
+        const bool more = it + 1 < T;
+        if constexpr (K == 1) {
+            bits[0] = (alpha[0] < 0.0f ? ~positive : positive) & valid;
+            csum[0] = alpha[0] < 0.0f ? -abs_w : abs_w;
+        } else if constexpr (K == 2) {
+            const TwoLevels t(alpha[0], alpha[1]);
+            const f32x2 minus = pack2(-t.mid, -t.mid);
+            uint32_t below = 0;
+            float s1 = 0.0f;
+            if (more) {
+                f32x2 s2 = 0ull;
+                SignWord<EPT> plane;
+#pragma unroll
+                for (int p = 0; p < EPT / 2; ++p) {
+                    float da, db;
+                    unpack2(fma2(pack2(unit_sign(w[2 * p]), unit_sign(w[2 * p + 1])), minus, w2[p]), da, db);
+                    const float sa = unit_sign(da), sb = unit_sign(db);
+                    s2 = fma2(pack2(sa, sb), w2[p], s2);
+                    plane.add(2 * p, sa);
+                    plane.add(2 * p + 1, sb);
+                }
+                s1 = pair_sum(s2);
+                below = ~plane.word();
+            } else {
+#pragma unroll
+                for (int p = EPT / 2 - 1; p >= 0; --p) {
+                    float da, db;
+                    unpack2(fma2(pack2(unit_sign(w[2 * p]), unit_sign(w[2 * p + 1])), minus, w2[p]), da, db);
+                    below = __funnelshift_l(__float_as_uint(db), below, 1);
+                    below = __funnelshift_l(__float_as_uint(da), below, 1);
+                }
+            }
+            t.planes(positive, ~below, valid, abs_w, s1, bits, csum);
+        } else {
+            float thr[(1 << K) - 1];
+            if (ascending_levels<K>(alpha, thr)) {
+                if (more) ascending_pass<K, EPT, true>(w, w2, thr, positive, abs_w, valid, bits, csum);
+                else ascending_pass<K, EPT, false>(w, w2, thr, positive, abs_w, valid, bits, csum);
+            } else {
+                sorted_pass<K, EPT>(w, alpha, positive, valid, more, thr, bits, csum);
+            }
+        }
+    }
+}
 
 // Quantize the vector held in w[] (positions past the end of the vector must hold 0 and have their bit
 // clear in `valid`; `pad_elems` = how many such positions lie in threads whose `valid` is not zero).  NW = 1: the group is the calling warp; NW > 1: the group is the whole CTA of up to NW
@@ -453,6 +793,10 @@ __device__ __forceinline__ void quantize_group(const float (&w_in)[EPT], uint32_
                                                int* flag = nullptr, int* parity_io = nullptr,
                                                const QuantTeam& team = QuantTeam::cta())
 {
+    if constexpr (NW == 1) {
+        quantize_warp<K, EPT>(w_in, valid, n, pad_elems, T, alpha, bits, sc);
+        return;
+    }
     constexpr int M = 1 << K;
     constexpr int NG = K * (K - 1) / 2;
     constexpr uint32_t SIGN = 0x80000000u;
@@ -544,13 +888,8 @@ __device__ __forceinline__ void quantize_group(const float (&w_in)[EPT], uint32_
             continue;
         }
         if constexpr (K == 2) {
-            // The sorted table in closed form, with the tree's two decisions as words of bits: the sign of w, and w against the
-            // midpoint of its half.  Which plane is which decision, and its sign, follow from the coefficients.
-            const float A = fabsf(alpha[0]), B = fabsf(alpha[K - 1]), d = A - B;
-            const uint32_t mid = __float_as_uint(0.5f * ((A + B) + fabsf(d)));         // >= 0
-            bool sa = alpha[0] < 0.0f, sb = alpha[K - 1] < 0.0f;
-            const bool first = d > 0.0f || (d == 0.0f && !sa);
-            if ((A + B) == fabsf(d)) { if (first) sb = false; else sa = false; }
+            const TwoLevels t(alpha[0], alpha[K - 1]);
+            const uint32_t mid = __float_as_uint(t.mid);
             uint32_t below = 0;
             float s1 = 0.0f;
 #pragma unroll
@@ -560,12 +899,7 @@ __device__ __forceinline__ void quantize_group(const float (&w_in)[EPT], uint32_
                 below = __funnelshift_l(db, below, 1);
                 if (more) s1 += __uint_as_float(wb ^ (db & SIGN));
             }
-            const uint32_t c1 = positive, c2 = ~below;
-            bits[0] = ((first ? c1 : c2) ^ (sa ? 0xffffffffu : 0u)) & valid;
-            bits[K - 1] = ((first ? c2 : c1) ^ (sb ? 0xffffffffu : 0u)) & valid;
-            const float sum0 = first ? abs_w : s1, sum1 = first ? s1 : abs_w;
-            csum[0] = sa ? -sum0 : sum0;
-            csum[K - 1] = sb ? -sum1 : sum1;
+            t.planes(positive, ~below, valid, abs_w, s1, bits, csum);
             continue;
         }
         if constexpr (QuantScratch<K, NW>::TABLE) {
@@ -612,44 +946,7 @@ __device__ __forceinline__ void quantize_group(const float (&w_in)[EPT], uint32_
             }
         }
         if constexpr (K >= 3) {
-            // Any other order of the levels.  The table is still antisymmetric (v and -v are levels together, of complementary codes, and
-            // ties are ordered alike), so the tree's decisions are the same comparisons with the sorted upper half; a plane is a
-            // function of the leaf, evaluated on whole words of decision bits.
-            constexpr int M2 = M / 2;
-            uint32_t code[M2];
-            upper_levels<K>(alpha, thr, code);
-            uint32_t below[K];
-#pragma unroll
-            for (int i = 0; i < K; ++i) below[i] = 0u;
-#pragma unroll
-            for (int j = EPT - 1; j >= 0; --j) tree_decisions<K, EPT>(w[j], thr, below);
-            // minterms of the leaf within the half: bit i of the leaf = decision i agrees with the sign of w
-            uint32_t leaf[M2];
-            {
-                const uint32_t u1 = positive ^ below[1], u2 = positive ^ below[2];          // (below: decision bits inverted)
-                const uint32_t q3 = u1 & u2, q2 = u1 & ~u2, q1 = ~u1 & u2, q0 = ~(u1 | u2);
-                if constexpr (K == 3) {
-                    leaf[0] = q0; leaf[1] = q1; leaf[2] = q2; leaf[3] = q3;
-                } else {
-                    const uint32_t u3 = positive ^ below[K - 1];
-                    leaf[0] = q0 & ~u3; leaf[1] = q0 & u3; leaf[2] = q1 & ~u3; leaf[3] = q1 & u3;
-                    leaf[M2 - 4] = q2 & ~u3; leaf[M2 - 3] = q2 & u3; leaf[M2 - 2] = q3 & ~u3; leaf[M2 - 1] = q3 & u3;
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < K; ++i) {
-                uint32_t f = 0u;
-#pragma unroll
-                for (int q = 0; q < M2; ++q) f |= leaf[q] & (0u - ((code[q] >> (K - 1 - i)) & 1u));
-                const uint32_t pb = ~(positive ^ f);        // the lower half has the complementary codes
-                bits[i] = pb & valid;
-                if (more) {
-                    float cs = 0.0f;
-#pragma unroll
-                    for (int j = EPT - 1; j >= 0; --j) cs += __uint_as_float(__float_as_uint(w[j]) ^ (~(pb << (31 - j)) & SIGN));
-                    csum[i] = cs;
-                }
-            }
+            sorted_pass<K, EPT>(w, alpha, positive, valid, more, thr, bits, csum);
         }
     }
     if (parity_io) *parity_io = parity;

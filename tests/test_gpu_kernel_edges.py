@@ -183,3 +183,28 @@ def test_quantizer_with_levels_out_of_order(amq, rows, n, k):
         got = ((x[r] - coeffs[r] @ b[r]) ** 2).sum()
         want = ((x[r] - oa @ ob) ** 2).sum()
         assert abs(got - want) <= 1e-3 * max(want, 1e-6 * (x[r].astype(np.float64) ** 2).sum()), r
+
+
+@pytest.mark.parametrize("n,k", [(1, 2), (7, 3), (9, 4), (31, 2), (33, 3), (255, 3), (256, 4), (257, 2), (258, 4), (1000, 3), (1023, 2), (1024, 4), (1024, 1)])
+def test_bulk_quantization_at_the_edges_of_a_warps_rows(amq, n, k):
+    """A warp per row: eight or thirty-two elements a thread, its last threads partly or wholly past the end; rows of ties (all of one
+    magnitude, whole numbers) beside random ones."""
+    x = synth.normal((1025, n), 0.05, 77 + n, k)
+    x[3] = 0.25
+    x[4] = -0.5
+    x[5] = np.round(x[5] * 40)
+    x[6] = 0.0
+
+    def gpu(v, kk, T):
+        codes, coeffs = amq.quantize(dev(v), kk, T)
+        rows = np.r_[0:40, 1024]                    # (the oracle is slow)
+        return codes.cpu().numpy().view(np.uint32)[rows], coeffs.cpu().numpy()[rows]
+
+    rows = np.r_[0:40, 1024]
+    random = [i for i, r in enumerate(rows) if r not in (3, 4, 5, 6)]
+    parity.compare_quantizer(x[rows][random], k, 2, lambda v, kk, T: tuple(a[random] for a in gpu(x, kk, T)))
+    # ties: several codes are correct, what they reconstruct is not free
+    codes, coeffs = gpu(x, k, 2)
+    bits = parity.unpack_rows(codes, n)
+    for r in (3, 4, 6):
+        assert np.abs(oracle.reconstruct(coeffs[r].astype(np.float64), bits[r]) - x[r]).max() <= 1e-6 * np.abs(x[r]).max()
