@@ -583,7 +583,74 @@ struct TwoLevels {
     }
 };
 
-// Codes for levels in any order, K >= 3.  The table is still antisymmetric (v and -v are levels together, of complementary codes, and
+// The table of three bits.  With the coefficients' magnitudes A >= B >= C the levels of its upper half are, in order, |A - B - C|, A - B + C,
+// A + B - C and A + B + C, whatever the coefficients: the planes of A, B and C are the tree's three decisions, but for the
+// elements at the innermost level on either side, all of whose signs are the opposite ones where A < B + C.  So any order of the
+// coefficients costs a sort of the four values (no codes travel with them) and a permutation of the finished words.  (On z = [x ; h] the
+// levels seldom ascend by code: with the codes sorted along and the planes evaluated leaf by leaf a cycle's codes took a team of eight warps
+// 1000 to 1130 clocks, where ascending levels take 300 to 470.)
+struct ThreeLevels {
+    float inner, mid, outer;        // midpoints of the upper half
+    int rank[3];                    // 0: the largest magnitude; among equals the smaller index first
+    bool neg[3], flip;
+    __device__ __forceinline__ ThreeLevels(const float (&a)[3])
+    {
+        const float m0 = fabsf(a[0]), m1 = fabsf(a[1]), m2 = fabsf(a[2]);
+        rank[0] = (m1 > m0) + (m2 > m0); rank[1] = (m0 >= m1) + (m2 > m1); rank[2] = (m0 >= m2) + (m1 >= m2);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) neg[i] = a[i] < 0.0f;
+        // (each value rounded as the sum in the order of the planes)
+        const float less = a[0] - a[1], more = a[0] + a[1];
+        const float v0 = fabsf(less - a[2]), v1 = fabsf(less + a[2]), v2 = fabsf(more - a[2]), v3 = fabsf(more + a[2]);
+        const float l1 = fminf(v0, v1), h1 = fmaxf(v0, v1), l2 = fminf(v2, v3), h2 = fmaxf(v2, v3);
+        const float x = fmaxf(l1, l2), y = fminf(h1, h2), q0 = fminf(l1, l2), q1 = fminf(x, y), q2 = fmaxf(x, y), q3 = fmaxf(h1, h2);
+        inner = (q0 + q1) * 0.5f; mid = (q1 + q2) * 0.5f; outer = (q2 + q3) * 0.5f;
+        flip = ((rank[0] == 0 ? m0 : -m0) + (rank[1] == 0 ? m1 : -m1)) + (rank[2] == 0 ? m2 : -m2) < 0.0f;
+    }
+    // Codes of a thread's elements; `sums`: also csum[i] = sum of b_i w.
+    template <int EPT>
+    __device__ __forceinline__ void pass(const float (&w)[EPT], uint32_t positive, float abs_w, uint32_t valid, bool sums,
+                                         uint32_t (&bits)[3], float (&csum)[3]) const
+    {
+        constexpr uint32_t SIGN = 0x80000000u;
+        uint32_t below1 = 0u, below2 = 0u;
+        float s1 = 0.0f, s2 = 0.0f, innermost = 0.0f;
+#pragma unroll
+        for (int j = EPT - 1; j >= 0; --j) {
+            const uint32_t wb = __float_as_uint(w[j]), sw = wb & SIGN;
+            const uint32_t d1 = __float_as_uint(w[j] - __uint_as_float(__float_as_uint(mid) | sw));
+            const float t2 = (int)(wb ^ d1) >= 0 ? outer : inner;           // the decision agrees with the sign: outer half
+            const uint32_t d2 = __float_as_uint(w[j] - __uint_as_float(__float_as_uint(t2) | sw));
+            below1 = __funnelshift_l(d1, below1, 1);
+            below2 = __funnelshift_l(d2, below2, 1);
+            if (sums) {
+                s1 += __uint_as_float(wb ^ (d1 & SIGN));
+                s2 += __uint_as_float(wb ^ (d2 & SIGN));
+            }
+        }
+        uint32_t plane[3] = {positive, ~below1, ~below2};
+        if (flip) {
+            const uint32_t leaf = (positive ^ plane[1]) & (positive ^ plane[2]);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) plane[i] ^= leaf;
+            if (sums) {
+#pragma unroll
+                for (int j = 0; j < EPT; ++j) innermost += (leaf >> j) & 1u ? fabsf(w[j]) : 0.0f;
+            }
+        }
+        // an innermost element adds |w|, -|w|, -|w| unflipped
+        const float sum[3] = {fmaf(-2.0f, innermost, abs_w), fmaf(2.0f, innermost, s1), fmaf(2.0f, innermost, s2)};
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const uint32_t b = rank[i] == 0 ? plane[0] : rank[i] == 1 ? plane[1] : plane[2];
+            const float c = rank[i] == 0 ? sum[0] : rank[i] == 1 ? sum[1] : sum[2];
+            bits[i] = (neg[i] ? ~b : b) & valid;
+            csum[i] = neg[i] ? -c : c;
+        }
+    }
+};
+
+// Codes of K >= 3 bits, levels in any order.  The table is still antisymmetric (v and -v are levels together, of complementary codes, and
 // ties are ordered alike), so the tree's decisions are the same comparisons with the sorted upper half; a plane is a function of the
 // leaf, evaluated on whole words of decision bits.  `sums`: also csum[i] = sum of b_i w.
 template <int K, int EPT>
@@ -592,40 +659,40 @@ __device__ __forceinline__ void sorted_pass(const float (&w)[EPT], const float (
 {
     constexpr uint32_t SIGN = 0x80000000u;
     constexpr int M2 = 1 << (K - 1);
-                uint32_t code[M2];
-                upper_levels<K>(alpha, thr, code);
-                uint32_t below[K];
+    uint32_t code[M2];
+    upper_levels<K>(alpha, thr, code);
+    uint32_t below[K];
 #pragma unroll
-                for (int i = 0; i < K; ++i) below[i] = 0u;
+    for (int i = 0; i < K; ++i) below[i] = 0u;
 #pragma unroll
-                for (int j = EPT - 1; j >= 0; --j) tree_decisions<K, EPT>(w[j], thr, below);
-                // minterms of the leaf within the half: bit i of the leaf = decision i agrees with the sign of w
-                uint32_t leaf[M2];
-                {
-                    const uint32_t u1 = positive ^ below[1], u2 = positive ^ below[2];          // (below: decision bits inverted)
-                    const uint32_t q3 = u1 & u2, q2 = u1 & ~u2, q1 = ~u1 & u2, q0 = ~(u1 | u2);
-                    if constexpr (K == 3) {
-                        leaf[0] = q0; leaf[1] = q1; leaf[2] = q2; leaf[3] = q3;
-                    } else {
-                        const uint32_t u3 = positive ^ below[K - 1];
-                        leaf[0] = q0 & ~u3; leaf[1] = q0 & u3; leaf[2] = q1 & ~u3; leaf[3] = q1 & u3;
-                        leaf[M2 - 4] = q2 & ~u3; leaf[M2 - 3] = q2 & u3; leaf[M2 - 2] = q3 & ~u3; leaf[M2 - 1] = q3 & u3;
-                    }
-                }
+    for (int j = EPT - 1; j >= 0; --j) tree_decisions<K, EPT>(w[j], thr, below);
+    // minterms of the leaf within the half: bit i of the leaf = decision i agrees with the sign of w
+    uint32_t leaf[M2];
+    {
+        const uint32_t u1 = positive ^ below[1], u2 = positive ^ below[2];          // (below: decision bits inverted)
+        const uint32_t q3 = u1 & u2, q2 = u1 & ~u2, q1 = ~u1 & u2, q0 = ~(u1 | u2);
+        if constexpr (K == 3) {
+            leaf[0] = q0; leaf[1] = q1; leaf[2] = q2; leaf[3] = q3;
+        } else {
+            const uint32_t u3 = positive ^ below[K - 1];
+            leaf[0] = q0 & ~u3; leaf[1] = q0 & u3; leaf[2] = q1 & ~u3; leaf[3] = q1 & u3;
+            leaf[M2 - 4] = q2 & ~u3; leaf[M2 - 3] = q2 & u3; leaf[M2 - 2] = q3 & ~u3; leaf[M2 - 1] = q3 & u3;
+        }
+    }
 #pragma unroll
-                for (int i = 0; i < K; ++i) {
-                    uint32_t f = 0u;
+    for (int i = 0; i < K; ++i) {
+        uint32_t f = 0u;
 #pragma unroll
-                    for (int q = 0; q < M2; ++q) f |= leaf[q] & (0u - ((code[q] >> (K - 1 - i)) & 1u));
-                    const uint32_t pb = ~(positive ^ f);        // the lower half has the complementary codes
-                    bits[i] = pb & valid;
-                    if (sums) {
-                        float cs = 0.0f;
+        for (int q = 0; q < M2; ++q) f |= leaf[q] & (0u - ((code[q] >> (K - 1 - i)) & 1u));
+        const uint32_t pb = ~(positive ^ f);        // the lower half has the complementary codes
+        bits[i] = pb & valid;
+        if (sums) {
+            float cs = 0.0f;
 #pragma unroll
-                        for (int j = EPT - 1; j >= 0; --j) cs += __uint_as_float(__float_as_uint(w[j]) ^ (~(pb << (31 - j)) & SIGN));
-                        csum[i] = cs;
-                    }
-                }
+            for (int j = EPT - 1; j >= 0; --j) cs += __uint_as_float(__float_as_uint(w[j]) ^ (~(pb << (31 - j)) & SIGN));
+            csum[i] = cs;
+        }
+    }
 }
 
 // quantize_group of a warp of its own: the same steps with two-wide multiply-adds (see above).
@@ -768,7 +835,8 @@ __device__ __forceinline__ void quantize_warp(const float (&w_in)[EPT], uint32_t
                 if (more) ascending_pass<K, EPT, true>(w, w2, thr, positive, abs_w, valid, bits, csum);
                 else ascending_pass<K, EPT, false>(w, w2, thr, positive, abs_w, valid, bits, csum);
             } else {
-                sorted_pass<K, EPT>(w, alpha, positive, valid, more, thr, bits, csum);
+                if constexpr (K == 3) ThreeLevels(alpha).template pass<EPT>(w, positive, abs_w, valid, more, bits, csum);
+                else sorted_pass<K, EPT>(w, alpha, positive, valid, more, thr, bits, csum);
             }
         }
     }
@@ -921,32 +989,35 @@ __device__ __forceinline__ void quantize_group(const float (&w_in)[EPT], uint32_
             for (int i = 0; i < K; ++i) bits[i] = pos_bits[i] & valid;
             continue;
         }
-        if constexpr (K >= 3) {
-            // ascending levels: code bit i is decision i of the tree, the sign of w minus the midpoint that decision compares with;
-            // plane 0 is the sign of w, whose sum is known
-            if (ascending_levels<K>(alpha, thr)) {
-                uint32_t below[K];
-                float s[K];
+        if constexpr (K == 3) {
+            // (Bulk rows of more than 1024, 32 elements a thread, nearly always ascend, and a thread's registers count: 8192 x 3000 72 us
+            // this way, 82 to 84 with ThreeLevels for all or for the other rows.)
+            if constexpr (EPT == 32) {
+                if (ascending_levels<K>(alpha, thr)) {
+                    uint32_t below[K];
+                    float sum[K];
 #pragma unroll
-                for (int i = 0; i < K; ++i) { below[i] = 0u; s[i] = 0.0f; }
+                    for (int i = 0; i < K; ++i) { below[i] = 0u; sum[i] = 0.0f; }
 #pragma unroll
-                for (int j = EPT - 1; j >= 0; --j) {
-                    uint32_t d[K];
-                    tree_decisions<K, EPT>(w[j], thr, below, d);
-                    if (more) {
+                    for (int j = EPT - 1; j >= 0; --j) {
+                        uint32_t d[K];
+                        tree_decisions<K, EPT>(w[j], thr, below, d);
+                        if (more) {
 #pragma unroll
-                        for (int i = 1; i < K; ++i) s[i] += __uint_as_float(__float_as_uint(w[j]) ^ (d[i] & SIGN));
+                            for (int i = 1; i < K; ++i) sum[i] += __uint_as_float(__float_as_uint(w[j]) ^ (d[i] & SIGN));
+                        }
                     }
-                }
-                bits[0] = positive & valid;
-                csum[0] = abs_w;
+                    bits[0] = positive & valid;
+                    csum[0] = abs_w;
 #pragma unroll
-                for (int i = 1; i < K; ++i) { bits[i] = ~below[i] & valid; csum[i] = s[i]; }
+                    for (int i = 1; i < K; ++i) { bits[i] = ~below[i] & valid; csum[i] = sum[i]; }
+                } else {
+                    sorted_pass<K, EPT>(w, alpha, positive, valid, more, thr, bits, csum);
+                }
                 continue;
             }
-        }
-        if constexpr (K >= 3) {
-            sorted_pass<K, EPT>(w, alpha, positive, valid, more, thr, bits, csum);
+            ThreeLevels(alpha).template pass<EPT>(w, positive, abs_w, valid, more, bits, csum);
+            continue;
         }
     }
     if (parity_io) *parity_io = parity;

@@ -208,3 +208,21 @@ def test_bulk_quantization_at_the_edges_of_a_warps_rows(amq, n, k):
     bits = parity.unpack_rows(codes, n)
     for r in (3, 4, 6):
         assert np.abs(oracle.reconstruct(coeffs[r].astype(np.float64), bits[r]) - x[r]).max() <= 1e-6 * np.abs(x[r]).max()
+
+
+@pytest.mark.parametrize("n,small", [(1, 1.0), (9, 0.1), (257, 0.02), (1025, 0.3), (2048, 0.1), (2049, 0.5)])
+def test_three_bits_whose_levels_do_not_ascend(amq, n, small):
+    """Vectors of large and of small elements, as [x ; h] is: the coefficients then come in any order of size, the smallest of them often
+    below the difference of the others."""
+    x = synth.normal((48, n), 1.0, 400 + n, 1)
+    x[:, n // 2:] *= small
+    x[24:, ::3] += 3.0
+
+    def gpu(v, k, T):
+        codes, coeffs = amq.quantize(dev(v), k, T)
+        return codes.cpu().numpy().view(np.uint32), coeffs.cpu().numpy()
+
+    parity.compare_quantizer(x, 3, 2, gpu)
+    a = np.abs(gpu(x, 3, 1)[1])                     # (what the last cycle's table is made of, but for one refit)
+    if n > 9:
+        assert (a[:, 0] < a[:, 1] + a[:, 2]).any() or (np.argsort(-a, axis=1) != np.arange(3)).any()
