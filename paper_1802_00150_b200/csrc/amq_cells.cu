@@ -227,8 +227,8 @@ amq_status enqueue_sequence(const CellCall& c, const CellWorkspace& ws, const fl
             if (chunks) AMQ_CUDA_TRY(cudaStreamWaitEvent(st, chunks->ready[q], 0));
             BatchedSequence b = batched_call(c, ws, x_seq + (size_t)s0 * c.batch * c.I, s1 - s0, q ? h_last : h0, q ? c_last : c0,
                                              h_seq ? h_seq + (size_t)s0 * state : nullptr, h_last, c_last);
-            b.counted = s0;
-            if (forced) { b.counted += forced->counted; b.late = forced->late; }
+            b.counted = s0; b.launched = q;
+            if (forced) { b.counted += forced->counted; b.launched += forced->counted; b.late = forced->late; }
             const amq_status r = launch_batched_sequence(b, form, shape, st);
             if (r != AMQ_OK) return r;
         }
@@ -495,7 +495,8 @@ amq_status amq_selftest_batched_sequence(const uint32_t* Wcodes, const float* Wa
     if (steps < 1 || !h0 || !h_last || (!c.gru && (!c0 || !c_last)) || (I > 0 && !x_seq) || h_last == h0 || (!c.gru && c_last == c0))
         return AMQ_ERR_INVALID_ARG;
     if (form < AMQ_FORM_CHAIN || form > AMQ_FORM_RESIDENT || counted < 0 || counted > 0x7fffffff - steps) return AMQ_ERR_INVALID_ARG;
-    if (late < 0 || late > 2 || (late > 0 && (form == AMQ_FORM_CHAIN || counted > 0)) || (late == 2 && steps < 2))
+    if (late < 0 || late > 3 || (late > 0 && (form == AMQ_FORM_CHAIN || counted > 0)) || (late >= 2 && steps < 2) ||
+        (late == 3 && form != AMQ_FORM_RESIDENT))
         return AMQ_ERR_INVALID_ARG;
     if (batch < 2) return AMQ_ERR_UNSUPPORTED;
     amq::CellWorkspace ws = amq::carve_cell_workspace(workspace, I, H, batch, k_a);

@@ -208,7 +208,8 @@ struct BatchedSequence {
     uint32_t* zcodes; float* zbeta; uint32_t* counters; uint32_t* status;
     int counted;                // timesteps that earlier launches have added to the counters since they were cleared
     int late;                   // self-test of the waits: the CTAs look for the counts of quantized shares (1) or of finished products (2) where
-                                // nobody counts; 0: none
+                                // nobody counts, for states (3, resident form) of another timestep; 0: none
+    int launched = 0;           // launches that have counted since the counters were cleared
 };
 // The ways to run one: a chain of launches per timestep, or one launch with the weights streamed past the activations (amq_rnn_batched.cu)
 // or held in tensor memory (amq_rnn_resident.cu).

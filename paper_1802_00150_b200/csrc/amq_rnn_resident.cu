@@ -41,12 +41,13 @@ struct RsParams {
     int I, k_w, gru, steps, batch;
     const float* x_seq; const float* h0; const float* c0;
     float* h_seq; float* h_last; float* c_last;
-    float* h[2];
+    unsigned long long* hx;     // [batch][H]: {h value, timestep}, from CTA to CTA
     const float* addend;        // [steps][batch][4H] added before the gates, or null
     uint32_t* counters;         // [blocks][64]: word 0 quantized shares, word 32 finished products
     int planes_word, h_word;    // where a block's CTAs look for them: 0 and 32 (the self-test of the waits: the next word, which stays 0)
+    uint32_t tag_bias;          // added to the timestep that is looked for in hx: 0 (self-test: 2^30)
     uint32_t* status;
-    int counted;                // timesteps in the counters at the start
+    int counted, launched;      // timesteps and launches in the counters at the start
     int P, block;               // CTAs and vectors of a block
     int upc, upt, tiles;        // units per CTA, per tile of 128 lanes
     int TB, N, NS;              // vectors and operand rows of a pass, slots of 256 positions
@@ -60,6 +61,61 @@ struct __align__(16) RsShared {
 };
 
 __device__ __forceinline__ uint32_t rs_upper_bits(int n) { return n >= 32 ? 0u : 0xffffffffu << (n < 0 ? 0 : n); }
+
+// h travels from the CTAs that compute it to those that quantize it as words {value, timestep}: value and "ready" arrive together, with no
+// fence in front of a counter and no load behind a wait (the same words as in amq_rnn_persistent.cu).  A reader never meets the words of
+// another call: it looks at them first in the second timestep, behind a counter, and a word is overwritten only after every
+// CTA of the block has seen the planes made of it.
+__device__ __forceinline__ unsigned long long rs_load_word(const unsigned long long* p)
+{
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ ulonglong2 rs_load_words(const unsigned long long* p)
+{
+    ulonglong2 v;
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void rs_store_word(unsigned long long* p, float value, uint32_t tag)
+{
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" :: "l"(p), "l"(((unsigned long long)tag << 32) | __float_as_uint(value)) : "memory");
+}
+
+// This thread's elements of h in z = [x ; h] from the words of timestep `tag`; false when they did not come.
+struct RsWords {
+    const unsigned long long* words;        // null: h is in memory as it is (the first timestep)
+    uint32_t tag;
+    unsigned limit;                         // looks at a word before giving up
+    template <int EPT>
+    __device__ __forceinline__ bool gather(const SeqVectors& a, int vector, int t0, float (&w)[EPT]) const
+    {
+        const unsigned long long* p = words + (size_t)vector * a.H + (t0 - a.xn);
+        const bool pairs = (reinterpret_cast<uintptr_t>(p) & 15u) == 0;
+        uint32_t pending = 0;
+#pragma unroll
+        for (int j = 0; j < EPT; ++j) pending |= (t0 + j >= a.xn && t0 + j < a.n ? 1u : 0u) << j;
+#pragma unroll 1
+        for (unsigned spins = 0; pending && spins < limit; ++spins) {
+            unsigned long long v[EPT];              // (all the loads, then all the looks: one round trip)
+            if (pairs && pending == (1u << EPT) - 1u) {
+#pragma unroll
+                for (int q = 0; q < EPT / 2; ++q) {
+                    const ulonglong2 two = rs_load_words(p + 2 * q);
+                    v[2 * q] = two.x; v[2 * q + 1] = two.y;
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < EPT; ++j) v[j] = (pending >> j) & 1u ? rs_load_word(p + j) : 0ull;
+            }
+#pragma unroll
+            for (int j = 0; j < EPT; ++j)
+                if (((pending >> j) & 1u) && (uint32_t)(v[j] >> 32) == tag) { w[j] = __uint_as_float((uint32_t)v[j]); pending &= ~(1u << j); }
+        }
+        return pending == 0;
+    }
+};
 
 // The CTA's plane-rows -> tensor memory, worker warp = (lane quarter, every fourth slot).  Bit 1 = -1 on both operands.
 __device__ __forceinline__ void rs_expand_weights(const RsParams& a, uint32_t a0, int u0, int warp, int lane)
@@ -197,24 +253,24 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
 #pragma unroll 1
     for (int t = 0; ok && t < a.steps; ++t) {
         const bool last = t + 1 == a.steps;
-        const float* h_prev = t == 0 ? a.h0 : (a.h_seq ? a.h_seq + (size_t)(t - 1) * a.batch * H : a.h[(t - 1) & 1]);
 
         // ---- 1. this CTA's share of the block's vectors ----
         if (part < quantizers) {                    // (uniform over the CTA)
-            if (t > 0) {
-                if (tid == 0) ok = seq_wait(counter + a.h_word, seq_target(a.counted + t, a.P));
+            if (t == 1) {                           // (the words of another call are gone)
+                if (tid == 0) ok = seq_wait(counter + a.h_word, seq_target(a.launched + 1, a.P));
                 if (__syncthreads_or(!ok)) { ok = false; break; }
             }
             const float* x = a.x_seq + (size_t)t * a.batch * a.z.xn;
 #pragma unroll 1
             for (int v = part + warp / NW * a.P; v < in_block; v += RS_WARPS / NW * a.P) {
-                seq_quantize<KA, 8, NW>(a.z, x, h_prev, b0 + v, scratch[warp / NW], quant, quant_parity);
+                ok &= seq_quantize<KA, 8, NW>(a.z, x, a.h0, b0 + v, scratch[warp / NW], quant, quant_parity,
+                                              RsWords{t == 0 ? nullptr : a.hx, (uint32_t)t + a.tag_bias, ok ? SEQ_POLL_LIMIT : 1u});
                 // the next timestep's inputs on their way into L2
                 const int e = (quant.warp * 32 + lane) * 8;
                 if (!last && e < a.z.xn)
                     asm volatile("prefetch.global.L2 [%0];" :: "l"(x + (size_t)(a.batch + b0 + v) * a.z.xn + e));
             }
-            __syncthreads();
+            if (__syncthreads_or(!ok)) { ok = false; break; }
             if (tid == 0) seq_publish(counter);
         }
         if (tid == 0) ok = seq_wait(counter + a.planes_word, seq_target(a.counted + t + 1, quantizers));
@@ -222,8 +278,7 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
         if (__syncthreads_or(!ok)) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
-        float* h_next = last ? a.h_last : (a.h_seq ? a.h_seq + (size_t)t * a.batch * H : a.h[t & 1]);
-        float* h_also = last && a.h_seq ? a.h_seq + (size_t)t * a.batch * H : nullptr;
+        float* h_seq = a.h_seq ? a.h_seq + (size_t)t * a.batch * H : nullptr;
 #pragma unroll 1
         for (int v0 = 0; v0 < in_block; v0 += a.TB, phase ^= 1u) {
             const int nv = in_block - v0 < a.TB ? in_block - v0 : a.TB, rows = nv * KA;
@@ -376,13 +431,14 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
                     h = (1.0f - zg) * cand + zg * *state;
                     *state = h;
                 }
-                h_next[o] = h;
-                if (h_also) h_also[o] = h;
+                if (last) a.h_last[o] = h;
+                else rs_store_word(a.hx + o, h, (uint32_t)t + 1);
+                if (h_seq) h_seq[o] = h;
             }
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         if (__syncthreads_or(!ok)) { ok = false; break; }
-        if (tid == 0) seq_publish(counter + 32);
+        if (t == 0 && tid == 0) seq_publish(counter + 32);
     }
 
     __syncwarp();
@@ -458,7 +514,9 @@ bool plan(const BatchedSequence& s, int sms, int only, RsPlan* out)
     a.z = SeqVectors{s.n, words_per_row(s.n), s.H, s.n - s.H, s.T, s.zcodes, s.zbeta, 16, (size_t)s.batch * s.k_a * 16};
     a.I = s.I; a.k_w = s.k_w; a.gru = s.gru; a.steps = s.steps; a.batch = s.batch;
     a.x_seq = s.x_seq; a.h0 = s.h0; a.c0 = s.c0; a.h_seq = s.h_seq; a.h_last = s.h_last; a.c_last = s.c_last;
-    a.h[0] = s.h[0]; a.h[1] = s.h[1]; a.addend = s.addend; a.counters = s.counters; a.counted = s.counted; a.status = s.status;
+    a.hx = reinterpret_cast<unsigned long long*>(s.h[0]);       // (the two states of the other forms, one behind the other)
+    a.launched = s.launched; a.tag_bias = s.late == 3 ? 1u << 30 : 0u;
+    a.addend = s.addend; a.counters = s.counters; a.counted = s.counted; a.status = s.status;
     a.planes_word = s.late == 1 ? 1 : 0; a.h_word = s.late == 2 ? 33 : 32;
     *out = p;
     return true;

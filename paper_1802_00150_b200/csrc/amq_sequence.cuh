@@ -37,21 +37,29 @@ struct SeqVectors {
     size_t row_bytes, half_bytes;       // distance of two plane-rows, of two 16-byte pieces of one
 };
 
-// Quantize one vector with a team of warps, thread g of the team owning the elements EPT g .. EPT g + EPT - 1.
-template <int KA, int EPT, int NW>
-__device__ __forceinline__ void seq_quantize(const SeqVectors& a, const float* x, const float* h, int vector,
-                                             QuantScratch<KA, NW>& sc, const QuantTeam& team, int& parity)
+// Where h is in memory as it is.
+struct SeqNoWords {
+    static constexpr void* words = nullptr;
+    template <int EPT> __device__ __forceinline__ bool gather(const SeqVectors&, int, int, float (&)[EPT]) const { return true; }
+};
+
+// Quantize one vector with a team of warps, thread g of the team owning the elements EPT g .. EPT g + EPT - 1.  Elements of h come from `h`,
+// or from `words` (whose gather may fail: false) where there are some.
+template <int KA, int EPT, int NW, typename Words = SeqNoWords>
+__device__ __forceinline__ bool seq_quantize(const SeqVectors& a, const float* x, const float* h, int vector,
+                                             QuantScratch<KA, NW>& sc, const QuantTeam& team, int& parity, const Words& words = Words{})
 {
     const int n = a.n, g = team.warp * 32 + ((int)threadIdx.x & 31), t0 = g * EPT;
     float w[EPT];
     uint32_t valid = 0;
     const float* xr = x + (size_t)vector * a.xn;
     const float* hr = h + (size_t)vector * a.H - a.xn;
+    const int end = words.words ? a.xn : n;         // elements read as they are
 #pragma unroll
     for (int q = 0; q < EPT / 4; ++q) {
         const int t = t0 + 4 * q;
         const float* p = (t < a.xn ? xr : hr) + t;
-        const bool one_piece = t + 3 < n && (t + 3 < a.xn || t >= a.xn) && (reinterpret_cast<uintptr_t>(p) & 15u) == 0;
+        const bool one_piece = t + 3 < end && (t + 3 < a.xn || t >= a.xn) && (reinterpret_cast<uintptr_t>(p) & 15u) == 0;
         if (one_piece) {
             const float4 v = __ldcg(reinterpret_cast<const float4*>(p));        // (h: written by other SMs)
             w[4 * q] = v.x; w[4 * q + 1] = v.y; w[4 * q + 2] = v.z; w[4 * q + 3] = v.w;
@@ -59,12 +67,12 @@ __device__ __forceinline__ void seq_quantize(const SeqVectors& a, const float* x
         } else {
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const bool ok = t + e < n;
-                w[4 * q + e] = ok ? __ldcg((t + e < a.xn ? xr : hr) + t + e) : 0.0f;
-                valid |= (ok ? 1u : 0u) << (4 * q + e);
+                w[4 * q + e] = t + e < end ? __ldcg((t + e < a.xn ? xr : hr) + t + e) : 0.0f;
+                valid |= (t + e < n ? 1u : 0u) << (4 * q + e);
             }
         }
     }
+    const bool ok = words.words ? words.gather(a, vector, t0, w) : true;
     float beta[KA];
     uint32_t bits[KA];
     quantize_group<KA, EPT, NW>(w, valid, n, quant_padding_consecutive(n, EPT), a.T, beta, bits, sc, nullptr, &parity, team);
@@ -81,6 +89,7 @@ __device__ __forceinline__ void seq_quantize(const SeqVectors& a, const float* x
         for (int i = 1; i < KA; ++i) b = (g == i) ? beta[i] : b;
         a.zbeta[(size_t)vector * KA + g] = b;
     }
+    return ok;
 }
 
 __device__ __forceinline__ float seq_logistic(float v) { return 1.0f / (1.0f + __expf(-v)); }

@@ -97,6 +97,54 @@ def test_batched_waits_that_run_out_set_the_status_and_leave_the_context_usable(
     assert all(torch.equal(g, w) for g, w in zip(got, want) if w is not None)
 
 
+@pytest.mark.parametrize("cell,I,H,batch,kw,ka", [
+    ("lstm", 64, 48, 9, 2, 2),              # words of h in pairs
+    ("gru", 301, 651, 150, 3, 2),           # single words, several vectors per team of warps
+    ("lstm", 1024, 1024, 64, 3, 3),
+])
+def test_states_that_never_come_set_the_status_and_leave_the_context_usable(amq, cell, I, H, batch, kw, ka):
+    """late 3 (weights in tensor memory): nobody sees the states of step 0 in step 1."""
+    steps, gru, form = 3, cell == "gru", 2
+    Wcodes, Walpha = amq.quantize(dev(synth.normal(((3 if gru else 4) * H, I + H), 0.08, 87, 1)), kw, 2)
+    xs = dev(synth.normal((steps, batch, I), 1.0, 87, 2))
+    h0, c0 = dev(synth.uniform((batch, H), -1, 1, 87, 3)), None if gru else dev(synth.uniform((batch, H), -1, 1, 87, 4))
+    args = (Wcodes, Walpha, None, I, H, xs, h0, c0, ka, 2)
+    ws = amq.new_workspace(I, H, batch, ka)
+    want = amq.selftest_batched_sequence(*args, amq.new_workspace(I, H, batch, ka), form)
+    h_seq, h_last, c_last = amq.selftest_batched_sequence(*args, ws, form, late=3)
+    assert amq.workspace_status(ws) == TIMEOUT
+    assert torch.all(h_last == 0) and (gru or torch.all(c_last == 0))       # outputs untouched
+    assert torch.equal(h_seq[0], want[0][0])                                # step 0 needs no state of another CTA
+    got = amq.selftest_batched_sequence(*args, ws, form)
+    assert amq.workspace_status(ws) == 0
+    assert all(torch.equal(g, w) for g, w in zip(got, want) if w is not None)
+
+
+@pytest.mark.parametrize("cell,I,H,batch,steps,kw,ka", [
+    ("lstm", 3, 1, 2, 9, 1, 1),             # one unit
+    ("gru", 7, 33, 5, 8, 2, 3),             # odd widths: single words
+    ("lstm", 0, 129, 17, 6, 3, 4),          # no inputs at all
+    ("lstm", 260, 256, 70, 5, 2, 2),        # a pair of words across x and h never
+    ("gru", 129, 127, 300, 4, 2, 2),        # several vectors per team, several passes
+])
+def test_states_travel_as_words_at_every_width(amq, cell, I, H, batch, steps, kw, ka):
+    """One launch, chunks of one step (each reads its state from memory, not from words) and the streaming form: the same steps.  Two calls on
+    one workspace: the words of the first are never taken for those of the second (the inputs differ)."""
+    gru = cell == "gru"
+    Wcodes, Walpha = amq.quantize(dev(synth.normal(((3 if gru else 4) * H, I + H), 0.08, 89, 1)), kw, 2)
+    ws = amq.new_workspace(I, H, batch, ka)
+    for seed in (2, 12):
+        xs = dev(synth.normal((steps, batch, I), 1.0, 89, seed)) if I else torch.empty((steps, batch, 0), device="cuda")
+        h, c = dev(synth.uniform((batch, H), -1, 1, 89, seed + 1)), None if gru else dev(synth.uniform((batch, H), -1, 1, 89, seed + 2))
+        h_seq, h_last, c_last = amq.selftest_batched_sequence(Wcodes, Walpha, None, I, H, xs, h, c, ka, 2, ws, 2)
+        assert amq.workspace_status(ws) == 0
+        fresh = amq.new_workspace(I, H, batch, ka)
+        for t in range(steps):
+            one, h, c = amq.selftest_batched_sequence(Wcodes, Walpha, None, I, H, xs[t:t + 1], h, c, ka, 2, fresh, 2)
+            assert torch.equal(one[0], h_seq[t])
+        assert torch.equal(h, h_last) and (gru or torch.equal(c, c_last))
+
+
 @pytest.mark.parametrize("late", [1, 2])
 @pytest.mark.parametrize("V,I,H", [(149, 33, 147), (3001, 96, 149), (42000, 1024, 1024)])
 def test_decoding_waits_that_run_out_set_the_status_and_leave_the_context_usable(amq, V, I, H, late):
