@@ -78,7 +78,7 @@ bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
             const int b = b0 + res_row_vector<KA>(q), j = res_row_plane<KA>(q);
             sBeta[q] = q < p.TB * KA && b < p.batch ? __ldcg(a.xbeta + (size_t)b * KA + j) : 0.0f;
         }
-        res_expand_activations<KA, 1>(p, a.xcodes, b0, sB);
+        res_expand_activations<KA, 1>(p, a.xcodes, (size_t)(p.wpr >> 2), 1, b0, sB);
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");

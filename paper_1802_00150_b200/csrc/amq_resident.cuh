@@ -168,10 +168,11 @@ template <int KA> __device__ __forceinline__ int res_row_vector(int row) { retur
 template <int KA> __device__ __forceinline__ int res_row_plane(int row) { return row / 8 % KA; }
 
 // Expand the planes of vectors b0 .. b0 + TB - 1 (all threads of the CTA; rows past the batch are zero nibbles).  The caller makes the
-// stores visible to the MMAs: every thread executes the proxy fence at the end, then a CTA barrier.  AHEAD (row, slot) pairs at a time:
+// stores visible to the MMAs: every thread executes the proxy fence at the end, then a CTA barrier.  `row_step`, `piece_step`: distance, in
+// 16-byte pieces, of two plane-rows and of two pieces of one.  AHEAD (row, slot) pairs at a time:
 // their loads overlap.
 template <int KA, int AHEAD>
-__device__ __forceinline__ void res_expand_activations(const ResProblem& p, const uint32_t* xcodes, int b0, uint32_t sB)
+__device__ __forceinline__ void res_expand_activations(const ResProblem& p, const uint32_t* xcodes, size_t row_step, size_t piece_step, int b0, uint32_t sB)
 {
     const int N = p.N;
     int row = (int)threadIdx.x % N, slot = (int)threadIdx.x / N;
@@ -189,10 +190,10 @@ __device__ __forceinline__ void res_expand_activations(const ResProblem& p, cons
 #pragma unroll
             for (int q = 0; q < 8; ++q) w[a][q] = 0;
             if (live[a]) {
-                const uint4* src = reinterpret_cast<const uint4*>(xcodes + ((size_t)b * KA + j) * p.wpr + w0);
+                const uint4* src = reinterpret_cast<const uint4*>(xcodes) + ((size_t)b * KA + j) * row_step + (size_t)(w0 >> 2) * piece_step;
                 const uint4 v0 = __ldcg(src);               // (other SMs wrote the planes: not through the read-only path)
                 w[a][0] = v0.x; w[a][1] = v0.y; w[a][2] = v0.z; w[a][3] = v0.w;
-                if (w0 + 4 < p.wpr) { const uint4 v1 = __ldcg(src + 1); w[a][4] = v1.x; w[a][5] = v1.y; w[a][6] = v1.z; w[a][7] = v1.w; }
+                if (w0 + 4 < p.wpr) { const uint4 v1 = __ldcg(src + piece_step); w[a][4] = v1.x; w[a][5] = v1.y; w[a][6] = v1.z; w[a][7] = v1.w; }
             }
             row += drow; slot += dslot;
             if (row >= N) { row -= N; ++slot; }

@@ -147,7 +147,7 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
             const int b = b0 + res_row_vector<KA>(tid), j = res_row_plane<KA>(tid);
             sh.beta[tid] = tid < p.TB * KA && b < p.batch ? __ldcg(a.z.zbeta + (size_t)b * KA + j) : 0.0f;
         }
-        res_expand_activations<KA, 2>(p, a.z.zcodes, b0, sB);
+        res_expand_activations<KA, 2>(p, a.z.zcodes, 1, (size_t)p.batch * KA, b0, sB);
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -292,7 +292,7 @@ bool plan(const BatchedSequence& s, int sms, int only, SeqPlan* out)
     const int blocks = (s.batch + a.p.TB - 1) / a.p.TB;
     a.b_bytes = a.p.NS * a.p.N * 128;
     a.bias = s.bias; a.H = s.H; a.steps = s.steps; a.k_a = s.k_a;
-    a.z = SeqVectors{s.n, a.p.wpr, s.H, s.n - s.H, s.T, s.zcodes, s.zbeta, (size_t)a.p.wpr * 4, 16};
+    a.z = SeqVectors{s.n, a.p.wpr, s.H, s.n - s.H, s.T, s.zcodes, s.zbeta, 16, (size_t)s.batch * s.k_a * 16};      // (pieces of all rows together: neighbouring lanes load neighbouring pieces)
     a.x_seq = s.x_seq; a.h0 = s.h0; a.c0 = s.c0; a.h_seq = s.h_seq; a.h_last = s.h_last; a.c_last = s.c_last;
     a.h[0] = s.h[0]; a.h[1] = s.h[1]; a.c = s.c; a.addend = s.addend;
     a.counters = s.counters; a.counted = s.counted; a.status = s.status;
