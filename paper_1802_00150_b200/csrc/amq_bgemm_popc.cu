@@ -254,7 +254,7 @@ amq_status product_call(const uint32_t* Wcodes, const float* Walpha, int m, int 
     GemmArgs a{};
     a.Wcodes = Wcodes; a.Walpha = Walpha; a.m = m; a.n = n; a.k_w = k_w;
     a.xcodes = xcodes; a.xbeta = xbeta; a.batch = batch; a.k_a = k_a;
-    a.bias = bias; a.epilogue = EPI_Y; a.y = y; a.ldy = ldy;
+    a.bias = bias; a.epilogue = EPI_Y; a.y = y; a.ldy = ldy; a.from_entry = true;
     *out = a;
     return AMQ_OK;
 }

@@ -19,6 +19,7 @@ struct ResGemmParams {
     float* y; int ldy;
     int mtiles, blocks;         // tiles of 128 rows, blocks of TB vectors
     int b_bytes;                // expanded activation operand
+    int early_weights;          // the kernel before does not write the weights: they may be fetched before it is through
     uint32_t* status;           // set when a bounded wait ran out
 };
 
@@ -95,7 +96,8 @@ bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
         auto start = [&](long long at) {
             feed.start(p, table, (int)(at % a.mtiles), 1, pass_tiles(at), r, ((warp >> 2) - first_step + R::GROUPS) % R::GROUPS);
         };
-        if (w < w_end) start(w);                    // (weights: no kernel of a chain writes them)
+        if (!a.early_weights) grid_dependency_wait();
+        if (w < w_end) start(w);                    // (no kernel of a chain writes the weights)
         grid_dependency_wait();                     // the planes and coefficients may come from the preceding kernel
         while (w < w_end) {
             load_block((int)(w / a.mtiles));
@@ -123,7 +125,7 @@ bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
         // coefficients of a tile's rows: thread te takes one of the 128 k_w, a tile ahead
         auto alpha_of = [&](int tile) {
             const int row = tile * 128 + (te & 127), plane = te >> 7;
-            return plane < p.k_w && row < p.units ? __ldg(p.Walpha + (size_t)row * p.k_w + plane) : 0.0f;
+            return plane < p.k_w && row < p.units ? __ldcg(p.Walpha + (size_t)row * p.k_w + plane) : 0.0f;
         };
         grid_dependency_wait();
         while (w < w_end) {
@@ -172,10 +174,10 @@ bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
                 const int row = (tile0 + t) * 128 + 4 * lane;
                 float4 bias = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
                 if (a.bias) {
-                    if (row < p.units) bias.x = __ldg(a.bias + row);
-                    if (row + 1 < p.units) bias.y = __ldg(a.bias + row + 1);
-                    if (row + 2 < p.units) bias.z = __ldg(a.bias + row + 2);
-                    if (row + 3 < p.units) bias.w = __ldg(a.bias + row + 3);
+                    if (row < p.units) bias.x = __ldcg(a.bias + row);
+                    if (row + 1 < p.units) bias.y = __ldcg(a.bias + row + 1);
+                    if (row + 2 < p.units) bias.z = __ldcg(a.bias + row + 2);
+                    if (row + 3 < p.units) bias.w = __ldcg(a.bias + row + 3);
                 }
                 ok = __all_sync(0xffffffffu, mbar_wait_relaxed(smem_u32(&sy.yfull), y_parity, &sy.failed));
                 y_parity ^= 1u;
@@ -244,6 +246,7 @@ bool plan(const GemmArgs& g, int sms, ResGemmPlan* out)
     const long long total = (long long)a.blocks * a.mtiles;
     out->grid = (int)(total < sms ? total : sms);
     out->smem = res_smem_bytes(a.p) + (size_t)a.p.TB * Y_LD * 4;
+    a.early_weights = !g.from_entry;
     out->vec_out = (reinterpret_cast<uintptr_t>(g.y) & 15) == 0 && g.ldy % 4 == 0;
     out->a = a;
     return true;
@@ -282,10 +285,10 @@ amq_status launch_binary_gemm_resident(const GemmArgs& g, cudaStream_t st)
     amq_status s = tc_status_word(&pl.a.status);
     if (s != AMQ_OK) return s;
     switch (g.k_a) {
-        case 1: return launch<1>(pl, g.overlap_with_previous, st);
-        case 2: return launch<2>(pl, g.overlap_with_previous, st);
-        case 3: return launch<3>(pl, g.overlap_with_previous, st);
-        case 4: return launch<4>(pl, g.overlap_with_previous, st);
+        case 1: return launch<1>(pl, g.overlap_with_previous || g.from_entry, st);
+        case 2: return launch<2>(pl, g.overlap_with_previous || g.from_entry, st);
+        case 3: return launch<3>(pl, g.overlap_with_previous || g.from_entry, st);
+        case 4: return launch<4>(pl, g.overlap_with_previous || g.from_entry, st);
     }
     return AMQ_ERR_UNSUPPORTED;
 }

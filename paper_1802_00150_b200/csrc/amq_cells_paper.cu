@@ -67,6 +67,7 @@ amq_status input_projection(const PaperCall& c, const uint32_t* xcodes, const fl
     a.Wcodes = c.Wi_codes; a.Walpha = c.Wi_alpha; a.m = 4 * c.H; a.n = c.I; a.k_w = c.k_w;
     a.xcodes = xcodes; a.xbeta = xbeta; a.batch = vectors; a.k_a = c.k_e;
     a.bias = c.bias; a.epilogue = EPI_Y; a.y = proj; a.ldy = 4 * c.H;
+    a.from_entry = true;
     a.same_for_any_batch = true;                // (a step and a sequence give the same bits)
     return launch_binary_gemm(a, st);
 }

@@ -215,5 +215,5 @@ extern "C" amq_status amq_quantize(const float* x, int rows, int n, int ldx, int
     if (rows == 0) return AMQ_OK;       // nothing to do; pointers of empty buffers may be NULL
     if (!x || !codes || !coeffs) return AMQ_ERR_INVALID_ARG;
     if (!amq::aligned16(codes)) return AMQ_ERR_ALIGNMENT;
-    return amq::launch_quantize(x, ldx, n, nullptr, 0, 0, rows, k, T, codes, coeffs, (cudaStream_t)stream);
+    return amq::launch_quantize(x, ldx, n, nullptr, 0, 0, rows, k, T, codes, coeffs, (cudaStream_t)stream, true);    // (waits first thing)
 }

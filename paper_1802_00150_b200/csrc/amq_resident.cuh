@@ -216,6 +216,14 @@ __device__ __forceinline__ void res_expand_activations(const ResProblem& p, cons
 constexpr int RES_TABLE = AMQ_MAX_K * 34;           // AMQ_MAX_N / 256 + 1 slots, in pairs
 constexpr uint32_t RES_STEP_NONE = 1u << 29, RES_STEP_HALF = 1u << 30, RES_STEP_H = 1u << 31;
 
+// (Not through the read-only path: with an overlapped launch the kernel before may still be writing the weights when this one starts.)
+__device__ __forceinline__ uint4 res_load(const uint4* p)
+{
+    uint4 v;
+    asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+
 // One group's share of the CTA's steps: the steps of all tiles in order are dealt to the groups in turn.  Thread = plane-row.  The
 // packed words of a step are fetched one of the group's steps ahead.  (Every instruction counts here: the expander warps
 // issue about one in ten clocks beside the other roles, and a group has three steps' time, some 1500 clocks, per step.)
@@ -266,17 +274,17 @@ struct ResFeeder {
         const uint4* src0 = reinterpret_cast<const uint4*>(row + (e.x & (RES_STEP_NONE - 1)));
         const uint4* src1 = reinterpret_cast<const uint4*>(row + (e.y & (RES_STEP_NONE - 1)));
         if (p.vec32) {
-            asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                          : "=r"(v[0][0].x), "=r"(v[0][0].y), "=r"(v[0][0].z), "=r"(v[0][0].w),
                            "=r"(v[0][1].x), "=r"(v[0][1].y), "=r"(v[0][1].z), "=r"(v[0][1].w) : "l"(src0));
-            asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                          : "=r"(v[1][0].x), "=r"(v[1][0].y), "=r"(v[1][0].z), "=r"(v[1][0].w),
                            "=r"(v[1][1].x), "=r"(v[1][1].y), "=r"(v[1][1].z), "=r"(v[1][1].w) : "l"(src1));
         } else {        // (a missing half keeps whatever was there: it meets zeros of the activation operand)
-            v[0][0] = __ldg(src0);
-            if (!(e.x & RES_STEP_HALF)) v[0][1] = __ldg(src0 + 1);
-            v[1][0] = __ldg(src1);
-            if (!(e.y & RES_STEP_HALF)) v[1][1] = __ldg(src1 + 1);
+            v[0][0] = res_load(src0);
+            if (!(e.x & RES_STEP_HALF)) v[0][1] = res_load(src0 + 1);
+            v[1][0] = res_load(src1);
+            if (!(e.y & RES_STEP_HALF)) v[1][1] = res_load(src1 + 1);
         }
         i += R::GROUPS;
         if (i >= n) next_tile(p, r);

@@ -192,5 +192,5 @@ extern "C" amq_status amq_log_softmax_argmax(const float* logits, int rows, int 
     if (rows < 0 || n < 1 || ld < n || (logp && ldp < n)) return AMQ_ERR_INVALID_ARG;
     if (rows == 0) return AMQ_OK;
     if (!logits || (!logp && !argmax)) return AMQ_ERR_INVALID_ARG;
-    return amq::launch_log_softmax_argmax(logits, rows, n, ld, logp, ldp, argmax, (cudaStream_t)stream, false);
+    return amq::launch_log_softmax_argmax(logits, rows, n, ld, logp, ldp, argmax, (cudaStream_t)stream, true);     // (waits first thing)
 }
