@@ -181,12 +181,15 @@ __device__ __forceinline__ float small_int_to_float(int v)
 }
 
 // Loads of what the preceding kernel of the stream may have produced (activation planes, their coefficients, added
-// pre-activations) are ordinary L2-cached loads (__ldcg), not read-only-path loads: with an overlapped launch this
+// pre-activations; from an entry point the weights too) are ordinary loads, not read-only-path loads: with an overlapped launch this
 // kernel is alive while those bytes are still being written, and a read-only load may be moved above the wait.
 
 __device__ __forceinline__ uint4 load_row_chunk(const uint4* p, bool weight_row)
 {
-    return weight_row ? __ldg(p) : __ldcg(p);       // weights are constant; activation planes: see above
+    if (!weight_row) return __ldcg(p);
+    uint4 v;
+    asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
 }
 
 // Two consecutive chunks of a packed row (32 bytes, 32-byte aligned) in one 256-bit load.  A warp-wide load of 16 bytes from
@@ -196,7 +199,7 @@ __device__ __forceinline__ uint4 load_row_chunk(const uint4* p, bool weight_row)
 __device__ __forceinline__ void load_row_chunk_pair(const uint4* p, bool weight_row, uint4& lo, uint4& hi)
 {
     if (weight_row)
-        asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                      : "=r"(lo.x), "=r"(lo.y), "=r"(lo.z), "=r"(lo.w), "=r"(hi.x), "=r"(hi.y), "=r"(hi.z), "=r"(hi.w) : "l"(p));
     else
         asm volatile("ld.global.cg.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
@@ -418,7 +421,7 @@ __device__ __forceinline__ void epilogue_smem_to_global(const TcParams& p, const
         if (a.epilogue == EPI_Y) {
             const int row = u0 + item;
             if (row >= a.m) continue;
-            const float bias = a.bias ? __ldg(a.bias + row) : 0.0f;
+            const float bias = a.bias ? __ldcg(a.bias + row) : 0.0f;
             const float* y0 = Yt + ((size_t)(mt * p.nseg) * TILE_M + li * k_w) * ldy;
             const int bend = (a.batch - b0 < TB) ? a.batch - b0 : TB;
             // four consecutive entries per item: one 128-bit load per plane, four stores (rows of y are entries)
@@ -438,7 +441,7 @@ __device__ __forceinline__ void epilogue_smem_to_global(const TcParams& p, const
             if (u >= H) continue;
             float bias4[4];
 #pragma unroll
-            for (int g = 0; g < 4; ++g) bias4[g] = a.bias ? __ldg(a.bias + g * H + u) : 0.0f;
+            for (int g = 0; g < 4; ++g) bias4[g] = a.bias ? __ldcg(a.bias + g * H + u) : 0.0f;
             const float* y0 = Yt + ((size_t)(mt * p.nseg) * TILE_M + li * 4 * k_w) * ldy;
             for (int bb = bsub; bb < TB && b0 + bb < a.batch; bb += bstep) {
                 float g4[4];
@@ -459,9 +462,9 @@ __device__ __forceinline__ void epilogue_smem_to_global(const TcParams& p, const
         } else {    // EPI_GRU
             const int H = a.H, u = u0 + item;
             if (u >= H) continue;
-            const float br = a.bias ? __ldg(a.bias + u) : 0.0f, bz = a.bias ? __ldg(a.bias + H + u) : 0.0f;
-            const float bnx = a.bias ? __ldg(a.bias + 2 * H + u) : 0.0f;
-            const float bnh = a.bias ? __ldg(a.bias + 3 * H + u) : 0.0f;
+            const float br = a.bias ? __ldcg(a.bias + u) : 0.0f, bz = a.bias ? __ldcg(a.bias + H + u) : 0.0f;
+            const float bnx = a.bias ? __ldcg(a.bias + 2 * H + u) : 0.0f;
+            const float bnh = a.bias ? __ldcg(a.bias + 3 * H + u) : 0.0f;
             const float* yx = Yt + ((size_t)(mt * 2 + 0) * TILE_M + li * 3 * k_w) * ldy;
             const float* yh = Yt + ((size_t)(mt * 2 + 1) * TILE_M + li * 3 * k_w) * ldy;
             for (int bb = bsub; bb < TB && b0 + bb < a.batch; bb += bstep) {
@@ -573,9 +576,9 @@ bgemm_tc_kernel(TcParams p)
                 if (j == 0) corr_src = coef_src;
             }
         }
-        // weight rows are fetched at once (no kernel of a chain writes them); everything the preceding kernel of the
+        // weight rows are fetched at once (no kernel of a chain writes them; from an entry point they wait as well); everything the preceding kernel of the
         // stream may have written (the activation planes and their coefficients, the state) is read after the wait
-        if (!weight_row) grid_dependency_wait();
+        if (!weight_row || a.from_entry) grid_dependency_wait();
         load_pair(grp, cur, cur2);                                  // own pairs: grp, grp + G, ..
         load_pair(grp + G, nxt, nxt2);
     }
@@ -890,7 +893,7 @@ bgemm_tc_persistent_kernel(TcParams p)
         };
         const int my_tiles = (ntiles - (int)blockIdx.x + tile_step - 1) / tile_step;
         const int total = my_tiles * STEPS;
-        if (!is_a) grid_dependency_wait();                          // activation planes come from the preceding kernel
+        if (!is_a || a.from_entry) grid_dependency_wait();                          // activation planes come from the preceding kernel
         uint4 cur, cur2, nxt, nxt2;
         pf_load(cur, cur2);
         pf_load(nxt, nxt2);
@@ -1012,7 +1015,7 @@ bgemm_tc_persistent_kernel(TcParams p)
                 const int l = div_small(r, k_w), i = r - l * k_w;
                 const int lg = div_small(l, p.gates);
                 const int u = u0 + mt * p.UT + lg, gate = l - lg * p.gates;
-                if (r < TMp && u < p.units) c_alpha = __ldg(a.Walpha + ((size_t)gate * p.units + u) * k_w + i);
+                if (r < TMp && u < p.units) c_alpha = __ldcg(a.Walpha + ((size_t)gate * p.units + u) * k_w + i);
             }
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
@@ -1233,7 +1236,7 @@ amq_status launch_ka(const TcPlan& pl, cudaStream_t st)
     auto kernel = pl.persistent ? (pl.p.fp4 ? bgemm_tc_persistent_kernel<KA, true> : bgemm_tc_persistent_kernel<KA, false>)
                                 : (pl.p.fp4 ? bgemm_tc_kernel<KA, true> : bgemm_tc_kernel<KA, false>);
     AMQ_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem));
-    if (pl.p.a.overlap_with_previous) {
+    if (pl.p.a.overlap_with_previous || pl.p.a.from_entry) {
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = pl.grid; cfg.blockDim = dim3((unsigned)pl.threads); cfg.dynamicSmemBytes = pl.smem; cfg.stream = st;
         cudaLaunchAttribute attr{};

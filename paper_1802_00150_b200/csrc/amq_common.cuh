@@ -109,8 +109,8 @@ struct GemmArgs {
     // the launch may start while the previous kernel of the stream (the on-line quantizer that produces xcodes / xbeta)
     // still runs: the kernel sets itself up, fetches weights, and waits for that kernel before it reads anything else
     bool overlap_with_previous;
-    // launched from an entry point behind whatever the caller's stream holds, which may be what writes the weights: an overlapped launch has to
-    // wait before it reads anything at all (the resident product does; the others are then not overlapped)
+    // launched from an entry point behind whatever the caller's stream holds, which may be what writes the weights: the two tensor-core products
+    // are overlapped all the same and wait before they read anything at all (the others are not overlapped)
     bool from_entry;
     // EPI_Y: the result of a vector may not depend on how many others are in the call (the two tensor-core products differ in the order of
     // their sums): the resident form wherever it covers the problem
