@@ -23,10 +23,11 @@ __device__ __forceinline__ float load_elem(const RowSource& s, int row, int t)
 // 32 l + 31 (eight 128-bit loads), so the sign word the quantizer leaves in a lane IS packed word l of the
 // plane and goes straight to memory, 128 contiguous bytes per warp and plane, with no ballot transposition.
 // Requires a single 16-byte-aligned source with a row stride that is a multiple of 4 elements.
-// At 3 and 4 bits 128 registers (four CTAs of four warps per SM) are faster than the 160 the compiler would take, at 2 bits 96 than 128:
-// 32768 x 1024 at 3 bits 62.4 us against 70.0, at 4 bits 160.7 against 168.5, at 2 bits 39.3 against 43.3.
+// At 3 bits 128 registers (four CTAs of four warps per SM) are faster than the 160 the compiler would take, at 2 bits 96 than 128:
+// 32768 x 1024 at 3 bits 62.4 us against 70.0, at 2 bits 39.3 against 43.3.  (Staged through shared memory, where a row is loaded in
+// contiguous pieces and the next one beside the quantizer, it took 68 to 74 us: registers.)
 template <int K>
-__global__ void __launch_bounds__(128, K >= 3 ? 4 : 5)
+__global__ void __launch_bounds__(128, K == 4 ? 0 : K == 3 ? 4 : 5)
 quantize_rows_consecutive_kernel(const float* __restrict__ x, int ldx, int rows, int n, int T,
                                  uint32_t* __restrict__ codes, float* __restrict__ coeffs)
 {

@@ -467,7 +467,7 @@ struct SignWord {
     }
 };
 
-// Codes of a thread's elements for levels that ascend by code index, K >= 3: plane i is decision i of the tree, the sign of w less the
+// Codes of a thread's elements for levels that ascend by code index, three bits: plane i is decision i of the tree, the sign of w less the
 // midpoint it compares with (the midpoints of the lower half are the negatives of the upper ones, `thr`).  SUMS: also csum[i] = sum of
 // b_i w, for which an element's own midpoints are chosen; without them every decision of a level is gathered as a word of bits and the
 // words are chosen from, which takes fewer instructions.
@@ -475,7 +475,8 @@ template <int K, int EPT, bool SUMS>
 __device__ __forceinline__ void ascending_pass(const float (&w)[EPT], const f32x2 (&w2)[EPT / 2], const float (&thr)[(1 << K) - 1],
                                                uint32_t positive, float abs_w, uint32_t valid, uint32_t (&bits)[K], float (&csum)[K])
 {
-    constexpr int M = 1 << K, M2 = M / 2;
+    static_assert(K == 3, "");
+    constexpr int M2 = 1 << (K - 1);
     const float t1 = thr[M2 - 1 + M2 / 2], t2o = thr[M2 - 1 + M2 / 2 + M2 / 4], t2i = thr[M2 - 1 + M2 / 4];
     bits[0] = positive & valid;
     csum[0] = abs_w;
@@ -506,17 +507,6 @@ __device__ __forceinline__ void ascending_pass(const float (&w)[EPT], const f32x
                 plane[2].add(2 * p, sa);
                 plane[2].add(2 * p + 1, sb);
             }
-            if constexpr (K == 4) {
-                unpack2(mul2(sw, d2), ea, eb);
-                const bool pa = (int)__float_as_uint(ea) >= 0, pb = (int)__float_as_uint(eb) >= 0;
-                const float ta = oa ? (pa ? thr[M - 2] : thr[M - 4]) : (pa ? thr[M2 + 2] : thr[M2]);
-                const float tb = ob ? (pb ? thr[M - 2] : thr[M - 4]) : (pb ? thr[M2 + 2] : thr[M2]);
-                unpack2(fma2(sw, pack2(-ta, -tb), w2[p]), da, db);
-                const float sa = unit_sign(da), sb = unit_sign(db);
-                s2[K - 1] = fma2(pack2(sa, sb), w2[p], s2[K - 1]);
-                plane[K - 1].add(2 * p, sa);
-                plane[K - 1].add(2 * p + 1, sb);
-            }
         }
 #pragma unroll
         for (int i = 1; i < K; ++i) {
@@ -544,11 +534,6 @@ __device__ __forceinline__ void ascending_pass(const float (&w)[EPT], const f32x
         const uint32_t b2 = (o1 & below[M2 / 2 + M2 / 4 - 1]) | (~o1 & below[M2 / 4 - 1]);
         bits[1] = ~b1 & valid;
         bits[2] = ~b2 & valid;
-        if constexpr (K == 4) {
-            const uint32_t o2 = positive ^ b2;
-            const uint32_t outer = (o2 & below[WORDS - 1]) | (~o2 & below[WORDS - 3]), inner = (o2 & below[2]) | (~o2 & below[0]);
-            bits[K - 1] = ~((o1 & outer) | (~o1 & inner)) & valid;
-        }
 #pragma unroll
         for (int i = 1; i < K; ++i) csum[i] = 0.0f;
     }
@@ -835,8 +820,7 @@ __device__ __forceinline__ void quantize_warp(const float (&w_in)[EPT], uint32_t
                 if (more) ascending_pass<K, EPT, true>(w, w2, thr, positive, abs_w, valid, bits, csum);
                 else ascending_pass<K, EPT, false>(w, w2, thr, positive, abs_w, valid, bits, csum);
             } else {
-                if constexpr (K == 3) ThreeLevels(alpha).template pass<EPT>(w, positive, abs_w, valid, more, bits, csum);
-                else sorted_pass<K, EPT>(w, alpha, positive, valid, more, thr, bits, csum);
+                ThreeLevels(alpha).template pass<EPT>(w, positive, abs_w, valid, more, bits, csum);
             }
         }
     }
@@ -861,7 +845,8 @@ __device__ __forceinline__ void quantize_group(const float (&w_in)[EPT], uint32_
                                                int* flag = nullptr, int* parity_io = nullptr,
                                                const QuantTeam& team = QuantTeam::cta())
 {
-    if constexpr (NW == 1) {
+    // (at four bits the warp's form gained 3 % on 32768 x 1024 and lost 7 % on 1704 x 896, where a row's chain of operations is what counts)
+    if constexpr (NW == 1 && K <= 3) {
         quantize_warp<K, EPT>(w_in, valid, n, pad_elems, T, alpha, bits, sc);
         return;
     }
@@ -989,35 +974,32 @@ __device__ __forceinline__ void quantize_group(const float (&w_in)[EPT], uint32_
             for (int i = 0; i < K; ++i) bits[i] = pos_bits[i] & valid;
             continue;
         }
-        if constexpr (K == 3) {
-            // (Bulk rows of more than 1024, 32 elements a thread, nearly always ascend, and a thread's registers count: 8192 x 3000 72 us
-            // this way, 82 to 84 with ThreeLevels for all or for the other rows.)
-            if constexpr (EPT == 32) {
-                if (ascending_levels<K>(alpha, thr)) {
-                    uint32_t below[K];
-                    float sum[K];
-#pragma unroll
-                    for (int i = 0; i < K; ++i) { below[i] = 0u; sum[i] = 0.0f; }
-#pragma unroll
-                    for (int j = EPT - 1; j >= 0; --j) {
-                        uint32_t d[K];
-                        tree_decisions<K, EPT>(w[j], thr, below, d);
-                        if (more) {
-#pragma unroll
-                            for (int i = 1; i < K; ++i) sum[i] += __uint_as_float(__float_as_uint(w[j]) ^ (d[i] & SIGN));
-                        }
-                    }
-                    bits[0] = positive & valid;
-                    csum[0] = abs_w;
-#pragma unroll
-                    for (int i = 1; i < K; ++i) { bits[i] = ~below[i] & valid; csum[i] = sum[i]; }
-                } else {
-                    sorted_pass<K, EPT>(w, alpha, positive, valid, more, thr, bits, csum);
-                }
-                continue;
-            }
+        if constexpr (K == 3 && EPT < 32) {
             ThreeLevels(alpha).template pass<EPT>(w, positive, abs_w, valid, more, bits, csum);
-            continue;
+        } else if constexpr (K >= 3) {
+            // A warp's rows of four bits, and bulk rows of more than 1024 at three bits, 32 elements a thread: they nearly always ascend, and a
+            // thread's registers count (8192 x 3000 at 3 bits 72 us this way, 82 to 84 with ThreeLevels for all or for the other rows).
+            if (ascending_levels<K>(alpha, thr)) {
+                uint32_t below[K];
+                float sum[K];
+#pragma unroll
+                for (int i = 0; i < K; ++i) { below[i] = 0u; sum[i] = 0.0f; }
+#pragma unroll
+                for (int j = EPT - 1; j >= 0; --j) {
+                    uint32_t d[K];
+                    tree_decisions<K, EPT>(w[j], thr, below, d);
+                    if (more) {
+#pragma unroll
+                        for (int i = 1; i < K; ++i) sum[i] += __uint_as_float(__float_as_uint(w[j]) ^ (d[i] & SIGN));
+                    }
+                }
+                bits[0] = positive & valid;
+                csum[0] = abs_w;
+#pragma unroll
+                for (int i = 1; i < K; ++i) { bits[i] = ~below[i] & valid; csum[i] = sum[i]; }
+            } else {
+                sorted_pass<K, EPT>(w, alpha, positive, valid, more, thr, bits, csum);
+            }
         }
     }
     if (parity_io) *parity_io = parity;

@@ -37,6 +37,16 @@ struct SeqVectors {
     size_t row_bytes, half_bytes;       // distance of two plane-rows, of two 16-byte pieces of one
 };
 
+// *p where `there`, else 0: a predicated load, so that several of them are in flight (as branches they were taken one after the other: a step
+// of GRU 64/479, two sequences, 14.2 us against 13.1).
+__device__ __forceinline__ float seq_load_if(const float* p, bool there)
+{
+    float v;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\tmov.f32 %0, 0f00000000;\n\t@p ld.global.cg.f32 %0, [%1];\n\t}"
+                 : "=f"(v) : "l"(p), "r"((int)there) : "memory");
+    return v;
+}
+
 // Where h is in memory as it is.
 struct SeqNoWords {
     static constexpr void* words = nullptr;
@@ -67,7 +77,7 @@ __device__ __forceinline__ bool seq_quantize(const SeqVectors& a, const float* x
         } else {
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                w[4 * q + e] = t + e < end ? __ldcg((t + e < a.xn ? xr : hr) + t + e) : 0.0f;
+                w[4 * q + e] = seq_load_if((t + e < a.xn ? xr : hr) + t + e, t + e < end);
                 valid |= (t + e < n ? 1u : 0u) << (4 * q + e);
             }
         }
