@@ -24,7 +24,7 @@ __device__ __forceinline__ float load_elem(const RowSource& s, int row, int t)
 // plane and goes straight to memory, 128 contiguous bytes per warp and plane, with no ballot transposition.
 // Requires a single 16-byte-aligned source with a row stride that is a multiple of 4 elements.
 // At 3 bits 128 registers (four CTAs of four warps per SM) are faster than the 160 the compiler would take, at 2 bits 96 than 128:
-// 32768 x 1024 at 3 bits 62.4 us against 70.0, at 2 bits 39.3 against 43.3.  (Staged through shared memory, where a row is loaded in
+// 32768 x 1024 at 3 bits 65.9 us against 70, at 2 bits 42.4 against 47.  (Staged through shared memory, where a row is loaded in
 // contiguous pieces and the next one beside the quantizer, it took 68 to 74 us: registers.)
 template <int K>
 __global__ void __launch_bounds__(128, K == 4 ? 0 : K == 3 ? 4 : 5)

@@ -16,8 +16,9 @@
 // logic operation; the refit sums of a cycle are accumulated in the same pass that assigns the codes.
 // A warp of its own (bulk quantization) is bound by the integer pipe, 64 lanes a clock, and by issue slots, while the fp32 pipe has 128
 // lanes and two-wide instructions: there one logic operation makes s = +-1 of a sign bit, a residue is r - a s, |r| is s r and
-// the refit sums add s w, multiply-adds for two elements at a time (the products are exact: rounded as the plain sums), and a word of
-// sign bits is the exact sum of s 2^j over sixteen elements.  32768 x 1024 at 3 bits 78 -> 62 us, at 2 bits 58 -> 39.  A team's
+// the refit sums add s w, multiply-adds (the products are exact: rounded as the plain sums, which are taken in the same order: the same
+// bits as a team's way of writing it), two elements wide where they are no sums, and a word of
+// sign bits is the exact sum of s 2^j over sixteen elements.  32768 x 1024 at 3 bits 78 -> 66 us, at 2 bits 58 -> 42.  A team's
 // quantizer is a chain of dependent operations, which the multiply-adds make longer: LSTM sequence 1024, one sequence, 154 -> 159 us,
 // decoding 674 -> 730; there it stays as it was.
 // Elements past the end of the vector are zeros that take part in every loop unmasked: their bits are
@@ -440,13 +441,6 @@ __device__ __forceinline__ int bst_leaf(float x, const float (&thr)[(1 << K) - 1
 // +1.0 or -1.0 with the sign of x
 __device__ __forceinline__ float unit_sign(float x) { return __uint_as_float((__float_as_uint(x) & 0x80000000u) | 0x3f800000u); }
 
-__device__ __forceinline__ float pair_sum(f32x2 v)
-{
-    float x, y;
-    unpack2(v, x, y);
-    return x + y;
-}
-
 // Signs s = +-1 of a thread's elements gathered as a word (bit j: s_j = +1).  Up to sixteen terms s_j 2^j plus 2^16 - 1 are twice that
 // word, exactly; halved and added to 2^23 it stands in the low bits of the sum.
 template <int EPT>
@@ -481,12 +475,12 @@ __device__ __forceinline__ void ascending_pass(const float (&w)[EPT], const f32x
     bits[0] = positive & valid;
     csum[0] = abs_w;
     if constexpr (SUMS) {
-        f32x2 s2[K];
+        float sum[K];
         SignWord<EPT> plane[K];
 #pragma unroll
-        for (int i = 1; i < K; ++i) s2[i] = 0ull;
+        for (int i = 1; i < K; ++i) sum[i] = 0.0f;
 #pragma unroll
-        for (int p = 0; p < EPT / 2; ++p) {
+        for (int p = EPT / 2 - 1; p >= 0; --p) {
             const f32x2 sw = pack2(unit_sign(w[2 * p]), unit_sign(w[2 * p + 1]));
             const f32x2 d1 = fma2(sw, pack2(-t1, -t1), w2[p]);
             float ea, eb, da, db;
@@ -495,7 +489,8 @@ __device__ __forceinline__ void ascending_pass(const float (&w)[EPT], const f32x
             const bool oa = (int)__float_as_uint(ea) >= 0, ob = (int)__float_as_uint(eb) >= 0;
             {
                 const float sa = unit_sign(da), sb = unit_sign(db);
-                s2[1] = fma2(pack2(sa, sb), w2[p], s2[1]);
+                sum[1] = fmaf(sb, w[2 * p + 1], sum[1]);
+                sum[1] = fmaf(sa, w[2 * p], sum[1]);
                 plane[1].add(2 * p, sa);
                 plane[1].add(2 * p + 1, sb);
             }
@@ -503,14 +498,15 @@ __device__ __forceinline__ void ascending_pass(const float (&w)[EPT], const f32x
             unpack2(d2, da, db);
             {
                 const float sa = unit_sign(da), sb = unit_sign(db);
-                s2[2] = fma2(pack2(sa, sb), w2[p], s2[2]);
+                sum[2] = fmaf(sb, w[2 * p + 1], sum[2]);
+                sum[2] = fmaf(sa, w[2 * p], sum[2]);
                 plane[2].add(2 * p, sa);
                 plane[2].add(2 * p + 1, sb);
             }
         }
 #pragma unroll
         for (int i = 1; i < K; ++i) {
-            csum[i] = pair_sum(s2[i]);
+            csum[i] = sum[i];
             bits[i] = plane[i].word() & valid;
         }
     } else {
@@ -599,7 +595,7 @@ struct ThreeLevels {
     {
         constexpr uint32_t SIGN = 0x80000000u;
         uint32_t below1 = 0u, below2 = 0u;
-        float s1 = 0.0f, s2 = 0.0f, innermost = 0.0f;
+        float s1 = 0.0f, s2 = 0.0f;
 #pragma unroll
         for (int j = EPT - 1; j >= 0; --j) {
             const uint32_t wb = __float_as_uint(w[j]), sw = wb & SIGN;
@@ -614,17 +610,19 @@ struct ThreeLevels {
             }
         }
         uint32_t plane[3] = {positive, ~below1, ~below2};
+        float sum[3] = {abs_w, s1, s2};
         if (flip) {
             const uint32_t leaf = (positive ^ plane[1]) & (positive ^ plane[2]);
 #pragma unroll
-            for (int i = 0; i < 3; ++i) plane[i] ^= leaf;
-            if (sums) {
+            for (int i = 0; i < 3; ++i) {
+                plane[i] ^= leaf;
+                if (sums) {                         // (element by element, in the order of the other sums)
+                    sum[i] = 0.0f;
 #pragma unroll
-                for (int j = 0; j < EPT; ++j) innermost += (leaf >> j) & 1u ? fabsf(w[j]) : 0.0f;
+                    for (int j = EPT - 1; j >= 0; --j) sum[i] += __uint_as_float(__float_as_uint(w[j]) ^ (~(plane[i] << (31 - j)) & SIGN));
+                }
             }
         }
-        // an innermost element adds |w|, -|w|, -|w| unflipped
-        const float sum[3] = {fmaf(-2.0f, innermost, abs_w), fmaf(2.0f, innermost, s1), fmaf(2.0f, innermost, s2)};
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             const uint32_t b = rank[i] == 0 ? plane[0] : rank[i] == 1 ? plane[1] : plane[2];
@@ -721,22 +719,21 @@ __device__ __forceinline__ void quantize_warp(const float (&w_in)[EPT], uint32_t
                 bits[0] = positive & valid;
                 csum[0] = abs_w = part;
             } else {
-                f32x2 part2 = 0ull, cs2 = 0ull;
+                float cs = 0.0f;
                 SignWord<EPT> plane;
 #pragma unroll
-                for (int p = 0; p < EPT / 2; ++p) {
+                for (int p = EPT / 2 - 1; p >= 0; --p) {
                     float ra, rb;
                     unpack2(r2[p], ra, rb);
                     const float sa = unit_sign(ra), sb = unit_sign(rb);
-                    const f32x2 s = pack2(sa, sb);
-                    part2 = fma2(s, r2[p], part2);                // |r|
-                    cs2 = fma2(s, w2[p], cs2);                    // b_i w
+                    part += fabsf(rb); part += fabsf(ra);
+                    cs = fmaf(sb, w[2 * p + 1], cs);              // b_i w
+                    cs = fmaf(sa, w[2 * p], cs);
                     plane.add(2 * p, sa);
                     plane.add(2 * p + 1, sb);
                 }
                 bits[i] = plane.word() & valid;
-                csum[i] = pair_sum(cs2);
-                part = pair_sum(part2);
+                csum[i] = cs;
             }
             part = holds_some ? part : 0.0f;
             if (i == K - 1 && T > 0) { last_abs = part; alpha[i] = 0.0f; break; }
@@ -745,14 +742,17 @@ __device__ __forceinline__ void quantize_warp(const float (&w_in)[EPT], uint32_t
             group_totals<1, 0, K, 1>(tot, none, sc, 0, nullptr, none_team);
             const float a = (tot[0] - padding * fabsf(rho)) * inv_n;
             alpha[i] = a;
-            const f32x2 minus = pack2(-a, -a);
-            rho = fmaf(unit_sign(rho), -a, rho);
+            const uint32_t ab = __float_as_uint(a);               // a >= 0, but for a rounding of a vanishing one
+            rho -= __uint_as_float(ab | (__float_as_uint(rho) & 0x80000000u));
             if (i == K - 1) break;                                // (T = 0: no residue is needed any more)
+            const uint32_t sign = ~ab & 0x80000000u;              // (a team takes a negative coefficient off every residue as it is)
+            const f32x2 minus = pack2(-a, -a);
 #pragma unroll
             for (int p = 0; p < EPT / 2; ++p) {                   // r - a sign(r)
                 float ra, rb;
                 unpack2(r2[p], ra, rb);
-                r2[p] = fma2(pack2(unit_sign(ra), unit_sign(rb)), minus, r2[p]);
+                r2[p] = fma2(pack2(__uint_as_float((__float_as_uint(ra) & sign) | 0x3f800000u), __uint_as_float((__float_as_uint(rb) & sign) | 0x3f800000u)),
+                             minus, r2[p]);
             }
         }
     }
@@ -791,18 +791,17 @@ __device__ __forceinline__ void quantize_warp(const float (&w_in)[EPT], uint32_t
             uint32_t below = 0;
             float s1 = 0.0f;
             if (more) {
-                f32x2 s2 = 0ull;
                 SignWord<EPT> plane;
 #pragma unroll
-                for (int p = 0; p < EPT / 2; ++p) {
+                for (int p = EPT / 2 - 1; p >= 0; --p) {
                     float da, db;
                     unpack2(fma2(pack2(unit_sign(w[2 * p]), unit_sign(w[2 * p + 1])), minus, w2[p]), da, db);
                     const float sa = unit_sign(da), sb = unit_sign(db);
-                    s2 = fma2(pack2(sa, sb), w2[p], s2);
+                    s1 = fmaf(sb, w[2 * p + 1], s1);
+                    s1 = fmaf(sa, w[2 * p], s1);
                     plane.add(2 * p, sa);
                     plane.add(2 * p + 1, sb);
                 }
-                s1 = pair_sum(s2);
                 below = ~plane.word();
             } else {
 #pragma unroll

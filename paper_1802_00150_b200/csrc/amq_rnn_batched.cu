@@ -13,8 +13,8 @@
 // machine, which had become longer than the kernels), the set-up of tensor memory and barriers, and the repeated expansion
 // of the activation planes by every tile of weight rows.  What bounds a timestep now: the steps of the weight pipeline (240-300
 // clocks per 256 bit positions of 128 plane-rows), the quantizer's chain of reductions, and the two waits (GRU 2048, 256 sequences,
-// 2/3 bits, clocks of a timestep: wait for h 1650, quantizer 12200, publish and wait for planes 2700, expansion of the activations
-// 8700, weights 42900, last epilogue 4500, publish 1650).
+// 2/3 bits, 32 vectors a block, clocks of a timestep: wait for h 1700, quantizer 12100, publish and wait for planes 2800, expansion of the
+// activations 4700, weights 37000, last epilogue 5900, publish 1100).
 #include "amq_resident.cuh"
 #include "amq_sequence.cuh"
 

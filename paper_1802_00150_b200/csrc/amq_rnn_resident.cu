@@ -16,9 +16,9 @@
 // are r, z and the x and h parts of the candidate: positions that a row does not have (the other part, past n) are zero nibbles,
 // which add nothing, so the activation operand needs no masks and no split.
 //
-// Measured (clocks of a timestep, 64 vectors, 1024 units, n = 2048, 3 bits; 147 CTAs, 394 us for 35 timesteps against 508 us): wait for h
-// 1150, quantizer 6750, publish 1550, wait for planes 1350, their loads 1350, expansion 2850, rest of the MMAs 2350, folding 1850,
-// gates 1950, publish 1050.
+// Measured (clocks of a timestep, 64 vectors, 1024 units, n = 2048, 3 bits; 147 CTAs, 368 us for 35 timesteps): words of h and quantizer 7050,
+// publish 1650, wait for planes 1500, their loads 1700, expansion 2400, rest of the MMAs 2250, folding 1850, gates 1850.  (With h in
+// memory behind a counter 394 us: wait for h 1150, publish 1050 more; streamed weights 508 us.)
 //
 // More vectors than one accumulator (N <= 256 operand rows) or shared memory holds are taken in passes over the same weights.
 #include "amq_sequence.cuh"
