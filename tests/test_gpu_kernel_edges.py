@@ -226,3 +226,25 @@ def test_three_bits_whose_levels_do_not_ascend(amq, n, small):
     a = np.abs(gpu(x, 3, 1)[1])                     # (what the last cycle's table is made of, but for one refit)
     if n > 9:
         assert (a[:, 0] < a[:, 1] + a[:, 2]).any() or (np.argsort(-a, axis=1) != np.arange(3)).any()
+
+
+@pytest.mark.parametrize("n,kw,ka", [
+    (13 * 128 - 5, 2, 2),               # four chunks of 128 bits for the first lane of a row's segment only
+    (16 * 128, 2, 3), (17 * 128, 2, 1),  # for all, and one left over
+    (6 * 128, 3, 2), (7 * 128, 3, 2),   # none, the first
+    (31 * 128 + 1, 4, 4),               # several groups and a remainder
+    (25 * 128, 1, 2),
+])
+def test_one_sequence_lstm_at_the_edges_of_its_groups_of_chunks(amq, n, kw, ka):
+    """Bit counts through full adders, sixteen words at a time, and word by word for what is left.  Tolerance: that of a step's state (three
+    times the product's 1e-3 of the largest possible pre-activation), on the device's own weight codes."""
+    H, I = 40, n - 40
+    Wc, Wa = quantized((4 * H, n), 0.03, kw, 500 + n, 1)
+    x, h, c = synth.normal((1, I), 1.0, 500 + n, 2), synth.uniform((1, H), -1, 1, 500 + n, 3), synth.uniform((1, H), -1, 1, 500 + n, 4)
+    bias = synth.normal((4 * H,), 0.1, 500 + n, 5)
+    got = amq.lstm_step(cdev(Wc), dev(Wa), dev(bias), I, H, dev(x), dev(h), dev(c), ka, 2, amq.new_workspace(I, H, 1, ka))
+    want = oracle.lstm_step(Wc, Wa, bias.astype(np.float64), I, H, x, h, c, ka, 2)
+    _, beta = oracle.quantize_rows(np.concatenate([x, h], axis=1).astype(np.float64), ka, 2)
+    tol = 3e-3 * np.abs(Wa).sum(axis=1).max() * np.abs(beta).sum()
+    for g, w in zip(got, want):
+        assert np.abs(g.cpu().numpy() - w).max() <= tol
