@@ -58,7 +58,9 @@ bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
     };
 
     if (tid == 0) res_sync_init<R>(sy);
+    res_fill_table(p, table);
     if (warp == R::MMA_WARP) {
+        if (!a.early_weights) grid_dependency_wait();       // (a foreign kernel in front may still want tensor memory)
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      :: "r"(smem_u32(&sy.tmem_slot)), "r"((uint32_t)RES_TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -68,8 +70,6 @@ bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = __shfl_sync(0xffffffffu, sy.tmem_slot, 0);
     if (warp < 4) write_unit_scales(tmem, p.ring * p.N, warp);
-
-    res_fill_table(p, table);
     __syncthreads();
 
     // expand the activations of block bb; all threads, ends with a CTA barrier

@@ -125,7 +125,9 @@ __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepco
 
 // Launch `kernel`, as a programmatic dependent of the preceding kernel of the stream when `overlap` is set (the kernel
 // must then execute grid_dependency_wait() before it reads or writes anything another kernel of the chain touches,
-// and read such data with ordinary loads, not through the read-only path).
+// and read such data with ordinary loads, not through the read-only path).  From an entry point the preceding kernel may be
+// anybody's, and may signal its dependents long before it is through: nothing that it may still need (tensor memory) is
+// taken before the wait, and no bounded wait begins before it.
 template <typename... Params, typename... Args>
 inline cudaError_t launch_kernel(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool overlap,
                                  Args... args)
