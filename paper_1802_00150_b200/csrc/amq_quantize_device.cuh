@@ -565,15 +565,21 @@ struct TwoLevels {
 };
 
 // The table of three bits.  With the coefficients' magnitudes A >= B >= C the levels of its upper half are, in order, |A - B - C|, A - B + C,
-// A + B - C and A + B + C, whatever the coefficients: the planes of A, B and C are the tree's three decisions, but for the
-// elements at the innermost level on either side, all of whose signs are the opposite ones where A < B + C.  So any order of the
-// coefficients costs a sort of the four values (no codes travel with them) and a permutation of the finished words.  (On z = [x ; h] the
-// levels seldom ascend by code: with the codes sorted along and the planes evaluated leaf by leaf a cycle's codes took a team of eight warps
-// 1000 to 1130 clocks, where ascending levels take 300 to 470.)
+// A + B - C and A + B + C: the planes of A, B and C are the tree's three decisions, but for the elements at the innermost level on either
+// side, all of whose signs are the opposite ones where A < B + C.  So any order of the coefficients costs the four values (no codes
+// travel with them) and a permutation of the finished words.  (On z = [x ; h] the levels seldom ascend by code: with the codes sorted along
+// and the planes evaluated leaf by leaf a cycle's codes took a team of eight warps 1000 to 1130 clocks, where ascending levels take 300 to 470.)
+// Levels that tie go by the order of their codes, and rounded sums of coefficients that differ by less than the rounding may tie or even come in
+// another order than the exact ones.  `regular`: the smallest magnitude, the differences of any two and the innermost level are all above
+// 2^-20 of the sum S, so that no two levels, each two sums within 2^-24 S of the exact ones, change places or meet.  Anything else,
+// infinities and NaN among it, is sorted: the same codes as without ThreeLevels, always.  (Told from the magnitudes and not from the sorted
+// levels, whose chain is the longer one.  35 steps of LSTM 1024, one sequence, 3/3 bits: 206 us without the question, 209.5 with it, 211.3
+// from the sorted levels, 232 with every table sorted; 64 sequences 374, 378, 377, 396; the sorting as a call of its own, behind the pass,
+// or sharing its loop over the elements: no faster there and slower in amq_quantize.)
 struct ThreeLevels {
     float inner, mid, outer;        // midpoints of the upper half
     int rank[3];                    // 0: the largest magnitude; among equals the smaller index first
-    bool neg[3], flip;
+    bool neg[3], flip, regular;
     __device__ __forceinline__ ThreeLevels(const float (&a)[3])
     {
         const float m0 = fabsf(a[0]), m1 = fabsf(a[1]), m2 = fabsf(a[2]);
@@ -587,6 +593,8 @@ struct ThreeLevels {
         const float x = fmaxf(l1, l2), y = fminf(h1, h2), q0 = fminf(l1, l2), q1 = fminf(x, y), q2 = fmaxf(x, y), q3 = fmaxf(h1, h2);
         inner = (q0 + q1) * 0.5f; mid = (q1 + q2) * 0.5f; outer = (q2 + q3) * 0.5f;
         flip = ((rank[0] == 0 ? m0 : -m0) + (rank[1] == 0 ? m1 : -m1)) + (rank[2] == 0 ? m2 : -m2) < 0.0f;
+        const float least = fminf(fminf(m0, fabsf(m0 - m1)), fminf(m1, fabsf(m1 - m2)));
+        regular = fminf(fminf(least, q0), fminf(m2, fabsf(m0 - m2))) > ((m0 + m1) + m2) * 0x1p-20f;     // (false where the sum is infinite or NaN)
     }
     // Codes of a thread's elements; `sums`: also csum[i] = sum of b_i w.
     template <int EPT>
@@ -676,6 +684,16 @@ __device__ __forceinline__ void sorted_pass(const float (&w)[EPT], const float (
             csum[i] = cs;
         }
     }
+}
+
+// Three bits, coefficients in any order: the same codes and sums as sorted_pass gives, by way of ThreeLevels where that is sure.
+template <int EPT>
+__device__ __forceinline__ void three_bit_codes(const float (&w)[EPT], const float (&alpha)[3], uint32_t positive, float abs_w, uint32_t valid,
+                                                bool sums, float (&thr)[7], uint32_t (&bits)[3], float (&csum)[3])
+{
+    const ThreeLevels t(alpha);
+    if (t.regular) t.template pass<EPT>(w, positive, abs_w, valid, sums, bits, csum);
+    else sorted_pass<3, EPT>(w, alpha, positive, valid, sums, thr, bits, csum);
 }
 
 // quantize_group of a warp of its own: the same steps with two-wide multiply-adds (see above).
@@ -819,7 +837,7 @@ __device__ __forceinline__ void quantize_warp(const float (&w_in)[EPT], uint32_t
                 if (more) ascending_pass<K, EPT, true>(w, w2, thr, positive, abs_w, valid, bits, csum);
                 else ascending_pass<K, EPT, false>(w, w2, thr, positive, abs_w, valid, bits, csum);
             } else {
-                ThreeLevels(alpha).template pass<EPT>(w, positive, abs_w, valid, more, bits, csum);
+                three_bit_codes<EPT>(w, alpha, positive, abs_w, valid, more, thr, bits, csum);
             }
         }
     }
@@ -974,7 +992,7 @@ __device__ __forceinline__ void quantize_group(const float (&w_in)[EPT], uint32_
             continue;
         }
         if constexpr (K == 3 && EPT < 32) {
-            ThreeLevels(alpha).template pass<EPT>(w, positive, abs_w, valid, more, bits, csum);
+            three_bit_codes<EPT>(w, alpha, positive, abs_w, valid, more, thr, bits, csum);
         } else if constexpr (K >= 3) {
             // A warp's rows of four bits, and bulk rows of more than 1024 at three bits, 32 elements a thread: they nearly always ascend, and a
             // thread's registers count (8192 x 3000 at 3 bits 72 us this way, 82 to 84 with ThreeLevels for all or for the other rows).
