@@ -4,13 +4,13 @@
 // lanes; expanded to E2M1 nibbles ONCE, they lie in tensor memory (n / 8 columns per tile) for the whole sequence.  A timestep is, in
 // every CTA: quantize the own share of the vectors z = [x_t ; h_{t-1}] (Algorithm 2), wait for the other shares, expand the planes
 // of all vectors into shared memory slot by slot while the MMAs of the finished slots run, fold the accumulators with the
-// coefficients, apply the gates, wait for the other CTAs' h.
+// coefficients, apply the gates, store h as words that the others' quantizers look for.
 //
 // Against streaming the packed weights through an expander every timestep (amq_rnn_batched.cu) this takes the weights out of the loop: at
 // n = 2048, 1024 units, 64 vectors, 3 bits each the product phase was 16600 of a timestep's 30000 clocks, most of it the expansion
 // of 128 plane-rows x 3 per CTA; here the CTAs expand the activations instead, which are fewer.  What bounds a timestep now: the
-// quantizer's chain of reductions, the two waits (an L2 round trip and an atomic each), the tensor pipe (N / 2 clocks per 64
-// positions) where N is large.
+// quantizer's chain of reductions, the wait for the words of h (an L2 round trip) and for the planes (that, a fence and an atomic), the tensor
+// pipe (N / 2 clocks per 64 positions) where N is large.
 //
 // Plane-rows: lane 4 k_w u + k_w g + i of a tile = plane i of gate g of unit u, as many whole units as fit 128 lanes.  The four "gates" of a GRU
 // are r, z and the x and h parts of the candidate: positions that a row does not have (the other part, past n) are zero nibbles,
@@ -66,6 +66,10 @@ __device__ __forceinline__ uint32_t rs_upper_bits(int n) { return n >= 32 ? 0u :
 // fence in front of a counter and no load behind a wait (the same words as in amq_rnn_persistent.cu).  A reader never meets the words of
 // another call: it looks at them first in the second timestep, behind a counter, and a word is overwritten only after every
 // CTA of the block has seen the planes made of it.
+// The words also keep the planes and coefficients of a timestep from being overwritten too soon, which no counter does: a vector's words are
+// stored only after the CTA has consumed all that vector's planes and coefficients (they are in its shared memory, multiplied and folded, by
+// the time its gates run), and the quantizer that writes the next ones waits for the words of every unit, so of every CTA of the block
+// (each has units).  Planes loaded ahead, or words stored before the fold, would break that: then they need a buffer per parity.
 __device__ __forceinline__ unsigned long long rs_load_word(const unsigned long long* p)
 {
     unsigned long long v;

@@ -128,8 +128,7 @@ def test_states_that_never_come_set_the_status_and_leave_the_context_usable(amq,
     ("gru", 129, 127, 300, 4, 2, 2),        # several vectors per team, several passes
 ])
 def test_states_travel_as_words_at_every_width(amq, cell, I, H, batch, steps, kw, ka):
-    """One launch, chunks of one step (each reads its state from memory, not from words) and the streaming form: the same steps.  Two calls on
-    one workspace: the words of the first are never taken for those of the second (the inputs differ)."""
+    """One launch and launches of one step each (which read their state from memory, not from words): the same steps, twice on one workspace."""
     gru = cell == "gru"
     Wcodes, Walpha = amq.quantize(dev(synth.normal(((3 if gru else 4) * H, I + H), 0.08, 89, 1)), kw, 2)
     ws = amq.new_workspace(I, H, batch, ka)
@@ -143,6 +142,52 @@ def test_states_travel_as_words_at_every_width(amq, cell, I, H, batch, steps, kw
             one, h, c = amq.selftest_batched_sequence(Wcodes, Walpha, None, I, H, xs[t:t + 1], h, c, ka, 2, fresh, 2)
             assert torch.equal(one[0], h_seq[t])
         assert torch.equal(h, h_last) and (gru or torch.equal(c, c_last))
+
+
+@pytest.mark.parametrize("cell,I,H,batch,kw,ka", [("lstm", 64, 48, 9, 2, 2), ("gru", 300, 650, 20, 3, 2), ("lstm", 1024, 1024, 64, 3, 3), ("gru", 129, 127, 300, 2, 2)])
+def test_words_of_an_earlier_call_are_not_taken_for_this_calls(amq, cell, I, H, batch, kw, ka):
+    """A call of two steps leaves words of timestep 1 behind, the ones that the next call on the workspace looks for in its second step: behind
+    the count of that call's first products, when they have been overwritten.  Other inputs every time, without a synchronisation in between."""
+    gru = cell == "gru"
+    Wcodes, Walpha = amq.quantize(dev(synth.normal(((3 if gru else 4) * H, I + H), 0.08, 90, 1)), kw, 2)
+    ws = amq.new_workspace(I, H, batch, ka)
+    calls = []
+    for r, steps in enumerate((2, 2, 5, 2, 3, 2, 2, 4)):
+        calls.append((dev(synth.normal((steps, batch, I), 1.0, 91, 3 * r)), dev(synth.uniform((batch, H), -1, 1, 91, 3 * r + 1)),
+                      None if gru else dev(synth.uniform((batch, H), -1, 1, 91, 3 * r + 2))))
+    run = lambda call, w: amq.selftest_batched_sequence(Wcodes, Walpha, None, I, H, *call, ka, 2, w, 2)
+    got = [run(call, ws) for call in calls]
+    assert amq.workspace_status(ws) == 0
+    for call, g in zip(calls, got):
+        fresh = amq.new_workspace(I, H, batch, ka)
+        want = run(call, fresh)
+        assert amq.workspace_status(fresh) == 0
+        assert all(torch.equal(a, b) for a, b in zip(g, want) if a is not None)
+
+
+@pytest.mark.parametrize("cell,kw,ka,steps", [("lstm", 2, 2, 13), ("lstm", 3, 3, 24), ("gru", 2, 3, 17)])
+def test_host_chunks_of_two_steps_do_not_read_each_others_words(amq, cell, kw, ka, steps):
+    """From 13 to 24 timesteps the first chunk of a host call is a launch of two steps: it leaves words of timestep 1, which the second chunk's
+    launch, on the same counters, looks for as well.  The host call equals the device call bit for bit."""
+    I = H = 1024
+    batch, gru = 96, cell == "gru"                              # 5 MB and more of inputs: copied in chunks
+    assert amq.selftest_sequence_plan(gru, I, H, kw, ka, batch)[0] == 2
+    Wcodes, Walpha = amq.quantize(dev(synth.normal(((3 if gru else 4) * H, I + H), 0.05, 92, 1)), kw, 2)
+    ws, staging = amq.new_workspace(I, H, batch, ka), amq.new_host_staging(I, H, batch, steps)
+    for seed in (2, 12, 22):
+        xs = torch.from_numpy(synth.normal((steps, batch, I), 1.0, 92, seed)).pin_memory()
+        h0, c0 = (torch.from_numpy(synth.uniform((batch, H), -1, 1, 92, seed + i)).pin_memory() for i in (1, 2))
+        h, c, seq = torch.empty_like(h0).pin_memory(), torch.empty_like(c0).pin_memory(), torch.empty((steps, batch, H)).pin_memory()
+        if gru:
+            amq.gru_sequence_host(Wcodes, Walpha, None, I, H, xs, h0, ka, 2, ws, staging, h, h_seq=seq)
+            want = amq.gru_sequence(Wcodes, Walpha, None, I, H, xs.cuda(), h0.cuda(), ka, 2, amq.new_workspace(I, H, batch, ka), want_h_seq=True)
+            got = (seq, h)
+        else:
+            amq.lstm_sequence_host(Wcodes, Walpha, None, I, H, xs, h0, c0, ka, 2, ws, staging, h, c, h_seq=seq)
+            want = amq.lstm_sequence(Wcodes, Walpha, None, I, H, xs.cuda(), h0.cuda(), c0.cuda(), ka, 2, amq.new_workspace(I, H, batch, ka), want_h_seq=True)
+            got = (seq, h, c)
+        assert amq.workspace_status(ws) == 0
+        assert all(torch.equal(g, w.cpu()) for g, w in zip(got, want))
 
 
 @pytest.mark.parametrize("late", [1, 2])
