@@ -412,8 +412,8 @@ AMQ_API amq_status amq_selftest_sequence_give_up(const uint32_t* Wcodes, const f
  * counters of the one-launch forms start as `counted` (0 .. 2^31 - 1 - steps) earlier timesteps would have left them.  Results are
  * those of the ordinary call in that form, whatever `counted` is.  AMQ_ERR_UNSUPPORTED where the form does not take the problem.
  *   late = 1, 2 or 3 (one-launch forms, counted = 0; 0: none): the CTAs look for the counts of quantized vectors (from step 0 on) or of finished
- *   products (from step 1 on: steps >= 2) where none of them counts; late = 3 (AMQ_FORM_RESIDENT): they look for states of a timestep that
- *   is not computed (from step 1 on).  Every wait runs out (a second or two: the ordinary limit),
+ *   products (from step 1 on: steps >= 2) where none of them counts; late = 3 (AMQ_FORM_RESIDENT, where the states travel as
+ *   words, AMQ_ERR_UNSUPPORTED elsewhere): they look for states of a timestep that is not computed (from step 1 on).  Every wait runs out (a second or two: the ordinary limit),
  *   every CTA records that in the workspace status word, gives its tensor memory back and returns; h_last and c_last are left unwritten.
  */
 #define AMQ_FORM_CHAIN 0

@@ -147,7 +147,7 @@ rnn_batched_kernel(const __grid_constant__ SeqParams a)
             const int b = b0 + res_row_vector<KA>(tid), j = res_row_plane<KA>(tid);
             sh.beta[tid] = tid < p.TB * KA && b < p.batch ? __ldcg(a.z.zbeta + (size_t)b * KA + j) : 0.0f;
         }
-        res_expand_activations<KA, 2>(p, a.z.zcodes, 1, (size_t)p.batch * KA, b0, sB);
+        res_expand_activations<KA, 2>(p, a.z.zcodes, a.z.row_bytes >> 4, a.z.half_bytes >> 4, b0, sB);
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");

@@ -42,6 +42,7 @@ struct RsParams {
     const float* x_seq; const float* h0; const float* c0;
     float* h_seq; float* h_last; float* c_last;
     unsigned long long* hx;     // [batch][H]: {h value, timestep}, from CTA to CTA
+    float* h[2];                // the states where there are no words and no h_seq
     const float* addend;        // [steps][batch][4H] added before the gates, or null
     uint32_t* counters;         // [blocks][64]: word 0 quantized shares, word 32 finished products
     int planes_word, h_word;    // where a block's CTAs look for them: 0 and 32 (the self-test of the waits: the next word, which stays 0)
@@ -188,7 +189,8 @@ __device__ __forceinline__ void rs_unit_sums(const float* folded, const float* a
     }
 }
 
-template <int KA, int NW>
+// WORDS: h travels as words, otherwise in memory behind a counter (two kernels: the one without the words' code is the smaller).
+template <int KA, int NW, bool WORDS>
 __global__ void __launch_bounds__(RS_THREADS, 1)
 rnn_resident_kernel(const __grid_constant__ RsParams a)
 {
@@ -260,15 +262,19 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
 
         // ---- 1. this CTA's share of the block's vectors ----
         if (part < quantizers) {                    // (uniform over the CTA)
-            if (t == 1) {                           // (the words of another call are gone)
-                if (tid == 0) ok = seq_wait(counter + a.h_word, seq_target(a.launched + 1, a.P));
+            if (WORDS ? t == 1 : t > 0) {           // (words: those of another call are gone)
+                if (tid == 0) ok = seq_wait(counter + a.h_word, seq_target(WORDS ? a.launched + 1 : a.counted + t, a.P));
                 if (__syncthreads_or(!ok)) { ok = false; break; }
             }
             const float* x = a.x_seq + (size_t)t * a.batch * a.z.xn;
+            const float* h_prev = t == 0 || WORDS ? a.h0 : (a.h_seq ? a.h_seq + (size_t)(t - 1) * a.batch * H : a.h[(t - 1) & 1]);
 #pragma unroll 1
             for (int v = part + warp / NW * a.P; v < in_block; v += RS_WARPS / NW * a.P) {
-                ok &= seq_quantize<KA, 8, NW>(a.z, x, a.h0, b0 + v, scratch[warp / NW], quant, quant_parity,
-                                              RsWords{t == 0 ? nullptr : a.hx, (uint32_t)t + a.tag_bias, ok ? SEQ_POLL_LIMIT : 1u});
+                if constexpr (WORDS)
+                    ok &= seq_quantize<KA, 8, NW, true>(a.z, x, h_prev, b0 + v, scratch[warp / NW], quant, quant_parity,
+                                                  RsWords{t == 0 ? nullptr : a.hx, (uint32_t)t + a.tag_bias, ok ? SEQ_POLL_LIMIT : 1u});
+                else
+                    seq_quantize<KA, 8, NW, false>(a.z, x, h_prev, b0 + v, scratch[warp / NW], quant, quant_parity);
                 // the next timestep's inputs on their way into L2
                 const int e = (quant.warp * 32 + lane) * 8;
                 if (!last && e < a.z.xn)
@@ -436,13 +442,14 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
                     *state = h;
                 }
                 if (last) a.h_last[o] = h;
-                else rs_store_word(a.hx + o, h, (uint32_t)t + 1);
+                else if (WORDS) rs_store_word(a.hx + o, h, (uint32_t)t + 1);
+                else if (!h_seq) a.h[t & 1][o] = h;
                 if (h_seq) h_seq[o] = h;
             }
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         if (__syncthreads_or(!ok)) { ok = false; break; }
-        if (t == 0 && tid == 0) seq_publish(counter + 32);
+        if (tid == 0 && (t == 0 || !WORDS)) seq_publish(counter + 32);
     }
 
     __syncwarp();
@@ -457,7 +464,7 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(sh.tmem_slot), "r"((uint32_t)RS_TMEM_COLS) : "memory");
 }
 
-struct RsPlan { RsParams a; int grid, warps; size_t smem; double clocks; };
+struct RsPlan { RsParams a; int grid, warps; bool words; size_t smem; double clocks; };
 
 // Estimated clocks of a timestep: quantizer rounds (by activation bits and warps per vector), per pass over the weights the tensor pipe, the
 // expansion of the activations, the folding and the gates, and the waits.  Fitted to 383 problems (LSTM and GRU, 1 to 4 bits, 2 to
@@ -518,7 +525,15 @@ bool plan(const BatchedSequence& s, int sms, int only, RsPlan* out)
     a.z = SeqVectors{s.n, words_per_row(s.n), s.H, s.n - s.H, s.T, s.zcodes, s.zbeta, 16, (size_t)s.batch * s.k_a * 16};
     a.I = s.I; a.k_w = s.k_w; a.gru = s.gru; a.steps = s.steps; a.batch = s.batch;
     a.x_seq = s.x_seq; a.h0 = s.h0; a.c0 = s.c0; a.h_seq = s.h_seq; a.h_last = s.h_last; a.c_last = s.c_last;
-    a.hx = reinterpret_cast<unsigned long long*>(s.h[0]);       // (the two states of the other forms, one behind the other)
+    // Words where a team of warps quantizes one vector a timestep: the time from a CTA's h to the planes made of it is what counts there.  Where it
+    // takes several in turn, twice the bytes and a look at every word count more; a single timestep has no words to look at.  Eight timesteps,
+    // words against none: 58 problems of one vector a team 0.94 to 1.01 of the time (LSTM 512/1024, 21 sequences, 3/3 bits 94 us against 97), 51 of
+    // 2 to 35 vectors 1.00 to 1.17 (GRU 128/128, 3530 sequences, 2/2 bits 217 us against 187; LSTM 1919/185, 1297 sequences, 2/3 bits 527 against 485).
+    const int teams = RS_WARPS / p.warps, vectors = (a.block + a.P - 1) / a.P;
+    p.words = s.steps > 1 && vectors <= teams;
+    if (s.late == 3 && !p.words) return false;
+    a.hx = reinterpret_cast<unsigned long long*>(s.h[0]);       // (the two states, one behind the other)
+    a.h[0] = s.h[0]; a.h[1] = s.h[1];
     a.launched = s.launched; a.tag_bias = s.late == 3 ? 1u << 30 : 0u;
     a.addend = s.addend; a.counters = s.counters; a.counted = s.counted; a.status = s.status;
     a.planes_word = s.late == 1 ? 1 : 0; a.h_word = s.late == 2 ? 33 : 32;
@@ -529,7 +544,7 @@ bool plan(const BatchedSequence& s, int sms, int only, RsPlan* out)
 template <int KA, int NW>
 amq_status launch(const RsPlan& pl, cudaStream_t st)
 {
-    auto kernel = rnn_resident_kernel<KA, NW>;
+    auto kernel = pl.words ? rnn_resident_kernel<KA, NW, true> : rnn_resident_kernel<KA, NW, false>;
     AMQ_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem));
     RsParams args = pl.a;
     void* params[] = {&args};

@@ -125,10 +125,12 @@ def test_states_that_never_come_set_the_status_and_leave_the_context_usable(amq,
     ("gru", 7, 33, 5, 8, 2, 3),             # odd widths: single words
     ("lstm", 0, 129, 17, 6, 3, 4),          # no inputs at all
     ("lstm", 260, 256, 70, 5, 2, 2),        # a pair of words across x and h never
-    ("gru", 129, 127, 300, 4, 2, 2),        # several vectors per team, several passes
+    ("gru", 129, 127, 300, 4, 2, 2),        # several vectors per team, several passes: states in memory, behind a counter
+    ("lstm", 33, 65, 1000, 3, 2, 3), ("gru", 64, 128, 700, 4, 2, 2),
 ])
 def test_states_travel_as_words_at_every_width(amq, cell, I, H, batch, steps, kw, ka):
-    """One launch and launches of one step each (which read their state from memory, not from words): the same steps, twice on one workspace."""
+    """One launch and launches of one step each (which read their state from memory): the same steps, twice on one workspace, by words and, where
+    a team quantizes several vectors, without."""
     gru = cell == "gru"
     Wcodes, Walpha = amq.quantize(dev(synth.normal(((3 if gru else 4) * H, I + H), 0.08, 89, 1)), kw, 2)
     ws = amq.new_workspace(I, H, batch, ka)
@@ -231,6 +233,11 @@ def test_give_up_selftest_rejects_what_it_cannot_run(amq):
             amq.selftest_batched_sequence(Wcodes, Walpha, None, I, H, torch.zeros((steps, 9, I), device="cuda"), h1, h1.clone(), ka, 2,
                                           amq.new_workspace(I, H, 9, ka), form, counted, late)
         assert e.value.status == -1
+    with pytest.raises(amq.AmqError) as e:      # no words: nothing of the kind to look for
+        h = torch.zeros((700, H), device="cuda")
+        amq.selftest_batched_sequence(Wcodes, Walpha, None, I, H, torch.zeros((3, 700, I), device="cuda"), h, h.clone(), ka, 2,
+                                      amq.new_workspace(I, H, 700, ka), 2, 0, 3)
+    assert e.value.status == -2
     with pytest.raises(amq.AmqError) as e:      # a single step waits for nothing: refused
         amq.selftest_sequence_give_up(Wcodes, Walpha, None, I, H, xs[:1], h0, h0.clone(), ka, 2, ws, 100)
     assert e.value.status == -1
