@@ -5,7 +5,7 @@
 // What bounds it: per tile of 128 rows (32768 x 1024, 512 vectors, 3/2 bits: some 5500 clocks, 3080 of them the tensor pipe's) the chain
 // commit - poll - barrier - read - release of every accumulator, and the issue slots that the roles share with the warp that issues the
 // MMAs.  That product took 59.8 us with a constant of every operand row added back in the epilogue (twice the instructions, and its
-// loads kept the load/store unit busy) and the polling warp on the issuing warp's scheduler; 53.5 us now.  Outputs leave through shared
+// loads kept the load/store unit busy) and the polling warp on the issuing warp's scheduler; 52.5 us now (behind a flush of L2 65.6 and 59.4).  Outputs leave through shared
 // memory as 16-byte pieces.
 #include "amq_resident.cuh"
 
@@ -129,7 +129,7 @@ bgemm_resident_kernel(const __grid_constant__ ResGemmParams a)
         };
         grid_dependency_wait();
         while (w < w_end) {
-            const int bb = (int)(w / a.mtiles), b0 = bb * p.TB, tile0 = (int)(w % a.mtiles), tiles = pass_tiles(w);
+            const int bb = (int)(w / a.mtiles), tile0 = (int)(w % a.mtiles), tiles = pass_tiles(w);
             float next_alpha = alpha_of(tile0);
             load_block(bb);
             f32x2 beta[NG][KA];

@@ -465,12 +465,11 @@ struct SignWord {
 // midpoint it compares with (the midpoints of the lower half are the negatives of the upper ones, `thr`).  SUMS: also csum[i] = sum of
 // b_i w, for which an element's own midpoints are chosen; without them every decision of a level is gathered as a word of bits and the
 // words are chosen from, which takes fewer instructions.
-template <int K, int EPT, bool SUMS>
-__device__ __forceinline__ void ascending_pass(const float (&w)[EPT], const f32x2 (&w2)[EPT / 2], const float (&thr)[(1 << K) - 1],
-                                               uint32_t positive, float abs_w, uint32_t valid, uint32_t (&bits)[K], float (&csum)[K])
+template <int EPT, bool SUMS>
+__device__ __forceinline__ void ascending_pass(const float (&w)[EPT], const f32x2 (&w2)[EPT / 2], const float (&thr)[7],
+                                               uint32_t positive, float abs_w, uint32_t valid, uint32_t (&bits)[3], float (&csum)[3])
 {
-    static_assert(K == 3, "");
-    constexpr int M2 = 1 << (K - 1);
+    constexpr int K = 3, M2 = 4;
     const float t1 = thr[M2 - 1 + M2 / 2], t2o = thr[M2 - 1 + M2 / 2 + M2 / 4], t2i = thr[M2 - 1 + M2 / 4];
     bits[0] = positive & valid;
     csum[0] = abs_w;
@@ -834,8 +833,8 @@ __device__ __forceinline__ void quantize_warp(const float (&w_in)[EPT], uint32_t
         } else {
             float thr[(1 << K) - 1];
             if (ascending_levels<K>(alpha, thr)) {
-                if (more) ascending_pass<K, EPT, true>(w, w2, thr, positive, abs_w, valid, bits, csum);
-                else ascending_pass<K, EPT, false>(w, w2, thr, positive, abs_w, valid, bits, csum);
+                if (more) ascending_pass<EPT, true>(w, w2, thr, positive, abs_w, valid, bits, csum);
+                else ascending_pass<EPT, false>(w, w2, thr, positive, abs_w, valid, bits, csum);
             } else {
                 three_bit_codes<EPT>(w, alpha, positive, abs_w, valid, more, thr, bits, csum);
             }

@@ -243,7 +243,8 @@ size_t seq_more_smem(const ResProblem& p)
 }
 
 // Estimated clocks of a timestep: quantizer rounds (by activation bits), steps and epilogues of a CTA's blocks of units, expansion of the
-// activations, waits.  Fitted to 415 problems (LSTM and GRU, 1 to 4 bits, 2 to 5000 sequences, widths 64 to 2048) on a B200, within 6 %
+// activations, waits.  Fitted to 415 problems (LSTM and GRU, 1 to 4 bits, 2 to 5000 sequences, widths 64 to 2048) on a B200 when the planes lay
+// row by row and the epilogue added a constant per operand row, within 6 %
 // (standard deviation; 19 % at worst).
 double streaming_clocks(const ResProblem& p, int k_a, int P, int unit_blocks, int unit_steps, int team_warps)
 {
@@ -343,18 +344,19 @@ amq_status launch_streaming_sequence(const BatchedSequence& s, const SequenceSha
 SequenceForm batched_sequence_form(const BatchedSequence& s, int sms, SequenceShape* out)
 {
     // The least estimated time.  The weights are worth keeping in tensor memory while the vectors of a block need few passes over them: 35
-    // timesteps of LSTM 1024/1024, 64 sequences, 3/3 bits take 394 us resident, 517 streamed; of GRU 1900/1900, 256 sequences, 2/3 bits
-    // (52 passes of five vectors) 7301 us resident, 1486 streamed.  Over 420 problems the choice costs 0.2 % on average against the
-    // best form of each, 12 % at worst (always the resident form: 8 %, and five times the time at worst).
+    // timesteps of LSTM 1024/1024, 64 sequences, 3/3 bits take 400 us resident, 482 streamed; of GRU 1900/1900, 256 sequences, 2/3 bits
+    // (52 passes of five vectors) 7268 us resident, 1264 streamed.  Over 122 problems (2 to 5000 sequences) the choice costs 0.3 % on
+    // average against the best form of each, 9 % at worst (always the resident form: 19 %, and six times the time at worst).
     if (sms < 1) sms = res_sm_count();
     SequenceShape shape;
     SequenceForm form = SEQ_CHAIN;
     double best = 0.0;
     if (resident_sequence_shape(s, sms, &shape)) { form = SEQ_RESIDENT; best = shape.clocks; *out = shape; }
     if (streaming_sequence_shape(s, sms, &shape) && (best == 0.0 || shape.clocks < best)) { form = SEQ_STREAMING; best = shape.clocks; *out = shape; }
-    // From eight tiles of 256 operand rows on the product of the chain fills the machine for longer than its launches take (GRU 1024/1024,
-    // 4096 sequences, 2/3 bits: 6976 us, streamed 7274, resident 10877); below, a one-launch form was at most 12 % behind it, and up
-    // to 27 times faster where the chain's product has to run on the CUDA cores.
+    // From eight tiles of 256 operand rows on the product of the chain fills the machine for longer than its launches take (LSTM 2048/2048,
+    // 2048 sequences, 2/2 bits: 6915 us, streamed 7669; GRU 1024/1024, 4096 sequences, 2/3 bits: 6991, streamed 7045, resident 10915);
+    // below, none of 69 problems was faster as a chain by more than 0.3 %, and where its product has to run on the CUDA cores it takes up to
+    // 12 times as long.
     if (best > 0.0 && (long long)s.batch * s.k_a >= 2048) {
         const double chain = chain_clocks(s, sms);
         if (chain > 0.0 && chain < best) form = SEQ_CHAIN;

@@ -17,8 +17,9 @@
 // which add nothing, so the activation operand needs no masks and no split.
 //
 // Measured (clocks of a timestep, 64 vectors, 1024 units, n = 2048, 3 bits; 147 CTAs, 368 us for 35 timesteps): words of h and quantizer 7050,
-// publish 1650, wait for planes 1500, their loads 1700, expansion 2400, rest of the MMAs 2250, folding 1850, gates 1850.  (With h in
-// memory behind a counter 394 us: wait for h 1150, publish 1050 more; streamed weights 508 us.)
+// publish 1650, wait for planes 1500, their loads 1700, expansion 2400, rest of the MMAs 2250, folding 1850, gates 1850.  (374 us and some 200
+// clocks more in the quantizer since it asks whether levels tie; with h in memory behind a counter 394 us: wait for h 1150, publish
+// 1050 more; streamed weights 482 us.)
 //
 // More vectors than one accumulator (N <= 256 operand rows) or shared memory holds are taken in passes over the same weights.
 #include "amq_sequence.cuh"
@@ -467,7 +468,7 @@ rnn_resident_kernel(const __grid_constant__ RsParams a)
 struct RsPlan { RsParams a; int grid, warps; bool words; size_t smem; double clocks; };
 
 // Estimated clocks of a timestep: quantizer rounds (by activation bits and warps per vector), per pass over the weights the tensor pipe, the
-// expansion of the activations, the folding and the gates, and the waits.  Fitted to 383 problems (LSTM and GRU, 1 to 4 bits, 2 to
+// expansion of the activations, the folding and the gates, and the waits.  Fitted, with h in memory behind a counter, to 383 problems (LSTM and GRU, 1 to 4 bits, 2 to
 // 5000 sequences, widths 64 to 2048) on a B200, within 6 % (standard deviation; 17 % at worst).
 double resident_clocks(int k_a, int warps, int block, int P, int TB, int N, int NS, int tiles, int upc)
 {

@@ -25,13 +25,11 @@ def dev(a):
 PROBLEMS = [(60, 130, 16, 2, 2), (2000, 300, 64, 2, 2), (5000, 1024, 96, 3, 3), (9999, 650, 200, 2, 2), (20000, 1024, 256, 4, 4), (300, 257, 2, 1, 2)]
 
 
-@pytest.mark.parametrize("m,n,batch,kw,ka", PROBLEMS)
-@pytest.mark.parametrize("form", [None, 1, 2])
+# (forms 1 and 2, the tensor-core kernels, start at 16 vectors here)
+@pytest.mark.parametrize("m,n,batch,kw,ka,form", [p + (f,) for p in PROBLEMS for f in (None, 1, 2) if f is None or p[2] >= 16])
 def test_products_wait_for_the_kernel_in_front(amq, m, n, batch, kw, ka, form):
     """The weights, the activations and the bias change between products that follow one another on the stream, written by this library's
     quantizer and by foreign kernels in turn; every product leaves the bits of one that had the GPU to itself."""
-    if form is not None and batch < 16:
-        pytest.skip("the tensor-core kernels start at 16 vectors here")
     product = lambda *a, **k: amq.binary_gemm(*a, **k) if form is None else amq.selftest_binary_gemm(*a, form, **k)
     w = [dev(synth.normal((m, n), 0.03, 600 + m, i)) for i in range(2)]
     x = [dev(synth.normal((batch, n), 1.0, 600 + m, 2 + i)) for i in range(2)]
