@@ -288,3 +288,46 @@ def test_one_sequence_lstm_at_the_edges_of_its_groups_of_chunks(amq, n, kw, ka):
     tol = 3e-3 * np.abs(Wa).sum(axis=1).max() * np.abs(beta).sum()
     for g, w in zip(got, want):
         assert np.abs(g.cpu().numpy() - w).max() <= tol
+
+
+@pytest.mark.parametrize("cell,I,H,batch", [
+    ("lstm", 96, 40, 1), ("gru", 128, 64, 1), ("lstm", 700, 900, 1),                # one sequence: teams of four and eight warps, sixteen elements a thread
+    ("lstm", 96, 40, 9), ("gru", 260, 252, 20), ("lstm", 500, 900, 33),             # the three forms of a batch
+])
+def test_steps_on_vectors_whose_levels_tie(amq, cell, I, H, batch):
+    """[x ; h] of as many +-1 as +-3: coefficients (2, 1, 0) at three bits, levels that tie in pairs, a table that is sorted inside the recurrent
+    kernels too, and an exact reconstruction whichever of a pair is taken, so that the step is the textbook one on [x ; h] itself.  Tolerance: the
+    pre-activations are sums of n terms of up to 3 |w| in fp32, some 1e-6 of their absolute sum; gates have slopes up to 1, c up to 3."""
+    n, gates = I + H, 4 if cell == "lstm" else 3
+    Wc, Wa = quantized((gates * H, n), 0.05, 2, 900 + n, 1)
+    W = np.einsum("rk,rkn->rn", Wa, parity.unpack_rows(Wc, n).astype(np.float64))
+    bias = synth.normal((4 * H,), 0.1, 900 + n, 2)
+    z = np.empty((batch, n))
+    for b in range(batch):
+        order = np.argsort(synth.uniform((n,), 0, 1, 900 + n, 10 + b))
+        z[b, order] = np.tile([1.0, -1.0, 3.0, -3.0], n // 4)
+    x, h = dev(z[None, :, :I]), dev(z[:, I:])
+    c = synth.uniform((batch, H), -1, 1, 900 + n, 3)
+    sig = lambda v: 1.0 / (1.0 + np.exp(-v))
+    if cell == "lstm":
+        i, f, o, g = (z @ W.T + bias).reshape(batch, 4, H).transpose(1, 0, 2)
+        c_ref = sig(f) * c + sig(i) * np.tanh(g)
+        want = (sig(o) * np.tanh(c_ref), c_ref)
+    else:
+        pre, b4 = (z @ W.T).reshape(batch, 3, H), bias.reshape(4, H)
+        nx, nh = z[:, :I] @ W[2 * H:, :I].T, z[:, I:] @ W[2 * H:, I:].T
+        r, u = sig(pre[:, 0] + b4[0]), sig(pre[:, 1] + b4[1])
+        want = ((1 - u) * np.tanh(nx + b4[2] + r * (nh + b4[3])) + u * z[:, I:],)
+    tol = 4e-6 * 3 * (np.abs(z) @ np.abs(W).T).max() + 1e-5
+    Wd = (cdev(Wc), dev(Wa), dev(bias), I, H)
+    ws = amq.new_workspace(I, H, batch, 3)
+    results = []
+    if batch == 1:
+        results.append(amq.lstm_step(*Wd, x[0], h, dev(c), 3, 2, ws) if cell == "lstm" else (amq.gru_step(*Wd, x[0], h, 3, 2, ws),))
+    else:
+        for form in (0, 1, 2):
+            results.append(amq.selftest_batched_sequence(*Wd, x, h, dev(c) if cell == "lstm" else None, 3, 2, ws, form)[1:])
+    assert amq.workspace_status(ws) == 0
+    for got in results:
+        for g, w in zip(got, want):
+            assert np.abs(g.cpu().numpy() - w).max() <= tol
